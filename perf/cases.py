@@ -323,3 +323,88 @@ def tolerance(c):
     if kind == "verify" and c["n_q"] * c["group"] > 32:
         return {"rel": 1.5e-3, "max": 8e-3}
     return {"rel": 3.2e-5, "max": 2.5e-4}
+
+
+# ------------------------------------------------------------------------------------------------ 64-bit results
+def _dequantised(p, full):
+    """Values float64 [blocks][heads][block][128] of quantised planes: the 8-bit code, or the middle of the Anchor's
+    bucket of 16 codes."""
+    def nibbles(t):
+        return torch.stack((t & 15, t >> 4), dim=-1).reshape(*t.shape[:-1], D).double()
+    level = nibbles(p.anchor) * 16 + (nibbles(p.residual) if full else 8)
+    return p.meta[..., 1:2].double() + p.meta[..., 0:1].double() * level
+
+
+def _pages(c, s, x_of, table, seq, n):
+    """The first n tokens of a sequence, [heads][n][128], from the blocks of its table."""
+    ids = table[seq, :(n + c["block"] - 1) // c["block"]].long()
+    return x_of(ids).permute(1, 0, 2, 3).reshape(c["heads"], -1, D)[:, :n]
+
+
+def _attend(c, s, parts):
+    """Softmax attention over the concatenation of key sets; a part is (K of block ids, V of block ids, table, lengths,
+    causal).  float64 [sequences][n_q][query heads][128]."""
+    q = s["q"].double()
+    B, n_q = q.shape[:2]
+    out = torch.empty(q.shape, dtype=torch.float64, device=q.device)
+    scale = float(torch.tensor(1.0 / math.sqrt(D), dtype=torch.float32))
+    for b in range(B):
+        qb = q[b].permute(1, 0, 2).reshape(c["heads"], c["group"] * n_q, D)     # rows: query head of the group, position
+        scores, values = [], []
+        for k_of, v_of, table, lens, causal in parts:
+            n = lens[b]
+            sc = qb @ _pages(c, s, k_of, table, b, n).transpose(1, 2) * scale
+            if causal:
+                last = n - n_q + torch.arange(n_q, device=q.device).repeat(c["group"])
+                sc.masked_fill_(torch.arange(n, device=q.device) > last[:, None], -math.inf)
+            scores.append(sc)
+            values.append(_pages(c, s, v_of, table, b, n))
+        o = torch.softmax(torch.cat(scores, 2), 2).nan_to_num_(0.0) @ torch.cat(values, 1)
+        out[b] = o.reshape(c["heads"] * c["group"], n_q, D).permute(1, 0, 2)
+    return out
+
+
+def _algorithm1(x):
+    """Algorithm 1 of pages [n][256][128] and its inverse: metadata and reconstruction (its packed codes left out)."""
+    x = x.double()
+    n, eps, log_a = x.shape[0], 1e-6, math.log(256.0)
+    g_min = x.amin(1)
+    g_scale = x.amax(1) - g_min
+    xv = ((x - g_min[:, None]) / (g_scale[:, None] + eps)).view(n, 8, 32, D)
+    mu = xv.mean(2)
+    cent = xv - mu[:, :, None]
+    sigma = cent.abs().amax(2)
+    raw = torch.round(torch.log1p(255.0 * (cent / (sigma[:, :, None] + eps)).abs()) / log_a * 120.0)
+    mag = torch.expm1(raw / 120.0 * log_a) / 255.0
+    back = torch.where(cent < 0, -mag, mag) * (sigma[:, :, None] + eps) + mu[:, :, None]
+    return [None, None, g_min, g_scale, mu, sigma, back.view(n, PAGE, D) * (g_scale[:, None] + eps) + g_min[:, None]]
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits; None for the integer planes of the quantiser, the codes of Algorithm 1 and the
+    index of the first rejected position."""
+    c = case
+    kind = c["kind"]
+    if kind in ("quantize", "quantize_blocks"):
+        return None
+    s = prepare(case, seed)
+    if kind == "algorithm1":
+        return [t for src in s["src"] for t in _algorithm1(src)]
+    lens = _lens(c) * c["layers"]
+
+    def rows(p, full):
+        return lambda ids: _dequantised(lynx.Planes(p.anchor[ids], p.residual[ids], p.meta[ids]), full)
+    if kind == "pages":
+        k, v = _dequantised(s["K"], True), _dequantised(s["V"], True)
+        kb, vb = k.float().to(torch.bfloat16), v.float().to(torch.bfloat16)
+        return k, v, _attend(c, s, [(lambda i: kb[i].double(), lambda i: vb[i].double(), s["table"], lens, c["causal"])])
+    full = kind == "verify"
+    planes = (rows(s["K"], full), rows(s["V"], full), s["table"], lens, c["causal"] and kind != "decode_tail")
+    if kind == "decode":
+        return _attend(c, s, [planes])
+    if kind == "decode_tail":
+        return _attend(c, s, [planes, (lambda i: s["tail_k"][i].double(), lambda i: s["tail_v"][i].double(),
+                                       s["tail_table"], _tail_lens(c), c["causal"])])
+    out = _attend(c, s, [planes])
+    dev = ((out - s["draft"].double()).abs() / (0.5 + 0.1 * out.abs())).amax((2, 3))
+    return out, None, dev

@@ -1,7 +1,7 @@
 // lynx_anchor_attention and lynx_merge_verify_attention: split-K decode attention over the
 // packed nibble planes, dequantised on chip (sm_100a).  This file holds what the kernels share
 // (parameters, PTX helpers, the end-of-piece merge and the accept / reject decision) and the host
-// side; the kernels are in attention_i8.cuh and attention_wide.cuh.
+// side; the kernels are in attention_i8.cuh and attention_f16.cuh.
 //
 // What is computed (Section 2 attention equation on the states of Section 4.2; accept/reject
 // of Section 4.3): for every (sequence, KV head) the G = Hq/Hkv query heads of each of the n_q
@@ -11,10 +11,9 @@
 //     q . K^_t        = scale_t * (q . level_t) + zero_t * sum_d q_d
 //     sum_t p_t V^_t  = sum_t (p_t scale_t) level_t + (sum_t p_t zero_t) * 1
 // so the two contractions run on the integer levels and the scalars are applied per token
-// outside.  Anchor attention (any column count) and verification with up to 16 columns per launch
-// (17..32 columns: two such launches) run both contractions as exact integer products on
-// tcgen05.mma kind::i8 (attention_i8.cuh); verification with 33..64 columns per launch runs them on
-// tcgen05.mma kind::f16 with two-term FP16 weights (attention_wide.cuh).
+// outside.  Anchor attention (any column count) and verification with up to 16 columns per launch run both contractions as exact integer products on
+// tcgen05.mma kind::i8 (attention_i8.cuh); verification with 17..64 columns per launch runs them on
+// tcgen05.mma kind::f16 with two-term FP16 weights (attention_f16.cuh).
 //
 // Common shape.  Persistent grid, one CTA per SM, flash-decoding split-K in stream-K form: the
 // (sequence, KV head, stage-unit) list is cut into equal contiguous ranges, one per CTA.
@@ -54,7 +53,6 @@ struct AttnParams {
   uint32_t* ws_chunk_ctr;  // [B*Hkv]
   uint32_t* ws_seq_ctr;    // [B]
   uint32_t* ws_group_ctr;  // [2 * CTAs of the largest grid]: tickets of the groups of partial slots
-  float* ws_shadow;        // FP32 copies of the O accumulators (see kFlushMmas), or null
   float* ws_dev;           // [B*Hkv][kMaxQ]
   float* ws_lse;           // [B][nq_stride][Hq] natural-log log-sum-exp of every output row's scores
   float* ws_part;          // [B*Hkv + CTAs][ncols_pad][kPartStride], slot = segment + CTA index
@@ -162,36 +160,7 @@ __device__ __forceinline__ uint2 lds64(uint32_t addr) {
   asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
   return v;
 }
-__device__ __forceinline__ float2 lds64f(uint32_t addr) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-  return v;
-}
 
-// Packed FP32 pairs (Blackwell fma/add/mul .f32x2: two lanes per instruction).
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 
 // Full codes of 8 elements from an anchor word and a residual word: ev = codes of elements
 // 0,2,4,6 (one per byte), od = codes of elements 1,3,5,7.
@@ -210,7 +179,6 @@ __device__ __forceinline__ void merge_codes(uint32_t xa, uint32_t xr, uint32_t& 
 __device__ __forceinline__ float lse_of(float M, float L) {
   return L > 0.0f ? (M + __log2f(L)) * 0.6931471805599453f : -INFINITY;
 }
-constexpr int kPieceUnits = 64;  // stage-units whose block ids are looked up at a time
 
 struct Item {  // one piece: a run of stage-units of one (sequence, KV head) given to one CTA
   int b, hkv, len, first_cta, n_contrib, pad0, pad1, pad2;  // pad0 = units, pad1 = first unit
@@ -224,7 +192,7 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
 // contributor of the (sequence, KV head) merges the slots, and for verification the CTA holding
 // the final outputs of a head takes part in the accept / reject decision (Section 4.3).
 // Called by all consumer threads of the CTA (named barrier 1).
-template <bool FULL, int kColsPad, int kConsThreads>
+template <bool FULL, int kColsPad, int kConsThreads, int kCols = kColsPad, int kFly = 8, int kMaxCC = 4>   // kCols: the most columns of a launch; kFly: row loads in flight per thread
 __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& item, bool direct, int tid,
                                              int* misc, int bar_id = 1) {
   const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
@@ -237,16 +205,16 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
   const bool decide = FULL && p.draft != nullptr;
   int* devs = misc + 16;
   if (decide && tid < kMaxQ) devs[tid] = 0;   // (free: the previous piece's were read before its last barrier)
-  auto draft_of = [&](int c) {
-    const int j = c / p.G, hh = c % p.G;
-    return __ldg(reinterpret_cast<const float4*>(
-        p.draft + (((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh) * LYNX_D) + lane);
+  // float offset of an output row of this head: column c = position c / G, query head c % G
+  auto row_off = [&](int c) {
+    const int j = c / p.G;
+    return ((uint32_t)(item.b * p.nq_stride + j) * (uint32_t)p.Hq + (uint32_t)(item.hkv * p.G + c - j * p.G));
   };
   auto deviation = [&](const float4& f, const float4& d, int j) {
-    float r = fabsf(f.x - d.x) / (p.atol + p.rtol * fabsf(f.x));
-    r = fmaxf(r, fabsf(f.y - d.y) / (p.atol + p.rtol * fabsf(f.y)));
-    r = fmaxf(r, fabsf(f.z - d.z) / (p.atol + p.rtol * fabsf(f.z)));
-    r = fmaxf(r, fabsf(f.w - d.w) / (p.atol + p.rtol * fabsf(f.w)));
+    const float fv[4] = {f.x, f.y, f.z, f.w}, dv[4] = {d.x, d.y, d.z, d.w};
+    float r = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r = fmaxf(r, fabsf(fv[i] - dv[i]) / (p.atol + p.rtol * fabsf(fv[i])));
     const int m = __reduce_max_sync(0xFFFFFFFFu, __float_as_int(r));   // r >= 0: integer order = float order
     if (lane == 0) atomicMax(devs + j, m);
   };
@@ -257,13 +225,12 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
     // neighbouring contributors merges the group into its first slot; the last group to finish
     // merges the group results into the output.  Every ticket resets itself; nobody waits.
     constexpr int kGroup = 8, kOneLevel = 24;   // up to kOneLevel slots are merged in one go
-    constexpr int kAhead = 6;                    // loads in flight per thread
     const int n = item.n_contrib;
     const int ng = (n + kGroup - 1) / kGroup;
     const int g = ((int)blockIdx.x - item.first_cta) / kGroup;
     const int gsize = min(kGroup, n - g * kGroup);
     float* seg = p.ws_part + (bh + (size_t)item.first_cta) * (size_t)kColsPad * kPartStride;
-    const size_t cstride = (size_t)kColsPad * kPartStride;
+    constexpr uint32_t cstride = kColsPad * kPartStride;   // (a segment has at most 592 slots: offsets fit 32 bits)
     named_bar(bar_id, kConsThreads);
     if (tid == 0) {
       bool last = true;   // of this CTA's group (n <= kOneLevel: of the whole segment)
@@ -285,51 +252,86 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
       __threadfence();
       const int first = top ? 0 : g * kGroup;
       const int count = top ? (n <= kOneLevel ? n : ng) : gsize;
-      const size_t sstride = (top && n > kOneLevel ? (size_t)kGroup : (size_t)1) * cstride;
-      // a warp per column, a lane per 4 dims; `count` slots from `first` on, merged online, kAhead
-      // loads ahead; the result goes to the output (normalised) or back to slot `first`
-      for (int c = tid >> 5; c < p.ncols; c += kConsThreads / 32) {
-        float* col = seg + (size_t)first * cstride + (size_t)c * kPartStride;
-        float M = -INFINITY, L = 0.0f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 dr = decide && top ? draft_of(c) : acc;   // (loaded with the slots)
-        for (int i0 = 0; i0 < count; i0 += kAhead) {
-          float mi[kAhead], li[kAhead];
-          float4 oi[kAhead];
+      const uint32_t sstride = (top && n > kOneLevel ? kGroup : 1) * cstride;
+      // A warp takes kCC columns at a time, a lane 4 dims of each; `count` slots from `first` on (at most 32: a grid has a
+      // CTA per SM); the result goes to the output (normalised) or back to slot `first`.  Lane i first takes the maximum
+      // and the sum of slot i (one load per column), so that the factors of all slots are known and the rows are
+      // independent loads, kFly in flight per thread.  (Column after column, each slot waiting for the one before: 16.5 us
+      // for 18 slots of 32 columns with the decision, 12 us this way.)
+      constexpr int kWarps = kConsThreads / 32, kPerWarp = (kCols + kWarps - 1) / kWarps;
+      constexpr int kCC = kPerWarp < kMaxCC ? kPerWarp : kMaxCC, kSS = kFly / kCC;
+#pragma unroll 1
+      for (int cw = (tid >> 5) * kCC; cw < p.ncols; cw += kWarps * kCC) {
+        float* col = seg + (uint32_t)first * cstride + (uint32_t)(cw * kPartStride);
+        float f[kCC], my_m = 0.0f, my_l = 0.0f;
+        float2 ml[kCC];
 #pragma unroll
-          for (int u = 0; u < kAhead; ++u) {
-            const bool in = i0 + u < count;
-            const float* src = col + (size_t)(in ? i0 + u : i0) * sstride;
-            mi[u] = in ? __ldcg(src + 128) : -INFINITY;
-            li[u] = __ldcg(src + 129);
-            oi[u] = __ldcg(reinterpret_cast<const float4*>(src) + lane);
-          }
-#pragma unroll
-          for (int u = 0; u < kAhead; ++u) {
-            const float Mn = fmaxf(M, mi[u]);
-            // an absent slot (mi = -inf) keeps fa = 1, fb = 0 once M is finite; while M is still
-            // -inf both factors are forced to 0 / taken from the slot without forming inf - inf
-            const float fa = M == -INFINITY ? 0.0f : ex2(M - Mn);
-            const float fb = mi[u] == -INFINITY ? 0.0f : ex2(mi[u] - Mn);
-            acc.x = acc.x * fa + oi[u].x * fb;
-            acc.y = acc.y * fa + oi[u].y * fb;
-            acc.z = acc.z * fa + oi[u].z * fb;
-            acc.w = acc.w * fa + oi[u].w * fb;
-            L = L * fa + li[u] * fb;
-            M = Mn;
-          }
+        for (int c = 0; c < kCC; ++c) {
+          ml[c] = make_float2(-INFINITY, 0.0f);
+          if (lane < count && cw + c < p.ncols)
+            ml[c] = __ldcg(reinterpret_cast<const float2*>(col + ((uint32_t)lane * sstride + (uint32_t)(c * kPartStride + 128))));
         }
-        if (top) {
-          const float inv = L > 0.0f ? 1.0f / L : 0.0f;
-          const int j = c / p.G, hh = c % p.G;
-          const size_t o = (((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh) * LYNX_D;
-          const float4 v = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-          reinterpret_cast<float4*>(p.out + o)[lane] = v;
-          if (decide) deviation(v, dr, j);
-          if (lane == 0) p.ws_lse[((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh] = lse_of(M, L);
-        } else {
-          reinterpret_cast<float4*>(col)[lane] = acc;
-          if (lane == 0) { col[128] = M; col[129] = L; }
+#pragma unroll
+        for (int c = 0; c < kCC; ++c) {
+          float M = ml[c].x;
+#pragma unroll
+          for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
+          f[c] = ml[c].x == -INFINITY ? 0.0f : ex2(ml[c].x - M);
+          float L = f[c] * ml[c].y;
+#pragma unroll
+          for (int off = 16; off >= 1; off >>= 1) L += __shfl_xor_sync(0xFFFFFFFFu, L, off);
+          if (top) f[c] *= L > 0.0f ? 1.0f / L : 0.0f;
+          if (lane == c) { my_m = M; my_l = L; }
+        }
+        float4 acc[kCC];
+#pragma unroll
+        for (int c = 0; c < kCC; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int i0 = 0; i0 < count; i0 += kSS) {
+          float4 oi[kSS][kCC];
+#pragma unroll
+          for (int u = 0; u < kSS; ++u) {
+            const float4* row = reinterpret_cast<const float4*>(col + (uint32_t)min(i0 + u, count - 1) * sstride) + lane;
+#pragma unroll
+            for (int c = 0; c < kCC; ++c)   // (columns beyond the last of the launch: the slots are padded)
+              oi[u][c] = __ldcg(row + c * (kPartStride / 4));
+          }
+#pragma unroll
+          for (int u = 0; u < kSS; ++u)
+#pragma unroll
+            for (int c = 0; c < kCC; ++c) {
+              const float fu = i0 + u < count ? __shfl_sync(0xFFFFFFFFu, f[c], i0 + u) : 0.0f;
+              if (fu != 0.0f) {
+                acc[c].x = fmaf(oi[u][c].x, fu, acc[c].x);
+                acc[c].y = fmaf(oi[u][c].y, fu, acc[c].y);
+                acc[c].z = fmaf(oi[u][c].z, fu, acc[c].z);
+                acc[c].w = fmaf(oi[u][c].w, fu, acc[c].w);
+              }
+            }
+        }
+        // lane c finishes column c's scalars and knows its row; the rows follow one by one (a loop: this code runs once per
+        // head, straight from a cold instruction cache, where unrolling it costs more than it saves)
+        const int my_c = min(cw + lane, p.ncols - 1);
+        const uint32_t my_row = row_off(my_c);
+        const int my_j = my_c / p.G;
+        if (lane < kCC && cw + lane < p.ncols) {
+          if (top) p.ws_lse[my_row] = lse_of(my_m, my_l);
+          else *reinterpret_cast<float2*>(col + (lane * kPartStride + 128)) = make_float2(my_m, my_l);
+        }
+        float4 dr[kCC];
+#pragma unroll
+        for (int c = 0; c < kCC; ++c)
+          if (decide && top)
+            dr[c] = __ldg(reinterpret_cast<const float4*>(p.draft + (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D) + lane);
+#pragma unroll 1
+        for (int c = 0; c < kCC && cw + c < p.ncols; ++c) {
+          float4 a = acc[0], d = dr[0];
+#pragma unroll
+          for (int i = 1; i < kCC; ++i)
+            if (c == i) { a = acc[i]; d = dr[i]; }
+          float* dst = top ? p.out + (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D : col + c * kPartStride;
+          reinterpret_cast<float4*>(dst)[lane] = a;
+          if (decide && top) deviation(a, d, __shfl_sync(0xFFFFFFFFu, my_j, c));
         }
       }
       if (top) {
@@ -350,12 +352,12 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
     named_bar(bar_id, kConsThreads);  // final outputs written; devs zeroed, or complete where slots were merged
     if (final_here) {
       if (direct) {
+#pragma unroll 1
         for (int c = tid >> 5; c < p.ncols; c += kConsThreads / 32) {
-          const int j = c / p.G, hh = c % p.G;
-          const float4 dr = draft_of(c);
-          const float4 f = reinterpret_cast<const float4*>(
-              p.out + (((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh) * LYNX_D)[lane];
-          deviation(f, dr, j);
+          const size_t o = (size_t)row_off(c) * LYNX_D;
+          const float4 dr = __ldg(reinterpret_cast<const float4*>(p.draft + o) + lane);
+          const float4 f = reinterpret_cast<const float4*>(p.out + o)[lane];
+          deviation(f, dr, c / p.G);
         }
         named_bar(bar_id, kConsThreads);
       }
@@ -461,8 +463,33 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
   return r;
 }
 
-#include "attention_wide.cuh"
+// Sequences with no token, by one warp of one CTA each: outputs are zero, nothing is rejected unless the draft is not zero.
+template <bool FULL, class ClampLen>
+__device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, int n_cta, int lane, ClampLen clamp_len) {
+  for (int b = cta; b < p.B; b += n_cta) {
+    if (clamp_len(b) != 0) continue;
+    const size_t n = (size_t)p.nq * p.Hq * LYNX_D;
+    for (size_t i = lane; i < n; i += 32) p.out[(size_t)b * p.nq_stride * p.Hq * LYNX_D + i] = 0.0f;
+    for (int i = lane; i < p.nq * p.Hq; i += 32) p.ws_lse[(size_t)b * p.nq_stride * p.Hq + i] = -INFINITY;
+    if (FULL && p.draft != nullptr) {
+      int fr = p.nq;
+      for (int j = p.nq - 1; j >= 0; --j) {
+        float worst = 0.0f;
+        for (int i = lane; i < p.Hq * LYNX_D; i += 32)
+          worst = fmaxf(worst, fabsf(__ldg(p.draft + ((size_t)b * p.nq_stride + j) * p.Hq * LYNX_D + i)) / p.atol);
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xFFFFFFFFu, worst, off));
+        if (lane == 0) p.dev[(size_t)b * p.nq_stride + j] = worst;
+        if (worst > 1.0f) fr = j;
+      }
+      if (lane == 0) p.first_reject[b] = fr;
+    }
+  }
+}
+
+#include "tc_common.cuh"
 #include "attention_i8.cuh"
+#include "attention_f16.cuh"
 
 // ------------------------------------------------------------------ host side
 constexpr int kMaxCtasPerSm = 4;
@@ -470,9 +497,6 @@ constexpr int kMaxCtasPerSm = 4;
 // Query positions per launch of a verification call: all of them up to kMaxQ positions and kMaxCols
 // columns, else as many whole positions as fit both.
 inline int verify_slice(int nq, int G) {
-  // (17..32 columns: two passes of the exact integer kernel at 16 columns measure as fast as one pass of the
-  // FP16 kernel at 32, without its limits on the value range)
-  if (nq * G > 16 && nq * G <= 32 && 16 / G > 0) return 16 / G;
   if (nq <= kMaxQ && nq * G <= kMaxCols) return nq;
   const int by_cols = kMaxCols / G > 0 ? kMaxCols / G : 1;
   return by_cols < kMaxQ ? by_cols : kMaxQ;
@@ -483,7 +507,6 @@ struct Plan {
   int ncols, variant;  // variant: 0: NT1 TW4 CG1; 1: NT2 TW4 CG1; 2: NT2 TW4 CG2; 3: NT2 TW2 CG4
   int cols_pad;
   size_t off_chunk_ctr, off_seq_ctr, off_group_ctr, off_dev, off_lse, off_part, bytes;
-  size_t shadow_bytes;   // optional tail of the workspace: FP32 copies of the accumulators (see kFlushMmas)
 };
 
 bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
@@ -518,9 +541,6 @@ bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
   pl->off_part = off;
   off += ((size_t)B * s->num_kv_heads + (size_t)sm_count() * kMaxCtasPerSm) * pl->cols_pad * kPartStride * 4;
   pl->bytes = (off + 255) & ~(size_t)255;
-  // FP32 copies of the accumulators of the FP16 kernel (verification with 33..64 columns per launch):
-  // 2 groups x 128 rows x 128 dims per CTA
-  pl->shadow_bytes = ncols > 32 ? (size_t)sm_count() * 131072 : 0;
   return true;
 }
 
@@ -582,11 +602,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
       !aligned16(V.meta) || !aligned16(workspace) || !aligned16(out) ||
       (full && (!aligned16(K.residual) || !aligned16(V.residual))))
     return LYNX_ERR_ALIGN;
-  // the FP16 kernels cut their accumulation chains into FP32 copies at the end of the workspace; the
-  // fixed-scratch entry point has no room for them and says so in its contract
-  const bool fp16_kernel = full && pl.ncols > 32;   // (pl.ncols: the columns of the widest launch)
-  const bool use_shadow = fp16_kernel && !fixed_scratch;
-  if (workspace_bytes < pl.bytes + (use_shadow ? pl.shadow_bytes : 0)) return LYNX_ERR_WORKSPACE;
+  if (workspace_bytes < pl.bytes) return LYNX_ERR_WORKSPACE;
   if (full && draft && !(atol > 0.0f && rtol >= 0.0f)) return LYNX_ERR_SHAPE;
 
   unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -600,7 +616,6 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.ws_chunk_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_chunk_ctr);
   p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_seq_ctr);
   p.ws_group_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_group_ctr);
-  p.ws_shadow = use_shadow ? reinterpret_cast<float*>(ws + pl.bytes) : nullptr;
   p.ws_dev = reinterpret_cast<float*>(ws + pl.off_dev);
   p.ws_lse = reinterpret_cast<float*>(ws + pl.off_lse);
   p.ws_part = reinterpret_cast<float*>(ws + pl.off_part);
@@ -633,7 +648,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     }
     return LYNX_OK;
   }
-  // verification: the integer kernels up to 16 columns, tcgen05 with FP16 operands (attention_wide.cuh) above.
+  // verification: the integer kernels up to 16 columns, tcgen05 with FP16 operands (attention_f16.cuh) above (one layer of
+  // 131072 tokens, 32 columns: 93 us by the FP16 kernel, 174 us as two passes of the integer kernel at 16).
   // A window of more than kMaxQ positions or kMaxCols columns runs as slices of whole positions, each a pass
   // of its own over the planes that writes its outputs and deviations; the index of the first rejected
   // position over the whole window then follows from the deviations.
@@ -647,7 +663,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     ps.ws_lse = p.ws_lse + (size_t)j0 * p.Hq;
     if (p.draft) { ps.draft = p.draft + (size_t)j0 * p.Hq * LYNX_D; ps.dev = p.dev + j0; }
     const lynx_status rc = ps.ncols <= 4 ? launch_i8<true, 4>(ps, st) : ps.ncols <= 8 ? launch_i8<true, 8>(ps, st)
-                         : ps.ncols <= 16 ? launch_i8<true, 16>(ps, st) : launch_wide<2, 1>(ps, st);
+                         : ps.ncols <= 16 ? launch_i8<true, 16>(ps, st) : ps.ncols <= 32 ? launch_f16<32>(ps, st)
+                         : launch_f16<64>(ps, st);
     if (rc != LYNX_OK) return rc;
   }
   if (p.draft && pl.per < nq) {
@@ -663,7 +680,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
 extern "C" size_t lynx_workspace_bytes(const lynx_shape* shape, int32_t batch, int32_t n_cols_q) {
   lynx::Plan pl;
   if (!lynx::make_plan(shape, batch, n_cols_q, &pl)) return 0;
-  return pl.bytes + pl.shadow_bytes;
+  return pl.bytes;
 }
 
 extern "C" lynx_status lynx_verify_decision(const float* out_full, const float* draft_out, int32_t batch, int32_t k,

@@ -1,0 +1,846 @@
+// Merge-verify attention for 17..64 columns on the fifth-generation tensor cores, FP16 operands with FP32
+// accumulators.  Included by attention.cu inside its namespace.
+//
+// A unit is 128 tokens.  Both contractions take the 8-bit codes centred, c - 128, which FP16 represents exactly:
+//   S^T[128 tokens x NC]      = (codes(K) - 128) . Q^T       A = K in tensor memory (a thread owns a token = a lane),
+//                                                            B = Q, FP16 after a power-of-two scale (exact for BF16
+//                                                                entries down to 2^-32 of the largest)
+//   O^T[128 dims x 2 x 32]   += (codes(V) - 128)^T . [h | r] A = V tile (MN-major), B = the weights as two FP16 terms,
+//                                                                w = h + r (22 bits), side by side in N
+// Centring costs one packed addition per two codes and is what keeps FP32 sufficient: the zero points, 128 steps below
+// the centre of a row, would otherwise be added and taken off again around results a hundred times smaller (error against
+// 64 bits, one layer of 131072 tokens: 2e-6 at 32 columns, 5e-6 at 64; the integer kernel, not centred, 8e-6 at 32).
+// x = s log2(e) + log2(scale_v), w = 2^(x - ref[c]); ref[c] is set so that the largest weight of a column's first unit is
+// 2^8 and raised (accumulators drained, rare) before a weight would leave FP16.  The tensor core's accumulation truncates
+// (0.46 ulp of the running sum per product): every kDrainUnits units the accumulators move into an FP32 copy.
+//
+// Warp roles, one CTA per SM; every hand-off is an mbarrier with a bounded wait, nothing waits on another CTA:
+//   warps 0-7    two softmax warpgroups of 32 columns each: scores -> weights -> P tile
+//   warps 8-11   K codes into tensor memory, and a piece's queries into the Q tile
+//   warps 12-15  V codes into the V tile
+//   warps 16-19  producers (tensor-map copies of 16-token sub-blocks): two warps for the K ring, two for the V ring
+//   warp 20      issues every tcgen05.mma
+//   warps 21, 22 the per-token scalars of the scores and weights (warp 23 completes the warpgroup, for the register split)
+// With 64 columns the groups take one half of the columns each of every unit; with 32 they alternate over the units
+// (separate accumulators, merged at the end of a piece), which spares the per-token work of a second group.
+// Why specialised warps here and teams in attention_i8.cuh: at these widths the accumulators of teams do not fit tensor
+// memory (integer digit planes: 224 columns per team at 32), while the expansions and the softmax of a unit are long
+// enough to overlap as pipeline stages with double-buffered S, K and V.
+//
+// What bounds it: instruction issue.  A unit takes 6200 warp instructions at 32 columns and 8000 at 64 (K expansion 1300,
+// V expansion 1400, softmax 1900 per 32 columns), at 2.2 per cycle; tensor pipe 15-20 %, DRAM under half.  What mattered on
+// the way: no register spills in the softmax loop (little L1 is left beside 227 KB of shared memory: 400 bytes of spills
+// per thread cost a factor of two; hence scores in the 16-lane layout, where a thread sums 8 columns over 4 tokens instead
+// of 32 columns over one), rolled expansion loops (the roles compete for the instruction caches: 118 -> 98 us at 32
+// columns), products issued by an elected lane (93 -> 30 cycles each).  One layer of 131072 tokens: 174 us as two passes of
+// the 16-column integer kernel -> 93 us (32 columns); 293 us by the previous kernel (M = columns, codes not centred) ->
+// 260 us (64 columns, batch 2).
+
+template <int NC>
+struct F16Cfg {
+  static_assert(NC == 32 || NC == 64, "padded column counts");
+  static constexpr bool kSplit = NC == 64;          // both groups score every unit (else they alternate)
+  static constexpr int kST = 128, kCG = 32, kNG = kCG / 8;
+  static constexpr int kPartCols = NC;
+  static constexpr int kStageBytes = kST * 128;     // Anchor and Residual of one tensor: [2][128 tokens][64 B]
+  static constexpr int kVTile = 32768;              // [2 dim blocks][128 tokens][128 B]
+  static constexpr int kPTile = 16384;              // [128 tokens][32 h | 32 r]
+  static constexpr int kQTile = NC * 256;           // [2 dim blocks][NC][128 B]
+  static constexpr int kRingK = 3, kRingV = 3;
+  static constexpr int kOffV = 0, kOffP = 2 * kVTile, kOffQ = kOffP + 2 * kPTile, kOffRK = kOffQ + kQTile,
+                       kOffRV = kOffRK + kRingK * kStageBytes, kOffScal = kOffRV + kRingV * kStageBytes;
+  // floats: qs[2][NC], limits[2][NC], exponents[2] (+ 2); per group: ref[32], fac[32], red[4][64], lz[64]
+  static constexpr int kGrpScal = 2 * 32 + 256 + 64;
+  static constexpr int kOffGrp = kOffScal + (4 * NC + 4) * 4;
+  static constexpr int kOffTok = kOffGrp + 2 * kGrpScal * 4;        // per-token scalars, 4 slots: [4][128] float4, [4][128] float
+  static constexpr int kOffBlk = kOffTok + 4 * 128 * 20;        // [4 producer warps][4 sub-blocks][kI8PieceUnits]
+  static constexpr int kOffItems = kOffBlk + 16 * kI8PieceUnits * 4;
+  static constexpr int kOffBars = kOffItems + 2 * 32;
+  static constexpr int kOffMisc = kOffBars + 44 * 8;
+  static constexpr int kSmem = kOffMisc + 256 + 1024;               // + alignment slack
+  static_assert(kSmem <= 227 * 1024, "shared memory");
+  static_assert(kOffScal % 16 == 0 && kOffGrp % 16 == 0 && kOffBars % 8 == 0, "alignment");
+  static constexpr int kTmS = 0, kTmK = 2 * NC, kTmO = kTmK + 128, kTmOF = kTmO + 128;   // [2][NC], [2][64], [2][64], [2][32]
+  static_assert(kTmOF + 64 <= 512, "tensor memory");
+  static constexpr int kThreads = 768;
+  // units between drains: each adds 8 truncating products to a sum.  (64 columns against 64 bits: 3.3e-4 by the previous
+  // FP16 kernel, 5e-6 here; a drain per 8 units costs 6 % of its time, one per 16 units 3 %.)
+  static constexpr int kDrainUnits = NC == 64 ? 16 : 8;
+  // registers per thread after the split (launched with 80 each): 256 * 136 + 256 * 64 + 128 * 56 + 128 * 24 = 768 * 80
+  static constexpr int kRegSoft = 128, kRegExp = 64, kRegProd = 56, kRegMma = 40;
+};
+template <int N>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
+// The bounded wait of mbar_wait without a call: ptxas cannot split the registers of a kernel that has calls.
+__device__ __forceinline__ void mbar_wait_in(uint32_t bar, uint32_t parity, volatile int* abort_word) {
+  if (mbar_test(bar, parity)) return;
+  uint64_t t0 = 0;
+  for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
+    if ((i & 255u) != 0) continue;
+    const uint64_t now = globaltimer_ns();
+    if (t0 == 0) t0 = now;
+    if (*abort_word || now - t0 > 2000000000ull) { *abort_word = 1; return; }
+  }
+}
+
+// position -> element within a group of 8: {0,4,2,6,1,5,3,7} (what the nibble expansion yields), its own inverse
+__host__ __device__ constexpr int f16_perm(int pos) { return ((pos & 1) << 2) | (pos & 2) | ((pos >> 2) & 1); }
+
+// Four centred FP16 pairs from a word of eight Anchor and a word of eight Residual nibbles: 0x64cc is 1024 + code.
+__device__ __forceinline__ uint32_t f16_centre(uint32_t x) {
+  uint32_t d;
+  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(x), "r"(0xE480E480u));   // - 1152
+  return d;
+}
+__device__ __forceinline__ void f16_codes(uint32_t xa, uint32_t xr, uint32_t* o) {
+  uint32_t ev, od;
+  merge_codes(xa, xr, ev, od);
+  o[0] = f16_centre((ev & 0x00FF00FFu) | 0x64006400u);
+  o[1] = f16_centre(prmt(ev, 0x64646464u, 0x4341));
+  o[2] = f16_centre((od & 0x00FF00FFu) | 0x64006400u);
+  o[3] = f16_centre(prmt(od, 0x64646464u, 0x4341));
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+
+// K codes of a token (thread r of 128 = TMEM lane r) into 64 columns of tensor memory.  The raw planes arrive with the
+// copy engine's 64-byte swizzle (see i8_expand_k_tmem).
+__device__ __forceinline__ void f16_expand_k(uint32_t raw, int r, uint32_t tm_k) {
+  const uint32_t s = ((uint32_t)r >> 1) & 3u, row = raw + (uint32_t)r * 64u;
+  // (a rolled loop, with the next chunk's loads ahead: five roles share an instruction cache of some 12 KB per scheduler)
+  uint4 xa = lds128(row + (s << 4)), xr = lds128(row + 8192u + (s << 4));
+#pragma unroll 1
+  for (int h = 0; h < 4; ++h) {
+    const uint32_t off = ((uint32_t)((h + 1) & 3) ^ s) << 4;
+    const uint4 na = lds128(row + off), nr = lds128(row + 8192u + off);
+    uint32_t regs[16];
+    f16_codes(xa.x, xr.x, regs);
+    f16_codes(xa.y, xr.y, regs + 4);
+    f16_codes(xa.z, xr.z, regs + 8);
+    f16_codes(xa.w, xr.w, regs + 12);
+    TmemRegs<16>::st(tm_k + h * 16, regs);
+    xa = na; xr = nr;
+  }
+}
+// V codes of a unit into the V tile by 128 threads: thread i takes the 16-byte chunk i & 3 (32 elements) of rows i >> 2 + 32 j.
+// Half of the threads take the two 8-byte halves of a chunk in the other order: the four threads of a row then store to
+// four chunk positions per instruction, and rows r and r + 2, which share their banks in the raw stage, read different halves.
+__device__ __forceinline__ void f16_expand_v(uint32_t raw, uint32_t tile, int i) {
+  const int cc = i & 3, row0 = i >> 2;
+  const uint32_t sw = (uint32_t)(((cc >> 1) ^ (row0 >> 1)) & 1) * 2u;
+  const uint32_t base = tile + (uint32_t)(cc >> 1) * 16384u + (uint32_t)row0 * 128u;
+  const uint32_t swz = (uint32_t)(((cc & 1) * 4) ^ (row0 & 7) ^ (int)sw) * 16u;
+  uint32_t a = raw + (uint32_t)(row0 * 64 + cc * 16);
+  uint2 xa[2] = {lds64(a + sw * 4u), lds64(a + (sw ^ 2u) * 4u)}, xr[2] = {lds64(a + 8192u + sw * 4u), lds64(a + 8192u + (sw ^ 2u) * 4u)};
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {   // (loads one step ahead, rolled: see f16_expand_k)
+    a = raw + (uint32_t)((row0 + 32 * ((j + 1) & 3)) * 64 + cc * 16);
+    const uint2 na[2] = {lds64(a + sw * 4u), lds64(a + (sw ^ 2u) * 4u)};
+    const uint2 nr[2] = {lds64(a + 8192u + sw * 4u), lds64(a + 8192u + (sw ^ 2u) * 4u)};
+    const uint32_t wa[4] = {xa[0].x, xa[0].y, xa[1].x, xa[1].y}, wr[4] = {xr[0].x, xr[0].y, xr[1].x, xr[1].y};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {   // register k holds word k ^ sw of the chunk
+      uint32_t o[4];
+      f16_codes(wa[k], wr[k], o);
+      sts128(base + (uint32_t)j * 4096u + (swz ^ (uint32_t)(k * 16)), o[0], o[1], o[2], o[3]);
+    }
+    xa[0] = na[0]; xa[1] = na[1]; xr[0] = nr[0]; xr[1] = nr[1];
+  }
+}
+
+// A producer warp: derives the CTA's range like the others (warp 0 publishes it, the pieces, and the results of empty
+// sequences) and copies its half of the sub-blocks of one tensor: warps 0, 1 the K planes, warps 2, 3 the V planes, eight
+// copies per unit (4 sub-blocks x Anchor / Residual) in one instruction.
+template <class C>
+__device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange& rng, int pw, int lane, uint32_t sbase, uint32_t full0,
+                                             uint32_t empty0, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
+                                             volatile int* abort_word, const I8Maps* maps) {
+  constexpr int ST = C::kST;
+  const int tensor = pw >> 1, nstage = tensor ? C::kRingV : C::kRingK;
+  const int sub0 = 4 * (pw & 1);
+  const int cap = p.max_blocks * p.bt;
+  auto clamp_len = [&](int b) {
+    int len = __ldg(p.seq_lens + b);
+    return len < 0 ? 0 : (len > cap ? cap : len);
+  };
+  const uint32_t dst0 = sbase + (tensor ? C::kOffRV : C::kOffRK) + (uint32_t)(sub0 * 1024);
+  const CUtensorMap *map_a = &maps->m[tensor], *map_r = &maps->m[2 + tensor];
+  uint32_t* my_blk = blk_s + pw * 4 * kI8PieceUnits;
+  int b = rng.b_lo, len = clamp_len(b), U = (len + ST - 1) / ST;
+  int hkv = (int)(rng.off_lo / U), u = (int)(rng.off_lo % U);
+  const int n_units = (int)(rng.hi - rng.lo);
+  int remaining = n_units, slot = 0, ic = 0;
+  uint32_t phase = 1;   // (a fresh barrier passes a wait for the phase before its first)
+  while (remaining > 0) {
+    const int n = min(remaining, U - u);
+    if (pw == 0) {
+      const int qi = ic & 1;
+      if (ic >= 2) mbar_wait_in(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word);
+      const long long seg0 = rng.lo + (n_units - remaining) - u;  // first unit of this segment
+      if (lane == 0) {
+        Item it;
+        it.b = b; it.hkv = hkv; it.len = len;
+        it.first_cta = (int)(seg0 / rng.q);
+        it.n_contrib = (int)((seg0 + U - 1) / rng.q) - it.first_cta + 1;
+        it.pad0 = n; it.pad1 = u; it.pad2 = 0;
+        items[qi] = it;
+        mbar_arrive(qfull0 + qi * 8);
+      }
+      __syncwarp();
+    }
+    for (int c0 = 0; c0 < n; c0 += kI8PieceUnits) {
+      const int cn = min(kI8PieceUnits, n - c0);
+      for (int i = lane; i < 4 * cn; i += 32) {
+        const int t0 = (u + c0 + (i >> 2)) * ST + (sub0 + (i & 3)) * 16;
+        uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
+        if (t0 < len) {
+          int blk = __ldg(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+          if (blk < 0 || blk >= p.num_blocks) {
+            atomicOr(p.ws_flags, kFlagBadBlock);
+            blk = blk < 0 ? 0 : p.num_blocks - 1;
+          }
+          row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 % p.bt));
+        }
+        my_blk[i] = row;
+      }
+      __syncwarp();
+      for (int k = 0; k < cn; ++k) {
+        mbar_wait_in(empty0 + slot * 8, phase, abort_word);
+        const uint4 rw = *reinterpret_cast<const uint4*>(my_blk + 4 * k);
+        // (one elected lane: with a copy per lane the compiler walks through the lanes, operands to the uniform
+        // datapath and back for each; only the sub-blocks at the end of a sequence can be absent)
+        if (tc_elect()) {
+          const uint32_t bar = full0 + slot * 8, dst = dst0 + (uint32_t)slot * C::kStageBytes;
+          const uint32_t rows[4] = {rw.x, rw.y, rw.z, rw.w};
+          uint32_t bytes = 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) bytes += rows[i] != 0xFFFFFFFFu ? 2048u : 0u;
+          if (bytes) mbar_expect_tx(bar, bytes);
+          else mbar_arrive(bar);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (rows[i] != 0xFFFFFFFFu) {
+              tma_rows16(dst + i * 1024, map_a, (int)rows[i], bar);
+              tma_rows16(dst + 8192 + i * 1024, map_r, (int)rows[i], bar);
+            }
+        }
+        __syncwarp();
+        if (++slot == nstage) { slot = 0; phase ^= 1; }
+      }
+      __syncwarp();  // my_blk is rewritten by the next round
+    }
+    remaining -= n;
+    u += n;
+    ++ic;
+    if (u == U && remaining > 0) {
+      u = 0;
+      if (++hkv == p.Hkv) {
+        hkv = 0;
+        do {
+          ++b;
+          len = b < p.B ? clamp_len(b) : 0;
+          U = (len + ST - 1) / ST;
+        } while (b < p.B && U == 0);
+        if (b >= p.B) break;  // cannot happen: the range ends inside the list
+      }
+    }
+  }
+}
+
+template <int NC>
+__global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const AttnParams p,
+                                                                           const __grid_constant__ I8Maps maps) {
+  using C = F16Cfg<NC>;
+  constexpr bool SPLIT = C::kSplit;
+  constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t sbase = smem_u32(smem);
+  float* scal = reinterpret_cast<float*>(smem + C::kOffScal);
+  Item* items = reinterpret_cast<Item*>(smem + C::kOffItems);
+  int* misc = reinterpret_cast<int*>(smem + C::kOffMisc);   // [0] abort, [7] units, [8] tensor memory base, [40 + g] accumulate
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // (known to be uniform)
+  const uint32_t kfull = sbase + C::kOffBars, kempty = kfull + 32, vfull = kempty + 32, vempty = vfull + 24;
+  const uint32_t qfull = vempty + 24, qempty = qfull + 16, qready = qempty + 16;   // [2]: piece published / left / queries in place
+  const uint32_t kready = qready + 16, sfull = kready + 16, sfree = sfull + 16;    // [2]: K in TMEM / scores valid / scores read
+  const uint32_t vready = sfree + 16, vfree = vready + 16;                         // [2]: V tile written / read
+  const uint32_t pready = vfree + 16, pvdone = pready + 16;                        // [group]: weights written / P.V complete
+  const uint32_t mready = pvdone + 16, mfree = mready + 32;                        // [4]: per-token scalars written / read
+  volatile int* abort_word = misc;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  if (warp == 16 && lane < 4) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.m[lane])) : "memory");
+  if (tid == 0) {
+    for (int i = 0; i < C::kRingK; ++i) { mbar_init(kfull + i * 8, 2); mbar_init(kempty + i * 8, 4); }
+    for (int i = 0; i < C::kRingV; ++i) { mbar_init(vfull + i * 8, 2); mbar_init(vempty + i * 8, 4); }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(qfull + i * 8, 1);
+      mbar_init(qempty + i * 8, 14);
+      mbar_init(qready + i * 8, 4);
+      mbar_init(kready + i * 8, 4);
+      mbar_init(sfull + i * 8, 1);
+      mbar_init(sfree + i * 8, SPLIT ? 8 : 4);
+      mbar_init(vready + i * 8, 4);
+      mbar_init(vfree + i * 8, SPLIT ? 2 : 1);
+      mbar_init(pready + i * 8, 4);
+      mbar_init(pvdone + i * 8, 1);
+    }
+    for (int i = 0; i < 4; ++i) { mbar_init(mready + i * 8, 2); mbar_init(mfree + i * 8, SPLIT ? 8 : 4); }
+    for (int i = 0; i < 64; ++i) misc[i] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = tid; i < 2 * C::kGrpScal; i += C::kThreads) reinterpret_cast<float*>(smem + C::kOffGrp)[i] = 0.0f;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(misc + 8)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem0 = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(misc + 8), 0);
+  // nothing in global memory has been touched so far: wait for the grids this one depends on
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  SkRange rng;
+  if (warp >= 16 && warp < 20) {
+    const int cap = p.max_blocks * p.bt;
+    auto clamp_len = [&](int b) {
+      int len = __ldg(p.seq_lens + b);
+      return len < 0 ? 0 : (len > cap ? cap : len);
+    };
+    rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, clamp_len);
+    if (warp == 16) {
+      if (lane == 0) misc[7] = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
+      empty_sequences<true>(p, blockIdx.x, gridDim.x, lane, clamp_len);
+    }
+  }
+  __syncthreads();  // (A) the range is published
+  const int n_units = misc[7];
+
+  // ================================================================================== softmax warpgroups
+  if (warp < 8) {
+    reg_inc<C::kRegSoft>();
+    const int g = warp >> 2, w4 = warp & 3, r = tid & 127;
+    const uint32_t lane_sel = (uint32_t)(w4 * 32) << 16;
+    const uint32_t tm_o = tmem0 + C::kTmO + g * 64 + lane_sel, tm_of = tmem0 + C::kTmOF + g * 32 + lane_sel;
+    // this thread's tokens of a unit: t0 + 8 k, k = 0..3; its columns 8 j + c2, + 1
+    const int t0 = w4 * 32 + (lane >> 2), c2 = (lane & 3) * 2;
+    // row lane & 7 of block lane >> 3 of a warp's first eight tokens in the P tile (the remainders: 64 bytes on, swizzled)
+    const uint32_t p_addr = sbase + C::kOffP + g * C::kPTile + (uint32_t)(w4 * 32 + (lane & 7)) * 128u +
+                            (uint32_t)((lane >> 3) ^ (lane & 7)) * 16u;
+    float* grp = reinterpret_cast<float*>(smem + C::kOffGrp) + g * C::kGrpScal;
+    float *ref_s = grp, *fac_s = grp + 32, *red_s = grp + 64, *lz_s = grp + 320;
+    const int bar_g = 1 + g;
+    const int col0 = SPLIT ? g * CG : 0;            // first column of this group
+    const int dim_out = (r & ~7) + f16_perm(r & 7);
+    const float4* tok4 = reinterpret_cast<const float4*>(smem + C::kOffTok) + t0;
+    const float* tok1 = reinterpret_cast<const float*>(smem + C::kOffTok + 4 * 128 * 16) + t0;
+    uint32_t n_own = 0;                             // units of this group so far
+    int gs_base = 0, ic = 0;
+    while (gs_base < n_units) {
+      const int qi = ic & 1;
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      const Item item = items[qi];
+      const int len = item.len, n_piece = item.pad0;
+      const int u_first = SPLIT ? 0 : (g ^ gs_base) & 1;
+      const bool have = u_first < n_piece;
+      uint64_t l2[NG], zs2[NG];                     // softmax sums of this thread's tokens, two columns per register pair
+      uint64_t qs2[NG], ref2[NG];                   // the columns' sums of q and reference exponents
+#pragma unroll
+      for (int j = 0; j < NG; ++j) { l2[j] = 0ull; zs2[j] = 0ull; ref2[j] = 0ull; }
+      bool have_of = false;
+      int units_in_acc = 0;
+      // Moves the accumulators (the group's last P.V is complete) into the FP32 copy, scaled by fac_s[] if asked.
+      auto drain = [&](bool scale) {
+        tc_fence_after();
+#pragma unroll 1
+        for (int c8 = 0; c8 < CG / 8; ++c8) {   // (a loop: the caller's values fill the registers)
+          uint32_t h[8], q[8], of[8];
+          TmemRegs<8>::ld(tm_o + c8 * 8, h);
+          TmemRegs<8>::ld(tm_o + 32 + c8 * 8, q);
+          TmemRegs<8>::ld(tm_of + c8 * 8, of);
+          tc_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            float v = 0.0f;   // (a piece's first drain finds the previous piece's copy; accumulators not restarted since the last drain)
+            if (have_of) v = __uint_as_float(of[k]);
+            if (units_in_acc > 0) v += __uint_as_float(h[k]) + __uint_as_float(q[k]);
+            if (scale) v *= fac_s[c8 * 8 + k];
+            of[k] = __float_as_uint(v);
+          }
+          TmemRegs<8>::st(tm_of + c8 * 8, of);
+        }
+        tc_wait_st();
+        have_of = true;
+        units_in_acc = 0;
+      };
+      if (have) {
+        const int full_lim = p.causal ? len - p.tail + 1 : len;
+        const int* lim_s = reinterpret_cast<const int*>(scal + 2 * NC + qi * NC) + col0;
+        bool fresh = true;
+        mbar_wait_in(qready + qi * 8, (ic >> 1) & 1, abort_word);
+#pragma unroll
+        for (int j = 0; j < NG; ++j) qs2[j] = *reinterpret_cast<const uint64_t*>(scal + qi * NC + col0 + 8 * j + c2);
+        for (int u = u_first; u < n_piece; u += STEP, ++n_own) {
+          const int gs = gs_base + u, sl = gs & 1;
+          const int unit_t0 = (item.pad1 + u) * C::kST;
+          // ---- scores: log2 of the weights relative to the columns' references ------------------------------
+          mbar_wait_in(mready + (gs & 3) * 8, (gs >> 2) & 1, abort_word);
+          mbar_wait_in(sfull + sl * 8, (gs >> 1) & 1, abort_word);
+          tc_fence_after();
+          uint64_t y2[4][NG];
+          bool scale = false;
+#pragma unroll 1
+          for (int pass = 0; pass < 2; ++pass) {   // (a second time, from tensor memory, after a change of the references)
+          if (scale || units_in_acc >= C::kDrainUnits) {   // (here, while few registers are live)
+            mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);
+            drain(scale);
+          }
+          uint32_t s[2][4 * NG];   // [tokens t0, t0 + 8 | t0 + 16, t0 + 24]
+          const uint32_t tm_s = tmem0 + C::kTmS + sl * NC + col0 + lane_sel;
+          tc_ld_16x256<NG>(tm_s, s[0]);
+          tc_ld_16x256<NG>(tm_s + (16u << 16), s[1]);
+          tc_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 ts = tok4[(gs & 3) * 128 + 8 * k];
+            const uint64_t al2 = f2_pack(ts.x, ts.x), be2 = f2_pack(ts.y, ts.y), lsv2 = f2_pack(ts.z, ts.z);
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              const uint32_t* sv = s[k >> 1] + 4 * j + 2 * (k & 1);
+              y2[k][j] = f2_fma(f2_pack(__uint_as_float(sv[0]), __uint_as_float(sv[1])), al2,
+                                f2_fma(be2, qs2[j], f2_sub(lsv2, ref2[j])));
+            }
+          }
+          if (unit_t0 + C::kST > full_lim) {
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              const int la = lim_s[8 * j + c2] - unit_t0 - t0, lb = lim_s[8 * j + c2 + 1] - unit_t0 - t0;
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                float a, b;
+                f2_unpack(y2[k][j], a, b);
+                if (8 * k >= la) a = -INFINITY;
+                if (8 * k >= lb) b = -INFINITY;
+                y2[k][j] = f2_pack(a, b);
+              }
+            }
+          }
+          float ymax = -INFINITY;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              float a, b;
+              f2_unpack(y2[k][j], a, b);
+              ymax = max3(ymax, a, b);
+            }
+          if (n_own > 0) mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // P free, accumulators current
+          // ---- a piece's first unit, or a weight that would leave FP16: new reference exponents ----------
+          if (!bar_or(bar_g, 128, fresh || ymax > 15.0f)) break;
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              float ma = -INFINITY, mb = -INFINITY;
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                float a, b;
+                f2_unpack(y2[k][j], a, b);
+                ma = fmaxf(ma, a);
+                mb = fmaxf(mb, b);
+              }
+#pragma unroll
+              for (int off = 4; off <= 16; off <<= 1) {
+                ma = fmaxf(ma, __shfl_xor_sync(0xFFFFFFFFu, ma, off));
+                mb = fmaxf(mb, __shfl_xor_sync(0xFFFFFFFFu, mb, off));
+              }
+              if (lane < 4) { red_s[w4 * CG + 8 * j + c2] = ma; red_s[w4 * CG + 8 * j + c2 + 1] = mb; }
+            }
+            named_bar(bar_g, 128);
+            if (r < CG) {
+              const float old = fresh ? 0.0f : ref_s[r];
+              const float mx = fmaxf(fmaxf(red_s[r], red_s[CG + r]), fmaxf(red_s[2 * CG + r], red_s[3 * CG + r])) + old;
+              float nw = old, f = 1.0f;
+              if (fresh) { nw = fmaxf(mx, -1.0e4f) - 8.0f; f = 0.0f; }
+              else if (mx - old > 15.0f) { nw = mx - 8.0f; f = ex2_full(old - nw); }
+              ref_s[r] = nw;
+              fac_s[r] = f;
+            }
+            named_bar(bar_g, 128);
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              const uint64_t f2 = *reinterpret_cast<const uint64_t*>(fac_s + 8 * j + c2);
+              const uint64_t nw2 = *reinterpret_cast<const uint64_t*>(ref_s + 8 * j + c2);
+              l2[j] = f2_mul(l2[j], f2);
+              zs2[j] = f2_mul(zs2[j], f2);
+              ref2[j] = nw2;
+            }
+            scale = !fresh;
+            fresh = false;
+          }
+          // ---- weights of this thread's tokens into the P tile --------------------------------------------------
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float ia = tok4[(gs & 3) * 128 + 8 * k].w, ib = tok1[(gs & 3) * 128 + 8 * k];
+            const uint64_t ia2 = f2_pack(ia, ia), ib2 = f2_pack(ib, ib);
+            uint32_t h[4], q[4];
+#pragma unroll
+            for (int j = 0; j < NG; ++j) {
+              float a, b, ha, hb;
+              f2_unpack(y2[k][j], a, b);
+              const float wa = ex2_ftz(a), wb = ex2_ftz(b);
+              const uint64_t w2 = f2_pack(wa, wb);
+              l2[j] = f2_fma(w2, ia2, l2[j]);
+              zs2[j] = f2_fma(w2, ib2, zs2[j]);
+              h[j] = pack_f16x2(wa, wb);
+              asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tcvt.f32.f16 %0, lo;\n\tcvt.f32.f16 %1, hi;\n\t}"
+                  : "=f"(ha), "=f"(hb) : "r"(h[j]));
+              f2_unpack(f2_sub(w2, f2_pack(ha, hb)), a, b);
+              q[j] = pack_f16x2(a, b);
+            }
+            stm_x4(p_addr + k * 1024, h[0], h[1], h[2], h[3]);
+            stm_x4((p_addr ^ 64u) + k * 1024, q[0], q[1], q[2], q[3]);
+          }
+          if (r == 0) misc[40 + g] = units_in_acc > 0 ? 1 : 0;
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) { mbar_arrive(sfree + sl * 8); mbar_arrive(mfree + (gs & 3) * 8); mbar_arrive(pready + g * 8); }
+          ++units_in_acc;
+        }
+        mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // the last P.V
+        drain(false);
+      }
+      // ---- end of the piece: totals over the 128 tokens of a unit, then the result -------------------------
+      if (have) {
+#pragma unroll
+        for (int j = 0; j < NG; ++j) {
+          float v[4];
+          f2_unpack(l2[j], v[0], v[1]);
+          f2_unpack(zs2[j], v[2], v[3]);
+#pragma unroll
+          for (int off = 4; off <= 16; off <<= 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] += __shfl_xor_sync(0xFFFFFFFFu, v[i], off);
+          if (lane < 4) {
+            float* d = red_s + w4 * 64 + 8 * j + c2;
+            d[0] = v[0]; d[1] = v[1]; d[32] = v[2]; d[33] = v[3];
+          }
+        }
+        named_bar(bar_g, 128);
+        if (r < 64) lz_s[r] = (red_s[r] + red_s[64 + r]) + (red_s[128 + r] + red_s[192 + r]);
+        named_bar(bar_g, 128);
+      } else {
+        if (r < 64) lz_s[r] = 0.0f;
+        if (r < CG) ref_s[r] = -INFINITY;
+        named_bar(bar_g, 128);
+      }
+      const bool direct = item.n_contrib == 1;
+      const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
+      float* part = p.ws_part + (bh + (size_t)blockIdx.x) * (size_t)C::kPartCols * kPartStride;
+      auto put = [&](int c, float v, float m, float l) {   // column c, this lane's dim
+        if (c >= p.ncols) return;
+        if (direct) {
+          const int j = c / p.G, hh = c % p.G;
+          p.out[(((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh) * LYNX_D + dim_out] = l > 0.0f ? v / l : 0.0f;
+          if (r == 0) p.ws_lse[((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh] = lse_of(m, l);
+        } else {
+          part[(size_t)c * kPartStride + dim_out] = v;
+          if (r == 0) { part[(size_t)c * kPartStride + 128] = m; part[(size_t)c * kPartStride + 129] = l; }
+        }
+      };
+      // (rolled loops, four columns of tensor memory at a time: this code runs once per piece, from a cold instruction cache)
+      auto o_cols = [&](int c, float* o) {
+        uint32_t t[4];
+        TmemRegs<4>::ld(tm_of + c, t);
+        tc_wait_ld();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[k] = have ? __uint_as_float(t[k]) : 0.0f;
+      };
+      if (SPLIT) {
+#pragma unroll 1
+        for (int c = 0; c < CG; c += 4) {
+          float o[4];
+          o_cols(c, o);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) put(col0 + c + k, o[k] + lz_s[32 + c + k], ref_s[c + k], lz_s[c + k]);
+        }
+      } else {
+        // each group hands the other one half of its columns through its idle P tile, and merges and writes the other half
+        float* mail = reinterpret_cast<float*>(smem + C::kOffP + g * C::kPTile);
+        const int g0 = 16 * g;   // first column of this group's half
+#pragma unroll 1
+        for (int c = 0; c < 16; c += 4) {
+          float o[4];
+          o_cols(16 - g0 + c, o);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) mail[(c + k) * 128 + r] = o[k];
+        }
+        named_bar(3, 256);
+        const float* omail = reinterpret_cast<const float*>(smem + C::kOffP + (g ^ 1) * C::kPTile);
+        const float* ogrp = reinterpret_cast<const float*>(smem + C::kOffGrp) + (g ^ 1) * C::kGrpScal;
+#pragma unroll 1
+        for (int c = 0; c < 16; c += 4) {
+          float o[4];
+          o_cols(g0 + c, o);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int cc = g0 + c + k;
+            const float m1 = ref_s[cc], m2 = ogrp[cc], M = fmaxf(m1, m2);
+            const float f1 = ex2_full(m1 - M), f2 = ex2_full(m2 - M);
+            const float l = lz_s[cc] * f1 + ogrp[320 + cc] * f2;
+            const float z = lz_s[32 + cc] * f1 + ogrp[320 + 32 + cc] * f2;
+            put(cc, (o[k] * f1 + omail[(c + k) * 128 + r] * f2) + z, M, l);
+          }
+        }
+      }
+      tc_fence_before();
+      __threadfence();
+      named_bar(3, 256);   // (the mail and the other group's totals have been read)
+      finish_piece<true, C::kPartCols, 256, NC, 12>(p, item, direct, tid, misc, 3);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(qempty + qi * 8);
+      gs_base += n_piece;
+      ++ic;
+    }
+    // ---- release the tensor memory: every product has been waited for ----------------------------------------
+    tc_fence_before();
+    named_bar(3, 256);
+    if (warp == 0) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem0), "r"(512u) : "memory");
+    }
+    if (tid == 0 && misc[0]) atomicOr(p.ws_flags, kFlagTimeout);
+    return;
+  }
+  // ================================================================================== K codes and queries
+  if (warp < 12) {
+    reg_dec<C::kRegExp>();
+    const int kt = tid - 256, w4 = warp & 3;
+    const uint32_t tm_k = tmem0 + C::kTmK + ((uint32_t)(w4 * 32) << 16);
+    float* amax_s = reinterpret_cast<float*>(misc + 48);
+    int gs = 0, ic = 0, slot = 0;
+    uint32_t phase = 0;
+    while (gs < n_units) {
+      const int qi = ic & 1;
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      const int ib = items[qi].b, ih = items[qi].hkv, len = items[qi].len, n_piece = items[qi].pad0;
+      // ---- the piece's queries: thread = 16-byte chunk kt & 15 of columns kt >> 4, + 8, ... ---------------------
+      {
+        constexpr int NI = NC / 8;
+        auto chunk_of = [&](int c) {
+          if (c >= p.ncols) return make_uint4(0u, 0u, 0u, 0u);
+          const int j = c / p.G, hh = c % p.G;
+          return __ldg(reinterpret_cast<const uint4*>(p.q + (((size_t)ib * p.nq_stride + j) * p.Hq + (size_t)ih * p.G + hh) * LYNX_D) + (kt & 15));
+        };
+        float amax = 0.0f;
+#pragma unroll 4
+        for (int i = 0; i < NI; ++i) {
+          const uint4 v = chunk_of(i * 8 + (kt >> 4));
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          float sum = 0.0f;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xFFFF0000u);
+            amax = fmaxf(amax, fmaxf(fabsf(lo), fabsf(hi)));
+            sum += lo + hi;
+          }
+#pragma unroll
+          for (int off = 8; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+          if ((kt & 15) == 0) scal[qi * NC + i * 8 + (kt >> 4)] = sum;
+        }
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, off));
+        if (lane == 0) amax_s[w4] = amax;
+        named_bar(4, 128);
+        amax = fmaxf(fmaxf(amax_s[0], amax_s[1]), fmaxf(amax_s[2], amax_s[3]));
+        // |q 2^e| in [2^14, 2^15) for the largest entry
+        int e = 0;
+        if (amax > 0.0f && amax < INFINITY) e = 14 - (((__float_as_int(amax) >> 23) & 0xFF) - 127);
+        e = max(-100, min(100, e));
+        const float up = __int_as_float((127 + e) << 23);
+        if (kt == 0) reinterpret_cast<int*>(scal)[4 * NC + qi] = e;
+        if (kt < NC) reinterpret_cast<int*>(scal)[2 * NC + qi * NC + kt] =
+            kt < p.ncols ? (p.causal ? len - p.tail + kt / p.G + 1 : len) : 0;
+        if (gs > 0) mbar_wait_in(sfull + ((gs - 1) & 1) * 8, ((gs - 1) >> 1) & 1, abort_word);   // the previous piece's last Q.K^T
+#pragma unroll 4
+        for (int i = 0; i < NI; ++i) {   // (read again, from the cache: 64 columns do not fit the registers)
+          const int c = i * 8 + (kt >> 4), ch = kt & 15;
+          const uint4 v = chunk_of(c);
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          float f[8];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            f[2 * k] = __uint_as_float(w[k] << 16) * up;
+            f[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u) * up;
+          }
+          sts128(sbase + C::kOffQ + (uint32_t)(ch >> 3) * (NC * 128u) + (uint32_t)c * 128u + (uint32_t)((ch & 7) ^ (c & 7)) * 16u,
+                 pack_f16x2(f[0], f[4]), pack_f16x2(f[2], f[6]), pack_f16x2(f[1], f[5]), pack_f16x2(f[3], f[7]));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        named_bar(4, 128);
+        if (lane == 0) { mbar_arrive(qready + qi * 8); mbar_arrive(qempty + qi * 8); }
+      }
+      for (int u = 0; u < n_piece; ++u, ++gs) {
+        mbar_wait_in(kfull + slot * 8, phase, abort_word);
+        if (gs >= 2) mbar_wait_in(sfull + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);   // Q.K^T of the unit before last
+        tc_fence_after();
+        f16_expand_k(sbase + C::kOffRK + (uint32_t)slot * C::kStageBytes, kt, tm_k + (uint32_t)(gs & 1) * 64u);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(kempty + slot * 8);
+        tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(kready + (gs & 1) * 8);
+        if (++slot == C::kRingK) { slot = 0; phase ^= 1; }
+      }
+      ++ic;
+    }
+    return;
+  }
+  // ================================================================================== V codes
+  if (warp < 16) {
+    reg_dec<C::kRegExp>();
+    const int vt = tid - 384;
+    int slot = 0;
+    uint32_t phase = 0;
+    for (int gs = 0; gs < n_units; ++gs) {
+      mbar_wait_in(vfull + slot * 8, phase, abort_word);
+      if (gs >= 2) mbar_wait_in(vfree + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);
+      f16_expand_v(sbase + C::kOffRV + (uint32_t)slot * C::kStageBytes, sbase + C::kOffV + (uint32_t)(gs & 1) * C::kVTile, vt);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) { mbar_arrive(vempty + slot * 8); mbar_arrive(vready + (gs & 1) * 8); }
+      if (++slot == C::kRingV) { slot = 0; phase ^= 1; }
+    }
+    return;
+  }
+  // ================================================================================== producers
+  if (warp < 20) {
+    reg_dec<C::kRegProd>();
+    const int pw = warp - 16;
+    if (n_units > 0)
+      f16_producer<C>(p, rng, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
+                      reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
+    return;
+  }
+  // ================================================================================== products
+  reg_dec<C::kRegMma>();
+  // ---- per-token scalars of the scores and weights (warps 21, 22: a lane has tokens 64 w + lane and 32 further on) ----
+  if (warp == 21 || warp == 22) {
+    const int i0 = (warp - 21) * 64 + lane;
+    float4* tok4 = reinterpret_cast<float4*>(smem + C::kOffTok) + i0;
+    float* tok1 = reinterpret_cast<float*>(smem + C::kOffTok + 4 * 128 * 16) + i0;
+    const int bt_shift = (p.bt & (p.bt - 1)) == 0 ? 31 - __clz(p.bt) : -1;
+    int gs = 0, ic = 0;
+    while (gs < n_units) {
+      const int qi = ic & 1;
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      const int ih = items[qi].hkv, len = items[qi].len, n_piece = items[qi].pad0, u0 = items[qi].pad1;
+      const int32_t* table = p.block_table + (size_t)items[qi].b * p.max_blocks;
+      // metadata is read two steps ahead: the block id of the unit after next, the (scale, zero) pairs of the next unit
+      auto blk_of = [&](int uu, int i) -> int {
+        const int t = (u0 + uu) * C::kST + i0 + 32 * i;
+        if (uu >= n_piece || t >= len) return 0;
+        return __ldg(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
+      };
+      auto meta_of = [&](int uu, int i, int blk, float2& k2, float2& v2) {
+        const int t = (u0 + uu) * C::kST + i0 + 32 * i;
+        k2 = make_float2(0.f, 0.f); v2 = k2;
+        if (uu >= n_piece || t >= len) return;
+        const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
+        blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
+        const uint32_t row = (uint32_t)(((size_t)blk * p.Hkv + ih) * p.bt + in_blk);
+        k2 = __ldg(reinterpret_cast<const float2*>(p.km) + row);
+        v2 = __ldg(reinterpret_cast<const float2*>(p.vm) + row);
+      };
+      int blk0[2], blk_n[2];
+      float2 km[2], vm[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) { blk0[i] = blk_of(0, i); blk_n[i] = blk_of(1, i); }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) meta_of(0, i, blk0[i], km[i], vm[i]);
+      mbar_wait_in(qready + qi * 8, (ic >> 1) & 1, abort_word);
+      const float ca = p.sm_log2 * __int_as_float((127 - reinterpret_cast<const int*>(scal)[4 * NC + qi]) << 23);
+      for (int u = 0; u < n_piece; ++u, ++gs) {
+        if (gs >= 4) mbar_wait_in(mfree + (gs & 3) * 8, ((gs >> 2) - 1) & 1, abort_word);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const bool valid = (u0 + u) * C::kST + i0 + 32 * i < len;
+          if (SPLIT && valid && !(vm[i].x < 16.0f)) atomicOr(p.ws_flags, kFlagRange);   // beyond the stated range of this width
+          const float sve = fmaxf(vm[i].x, 9.094947e-13f);   // floor 2^-40
+          const float ia = valid ? rcp_approx(sve) : 0.0f;
+          tok4[(gs & 3) * 128 + 32 * i] = make_float4(km[i].x * ca, fmaf(km[i].x, 128.0f, km[i].y) * p.sm_log2, lg2_approx(sve), ia);
+          tok1[(gs & 3) * 128 + 32 * i] = fmaf(sve, 128.0f, vm[i].y) * ia;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(mready + (gs & 3) * 8);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          meta_of(u + 1, i, blk_n[i], km[i], vm[i]);
+          blk_n[i] = blk_of(u + 2, i);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(qempty + qi * 8);
+      ++ic;
+    }
+    return;
+  }
+  if (warp == 20) {
+    constexpr uint32_t kIdescS = tc_idesc(NC, false), kIdescO = tc_idesc(64, true) | (1u << 15);
+    // (low words of the operand descriptors; the issuing thread keeps them in registers)
+    constexpr uint32_t kHi = i8_desc_hi(1024u, 2u);
+    const uint32_t q_lo = i8_desc_lo(sbase + C::kOffQ, 16u), v_lo = i8_desc_lo(sbase + C::kOffV, 16384u),
+                   p_lo = i8_desc_lo(sbase + C::kOffP, 16384u);
+    auto qk = [&](int gs) {
+      const int sl = gs & 1;
+      mbar_wait_in(kready + sl * 8, (gs >> 1) & 1, abort_word);
+      if (gs >= 2) mbar_wait_in(sfree + sl * 8, ((gs >> 1) - 1) & 1, abort_word);
+      tc_fence_after();
+      if (tc_elect()) {
+        const uint32_t d = tmem0 + C::kTmS + sl * NC, a = tmem0 + C::kTmK + sl * 64;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+          tc_mma_ts(d, a + ks * 8u, i8_pack(q_lo + (uint32_t)(((ks >> 2) * NC * 128 + (ks & 3) * 32) >> 4), kHi), kIdescS, ks > 0 ? 1u : 0u);
+        tc_commit(sfull + sl * 8);
+      }
+      __syncwarp();
+    };
+    auto pv = [&](int gs) {
+      const int sl = gs & 1;
+      mbar_wait_in(vready + sl * 8, (gs >> 1) & 1, abort_word);
+#pragma unroll 1
+      for (int g = SPLIT ? 0 : sl; g < (SPLIT ? 2 : sl + 1); ++g) {
+        mbar_wait_in(pready + g * 8, (SPLIT ? gs : gs >> 1) & 1, abort_word);
+        tc_fence_after();
+        const uint32_t acc = *reinterpret_cast<volatile int*>(misc + 40 + g) ? 1u : 0u;
+        if (tc_elect()) {
+          const uint32_t d = tmem0 + C::kTmO + g * 64, vl = v_lo + sl * (C::kVTile >> 4), pl = p_lo + g * (C::kPTile >> 4);
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            tc_mma_ss(d, i8_pack(vl + ks * 128u, kHi), i8_pack(pl + ks * 128u, kHi), kIdescO, ks > 0 ? 1u : acc);
+          tc_commit(pvdone + g * 8);
+          tc_commit(vfree + sl * 8);
+        }
+        __syncwarp();
+      }
+    };
+    if (n_units > 0) qk(0);
+#pragma unroll 1
+    for (int gs = 0; gs < n_units; ++gs) {
+      if (gs + 1 < n_units) qk(gs + 1);
+      pv(gs);
+    }
+  }
+}
+
+template <int NC>
+lynx_status launch_f16(const AttnParams& p, cudaStream_t st) {
+  using C = F16Cfg<NC>;
+  return launch_units<true, C::kSmem, C::kThreads, C::kST, attn_f16_kernel<NC>>(p, st);
+}

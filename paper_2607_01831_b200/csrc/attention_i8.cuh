@@ -341,26 +341,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   const int b_lo = rng.b_lo;
   if (pw == 0) {
     if (lane == 0) misc[7] = lo < hi ? (int)(hi - lo) : 0;
-    // sequences with no token: outputs are zero, nothing is rejected unless the draft is not zero
-    for (int b = cta; b < p.B; b += n_cta) {
-      if (clamp_len(b) != 0) continue;
-      const size_t n = (size_t)p.nq * p.Hq * LYNX_D;
-      for (size_t i = lane; i < n; i += 32) p.out[(size_t)b * p.nq_stride * p.Hq * LYNX_D + i] = 0.0f;
-      for (int i = lane; i < p.nq * p.Hq; i += 32) p.ws_lse[(size_t)b * p.nq_stride * p.Hq + i] = -INFINITY;
-      if (FULL && p.draft != nullptr) {
-        int fr = p.nq;
-        for (int j = p.nq - 1; j >= 0; --j) {
-          float worst = 0.0f;
-          for (int i = lane; i < p.Hq * LYNX_D; i += 32)
-            worst = fmaxf(worst, fabsf(__ldg(p.draft + ((size_t)b * p.nq_stride + j) * p.Hq * LYNX_D + i)) / p.atol);
-#pragma unroll
-          for (int off = 16; off >= 1; off >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xFFFFFFFFu, worst, off));
-          if (lane == 0) p.dev[(size_t)b * p.nq_stride + j] = worst;
-          if (worst > 1.0f) fr = j;
-        }
-        if (lane == 0) p.first_reject[b] = fr;
-      }
-    }
+    empty_sequences<FULL>(p, cta, n_cta, lane, clamp_len);
   }
   __syncthreads();  // (A) the range is published
   const int n_units = (int)(lo < hi ? hi - lo : 0);
@@ -833,15 +814,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         }
         tc_fence_before();
         named_bar(bar_tm, TT);
-        if (tt == 0) {
+        if (tw == 0) {
           if (u == u_first) mbar_wait(qready0 + qi * 8, (ic >> 1) & 1, abort_word);   // the piece's query planes
           tc_fence_after();
-          const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmS;
-          const uint32_t qd_lo = qd_lo0 + (uint32_t)qi * (C::kQTile >> 4);
+          if (lane == 0) {
+            const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmS;
+            const uint32_t qd_lo = qd_lo0 + (uint32_t)qi * (C::kQTile >> 4);
 #pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4)
-            i8_mma_ts(d, tm_k + (uint32_t)k4 * 8u, i8_pack(qd_lo + (uint32_t)k4 * 2u, kQdHi), kIdescS, k4 > 0 ? 1u : 0u);
-          tc_commit(sfull0 + tm * 8);
+            for (int k4 = 0; k4 < 4; ++k4)
+              i8_mma_ts(d, tm_k + (uint32_t)k4 * 8u, i8_pack(qd_lo + (uint32_t)k4 * 2u, kQdHi), kIdescS, k4 > 0 ? 1u : 0u);
+            tc_commit(sfull0 + tm * 8);
+          }
         }
         __syncwarp();
         if (G == 1 || grp == 0) {   // (the other group has waited already)
@@ -991,15 +974,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             weights(over);
           }
         }
-        if (tt == 0) {
+        if (tw == 0) {
           tc_fence_after();
-          const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmO;
+          if (lane == 0) {
+            const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmO;
 #pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4)
-            i8_mma_ss(d, i8_pack(vd_lo + (uint32_t)k4 * (4096u >> 4), kVdHi),
-                      i8_pack(pd_lo + (uint32_t)k4 * ((32u * C::kPRow) >> 4), kPdHi),
-                      kIdescO, (units_in_acc > 0 || k4 > 0) ? 1u : 0u);
-          tc_commit(pvdone0 + tm * 8);
+            for (int k4 = 0; k4 < 4; ++k4)
+              i8_mma_ss(d, i8_pack(vd_lo + (uint32_t)k4 * (4096u >> 4), kVdHi),
+                        i8_pack(pd_lo + (uint32_t)k4 * ((32u * C::kPRow) >> 4), kPdHi),
+                        kIdescO, (units_in_acc > 0 || k4 > 0) ? 1u : 0u);
+            tc_commit(pvdone0 + tm * 8);
+          }
         }
         __syncwarp();
         ++units_in_acc;
@@ -1108,7 +1093,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           }
         }
         __threadfence();
-        finish_piece<FULL, C::kPartCols, TT>(p, item, direct, tt, my_misc, bar_tm);
+        finish_piece<FULL, C::kPartCols, TT, CP, 8, 2>(p, item, direct, tt, my_misc, bar_tm);
       }
     }
     // every team keeps count of every team's deposits (the phase of its deposit barrier)
@@ -1131,19 +1116,18 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   if (tid == 0 && misc[0]) atomicOr(p.ws_flags, kFlagTimeout);
 }
 
-template <bool FULL, int CP>
-lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
-  using C = I8Cfg<FULL, CP>;
-  auto kern = attn_i8_kernel<FULL, CP>;
+// Launches one of the persistent attention kernels: SMEM bytes, THREADS per CTA, units of ST tokens.
+template <bool FULL, int SMEM, int THREADS, int ST, auto KERN>
+lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
   static bool configured[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess)
       return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  const long long cap_units = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + C::kST - 1) / C::kST);
+  const long long cap_units = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + ST - 1) / ST);
   long long grid = (cap_units + 3) / 4;
   const long long full = sm_count();   // one CTA per SM
   grid = grid < 1 ? 1 : (grid > full ? full : grid);
@@ -1153,8 +1137,8 @@ lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
   // griddepcontrol.wait, i.e. before that kernel has completed and its memory is visible.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(C::kThreads);
-  cfg.dynamicSmemBytes = C::kSmem;
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1172,6 +1156,12 @@ lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
     maps.m[2] = maps.m[0];
     maps.m[3] = maps.m[1];
   }
-  if (cudaLaunchKernelEx(&cfg, kern, p, maps) != cudaSuccess) return LYNX_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, KERN, p, maps) != cudaSuccess) return LYNX_ERR_CUDA;
   return launch_status();
+}
+
+template <bool FULL, int CP>
+lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
+  using C = I8Cfg<FULL, CP>;
+  return launch_units<FULL, C::kSmem, C::kThreads, C::kST, attn_i8_kernel<FULL, CP>>(p, st);
 }

@@ -111,10 +111,10 @@ struct I8Cfg {
   static constexpr int kGroups = CP == 32 ? 2 : 1;
   static constexpr int kCG = CP / kGroups;               // columns of a column group
   static constexpr int kTeamWarps = 4 * kGroups, kTeamThreads = 32 * kTeamWarps;
-  // (4 columns: four teams at 95 registers without spills and an 8-stage ring measure 2 % below five teams at
-  // 80 registers on one launch over 32 flattened layers, but 11 % faster on one launch per layer and 3-12 %
-  // faster on short and ragged contexts, where pieces end often)
-  static constexpr int kTeams = CP == 32 ? 2 : (FULL || CP == 16) ? 3 : CP == 4 ? 4 : 5;
+  // (4 and 8 columns: four teams.  Five teams have 80 registers a thread and spill: at 4 columns 11 % slower on one launch
+  // per layer and 3-12 % on short and ragged contexts; at 8 columns, 16 flattened layers of two sequences of 131072
+  // tokens, 1095 us with products issued behind a lane test and 1310 us by an elected lane, against 1055 us for four teams.)
+  static constexpr int kTeams = CP == 32 ? 2 : (FULL || CP == 16) ? 3 : 4;
   static constexpr int kProdWarps = CP == 32 ? 2 : 4;
   static constexpr int kProdWarp0 = kTeamWarps * kTeams;
   static constexpr int kThreads = (kProdWarp0 + kProdWarps) * 32;
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   float* my_lz = my_scal + 16 * CP;               // [2 CP]
   const int tw = grp * 4 + w4;                    // warp of the team
   int* my_misc = misc + 64 * (1 + tm);
-  const int bar_tm = 1 + tm;                      // named barrier of this team
+  const int bar_tm = 1 + tm, bar_k = 10 + tm;     // named barriers of this team
   const uint32_t vtile = sbase + tm * C::kTeamBytes, ptile = vtile + C::kTile;
   float* my_hdr = reinterpret_cast<float*>(smem + tm * C::kTeamBytes + C::kTile);   // [3 CP] l, zs, ref of this team's deposit (in its idle P tile)
   const uint32_t tm_k = tmem0 + tm * C::kTmTeam + C::kTmK;
@@ -813,11 +813,15 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           i8_expand<FULL>(st + C::kOffVA, st + C::kOffVR, vtile, w4, lane);
         }
         tc_fence_before();
-        named_bar(bar_tm, TT);
+        // (only the issuing warp waits for the others' K levels: they go on to the V tile.  An elected lane issues: the
+        // operands stay on the uniform datapath, see tc_elect.  Both together: one layer of 131072 tokens 42.4 -> 40.0 us
+        // at 4 columns, 16 ragged sequences at 16 columns 340 -> 335 us, 4096 tokens at 16 columns 29.0 -> 27.8 us.)
+        if (tw != 0) bar_arrive(bar_k, TT);
+        else named_bar(bar_k, TT);
         if (tw == 0) {
           if (u == u_first) mbar_wait(qready0 + qi * 8, (ic >> 1) & 1, abort_word);   // the piece's query planes
           tc_fence_after();
-          if (lane == 0) {
+          if (tc_elect()) {
             const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmS;
             const uint32_t qd_lo = qd_lo0 + (uint32_t)qi * (C::kQTile >> 4);
 #pragma unroll
@@ -959,7 +963,10 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
                            "r"(wi[4 * j + 2]), "r"(wi[4 * j + 3]) : "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_before();
-          named_bar(bar_tm, TT);     // the P tile and the V tile are complete, S has been read
+          // the P tile and the V tile are complete, S has been read: the issuing warp waits for it, the others only where
+          // the restart flag is looked at afterwards
+          if (C::kVoteFirst && tw != 0) bar_arrive(bar_tm, TT);
+          else named_bar(bar_tm, TT);
         };
         if (C::kVoteFirst) {   // (every instance but the 4-column anchor one measures faster with the question asked first)
           if (bar_or(bar_tm, TT, forced || over)) restart();
@@ -976,7 +983,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         }
         if (tw == 0) {
           tc_fence_after();
-          if (lane == 0) {
+          if (tc_elect()) {
             const uint32_t d = tmem0 + tm * C::kTmTeam + C::kTmO;
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4)

@@ -144,17 +144,10 @@ class Workload:
         return n
 
     def verify_kernels(self, k):
-        """Kernels of one merge-verify call: one attention launch per slice of the window (the library takes up
-        to 16 columns per launch on the integer kernel and runs 17..32 columns as two such passes; up to 16
-        positions and 64 columns on the FP16 kernel), plus the decision kernel when there is more than one."""
+        """Kernels of one merge-verify call: one attention launch per slice of the window (a launch takes up to 16
+        positions and 64 columns), plus the decision kernel when there is more than one."""
         G = self.wl.num_q_heads // self.wl.num_kv_heads
-        cols = k * G
-        if 16 < cols <= 32 and 16 // G > 0:
-            per = 16 // G
-        elif k <= 16 and cols <= 64:
-            per = k
-        else:
-            per = min(16, max(1, 64 // G))
+        per = k if k <= 16 and k * G <= 64 else min(16, max(1, 64 // G))
         slices = -(-k // per)
         return slices + (1 if slices > 1 else 0)
 

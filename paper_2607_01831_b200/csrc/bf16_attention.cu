@@ -48,6 +48,7 @@ __device__ __forceinline__ float ex2f(float x) {
 // COLS query columns (padded), LPT lanes per token
 template <int COLS, int LPT>
 __global__ void __launch_bounds__(kWarps * 32, COLS <= 4 ? 2 : 1) bf16_decode_kernel(const BfParams p) {
+  pdl_begin();
   constexpr int DPL = LYNX_D / LPT;      // dims per lane: 16 or 8
   constexpr int TPP = 32 / LPT;          // tokens per pass of a warp: 4 or 2
   constexpr int NV = DPL / 8;            // 128-bit loads per row and lane
@@ -244,6 +245,7 @@ __device__ __forceinline__ uint32_t bf16x2_of(float lo, float hi) {
 template <int COLS>
 __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const BfParams p) {
   extern __shared__ __align__(128) unsigned char smem_tc[];
+  pdl_begin();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int chunk = blockIdx.x % p.chunks, bh = blockIdx.x / p.chunks;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv;
@@ -406,6 +408,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
 // One CTA per (sequence, KV head, column): merges the chunk partials, normalises, writes the output.
 template <int COLS>
 __global__ void __launch_bounds__(LYNX_D) bf16_combine_kernel(const BfParams p) {
+  pdl_begin();
   const int c = blockIdx.x % COLS, bh = blockIdx.x / COLS;
   if (c >= p.ncols) return;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv, d = threadIdx.x;
@@ -442,11 +445,9 @@ __global__ void __launch_bounds__(LYNX_D) bf16_combine_kernel(const BfParams p) 
 
 template <int COLS, int LPT>
 lynx_status launch_bf16(const BfParams& p, cudaStream_t st) {
-  bf16_decode_kernel<COLS, LPT><<<(unsigned)(p.B * p.Hkv * p.chunks), kWarps * 32, 0, st>>>(p);
-  lynx_status rc = launch_status();
+  const lynx_status rc = launch_pdl(bf16_decode_kernel<COLS, LPT>, (unsigned)(p.B * p.Hkv * p.chunks), kWarps * 32, 0, st, p);
   if (rc != LYNX_OK) return rc;
-  bf16_combine_kernel<COLS><<<(unsigned)(p.B * p.Hkv * COLS), LYNX_D, 0, st>>>(p);
-  return launch_status();
+  return launch_pdl(bf16_combine_kernel<COLS>, (unsigned)(p.B * p.Hkv * COLS), LYNX_D, 0, st, p);
 }
 
 template <int COLS>
@@ -461,11 +462,9 @@ lynx_status launch_bf16_tc(const BfParams& p, cudaStream_t st) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  kern<<<(unsigned)(p.B * p.Hkv * p.chunks), kTcWarps * 32, kSmem, st>>>(p);
-  lynx_status rc = launch_status();
+  const lynx_status rc = launch_pdl(kern, (unsigned)(p.B * p.Hkv * p.chunks), kTcWarps * 32, kSmem, st, p);
   if (rc != LYNX_OK) return rc;
-  bf16_combine_kernel<COLS><<<(unsigned)(p.B * p.Hkv * COLS), LYNX_D, 0, st>>>(p);
-  return launch_status();
+  return launch_pdl(bf16_combine_kernel<COLS>, (unsigned)(p.B * p.Hkv * COLS), LYNX_D, 0, st, p);
 }
 
 // bytes of the chunk partials, rounded up to 256: the log-sum-exps follow them in the workspace

@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
   const uint32_t page_s = (uint32_t)__cvta_generic_to_shared(smem);
   const int tid = threadIdx.x, q = tid & 15, half = (tid >> 4) & 1, ch = tid >> 5;
   const int row0 = ch * kC + half * (kC / 2);
+  pdl_begin();
   for (int pg = blockIdx.x; pg < n_pages; pg += gridDim.x) {
     const uint4* gsrc = reinterpret_cast<const uint4*>(src + (size_t)pg * kP * LYNX_D);
     __syncthreads();                                                  // the previous page is done with shared memory
@@ -297,6 +298,7 @@ __global__ void __launch_bounds__(128, FULL ? 4 : 6) hier_dequantize_kernel(cons
     for (int i = tid; i < kEntries * kCopies; i += 128) table[i] = table[i & ~(kCopies - 1)];
     __syncthreads();
   }
+  pdl_begin();   // (the table above does not depend on anything before this kernel)
   const uint32_t lane4 = (uint32_t)(tid & 31) << 2;
   const int ch = tid >> 4, oc = tid & 15;                                     // chunk, octet of channels
   constexpr int kB = 8;                                                       // tokens per batch of loads
@@ -387,9 +389,8 @@ extern "C" lynx_status lynx_hier_quantize(const void* src_bf16, int64_t n_pages,
     configured[dev] = true;
   }
   const int64_t grid = n_pages < (int64_t)sm_count() * 3 ? n_pages : (int64_t)sm_count() * 3;
-  hier_quantize_kernel<<<(unsigned)grid, 256, kSmem, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __nv_bfloat16*>(src_bf16), (int)n_pages, q_anc, q_res, gamma_min, gamma_scale, mu, sigma);
-  return launch_status();
+  return launch_pdl(hier_quantize_kernel, (unsigned)grid, 256, kSmem, stream, static_cast<const __nv_bfloat16*>(src_bf16), (int)n_pages,
+                    q_anc, q_res, gamma_min, gamma_scale, mu, sigma);
 }
 
 extern "C" lynx_status lynx_hier_dequantize(const uint8_t* q_anc, const uint8_t* q_res, int64_t n_pages,
@@ -403,11 +404,6 @@ extern "C" lynx_status lynx_hier_dequantize(const uint8_t* q_anc, const uint8_t*
     return LYNX_ERR_ALIGN;
   if (!aligned16(q_anc) || (q_res && !aligned16(q_res))) return LYNX_ERR_ALIGN;
   const int64_t grid = n_pages < (int64_t)sm_count() * 16 ? n_pages : (int64_t)sm_count() * 16;
-  if (q_res)
-    hier_dequantize_kernel<true><<<(unsigned)grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        q_anc, q_res, (int)n_pages, gamma_min, gamma_scale, mu, sigma, static_cast<__nv_bfloat16*>(dst_bf16));
-  else
-    hier_dequantize_kernel<false><<<(unsigned)grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        q_anc, q_anc, (int)n_pages, gamma_min, gamma_scale, mu, sigma, static_cast<__nv_bfloat16*>(dst_bf16));
-  return launch_status();
+  return launch_pdl(q_res ? hier_dequantize_kernel<true> : hier_dequantize_kernel<false>, (unsigned)grid, 128, 0, stream, q_anc,
+                    q_res ? q_res : q_anc, (int)n_pages, gamma_min, gamma_scale, mu, sigma, static_cast<__nv_bfloat16*>(dst_bf16));
 }

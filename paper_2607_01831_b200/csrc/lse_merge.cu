@@ -14,6 +14,7 @@ namespace {
 __global__ void __launch_bounds__(256) lse_merge_kernel(const float4* __restrict__ out_a, const float* __restrict__ lse_a,
                                                         const float4* __restrict__ out_b, const float* __restrict__ lse_b,
                                                         int64_t n_rows, float4* out, float* lse_out) {
+  pdl_begin();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= n_rows) return;
   const int lane = threadIdx.x & 31;
@@ -44,8 +45,6 @@ extern "C" lynx_status lynx_lse_merge(const float* out_a, const float* lse_a, co
   if (n_rows < 0 || n_rows > (1ll << 40)) return LYNX_ERR_SHAPE;
   if (!out_a || !lse_a || !out_b || !lse_b || !out) return LYNX_ERR_NULL;
   if (!aligned16(out_a) || !aligned16(out_b) || !aligned16(out)) return LYNX_ERR_ALIGN;
-  lse_merge_kernel<<<(unsigned)((n_rows + 7) / 8), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<const float4*>(out_a), lse_a, reinterpret_cast<const float4*>(out_b), lse_b, n_rows,
-      reinterpret_cast<float4*>(out), lse_out);
-  return launch_status();
+  return launch_pdl(lse_merge_kernel, (unsigned)((n_rows + 7) / 8), 256, 0, stream, reinterpret_cast<const float4*>(out_a), lse_a,
+                    reinterpret_cast<const float4*>(out_b), lse_b, n_rows, reinterpret_cast<float4*>(out), lse_out);
 }

@@ -80,6 +80,7 @@ split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
                       const int32_t* __restrict__ block_ids, uint32_t rows_per_block,
                       int64_t n_blocks_total, uint32_t* __restrict__ anchor,
                       uint32_t* __restrict__ residual, float2* __restrict__ meta) {
+  pdl_begin();
   const int ln = threadIdx.x & (kLanesPerRow - 1);
   const int64_t grp = (int64_t)blockIdx.x * (kThreads / kLanesPerRow) + (threadIdx.x / kLanesPerRow);
   const int64_t grp_total = (int64_t)gridDim.x * (kThreads / kLanesPerRow);
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(kThreads)
 recombine_kernel(const uint32_t* __restrict__ anchor, const uint32_t* __restrict__ residual,
                  const float2* __restrict__ meta, int64_t n_rows, uint2* __restrict__ codes,
                  uint4* __restrict__ deq) {
+  pdl_begin();
   const int64_t n_items = n_rows * 16;  // 16 lanes per row, 8 elements per lane
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   constexpr int kAhead = 4;             // items per thread and trip: their loads are issued together
@@ -209,7 +211,6 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
   if (!aligned16(src_bf16) || !aligned16(anchor) || !aligned16(residual) ||
       (reinterpret_cast<uintptr_t>(meta) & 7u))
     return LYNX_ERR_ALIGN;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int rows_per_cta_trip = (kThreads / kLanesPerRow) * (block_ids ? kRowsInFlightIds : kRowsInFlight);
   if (block_ids) {
     if (n_block_ids < 0 || rows_per_block <= 0 || n_rows % rows_per_block != 0) return LYNX_ERR_SHAPE;
@@ -217,18 +218,14 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
     const int64_t logical = (int64_t)n_block_ids * rows_per_block;
     if (logical >= (1ll << 31)) return LYNX_ERR_UNSUPPORTED;
     const int grid = grid_for((logical + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
-    split_quantize_kernel<true><<<grid, kThreads, 0, st>>>(
-        static_cast<const uint4*>(src_bf16), logical, block_ids, (uint32_t)rows_per_block,
-        n_rows / rows_per_block, reinterpret_cast<uint32_t*>(anchor),
-        reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta));
-  } else {
-    const int grid = grid_for((n_rows + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
-    split_quantize_kernel<false><<<grid, kThreads, 0, st>>>(
-        static_cast<const uint4*>(src_bf16), n_rows, nullptr, 1u, n_rows,
-        reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),
-        reinterpret_cast<float2*>(meta));
+    return launch_pdl(split_quantize_kernel<true>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), logical, block_ids,
+                      (uint32_t)rows_per_block, n_rows / rows_per_block, reinterpret_cast<uint32_t*>(anchor),
+                      reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta));
   }
-  return launch_status();
+  const int grid = grid_for((n_rows + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
+  return launch_pdl(split_quantize_kernel<false>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), n_rows, nullptr, 1u,
+                    n_rows, reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),
+                    reinterpret_cast<float2*>(meta));
 }
 
 extern "C" lynx_status lynx_recombine(const uint8_t* anchor, const uint8_t* residual,
@@ -242,18 +239,13 @@ extern "C" lynx_status lynx_recombine(const uint8_t* anchor, const uint8_t* resi
   if (!aligned16(anchor) || !aligned16(residual) || !aligned16(codes_u8) ||
       !aligned16(dequant_bf16) || (reinterpret_cast<uintptr_t>(meta) & 7u))
     return LYNX_ERR_ALIGN;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int grid = grid_for((n_rows * 16 + kThreads - 1) / kThreads, 8);
   const uint32_t* a = reinterpret_cast<const uint32_t*>(anchor);
   const uint32_t* r = reinterpret_cast<const uint32_t*>(residual);
   const float2* m = reinterpret_cast<const float2*>(meta);
   uint2* c = reinterpret_cast<uint2*>(codes_u8);
   uint4* d = static_cast<uint4*>(dequant_bf16);
-  if (codes_u8 && dequant_bf16)
-    recombine_kernel<true, true><<<grid, kThreads, 0, st>>>(a, r, m, n_rows, c, d);
-  else if (codes_u8)
-    recombine_kernel<true, false><<<grid, kThreads, 0, st>>>(a, r, m, n_rows, c, d);
-  else
-    recombine_kernel<false, true><<<grid, kThreads, 0, st>>>(a, r, m, n_rows, c, d);
-  return launch_status();
+  if (codes_u8 && dequant_bf16) return launch_pdl(recombine_kernel<true, true>, grid, kThreads, 0, stream, a, r, m, n_rows, c, d);
+  if (codes_u8) return launch_pdl(recombine_kernel<true, false>, grid, kThreads, 0, stream, a, r, m, n_rows, c, d);
+  return launch_pdl(recombine_kernel<false, true>, grid, kThreads, 0, stream, a, r, m, n_rows, c, d);
 }

@@ -5,10 +5,10 @@
 // byte, one-contiguous-buffer-per-stream packing of the Compression Kernel paragraph.
 // Recombine is the Residual-phase refinement to Q_full of Section 4.2.
 //
-// Mapping: a row is 256 B of BF16; a quarter-warp (8 lanes) owns a row: two 128-bit streaming
-// loads per lane (each instruction covers 128 contiguous bytes of the row), min/max on packed
-// BF16 pairs and three xor-shuffles, 16 codes per lane, 2 x 4 B of each plane per lane.
-// Eight rows are in flight per quarter-warp.
+// Mapping: a row is 256 B of BF16; a quarter-warp (8 lanes) owns a row: a 256-bit streaming load
+// per lane (two 128-bit ones where the source is only 16-byte aligned), min/max on packed BF16
+// pairs and three xor-shuffles, 16 consecutive codes per lane, 8 B of each plane per lane.
+// Four rows are in flight per quarter-warp.
 #include <cuda_bf16.h>
 
 #include "lynx_common.cuh"
@@ -18,10 +18,11 @@ namespace lynx {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kLanesPerRow = 8;   // a quarter-warp owns a row: 2 x 16 B per lane
-// rows per quarter-warp per loop trip: dense rows 8 (2: 0.84, 4: 0.87, 8: 0.90 of the copy rate; 12:
-// spills); rows of listed blocks 4 (2: 0.81, 4: 0.87, 8: 0.77: the block lookups cost registers)
-constexpr int kRowsInFlight = 8;
+constexpr int kLanesPerRow = 8;   // a quarter-warp owns a row: 32 B per lane
+// rows per quarter-warp per loop trip.  Dense rows 4: with the 256-bit loads more warps per SM are worth more than more
+// rows per warp (6.6 GB of planes and source: 8 rows 1215 us, 4 rows 1111 us, 0.90 of the copy rate).  Rows of listed
+// blocks 4 (2: 0.81, 4: 0.87, 8: 0.77 with 128-bit loads: the block lookups cost registers)
+constexpr int kRowsInFlight = 4;
 constexpr int kRowsInFlightIds = 4;
 
 // Round-half-even of the exact product u*inv, as the low byte of an FP32 whose ulp is 1:
@@ -38,6 +39,12 @@ __device__ __forceinline__ uint32_t bf2max(uint32_t a, uint32_t b) {
   uint32_t d;
   asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
+}
+
+// 32 contiguous bytes per lane in one instruction (the address must be 32-byte aligned)
+__device__ __forceinline__ void ld256_cs(const void* p, uint4& a, uint4& b) {
+  asm volatile("ld.global.cs.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
 }
 
 // Two FP32 values in a register pair, one instruction for both (IEEE round-to-nearest per element, as the
@@ -79,7 +86,7 @@ __global__ void __launch_bounds__(kThreads)
 split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
                       const int32_t* __restrict__ block_ids, uint32_t rows_per_block,
                       int64_t n_blocks_total, uint32_t* __restrict__ anchor,
-                      uint32_t* __restrict__ residual, float2* __restrict__ meta) {
+                      uint32_t* __restrict__ residual, float2* __restrict__ meta, bool wide) {
   pdl_begin();
   const int ln = threadIdx.x & (kLanesPerRow - 1);
   const int64_t grp = (int64_t)blockIdx.x * (kThreads / kLanesPerRow) + (threadIdx.x / kLanesPerRow);
@@ -104,9 +111,14 @@ split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
         }
       }
       lo[u] = hi[u] = make_uint4(0, 0, 0, 0);
-      if (row[u] >= 0) {
-        lo[u] = __ldcs(src + row[u] * 16 + ln);      // elements 8*ln .. 8*ln+7
-        hi[u] = __ldcs(src + row[u] * 16 + 8 + ln);  // elements 64+8*ln .. 64+8*ln+7
+      if (row[u] >= 0) {   // elements 16*ln .. 16*ln+7 and 16*ln+8 .. 16*ln+15
+        const uint4* p = src + row[u] * 16 + 2 * ln;
+        if (wide) {
+          ld256_cs(p, lo[u], hi[u]);
+        } else {
+          lo[u] = __ldcs(p);
+          hi[u] = __ldcs(p + 1);
+        }
       }
     }
 #pragma unroll
@@ -136,10 +148,8 @@ split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
       codes8(wl, mn, inv, a_lo, r_lo);
       codes8(wh, mn, inv, a_hi, r_hi);
       if (row[u] >= 0) {
-        __stcs(anchor + row[u] * 16 + ln, a_lo);
-        __stcs(anchor + row[u] * 16 + 8 + ln, a_hi);
-        __stcs(residual + row[u] * 16 + ln, r_lo);
-        __stcs(residual + row[u] * 16 + 8 + ln, r_hi);
+        __stcs(reinterpret_cast<uint2*>(anchor) + row[u] * 8 + ln, make_uint2(a_lo, a_hi));
+        __stcs(reinterpret_cast<uint2*>(residual) + row[u] * 8 + ln, make_uint2(r_lo, r_hi));
         if (ln == 0) __stcs(meta + row[u], make_float2(scale, zero));
       }
     }
@@ -211,6 +221,7 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
   if (!aligned16(src_bf16) || !aligned16(anchor) || !aligned16(residual) ||
       (reinterpret_cast<uintptr_t>(meta) & 7u))
     return LYNX_ERR_ALIGN;
+  const bool wide = (reinterpret_cast<uintptr_t>(src_bf16) & 31u) == 0;   // 256-bit loads of the source rows
   const int rows_per_cta_trip = (kThreads / kLanesPerRow) * (block_ids ? kRowsInFlightIds : kRowsInFlight);
   if (block_ids) {
     if (n_block_ids < 0 || rows_per_block <= 0 || n_rows % rows_per_block != 0) return LYNX_ERR_SHAPE;
@@ -220,12 +231,12 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
     const int grid = grid_for((logical + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
     return launch_pdl(split_quantize_kernel<true>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), logical, block_ids,
                       (uint32_t)rows_per_block, n_rows / rows_per_block, reinterpret_cast<uint32_t*>(anchor),
-                      reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta));
+                      reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta), wide);
   }
   const int grid = grid_for((n_rows + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
   return launch_pdl(split_quantize_kernel<false>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), n_rows, nullptr, 1u,
                     n_rows, reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),
-                    reinterpret_cast<float2*>(meta));
+                    reinterpret_cast<float2*>(meta), wide);
 }
 
 extern "C" lynx_status lynx_recombine(const uint8_t* anchor, const uint8_t* residual,

@@ -20,7 +20,8 @@
 //   warps 12-15  V codes into the V tile
 //   warps 16-19  producers (tensor-map copies of 16-token sub-blocks): two warps for the K ring, two for the V ring
 //   warp 20      issues every tcgen05.mma
-//   warps 21, 22 the per-token scalars of the scores and weights (warp 23 completes the warpgroup, for the register split)
+//   warps 21, 22 the per-token scalars of the scores and weights at 32 columns (the rest completes the warpgroup, for the
+//                register split)
 // With 64 columns the groups take one half of the columns each of every unit; with 32 they alternate over the units
 // (separate accumulators, merged at the end of a piece), which spares the per-token work of a second group.
 // Why specialised warps here and teams in attention_i8.cuh: at these widths the accumulators of teams do not fit tensor
@@ -34,7 +35,7 @@
 // of 32 columns over one), rolled expansion loops (the roles compete for the instruction caches: 118 -> 98 us at 32
 // columns), products issued by an elected lane (93 -> 30 cycles each).  One layer of 131072 tokens: 174 us as two passes of
 // the 16-column integer kernel -> 93 us (32 columns); 293 us by the previous kernel (M = columns, codes not centred) ->
-// 260 us (64 columns, batch 2).
+// 251 us (64 columns, batch 2).
 
 template <int NC>
 struct F16Cfg {
@@ -66,6 +67,9 @@ struct F16Cfg {
   // units between drains: each adds 8 truncating products to a sum.  (64 columns against 64 bits: 3.3e-4 by the previous
   // FP16 kernel, 5e-6 here; a drain per 8 units costs 6 % of its time, one per 16 units 3 %.)
   static constexpr int kDrainUnits = NC == 64 ? 16 : 8;
+  // who computes the per-token scalars: with 64 columns the K warps have the time (261 -> 256 us), with 32 they are the
+  // slower stage and two spare warps do it (96.1 us, 97.4 us in the K warps)
+  static constexpr bool kMetaK = kSplit;
   // registers per thread after the split (launched with 80 each): 256 * 136 + 256 * 64 + 128 * 56 + 128 * 24 = 768 * 80
   static constexpr int kRegSoft = 128, kRegExp = 64, kRegProd = 56, kRegMma = 40;
 };
@@ -221,12 +225,14 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
           for (int i = 0; i < 4; ++i) bytes += rows[i] != 0xFFFFFFFFu ? 2048u : 0u;
           if (bytes) mbar_expect_tx(bar, bytes);
           else mbar_arrive(bar);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (rows[i] != 0xFFFFFFFFu) {
-              tma_rows16(dst + i * 1024, map_a, (int)rows[i], bar);
-              tma_rows16(dst + 8192 + i * 1024, map_r, (int)rows[i], bar);
+#pragma unroll 1
+          for (int i = 0; i < 4; ++i) {   // (rolled, for the instruction caches: 256 -> 251 us at 64 columns)
+            const uint32_t row = my_blk[4 * k + i];
+            if (row != 0xFFFFFFFFu) {
+              tma_rows16(dst + i * 1024, map_a, (int)row, bar);
+              tma_rows16(dst + 8192 + i * 1024, map_r, (int)row, bar);
             }
+          }
         }
         __syncwarp();
         if (++slot == nstage) { slot = 0; phase ^= 1; }
@@ -250,6 +256,67 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
     }
   }
 }
+
+// The per-token scalars of a unit, for N tokens (32 apart) of a thread: scale and offset of the scores, log2 of the value
+// scale, its reciprocal and the zero point in units of it.  Metadata is read two steps ahead: the block id of the unit after
+// next, the (scale, zero) pairs of the next unit.
+template <class C, int N>
+struct F16Meta {
+  float4* tok4;
+  float* tok1;
+  const int32_t* table;
+  int i0, bt_shift, ih, len, n_piece, u0;
+  int blk_n[N];
+  float2 km[N], vm[N];
+  __device__ __forceinline__ void init(const AttnParams& p, unsigned char* smem, int first) {
+    i0 = first;
+    tok4 = reinterpret_cast<float4*>(smem + C::kOffTok) + i0;
+    tok1 = reinterpret_cast<float*>(smem + C::kOffTok + 4 * 128 * 16) + i0;
+    bt_shift = (p.bt & (p.bt - 1)) == 0 ? 31 - __clz(p.bt) : -1;
+  }
+  __device__ __forceinline__ int blk_of(const AttnParams& p, int uu, int i) const {
+    const int t = (u0 + uu) * C::kST + i0 + 32 * i;
+    if (uu >= n_piece || t >= len) return 0;
+    return __ldg(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
+  }
+  __device__ __forceinline__ void meta_of(const AttnParams& p, int uu, int i, int blk) {
+    const int t = (u0 + uu) * C::kST + i0 + 32 * i;
+    km[i] = make_float2(0.f, 0.f); vm[i] = km[i];
+    if (uu >= n_piece || t >= len) return;
+    const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
+    blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
+    const uint32_t row = (uint32_t)(((size_t)blk * p.Hkv + ih) * p.bt + in_blk);
+    km[i] = __ldg(reinterpret_cast<const float2*>(p.km) + row);
+    vm[i] = __ldg(reinterpret_cast<const float2*>(p.vm) + row);
+  }
+  __device__ __forceinline__ void piece(const AttnParams& p, const Item& it) {
+    ih = it.hkv; len = it.len; n_piece = it.pad0; u0 = it.pad1;
+    table = p.block_table + (size_t)it.b * p.max_blocks;
+    int blk0[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) { blk0[i] = blk_of(p, 0, i); blk_n[i] = blk_of(p, 1, i); }
+#pragma unroll
+    for (int i = 0; i < N; ++i) meta_of(p, 0, i, blk0[i]);
+  }
+  __device__ __forceinline__ void unit(const AttnParams& p, int u, int gs, float ca) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const bool valid = (u0 + u) * C::kST + i0 + 32 * i < len;
+      if (C::kSplit && valid && !(vm[i].x < 16.0f)) atomicOr(p.ws_flags, kFlagRange);   // beyond the stated range of this width
+      const float sve = fmaxf(vm[i].x, 9.094947e-13f);   // floor 2^-40
+      const float ia = valid ? rcp_approx(sve) : 0.0f;
+      tok4[(gs & 3) * 128 + 32 * i] = make_float4(km[i].x * ca, fmaf(km[i].x, 128.0f, km[i].y) * p.sm_log2, lg2_approx(sve), ia);
+      tok1[(gs & 3) * 128 + 32 * i] = fmaf(sve, 128.0f, vm[i].y) * ia;
+    }
+  }
+  __device__ __forceinline__ void next(const AttnParams& p, int u) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      meta_of(p, u + 1, i, blk_n[i]);
+      blk_n[i] = blk_of(p, u + 2, i);
+    }
+  }
+};
 
 template <int NC>
 __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const AttnParams p,
@@ -280,7 +347,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     for (int i = 0; i < C::kRingV; ++i) { mbar_init(vfull + i * 8, 2); mbar_init(vempty + i * 8, 4); }
     for (int i = 0; i < 2; ++i) {
       mbar_init(qfull + i * 8, 1);
-      mbar_init(qempty + i * 8, 14);
+      mbar_init(qempty + i * 8, C::kMetaK ? 12 : 14);
       mbar_init(qready + i * 8, 4);
       mbar_init(kready + i * 8, 4);
       mbar_init(sfull + i * 8, 1);
@@ -290,7 +357,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       mbar_init(pready + i * 8, 4);
       mbar_init(pvdone + i * 8, 1);
     }
-    for (int i = 0; i < 4; ++i) { mbar_init(mready + i * 8, 2); mbar_init(mfree + i * 8, SPLIT ? 8 : 4); }
+    for (int i = 0; i < 4; ++i) { mbar_init(mready + i * 8, C::kMetaK ? 4 : 2); mbar_init(mfree + i * 8, SPLIT ? 8 : 4); }
     for (int i = 0; i < 64; ++i) misc[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -623,6 +690,9 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     const int kt = tid - 256, w4 = warp & 3;
     const uint32_t tm_k = tmem0 + C::kTmK + ((uint32_t)(w4 * 32) << 16);
     float* amax_s = reinterpret_cast<float*>(misc + 48);
+    F16Meta<C, 1> meta;
+    float ca = 0.0f;
+    if (C::kMetaK) meta.init(p, smem, kt);
     int gs = 0, ic = 0, slot = 0;
     uint32_t phase = 0;
     while (gs < n_units) {
@@ -663,7 +733,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         if (amax > 0.0f && amax < INFINITY) e = 14 - (((__float_as_int(amax) >> 23) & 0xFF) - 127);
         e = max(-100, min(100, e));
         const float up = __int_as_float((127 + e) << 23);
-        if (kt == 0) reinterpret_cast<int*>(scal)[4 * NC + qi] = e;
+        if (C::kMetaK) ca = p.sm_log2 * __int_as_float((127 - e) << 23);
+        else if (kt == 0) reinterpret_cast<int*>(scal)[4 * NC + qi] = e;
         if (kt < NC) reinterpret_cast<int*>(scal)[2 * NC + qi * NC + kt] =
             kt < p.ncols ? (p.causal ? len - p.tail + kt / p.G + 1 : len) : 0;
         if (gs > 0) mbar_wait_in(sfull + ((gs - 1) & 1) * 8, ((gs - 1) >> 1) & 1, abort_word);   // the previous piece's last Q.K^T
@@ -685,7 +756,16 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         named_bar(4, 128);
         if (lane == 0) { mbar_arrive(qready + qi * 8); mbar_arrive(qempty + qi * 8); }
       }
+      // (the item is still there: the softmax groups have not left the piece)
+      if (C::kMetaK) meta.piece(p, items[qi]);
       for (int u = 0; u < n_piece; ++u, ++gs) {
+        if (C::kMetaK) {
+          if (gs >= 4) mbar_wait_in(mfree + (gs & 3) * 8, ((gs >> 2) - 1) & 1, abort_word);
+          meta.unit(p, u, gs, ca);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(mready + (gs & 3) * 8);
+          meta.next(p, u);
+        }
         mbar_wait_in(kfull + slot * 8, phase, abort_word);
         if (gs >= 2) mbar_wait_in(sfull + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);   // Q.K^T of the unit before last
         tc_fence_after();
@@ -731,59 +811,23 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   // ================================================================================== products
   reg_dec<C::kRegMma>();
   // ---- per-token scalars of the scores and weights (warps 21, 22: a lane has tokens 64 w + lane and 32 further on) ----
-  if (warp == 21 || warp == 22) {
-    const int i0 = (warp - 21) * 64 + lane;
-    float4* tok4 = reinterpret_cast<float4*>(smem + C::kOffTok) + i0;
-    float* tok1 = reinterpret_cast<float*>(smem + C::kOffTok + 4 * 128 * 16) + i0;
-    const int bt_shift = (p.bt & (p.bt - 1)) == 0 ? 31 - __clz(p.bt) : -1;
+  if (!C::kMetaK && (warp == 21 || warp == 22)) {
+    F16Meta<C, 2> meta;
+    meta.init(p, smem, (warp - 21) * 64 + lane);
     int gs = 0, ic = 0;
     while (gs < n_units) {
       const int qi = ic & 1;
       mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
-      const int ih = items[qi].hkv, len = items[qi].len, n_piece = items[qi].pad0, u0 = items[qi].pad1;
-      const int32_t* table = p.block_table + (size_t)items[qi].b * p.max_blocks;
-      // metadata is read two steps ahead: the block id of the unit after next, the (scale, zero) pairs of the next unit
-      auto blk_of = [&](int uu, int i) -> int {
-        const int t = (u0 + uu) * C::kST + i0 + 32 * i;
-        if (uu >= n_piece || t >= len) return 0;
-        return __ldg(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
-      };
-      auto meta_of = [&](int uu, int i, int blk, float2& k2, float2& v2) {
-        const int t = (u0 + uu) * C::kST + i0 + 32 * i;
-        k2 = make_float2(0.f, 0.f); v2 = k2;
-        if (uu >= n_piece || t >= len) return;
-        const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
-        blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
-        const uint32_t row = (uint32_t)(((size_t)blk * p.Hkv + ih) * p.bt + in_blk);
-        k2 = __ldg(reinterpret_cast<const float2*>(p.km) + row);
-        v2 = __ldg(reinterpret_cast<const float2*>(p.vm) + row);
-      };
-      int blk0[2], blk_n[2];
-      float2 km[2], vm[2];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) { blk0[i] = blk_of(0, i); blk_n[i] = blk_of(1, i); }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) meta_of(0, i, blk0[i], km[i], vm[i]);
+      meta.piece(p, items[qi]);
+      const int n_piece = items[qi].pad0;
       mbar_wait_in(qready + qi * 8, (ic >> 1) & 1, abort_word);
       const float ca = p.sm_log2 * __int_as_float((127 - reinterpret_cast<const int*>(scal)[4 * NC + qi]) << 23);
       for (int u = 0; u < n_piece; ++u, ++gs) {
         if (gs >= 4) mbar_wait_in(mfree + (gs & 3) * 8, ((gs >> 2) - 1) & 1, abort_word);
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const bool valid = (u0 + u) * C::kST + i0 + 32 * i < len;
-          if (SPLIT && valid && !(vm[i].x < 16.0f)) atomicOr(p.ws_flags, kFlagRange);   // beyond the stated range of this width
-          const float sve = fmaxf(vm[i].x, 9.094947e-13f);   // floor 2^-40
-          const float ia = valid ? rcp_approx(sve) : 0.0f;
-          tok4[(gs & 3) * 128 + 32 * i] = make_float4(km[i].x * ca, fmaf(km[i].x, 128.0f, km[i].y) * p.sm_log2, lg2_approx(sve), ia);
-          tok1[(gs & 3) * 128 + 32 * i] = fmaf(sve, 128.0f, vm[i].y) * ia;
-        }
+        meta.unit(p, u, gs, ca);
         __syncwarp();
         if (lane == 0) mbar_arrive(mready + (gs & 3) * 8);
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          meta_of(u + 1, i, blk_n[i], km[i], vm[i]);
-          blk_n[i] = blk_of(u + 2, i);
-        }
+        meta.next(p, u);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(qempty + qi * 8);

@@ -138,7 +138,8 @@ lynx_status lynx_anchor_attention(const lynx_shape* shape, const void* q_bf16, i
  * and first_reject[b] = smallest j with dev[b][j] > 1, or k if none (the longest agreeing
  * prefix; out_full at that position is the correction).
  * draft_out : [batch][k][Hq][128] float, the Anchor-state results being verified; may be NULL,
- * then dev / first_reject are not written (and may be NULL).  out_full : same shape, float.
+ * then dev / first_reject are not written (and may be NULL).  It needs the alignment of a float only (a view into a
+ * larger buffer); 16-byte alignment is read faster.  out_full : same shape, float.
  * k must be <= 64.  Up to 16 columns k * (Hq/Hkv) are one launch of the exact integer kernel and 17..32 two
  * passes of it; 33..64 columns (up to 16 positions) are one launch of a kernel whose weights are FP16
  * numbers; a longer window runs as slices of whole positions (a pass over the planes each).  With several

@@ -63,6 +63,7 @@ struct AttnParams {
   // position j0): nq_stride = the caller's n_q (positions per sequence in q and out), tail = n_q - j0
   // (the causal limit of position j of the slice is len - tail + j + 1).  Unsliced: both equal nq.
   int nq_stride, tail;
+  int draft_vec;   // draft is 16-byte aligned: its rows are read four values at a time
 };
 
 // ------------------------------------------------------------------ PTX helpers
@@ -178,6 +179,14 @@ __device__ __forceinline__ void merge_codes(uint32_t xa, uint32_t xr, uint32_t& 
 // and the sum L of 2^(score - M); -inf for a row that saw no token.
 __device__ __forceinline__ float lse_of(float M, float L) {
   return L > 0.0f ? (M + __log2f(L)) * 0.6931471805599453f : -INFINITY;
+}
+
+// Values 4 lane .. 4 lane + 3 of the draft row at float offset `off`.  The interface asks for no more than the alignment
+// of a float: callers hold the draft inside larger buffers.
+__device__ __forceinline__ float4 draft_row(const AttnParams& p, size_t off, int lane) {
+  const float* d = p.draft + off + 4 * lane;
+  if (p.draft_vec) return __ldg(reinterpret_cast<const float4*>(d));
+  return make_float4(__ldg(d), __ldg(d + 1), __ldg(d + 2), __ldg(d + 3));
 }
 
 struct Item {  // one piece: a run of stage-units of one (sequence, KV head) given to one CTA
@@ -322,7 +331,7 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
 #pragma unroll
         for (int c = 0; c < kCC; ++c)
           if (decide && top)
-            dr[c] = __ldg(reinterpret_cast<const float4*>(p.draft + (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D) + lane);
+            dr[c] = draft_row(p, (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D, lane);
 #pragma unroll 1
         for (int c = 0; c < kCC && cw + c < p.ncols; ++c) {
           float4 a = acc[0], d = dr[0];
@@ -355,7 +364,7 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
 #pragma unroll 1
         for (int c = tid >> 5; c < p.ncols; c += kConsThreads / 32) {
           const size_t o = (size_t)row_off(c) * LYNX_D;
-          const float4 dr = __ldg(reinterpret_cast<const float4*>(p.draft + o) + lane);
+          const float4 dr = draft_row(p, o, lane);
           const float4 f = reinterpret_cast<const float4*>(p.out + o)[lane];
           deviation(f, dr, c / p.G);
         }
@@ -612,6 +621,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.va = V.anchor; p.vr = V.residual; p.vm = V.meta;
   p.block_table = block_table; p.seq_lens = seq_lens;
   p.out = out; p.draft = full ? draft : nullptr; p.first_reject = first_reject; p.dev = dev;
+  p.draft_vec = p.draft && aligned16(p.draft);   // (a slice starts whole rows of 512 bytes further on)
   p.ws_flags = reinterpret_cast<uint32_t*>(ws);
   p.ws_chunk_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_chunk_ctr);
   p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_seq_ctr);

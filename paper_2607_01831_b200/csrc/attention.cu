@@ -183,10 +183,13 @@ __device__ __forceinline__ float lse_of(float M, float L) {
 
 // Values 4 lane .. 4 lane + 3 of the draft row at float offset `off`.  The interface asks for no more than the alignment
 // of a float: callers hold the draft inside larger buffers.
+__device__ __forceinline__ float4 draft_row_vec(const AttnParams& p, size_t off, int lane) {
+  return ld_dep(reinterpret_cast<const float4*>(p.draft + off) + lane);
+}
 __device__ __forceinline__ float4 draft_row(const AttnParams& p, size_t off, int lane) {
+  if (p.draft_vec) return draft_row_vec(p, off, lane);
   const float* d = p.draft + off + 4 * lane;
-  if (p.draft_vec) return __ldg(reinterpret_cast<const float4*>(d));
-  return make_float4(__ldg(d), __ldg(d + 1), __ldg(d + 2), __ldg(d + 3));
+  return make_float4(ld_dep(d), ld_dep(d + 1), ld_dep(d + 2), ld_dep(d + 3));
 }
 
 struct Item {  // one piece: a run of stage-units of one (sequence, KV head) given to one CTA
@@ -330,15 +333,17 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
         float4 dr[kCC];
 #pragma unroll
         for (int c = 0; c < kCC; ++c)
-          if (decide && top)
-            dr[c] = draft_row(p, (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D, lane);
+          if (decide && top && p.draft_vec)   // (ahead of the stores; a draft that is not aligned is read row by row below)
+            dr[c] = draft_row_vec(p, (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D, lane);
 #pragma unroll 1
         for (int c = 0; c < kCC && cw + c < p.ncols; ++c) {
           float4 a = acc[0], d = dr[0];
 #pragma unroll
           for (int i = 1; i < kCC; ++i)
             if (c == i) { a = acc[i]; d = dr[i]; }
-          float* dst = top ? p.out + (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D : col + c * kPartStride;
+          const size_t off = (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D;
+          if (decide && top && !p.draft_vec) d = draft_row(p, off, lane);
+          float* dst = top ? p.out + off : col + c * kPartStride;
           reinterpret_cast<float4*>(dst)[lane] = a;
           if (decide && top) deviation(a, d, __shfl_sync(0xFFFFFFFFu, my_j, c));
         }
@@ -485,7 +490,7 @@ __device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, in
       for (int j = p.nq - 1; j >= 0; --j) {
         float worst = 0.0f;
         for (int i = lane; i < p.Hq * LYNX_D; i += 32)
-          worst = fmaxf(worst, fabsf(__ldg(p.draft + ((size_t)b * p.nq_stride + j) * p.Hq * LYNX_D + i)) / p.atol);
+          worst = fmaxf(worst, fabsf(ld_dep(p.draft + ((size_t)b * p.nq_stride + j) * p.Hq * LYNX_D + i)) / p.atol);
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xFFFFFFFFu, worst, off));
         if (lane == 0) p.dev[(size_t)b * p.nq_stride + j] = worst;
@@ -555,7 +560,7 @@ bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
 
 // Section 4.3's longest agreeing prefix over a window that was verified in slices: the smallest position
 // whose deviation exceeds 1, or the number of positions.
-__global__ void first_reject_kernel(const float* __restrict__ dev, int B, int nq, int32_t* __restrict__ first_reject) {
+__global__ void first_reject_kernel(const float* dev, int B, int nq, int32_t* __restrict__ first_reject) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   int fr = nq;
@@ -567,13 +572,13 @@ __global__ void first_reject_kernel(const float* __restrict__ dev, int B, int nq
 // Section 4.3's agreement test on outputs that are already in memory (a verification pass whose result was joined
 // with a BF16 tail first): dev[b][j] = max over heads and dims of |f - d| / (atol + rtol |f|), the arithmetic of
 // the decision fused into the verification kernels.  One CTA per (sequence, position).
-__global__ void __launch_bounds__(256) deviation_kernel(const float4* __restrict__ out_full, const float4* __restrict__ draft,
+__global__ void __launch_bounds__(256) deviation_kernel(const float4* out_full, const float4* draft,
                                                         int row_f4, float atol, float rtol, float* __restrict__ dev) {
   const float4* f = out_full + (size_t)blockIdx.x * row_f4;
   const float4* d = draft + (size_t)blockIdx.x * row_f4;
   float worst = 0.0f;
   for (int i = threadIdx.x; i < row_f4; i += 256) {
-    const float4 a = f[i], b = __ldg(d + i);
+    const float4 a = f[i], b = ld_dep(d + i);
     worst = fmaxf(worst, fabsf(a.x - b.x) / (atol + rtol * fabsf(a.x)));
     worst = fmaxf(worst, fabsf(a.y - b.y) / (atol + rtol * fabsf(a.y)));
     worst = fmaxf(worst, fabsf(a.z - b.z) / (atol + rtol * fabsf(a.z)));

@@ -168,7 +168,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
   const int sub0 = 4 * (pw & 1);
   const int cap = p.max_blocks * p.bt;
   auto clamp_len = [&](int b) {
-    int len = __ldg(p.seq_lens + b);
+    int len = ld_dep(p.seq_lens + b);
     return len < 0 ? 0 : (len > cap ? cap : len);
   };
   const uint32_t dst0 = sbase + (tensor ? C::kOffRV : C::kOffRK) + (uint32_t)(sub0 * 1024);
@@ -202,7 +202,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         const int t0 = (u + c0 + (i >> 2)) * ST + (sub0 + (i & 3)) * 16;
         uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
         if (t0 < len) {
-          int blk = __ldg(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
           if (blk < 0 || blk >= p.num_blocks) {
             atomicOr(p.ws_flags, kFlagBadBlock);
             blk = blk < 0 ? 0 : p.num_blocks - 1;
@@ -277,7 +277,7 @@ struct F16Meta {
   __device__ __forceinline__ int blk_of(const AttnParams& p, int uu, int i) const {
     const int t = (u0 + uu) * C::kST + i0 + 32 * i;
     if (uu >= n_piece || t >= len) return 0;
-    return __ldg(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
+    return ld_dep(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
   }
   __device__ __forceinline__ void meta_of(const AttnParams& p, int uu, int i, int blk) {
     const int t = (u0 + uu) * C::kST + i0 + 32 * i;
@@ -286,8 +286,8 @@ struct F16Meta {
     const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
     blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
     const uint32_t row = (uint32_t)(((size_t)blk * p.Hkv + ih) * p.bt + in_blk);
-    km[i] = __ldg(reinterpret_cast<const float2*>(p.km) + row);
-    vm[i] = __ldg(reinterpret_cast<const float2*>(p.vm) + row);
+    km[i] = ld_dep(reinterpret_cast<const float2*>(p.km) + row);
+    vm[i] = ld_dep(reinterpret_cast<const float2*>(p.vm) + row);
   }
   __device__ __forceinline__ void piece(const AttnParams& p, const Item& it) {
     ih = it.hkv; len = it.len; n_piece = it.pad0; u0 = it.pad1;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   if (warp >= 16 && warp < 20) {
     const int cap = p.max_blocks * p.bt;
     auto clamp_len = [&](int b) {
-      int len = __ldg(p.seq_lens + b);
+      int len = ld_dep(p.seq_lens + b);
       return len < 0 ? 0 : (len > cap ? cap : len);
     };
     rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, clamp_len);
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         auto chunk_of = [&](int c) {
           if (c >= p.ncols) return make_uint4(0u, 0u, 0u, 0u);
           const int j = c / p.G, hh = c % p.G;
-          return __ldg(reinterpret_cast<const uint4*>(p.q + (((size_t)ib * p.nq_stride + j) * p.Hq + (size_t)ih * p.G + hh) * LYNX_D) + (kt & 15));
+          return ld_dep(reinterpret_cast<const uint4*>(p.q + (((size_t)ib * p.nq_stride + j) * p.Hq + (size_t)ih * p.G + hh) * LYNX_D) + (kt & 15));
         };
         float amax = 0.0f;
 #pragma unroll 4

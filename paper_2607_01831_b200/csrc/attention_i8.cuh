@@ -333,7 +333,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   const int n_cta = gridDim.x, cta = blockIdx.x;
   const int cap = p.max_blocks * p.bt;
   auto clamp_len = [&](int b) {
-    int len = __ldg(p.seq_lens + b);
+    int len = ld_dep(p.seq_lens + b);
     return len < 0 ? 0 : (len > cap ? cap : len);
   };
   const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, clamp_len);
@@ -387,7 +387,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         const int t0 = (u + c0 + i) * ST + (sub_first + (i2 % SPW)) * 16;
         uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
         if (t0 < len) {
-          int blk = __ldg(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
           if (blk < 0 || blk >= p.num_blocks) {
             atomicOr(p.ws_flags, kFlagBadBlock);
             blk = blk < 0 ? 0 : p.num_blocks - 1;
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         const int t = (item.pad1 + uu) * C::kST + r;
         if (uu >= n_piece || t >= len) return 0;
         const int bi = bt_shift >= 0 ? t >> bt_shift : t / p.bt;
-        return __ldg(p.block_table + (size_t)item.b * p.max_blocks + bi);
+        return ld_dep(p.block_table + (size_t)item.b * p.max_blocks + bi);
       };
       auto row_of = [&](int uu, int blk) -> uint32_t {
         const int t = (item.pad1 + uu) * C::kST + r;
@@ -775,8 +775,8 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       auto meta_of = [&](uint32_t row, float2& k2, float2& v2) {
         k2 = make_float2(0.f, 0.f); v2 = k2;
         if (row != 0xFFFFFFFFu) {
-          k2 = __ldg(reinterpret_cast<const float2*>(p.km) + row);
-          v2 = __ldg(reinterpret_cast<const float2*>(p.vm) + row);
+          k2 = ld_dep(reinterpret_cast<const float2*>(p.km) + row);
+          v2 = ld_dep(reinterpret_cast<const float2*>(p.vm) + row);
         }
       };
       int blk_n1 = blk_of(u_first + T), blk_n2 = blk_of(u_first + 2 * T);

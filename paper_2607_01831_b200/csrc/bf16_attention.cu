@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kWarps * 32, COLS <= 4 ? 2 : 1) bf16_decode_ke
   const int bh = blockIdx.x / p.chunks;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv;
   const int cap = p.max_blocks * p.bt;
-  int len = __ldg(p.seq_lens + b);
+  int len = ld_dep(p.seq_lens + b);
   len = len < 0 ? 0 : (len > cap ? cap : len);
   float* part = p.part + ((size_t)bh * p.chunks + chunk) * (size_t)COLS * kPartStrideB;
   const int t_begin = chunk * kChunk, t_end = min(len, t_begin + kChunk);
@@ -96,13 +96,13 @@ __global__ void __launch_bounds__(kWarps * 32, COLS <= 4 ? 2 : 1) bf16_decode_ke
 #pragma unroll
       for (int i = 0; i < NV; ++i) { kxu[u][i] = make_uint4(0, 0, 0, 0); vxu[u][i] = kxu[u][i]; }
       if (validu[u]) {
-        int blk = __ldg(p.block_table + (size_t)b * p.max_blocks + t / p.bt);
+        int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t / p.bt);
         blk = min(max(blk, 0), p.num_blocks - 1);
         const size_t row = ((size_t)blk * p.Hkv + hkv) * p.bt + (t % p.bt);
         const uint4* kp = reinterpret_cast<const uint4*>(p.k + row * LYNX_D + sl * DPL);
         const uint4* vp = reinterpret_cast<const uint4*>(p.v + row * LYNX_D + sl * DPL);
 #pragma unroll
-        for (int i = 0; i < NV; ++i) { kxu[u][i] = __ldg(kp + i); vxu[u][i] = __ldg(vp + i); }
+        for (int i = 0; i < NV; ++i) { kxu[u][i] = ld_dep(kp + i); vxu[u][i] = ld_dep(vp + i); }
       }
     }
 #pragma unroll
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
   const int chunk = blockIdx.x % p.chunks, bh = blockIdx.x / p.chunks;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv;
   const int cap = p.max_blocks * p.bt;
-  int len = __ldg(p.seq_lens + b);
+  int len = ld_dep(p.seq_lens + b);
   len = len < 0 ? 0 : (len > cap ? cap : len);
   float* part = p.part + ((size_t)bh * p.chunks + chunk) * (size_t)COLS * kPartStrideB;
   const int t_begin = chunk * kChunk, t_end = min(len, t_begin + kChunk);
@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
         p.q + (((size_t)b * p.nq_stride + (in ? j : 0)) * p.Hq + hkv * p.G + (in ? hh : 0)) * LYNX_D);
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      qa[ks][0] = in ? __ldg(qp + 8 * ks + t) : 0u;
-      qa[ks][1] = in ? __ldg(qp + 8 * ks + 4 + t) : 0u;
+      qa[ks][0] = in ? ld_dep(qp + 8 * ks + t) : 0u;
+      qa[ks][1] = in ? ld_dep(qp + 8 * ks + 4 + t) : 0u;
     }
   }
   float o[16][4];
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
     const int tile = warp + kTcWarps * i;
     if (tile < n_tiles) {
       const int t0 = t_begin + tile * kTcTile;
-      int blk = __ldg(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+      int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
       blk = min(max(blk, 0), p.num_blocks - 1);
       const size_t row0 = ((size_t)blk * p.Hkv + hkv) * p.bt + (t0 % p.bt);
       const uint32_t st = ring + (uint32_t)(i % kTcStages) * kTcStageBytes;
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(LYNX_D) bf16_combine_kernel(const BfParams p) 
   if (c >= p.ncols) return;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv, d = threadIdx.x;
   const int cap = p.max_blocks * p.bt;
-  int len = __ldg(p.seq_lens + b);
+  int len = ld_dep(p.seq_lens + b);
   len = len < 0 ? 0 : (len > cap ? cap : len);
   const int n = (len + kChunk - 1) / kChunk;
   const float* part = p.part + (size_t)bh * p.chunks * (size_t)COLS * kPartStrideB + (size_t)c * kPartStrideB;

@@ -119,7 +119,7 @@ __device__ __forceinline__ void hier_nibbles4(const uint32_t* r, const uint32_t*
 // (stage 1) and, with them, every chunk's mean and largest deviation (stage 2: max |x - mean| =
 // max(max - mean, mean - min)); then the codes.  The reciprocals are split between the two halves of a chunk and
 // exchanged by shuffles.
-__global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat16* __restrict__ src, int n_pages,
+__global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat16* src, int n_pages,
                                                                uint8_t* __restrict__ q_anc, uint8_t* __restrict__ q_res,
                                                                float* __restrict__ g_min, float* __restrict__ g_scale,
                                                                float* __restrict__ mu, float* __restrict__ sigma) {
@@ -273,12 +273,12 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
 // the table indices of four channels at a time by one bit-select, eight look-ups, four packed multiply-adds, one
 // 16-byte store.
 template <bool FULL>
-__global__ void __launch_bounds__(128, FULL ? 4 : 6) hier_dequantize_kernel(const uint8_t* __restrict__ q_anc,
-                                                              const uint8_t* __restrict__ q_res, int n_pages,
-                                                              const float* __restrict__ g_min,
-                                                              const float* __restrict__ g_scale,
-                                                              const float* __restrict__ mu,
-                                                              const float* __restrict__ sigma,
+__global__ void __launch_bounds__(128, FULL ? 4 : 6) hier_dequantize_kernel(const uint8_t* q_anc,
+                                                              const uint8_t* q_res, int n_pages,
+                                                              const float* g_min,
+                                                              const float* g_scale,
+                                                              const float* mu,
+                                                              const float* sigma,
                                                               __nv_bfloat16* __restrict__ dst) {
   // FULL: every lane has its own copy of the 256 entries (entry e of lane l at e * 32 + l), so that the eight
   // look-ups of a token never meet in a bank; the 16 entries of the Anchor-only case sit in 16 banks anyway.
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(128, FULL ? 4 : 6) hier_dequantize_kernel(cons
       const float4* d = reinterpret_cast<const float4*>(g_min + (size_t)pg * LYNX_D) + oc * 2;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float4 va = __ldg(a + h), vb = __ldg(b + h), vc = __ldg(c + h), vd = __ldg(d + h);
+        const float4 va = ld_dep(a + h), vb = ld_dep(b + h), vc = ld_dep(c + h), vd = ld_dep(d + h);
         const float sc0 = vc.x + kEps, sc1 = vc.y + kEps, sc2 = vc.z + kEps, sc3 = vc.w + kEps;
         S2[2 * h] = pack2((va.x + kEps) * sc0, (va.y + kEps) * sc1);
         S2[2 * h + 1] = pack2((va.z + kEps) * sc2, (va.w + kEps) * sc3);

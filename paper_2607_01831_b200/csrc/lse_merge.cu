@@ -11,14 +11,14 @@
 namespace lynx {
 namespace {
 
-__global__ void __launch_bounds__(256) lse_merge_kernel(const float4* __restrict__ out_a, const float* __restrict__ lse_a,
-                                                        const float4* __restrict__ out_b, const float* __restrict__ lse_b,
+__global__ void __launch_bounds__(256) lse_merge_kernel(const float4* out_a, const float* lse_a,
+                                                        const float4* out_b, const float* lse_b,
                                                         int64_t n_rows, float4* out, float* lse_out) {
   pdl_begin();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= n_rows) return;
   const int lane = threadIdx.x & 31;
-  const float la = __ldg(lse_a + row), lb = __ldg(lse_b + row);
+  const float la = ld_dep(lse_a + row), lb = ld_dep(lse_b + row);
   const float m = fmaxf(la, lb);
   float wa = 0.0f, wb = 0.0f, l = -INFINITY;
   if (m > -INFINITY) {   // (an empty part has lse = -inf and weight 0; two empty parts give a zero row)

@@ -50,6 +50,22 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// What a kernel launched this way reads of earlier kernels' results goes through ordinary (coherent) loads: such a kernel is
+// alive while they still write, and the read-only path (__ldg, const __restrict__ parameters) is defined only for data that
+// does not change during the kernel's whole life.  ld_dep is volatile, so it also stays behind the wait.  Any of 4, 8 or 16
+// bytes, at an address aligned to as many.
+template <class T>
+__device__ __forceinline__ T ld_dep(const T* p) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "a register, a pair or four");
+  union { uint32_t r[sizeof(T) / 4]; T v; } u;
+  if constexpr (sizeof(T) == 4)
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(u.r[0]) : "l"(p));
+  else if constexpr (sizeof(T) == 8)
+    asm volatile("ld.global.v2.b32 {%0,%1}, [%2];" : "=r"(u.r[0]), "=r"(u.r[1]) : "l"(p));
+  else
+    asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(u.r[0]), "=r"(u.r[1]), "=r"(u.r[2]), "=r"(u.r[3]) : "l"(p));
+  return u.v;
+}
 
 // Number of SMs of the current device (cached per device id).
 __host__ int sm_count();

@@ -83,8 +83,8 @@ __device__ __forceinline__ void codes8(const uint32_t (&w)[4], float mn, float i
 
 template <bool kIds>
 __global__ void __launch_bounds__(kThreads)
-split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
-                      const int32_t* __restrict__ block_ids, uint32_t rows_per_block,
+split_quantize_kernel(const uint4* src, int64_t n_logical_rows,
+                      const int32_t* block_ids, uint32_t rows_per_block,
                       int64_t n_blocks_total, uint32_t* __restrict__ anchor,
                       uint32_t* __restrict__ residual, float2* __restrict__ meta, bool wide) {
   pdl_begin();
@@ -104,7 +104,7 @@ split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
         if (kIds) {
           uint32_t lb = (uint32_t)lr / rows_per_block;
           uint32_t in = (uint32_t)lr - lb * rows_per_block;
-          int32_t blk = __ldg(block_ids + lb);
+          int32_t blk = ld_dep(block_ids + lb);
           if (blk >= 0 && blk < n_blocks_total) row[u] = (int64_t)blk * rows_per_block + in;
         } else {
           row[u] = lr;
@@ -158,8 +158,8 @@ split_quantize_kernel(const uint4* __restrict__ src, int64_t n_logical_rows,
 
 template <bool kCodes, bool kBf16>
 __global__ void __launch_bounds__(kThreads)
-recombine_kernel(const uint32_t* __restrict__ anchor, const uint32_t* __restrict__ residual,
-                 const float2* __restrict__ meta, int64_t n_rows, uint2* __restrict__ codes,
+recombine_kernel(const uint32_t* anchor, const uint32_t* residual,
+                 const float2* meta, int64_t n_rows, uint2* __restrict__ codes,
                  uint4* __restrict__ deq) {
   pdl_begin();
   const int64_t n_items = n_rows * 16;  // 16 lanes per row, 8 elements per lane
@@ -185,7 +185,7 @@ recombine_kernel(const uint32_t* __restrict__ anchor, const uint32_t* __restrict
     const uint32_t c1 = __byte_perm(ev, od, 0x7362);  // elements 4..7
     if (kCodes) __stcs(codes + i, make_uint2(c0, c1));
     if (kBf16) {
-      const float2 m = __ldg(meta + (i >> 4));
+      const float2 m = ld_dep(meta + (i >> 4));
       uint32_t o[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {

@@ -23,11 +23,12 @@ __host__ inline lynx_status launch_status() {
 }
 
 // Programmatic dependent launch: a kernel launched this way may become resident while the last CTAs of the kernel before it
-// in the stream are still running, and must call pdl_begin() before it touches global memory.  pdl_begin() lets the
-// kernel after it do the same, then waits until everything before it in the stream has completed and is visible.  It
-// takes the launch gap and the ramp of a grid off chains of short kernels (planes to pages and attention on them, 32768
-// tokens, four kernels: 76.3 -> 74.4 us; Algorithm 1 and its inverse on K and V: 96.0 -> 93.9 us; two small quantisations: 19.6 ->
-// 18.8 us).
+// in the stream are still running, and must call pdl_wait() before it touches global memory.  pdl_trigger() lets the kernel
+// after it do the same; pdl_wait() waits until everything before it in the stream has completed and is visible; pdl_begin()
+// is both, for kernels whose CTAs are short.  It takes the launch gap and the ramp of a grid off chains of kernels (planes to
+// pages and attention on them, four kernels: 41.0 -> 35.1 us for 4096 tokens, 75.3 -> 73.7 us for 32768, 247.3 -> 243.3 us
+// for 131072, equal at 524288; two small quantisations 10.9 -> 9.9 us).  Where a grid's CTAs run long, the trigger belongs
+// behind their work: see hier_quantize.cu.
 template <class... P, class... A>
 __host__ inline lynx_status launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, void* stream, A... args) {
   cudaLaunchConfig_t cfg = {};
@@ -46,9 +47,11 @@ __host__ inline lynx_status launch_pdl(void (*kernel)(P...), unsigned grid, unsi
   }
   return launch_status();
 }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_trigger();
+  pdl_wait();
 }
 // What a kernel launched this way reads of earlier kernels' results goes through ordinary (coherent) loads: such a kernel is
 // alive while they still write, and the read-only path (__ldg, const __restrict__ parameters) is defined only for data that

@@ -21,7 +21,7 @@ def _includes(name):
 def _dependents():
     """Files with a kernel that waits for the grids before it, what they include and what includes them."""
     names = [n for n in sorted(os.listdir(CSRC)) if n.endswith((".cu", ".cuh"))]
-    own = {n for n in names if n != "lynx_common.cuh" and re.search(r"\bpdl_begin\(\)|griddepcontrol\.wait", _code(n))}
+    own = {n for n in names if n != "lynx_common.cuh" and re.search(r"\bpdl_(?:begin|wait)\(\)|griddepcontrol\.wait", _code(n))}
     units = own | {n for n in names if _includes(n) & own}
     return sorted(units.union(*(_includes(n) for n in units)))
 

@@ -4,15 +4,23 @@
 // A unit is 128 tokens.  Both contractions take the 8-bit codes centred, c - 128, which FP16 represents exactly:
 //   S^T[128 tokens x NC]      = (codes(K) - 128) . Q^T       A = K in tensor memory (a thread owns a token = a lane),
 //                                                            B = Q, FP16 after a power-of-two scale (exact for BF16
-//                                                                entries down to 2^-32 of the largest)
+//                                                                entries down to 2^-32 of the largest); up to 32 columns
+//                                                                in two parts side by side in N (f16_split_q)
 //   O^T[128 dims x 2 x 32]   += (codes(V) - 128)^T . [h | r] A = V tile (MN-major), B = the weights as two FP16 terms,
 //                                                                w = h + r (22 bits), side by side in N
 // Centring costs one packed addition per two codes and is what keeps FP32 sufficient: the zero points, 128 steps below
-// the centre of a row, would otherwise be added and taken off again around results a hundred times smaller (error against
-// 64 bits, one layer of 131072 tokens: 2e-6 at 32 columns, 5e-6 at 64; the integer kernel, not centred, 8e-6 at 32).
+// the centre of a row, would otherwise be added and taken off again around results a hundred times smaller.
 // x = s log2(e) + log2(scale_v), w = 2^(x - ref[c]); ref[c] is set so that the largest weight of a column's first unit is
 // 2^8 and raised (accumulators drained, rare) before a weight would leave FP16.  The tensor core's accumulation truncates
-// (0.46 ulp of the running sum per product): every kDrainUnits units the accumulators move into an FP32 copy.
+// (0.46 ulp of the running sum per product).  Scores: the high part of a query is a multiple of 2^-10 of the largest entry,
+// so that its products with the codes sum up exactly, and the truncation acts on the low part, a thousand times smaller.
+// Values: every kDrainUnits units the accumulators move into an FP32 copy.
+//
+// Error against 64 bits (2-norm; ten 64-column and fifty other cases of one layer, 64 to 131072 tokens, normal, heavy-tailed
+// and outlier values).  17..32 columns, against the exact integer products of attention_i8.cuh in two passes: 0.29 times on
+// the geometric mean, at most 0.97 times, largest 1.4e-6 (7.5e-6); log-sum-exps 0.54 times, largest 9e-6 (4.4e-5).  With
+// whole queries and a drain per 8 units it was 0.42 times on the mean but up to 2.0 times on heavy-tailed keys and long
+// contexts.  33..64 columns, against the uncentred kernel before it: 0.09 times, largest 1.2e-5 (3.4e-4).
 //
 // Warp roles, one CTA per SM; every hand-off is an mbarrier with a bounded wait, nothing waits on another CTA:
 //   warps 0-7    two softmax warpgroups of 32 columns each: scores -> weights -> P tile
@@ -34,8 +42,8 @@
 // per thread cost a factor of two; hence scores in the 16-lane layout, where a thread sums 8 columns over 4 tokens instead
 // of 32 columns over one), rolled expansion loops (the roles compete for the instruction caches: 118 -> 98 us at 32
 // columns), products issued by an elected lane (93 -> 30 cycles each).  One layer of 131072 tokens: 174 us as two passes of
-// the 16-column integer kernel -> 93 us (32 columns); 293 us by the previous kernel (M = columns, codes not centred) ->
-// 251 us (64 columns, batch 2).
+// the 16-column integer kernel -> 96 us (32 columns); 293 us by the previous kernel (M = columns, codes not centred) ->
+// 245 us (64 columns, batch 2).
 
 template <int NC>
 struct F16Cfg {
@@ -46,7 +54,9 @@ struct F16Cfg {
   static constexpr int kStageBytes = kST * 128;     // Anchor and Residual of one tensor: [2][128 tokens][64 B]
   static constexpr int kVTile = 32768;              // [2 dim blocks][128 tokens][128 B]
   static constexpr int kPTile = 16384;              // [128 tokens][32 h | 32 r]
-  static constexpr int kQTile = NC * 256;           // [2 dim blocks][NC][128 B]
+  static constexpr int kQP = NC == 32 ? 2 : 1;      // parts of the queries (see f16_split_q)
+  static constexpr int kSCols = kQP * NC;           // columns of Q.K^T: the queries' high parts, then the low ones
+  static constexpr int kQTile = kSCols * 256;       // [2 dim blocks][kSCols][128 B]
   static constexpr int kRingK = 3, kRingV = 3;
   static constexpr int kOffV = 0, kOffP = 2 * kVTile, kOffQ = kOffP + 2 * kPTile, kOffRK = kOffQ + kQTile,
                        kOffRV = kOffRK + kRingK * kStageBytes, kOffScal = kOffRV + kRingV * kStageBytes;
@@ -61,16 +71,17 @@ struct F16Cfg {
   static constexpr int kSmem = kOffMisc + 256 + 1024;               // + alignment slack
   static_assert(kSmem <= 227 * 1024, "shared memory");
   static_assert(kOffScal % 16 == 0 && kOffGrp % 16 == 0 && kOffBars % 8 == 0, "alignment");
-  static constexpr int kTmS = 0, kTmK = 2 * NC, kTmO = kTmK + 128, kTmOF = kTmO + 128;   // [2][NC], [2][64], [2][64], [2][32]
+  static constexpr int kTmS = 0, kTmK = 2 * kSCols, kTmO = kTmK + 128, kTmOF = kTmO + 128;   // [2][kSCols], [2][64], [2][64], [2][32]
   static_assert(kTmOF + 64 <= 512, "tensor memory");
   static constexpr int kThreads = 768;
-  // units between drains: each adds 8 truncating products to a sum.  (64 columns against 64 bits: 3.3e-4 by the previous
-  // FP16 kernel, 5e-6 here; a drain per 8 units costs 6 % of its time, one per 16 units 3 %.)
-  static constexpr int kDrainUnits = NC == 64 ? 16 : 8;
+  // units between drains: each adds 8 truncating products to a sum.  32 columns, one layer of 131072 tokens: a drain per 8
+  // units 92.7 us (largest error 3.4e-6), per 4 units 94.0 us (2.2e-6), per 2 units 96.2 us (1.4e-6), by when it is below the
+  // integer kernel's in every case; 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
+  static constexpr int kDrainUnits = NC == 64 ? 16 : 2;
   // who computes the per-token scalars: with 64 columns the K warps have the time (261 -> 256 us), with 32 they are the
   // slower stage and two spare warps do it (96.1 us, 97.4 us in the K warps)
   static constexpr bool kMetaK = kSplit;
-  // registers per thread after the split (launched with 80 each): 256 * 136 + 256 * 64 + 128 * 56 + 128 * 24 = 768 * 80
+  // registers per thread after the split (launched with 80 each): 256 * 128 + 256 * 64 + 128 * 56 + 128 * 40 = 768 * 80
   static constexpr int kRegSoft = 128, kRegExp = 64, kRegProd = 56, kRegMma = 40;
 };
 template <int N>
@@ -106,6 +117,16 @@ __device__ __forceinline__ void f16_codes(uint32_t xa, uint32_t xr, uint32_t* o)
   o[1] = f16_centre(prmt(ev, 0x64646464u, 0x4341));
   o[2] = f16_centre((od & 0x00FF00FFu) | 0x64006400u);
   o[3] = f16_centre(prmt(od, 0x64646464u, 0x4341));
+}
+// A scaled query entry, |f| < 2^15, in two parts: f becomes a multiple of 32, lo what is left, |lo| <= 16.  The sum of 128
+// products of codes (|c - 128| <= 128) with multiples of 32 up to 2^15 stays below 2^24 times 32: exact in FP32 in any order.
+// Both parts are exact in FP16: an entry has eight bits, and those above 2^12 are multiples of 32 themselves.  (Against whole
+// queries, 32 columns: 92.2 -> 93.5 us for one layer of 131072 tokens.)
+__device__ __forceinline__ void f16_split_q(float& f, float& lo) {
+  constexpr float kRound = 402653184.0f;   // 1.5 * 2^23 * 32
+  const float hi = (f + kRound) - kRound;
+  lo = f - hi;
+  f = hi;
 }
 __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
@@ -323,7 +344,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
                                                                            const __grid_constant__ I8Maps maps) {
   using C = F16Cfg<NC>;
   constexpr bool SPLIT = C::kSplit;
-  constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2;
+  constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2, kDW = 16;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -425,22 +446,24 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       // Moves the accumulators (the group's last P.V is complete) into the FP32 copy, scaled by fac_s[] if asked.
       auto drain = [&](bool scale) {
         tc_fence_after();
+        // (a loop: the caller's values fill the registers; 16 columns at a time, a drain per 2 units at 32 columns 96.2 us, 8 at a
+        // time 102 us, and 64 columns 220 -> 215 us)
 #pragma unroll 1
-        for (int c8 = 0; c8 < CG / 8; ++c8) {   // (a loop: the caller's values fill the registers)
-          uint32_t h[8], q[8], of[8];
-          TmemRegs<8>::ld(tm_o + c8 * 8, h);
-          TmemRegs<8>::ld(tm_o + 32 + c8 * 8, q);
-          TmemRegs<8>::ld(tm_of + c8 * 8, of);
+        for (int c = 0; c < CG; c += kDW) {
+          uint32_t h[kDW], q[kDW], of[kDW];
+          TmemRegs<kDW>::ld(tm_o + c, h);
+          TmemRegs<kDW>::ld(tm_o + 32 + c, q);
+          TmemRegs<kDW>::ld(tm_of + c, of);
           tc_wait_ld();
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
+          for (int k = 0; k < kDW; ++k) {
             float v = 0.0f;   // (a piece's first drain finds the previous piece's copy; accumulators not restarted since the last drain)
             if (have_of) v = __uint_as_float(of[k]);
             if (units_in_acc > 0) v += __uint_as_float(h[k]) + __uint_as_float(q[k]);
-            if (scale) v *= fac_s[c8 * 8 + k];
+            if (scale) v *= fac_s[c + k];
             of[k] = __float_as_uint(v);
           }
-          TmemRegs<8>::st(tm_of + c8 * 8, of);
+          TmemRegs<kDW>::st(tm_of + c, of);
         }
         tc_wait_st();
         have_of = true;
@@ -468,20 +491,31 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
             mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);
             drain(scale);
           }
-          uint32_t s[2][4 * NG];   // [tokens t0, t0 + 8 | t0 + 16, t0 + 24]
-          const uint32_t tm_s = tmem0 + C::kTmS + sl * NC + col0 + lane_sel;
-          tc_ld_16x256<NG>(tm_s, s[0]);
-          tc_ld_16x256<NG>(tm_s + (16u << 16), s[1]);
-          tc_wait_ld();
+          const uint32_t tm_s = tmem0 + C::kTmS + sl * C::kSCols + col0 + lane_sel;
+          uint32_t s[2][4 * NG];   // one part: tokens t0, t0 + 8 | t0 + 16, t0 + 24; two parts: the parts of one half
+          if (C::kQP == 1) {
+            tc_ld_16x256<NG>(tm_s, s[0]);
+            tc_ld_16x256<NG>(tm_s + (16u << 16), s[1]);
+            tc_wait_ld();
+          }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
+            if (C::kQP == 2 && (k & 1) == 0) {
+              tc_ld_16x256<NG>(tm_s + ((uint32_t)(8 * k) << 16), s[0]);
+              tc_ld_16x256<NG>(tm_s + NC + ((uint32_t)(8 * k) << 16), s[1]);
+              tc_wait_ld();
+            }
             const float4 ts = tok4[(gs & 3) * 128 + 8 * k];
             const uint64_t al2 = f2_pack(ts.x, ts.x), be2 = f2_pack(ts.y, ts.y), lsv2 = f2_pack(ts.z, ts.z);
 #pragma unroll
             for (int j = 0; j < NG; ++j) {
-              const uint32_t* sv = s[k >> 1] + 4 * j + 2 * (k & 1);
-              y2[k][j] = f2_fma(f2_pack(__uint_as_float(sv[0]), __uint_as_float(sv[1])), al2,
-                                f2_fma(be2, qs2[j], f2_sub(lsv2, ref2[j])));
+              const uint32_t* sv = s[C::kQP == 2 ? 0 : k >> 1] + 4 * j + 2 * (k & 1);
+              uint64_t rest = f2_fma(be2, qs2[j], f2_sub(lsv2, ref2[j]));
+              if (C::kQP == 2) {
+                const uint32_t* lv = s[1] + 4 * j + 2 * (k & 1);
+                rest = f2_fma(f2_pack(__uint_as_float(lv[0]), __uint_as_float(lv[1])), al2, rest);
+              }
+              y2[k][j] = f2_fma(f2_pack(__uint_as_float(sv[0]), __uint_as_float(sv[1])), al2, rest);
             }
           }
           if (unit_t0 + C::kST > full_lim) {
@@ -749,8 +783,15 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
             f[2 * k] = __uint_as_float(w[k] << 16) * up;
             f[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u) * up;
           }
-          sts128(sbase + C::kOffQ + (uint32_t)(ch >> 3) * (NC * 128u) + (uint32_t)c * 128u + (uint32_t)((ch & 7) ^ (c & 7)) * 16u,
-                 pack_f16x2(f[0], f[4]), pack_f16x2(f[2], f[6]), pack_f16x2(f[1], f[5]), pack_f16x2(f[3], f[7]));
+          const uint32_t dst = sbase + C::kOffQ + (uint32_t)(ch >> 3) * (C::kSCols * 128u) + (uint32_t)c * 128u +
+                               (uint32_t)((ch & 7) ^ (c & 7)) * 16u;
+          if (C::kQP == 2) {
+            float lo[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) f16_split_q(f[k], lo[k]);
+            sts128(dst + NC * 128u, pack_f16x2(lo[0], lo[4]), pack_f16x2(lo[2], lo[6]), pack_f16x2(lo[1], lo[5]), pack_f16x2(lo[3], lo[7]));
+          }
+          sts128(dst, pack_f16x2(f[0], f[4]), pack_f16x2(f[2], f[6]), pack_f16x2(f[1], f[5]), pack_f16x2(f[3], f[7]));
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         named_bar(4, 128);
@@ -836,7 +877,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     return;
   }
   if (warp == 20) {
-    constexpr uint32_t kIdescS = tc_idesc(NC, false), kIdescO = tc_idesc(64, true) | (1u << 15);
+    constexpr uint32_t kIdescS = tc_idesc(C::kSCols, false), kIdescO = tc_idesc(64, true) | (1u << 15);
     // (low words of the operand descriptors; the issuing thread keeps them in registers)
     constexpr uint32_t kHi = i8_desc_hi(1024u, 2u);
     const uint32_t q_lo = i8_desc_lo(sbase + C::kOffQ, 16u), v_lo = i8_desc_lo(sbase + C::kOffV, 16384u),
@@ -847,10 +888,10 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       if (gs >= 2) mbar_wait_in(sfree + sl * 8, ((gs >> 1) - 1) & 1, abort_word);
       tc_fence_after();
       if (tc_elect()) {
-        const uint32_t d = tmem0 + C::kTmS + sl * NC, a = tmem0 + C::kTmK + sl * 64;
+        const uint32_t d = tmem0 + C::kTmS + sl * C::kSCols, a = tmem0 + C::kTmK + sl * 64;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
-          tc_mma_ts(d, a + ks * 8u, i8_pack(q_lo + (uint32_t)(((ks >> 2) * NC * 128 + (ks & 3) * 32) >> 4), kHi), kIdescS, ks > 0 ? 1u : 0u);
+          tc_mma_ts(d, a + ks * 8u, i8_pack(q_lo + (uint32_t)(((ks >> 2) * C::kSCols * 128 + (ks & 3) * 32) >> 4), kHi), kIdescS, ks > 0 ? 1u : 0u);
         tc_commit(sfull + sl * 8);
       }
       __syncwarp();

@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  named_bar(8, T * TT);
+  named_bar(14, T * TT);
   tc_fence_after();
   const uint32_t tmem0 = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(misc + 8), 0);   // (known to be uniform)
   constexpr uint32_t kIdescS = i8_idesc(C::kNQK, false, true), kIdescO = i8_idesc(C::kNPV, true, false);
@@ -589,7 +589,11 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   float* my_lz = my_scal + 16 * CP;               // [2 CP]
   const int tw = grp * 4 + w4;                    // warp of the team
   int* my_misc = misc + 64 * (1 + tm);
-  const int bar_tm = 1 + tm, bar_k = 10 + tm;     // named barriers of this team
+  // named barriers of this team.  On bar_k and bar_p all but the issuing warp only arrive; each has an id of its own, so that
+  // between two arrivals of a warp there lies a barrier at which all warps synchronise (the restart question, or bar_p itself
+  // where they synchronise there): the phases stay apart even if the waits for products in between have given up.
+  static_assert(T <= 4, "barrier ids: 1.. bar_tm, 5.. bar_p, 9 and 14 all teams, 10.. bar_k");
+  const int bar_tm = 1 + tm, bar_p = 5 + tm, bar_k = 10 + tm;
   const uint32_t vtile = sbase + tm * C::kTeamBytes, ptile = vtile + C::kTile;
   float* my_hdr = reinterpret_cast<float*>(smem + tm * C::kTeamBytes + C::kTile);   // [3 CP] l, zs, ref of this team's deposit (in its idle P tile)
   const uint32_t tm_k = tmem0 + tm * C::kTmTeam + C::kTmK;
@@ -965,8 +969,8 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           tc_fence_before();
           // the P tile and the V tile are complete, S has been read: the issuing warp waits for it, the others only where
           // the restart flag is looked at afterwards
-          if (C::kVoteFirst && tw != 0) bar_arrive(bar_tm, TT);
-          else named_bar(bar_tm, TT);
+          if (C::kVoteFirst && tw != 0) bar_arrive(bar_p, TT);
+          else named_bar(bar_p, TT);
         };
         if (C::kVoteFirst) {   // (every instance but the 4-column anchor one measures faster with the question asked first)
           if (bar_or(bar_tm, TT, forced || over)) restart();

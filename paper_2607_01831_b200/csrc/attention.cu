@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "bounded_wait.cuh"
 #include "lynx_common.cuh"
 
 namespace lynx {
@@ -105,17 +106,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 // loop has a fixed trip count, so the kernel still ends) and the host is told through the
 // workspace status word.  Nothing in this kernel waits on another CTA.
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_word) {
-  if (*abort_word) return false;
-  const uint64_t t0 = globaltimer_ns();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_word) return false;
-    if (globaltimer_ns() - t0 > 2000000000ull) {
-      *abort_word = 1;
-      return false;
-    }
-  }
+  return !*abort_word && bounded_wait([=] { return mbar_try_wait(bar, parity); }, [] { return globaltimer_ns(); }, abort_word);
 }
 // One non-blocking probe of an mbarrier phase.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {

@@ -90,15 +90,9 @@ template <int N>
 __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // The bounded wait of mbar_wait without a call: ptxas cannot split the registers of a kernel that has calls.
-__device__ __forceinline__ void mbar_wait_in(uint32_t bar, uint32_t parity, volatile int* abort_word) {
-  if (mbar_test(bar, parity)) return;
-  uint64_t t0 = 0;
-  for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
-    if ((i & 255u) != 0) continue;
-    const uint64_t now = globaltimer_ns();
-    if (t0 == 0) t0 = now;
-    if (*abort_word || now - t0 > 2000000000ull) { *abort_word = 1; return; }
-  }
+__device__ __forceinline__ bool mbar_wait_in(uint32_t bar, uint32_t parity, volatile int* abort_word) {
+  if (mbar_test(bar, parity)) return true;
+  return bounded_wait([=] { return mbar_try_wait(bar, parity); }, [] { return globaltimer_ns(); }, abort_word);
 }
 
 // position -> element within a group of 8: {0,4,2,6,1,5,3,7} (what the nibble expansion yields), its own inverse

@@ -102,11 +102,15 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 // Bounded wait: gives up after ~2 s (at once if another thread of the CTA already gave up),
-// records it in the CTA's abort word and returns false.  Callers carry on without the data (every
-// loop has a fixed trip count, so the kernel still ends) and the host is told through the
-// workspace status word.  Nothing in this kernel waits on another CTA.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_word) {
-  return !*abort_word && bounded_wait([=] { return mbar_try_wait(bar, parity); }, [] { return globaltimer_ns(); }, abort_word);
+// records it in the CTA's abort word and returns false.  Callers carry on without the data and the host is told through the workspace status word.  The kernel still
+// ends: trip counts follow from the pieces alone, and the hand-offs of pieces between the producer and the
+// other warps, which need no data to arrive, have an abort word of their own (kItemAbort words behind the
+// other): they stay in step after a wait for data has given up.  Nothing in this kernel waits on another CTA.
+constexpr int kItemAbort = 9;
+template <int WORD>
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_words) {
+  return !abort_words[WORD] &&
+         bounded_wait([=] { return mbar_try_wait(bar, parity); }, [] { return globaltimer_ns(); }, abort_words + WORD);
 }
 // One non-blocking probe of an mbarrier phase.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
@@ -118,10 +122,11 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+template <int WORD = 0>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_word) {
   if (mbar_test(bar, parity)) return true;   // (a plain probe is several times quicker than one that may suspend)
   if (mbar_try_wait(bar, parity)) return true;
-  return mbar_wait_slow(bar, parity, abort_word);
+  return mbar_wait_slow<WORD>(bar, parity, abort_word);
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(

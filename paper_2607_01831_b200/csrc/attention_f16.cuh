@@ -73,7 +73,7 @@ struct F16Cfg {
   static_assert(kOffScal % 16 == 0 && kOffGrp % 16 == 0 && kOffBars % 8 == 0, "alignment");
   static constexpr int kTmS = 0, kTmK = 2 * kSCols, kTmO = kTmK + 128, kTmOF = kTmO + 128;   // [2][kSCols], [2][64], [2][64], [2][32]
   static_assert(kTmOF + 64 <= 512, "tensor memory");
-  static constexpr int kThreads = 768;
+  static constexpr int kThreads = 768, kDoneThreads = 256 + 128 + 32;   // softmax warpgroups, producers, products
   // units between drains: each adds 8 truncating products to a sum.  32 columns, one layer of 131072 tokens: a drain per 8
   // units 92.7 us (largest error 3.4e-6), per 4 units 94.0 us (2.2e-6), per 2 units 96.2 us (1.4e-6), by when it is below the
   // integer kernel's in every case; 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
@@ -198,7 +198,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
     const int n = min(remaining, U - u);
     if (pw == 0) {
       const int qi = ic & 1;
-      if (ic >= 2) mbar_wait_in(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word);
+      if (ic >= 2) mbar_wait_in(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word + kItemAbort);
       const long long seg0 = rng.lo + (n_units - remaining) - u;  // first unit of this segment
       if (lane == 0) {
         Item it;
@@ -270,6 +270,8 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
       }
     }
   }
+  __syncwarp();
+  bar_arrive(5, C::kDoneThreads);
 }
 
 // The per-token scalars of a unit, for N tokens (32 apart) of a thread: scale and offset of the scores, log2 of the value
@@ -344,7 +346,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   const uint32_t sbase = smem_u32(smem);
   float* scal = reinterpret_cast<float*>(smem + C::kOffScal);
   Item* items = reinterpret_cast<Item*>(smem + C::kOffItems);
-  int* misc = reinterpret_cast<int*>(smem + C::kOffMisc);   // [0] abort, [7] units, [8] tensor memory base, [40 + g] accumulate
+  int* misc = reinterpret_cast<int*>(smem + C::kOffMisc);   // [0], [kItemAbort] abort, [7] units, [8] tensor memory base, [40 + g] accumulate
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // (known to be uniform)
   const uint32_t kfull = sbase + C::kOffBars, kempty = kfull + 32, vfull = kempty + 32, vempty = vfull + 24;
@@ -426,7 +428,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     int gs_base = 0, ic = 0;
     while (gs_base < n_units) {
       const int qi = ic & 1;
-      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word + kItemAbort);
       const Item item = items[qi];
       const int len = item.len, n_piece = item.pad0;
       const int u_first = SPLIT ? 0 : (g ^ gs_base) & 1;
@@ -702,14 +704,15 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       gs_base += n_piece;
       ++ic;
     }
-    // ---- release the tensor memory: every product has been waited for ----------------------------------------
+    // ---- release the tensor memory: every product has been waited for, and the warps that issue copies and products are done
     tc_fence_before();
-    named_bar(3, 256);
+    named_bar(5, C::kDoneThreads);
     if (warp == 0) {
+      land_after_abort([] { return globaltimer_ns(); }, abort_word);
       tc_fence_after();
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem0), "r"(512u) : "memory");
     }
-    if (tid == 0 && misc[0]) atomicOr(p.ws_flags, kFlagTimeout);
+    if (tid == 0 && (misc[0] || misc[kItemAbort])) atomicOr(p.ws_flags, kFlagTimeout);
     return;
   }
   // ================================================================================== K codes and queries
@@ -725,7 +728,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     uint32_t phase = 0;
     while (gs < n_units) {
       const int qi = ic & 1;
-      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word + kItemAbort);
       const int ib = items[qi].b, ih = items[qi].hkv, len = items[qi].len, n_piece = items[qi].pad0;
       // ---- the piece's queries: thread = 16-byte chunk kt & 15 of columns kt >> 4, + 8, ... ---------------------
       {
@@ -838,7 +841,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   if (warp < 20) {
     reg_dec<C::kRegProd>();
     const int pw = warp - 16;
-    if (n_units > 0)
+    if (n_units == 0) bar_arrive(5, C::kDoneThreads);
+    else
       f16_producer<C>(p, rng, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
                       reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
     return;
@@ -852,7 +856,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     int gs = 0, ic = 0;
     while (gs < n_units) {
       const int qi = ic & 1;
-      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word);
+      mbar_wait_in(qfull + qi * 8, (ic >> 1) & 1, abort_word + kItemAbort);
       meta.piece(p, items[qi]);
       const int n_piece = items[qi].pad0;
       mbar_wait_in(qready + qi * 8, (ic >> 1) & 1, abort_word);
@@ -915,6 +919,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       if (gs + 1 < n_units) qk(gs + 1);
       pv(gs);
     }
+    bar_arrive(5, C::kDoneThreads);
   }
 }
 

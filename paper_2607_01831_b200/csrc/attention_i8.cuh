@@ -363,7 +363,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
     const int n = min(remaining, U - u);
     const int qi = ic & 1;
     if (pw == 0) {
-      if (ic >= 2) mbar_wait(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word);
+      if (ic >= 2) mbar_wait<kItemAbort>(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word);
       const long long seg0 = lo + (n_units - remaining) - u;  // first unit of this segment
       if (lane == 0) {
         Item it;
@@ -431,6 +431,8 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
       }
     }
   }
+  __syncwarp();
+  bar_arrive(9, C::kThreads);
 }
 
 // Largest |q| of a piece's raw queries, by 128 threads (index i of 0..127), reduced over the
@@ -516,7 +518,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   const uint32_t pvdone0 = sfull0 + T * 8;        // [team]  P.V complete: P and V tiles free, accumulators current
   volatile int* abort_word = misc;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a dependent grid may be scheduled as SMs become free
-  // misc[8] = tensor memory base; misc[16 + t] = deposits written by team t, misc[24 + t] = deposits of team t read;
+  // misc[0], misc[kItemAbort]: abort words; misc[8] = tensor memory base; misc[16 + t] = deposits written by team t, misc[24 + t] = deposits of team t read;
   // misc[32 + s] = completed phases of raw stage s
 
   if (tid == 0) {
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   int gs_base = 0, ic = 0;
   while (gs_base < n_units) {
     const int qi = ic & 1;
-    mbar_wait(qfull0 + qi * 8, (ic >> 1) & 1, abort_word);
+    mbar_wait<kItemAbort>(qfull0 + qi * 8, (ic >> 1) & 1, abort_word);
     const Item item = items[qi];
     const int len = item.len, n_piece = item.pad0;
     const int team0 = gs_base % T;                        // team of the piece's first unit
@@ -1118,13 +1120,14 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   }
   // ---- release the tensor memory ---------------------------------------------------------------
   tc_fence_before();
-  named_bar(9, T * TT);
+  named_bar(9, C::kThreads);   // (the producers have arrived there behind their last copy)
   if (warp == 0) {
+    land_after_abort([] { return globaltimer_ns(); }, abort_word);
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem0), "r"((uint32_t)C::kTmCols)
                  : "memory");
   }
-  if (tid == 0 && misc[0]) atomicOr(p.ws_flags, kFlagTimeout);
+  if (tid == 0 && (misc[0] || misc[kItemAbort])) atomicOr(p.ws_flags, kFlagTimeout);
 }
 
 // Launches one of the persistent attention kernels: SMEM bytes, THREADS per CTA, units of ST tokens.

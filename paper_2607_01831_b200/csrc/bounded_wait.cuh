@@ -33,4 +33,13 @@ LYNX_HD bool bounded_wait(Probe probe, Clock now_ns, volatile int* abort_word) {
   return true;
 }
 
+// What follows a wait that gave up, behind the last copy and product of the CTA and before it gives back the memory that they
+// write to: a millisecond, a thousand times what one of them takes.
+constexpr uint64_t kLandNs = 1000000ull;
+template <class Clock>
+LYNX_HD void land_after_abort(Clock now_ns, volatile int* abort_word) {
+  if (!*abort_word) return;
+  for (const uint64_t t0 = now_ns(); now_ns() - t0 < kLandNs;) {}
+}
+
 }  // namespace lynx

@@ -31,6 +31,13 @@ int main() {
   auto late = [&] { now += kProbeNs; return ++probes == 1000; };
   r = lynx::bounded_wait(late, clock, &abort_word);                             // it comes after all
   std::printf("%d %d %ld %llu\n", r, (int)abort_word, probes, (unsigned long long)now);
+  auto tick = [&] { return now += 100; };
+  now = 0; abort_word = 0;
+  lynx::land_after_abort(tick, &abort_word);                                    // nothing has given up: not a moment
+  std::printf("%llu ", (unsigned long long)now);
+  abort_word = 1;
+  lynx::land_after_abort(tick, &abort_word);                                    // time for what is in flight
+  std::printf("%llu\n", (unsigned long long)now);
 }
 """
 
@@ -45,6 +52,18 @@ def test_waiting_loop(tmp_path):
     assert after[:2] == [0, 1] and after[2] <= 16                  # within a few probes
     assert during[:2] == [0, 1] and during[2] <= 100 + 16          # within a few probes of the other's giving up
     assert late[:3] == [1, 0, 1000]
+    untouched, landed = (int(x) for x in out[4].split())
+    assert untouched == 0 and 1.0e6 <= landed <= 1.1e6
+
+
+def test_memory_is_given_back_behind_what_is_in_flight():
+    """The warps that issue copies and products arrive at a barrier behind their last one; tensor memory is released, and with it
+    the CTA can end, behind that barrier and the pause."""
+    for name, bar in (("attention_i8.cuh", r"named_bar\(9, C::kThreads\)"), ("attention_f16.cuh", r"named_bar\(5, C::kDoneThreads\)")):
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        done, land, free = (re.search(x, code).start() for x in (bar, r"land_after_abort\(", r"tcgen05\.dealloc"))
+        assert done < land < free
+        assert re.search(bar.replace("named_bar", "bar_arrive"), code), "the producers arrive there"
 
 
 def test_every_wait_of_the_kernels_goes_through_it():

@@ -88,7 +88,7 @@ def test_a_shared_barrier_would_mix():
 
 def test_barrier_ids_are_distinct():
     ids, text = _team_barriers()
-    fixed = [int(x) for x in re.findall(r"named_bar\((\d+), T \* TT\)", text)]
+    fixed = [int(x) for x in re.findall(r"named_bar\((\d+), (?:T \* TT|C::kThreads)\)", text)]
     assert len(fixed) == 2
     every = [0] + fixed + [f(tm) for f in ids.values() for tm in range(4)]
     assert len(set(every)) == len(every) and max(every) < 16

@@ -228,8 +228,8 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
   };
   if (!direct) {
     // The partial slots of this (sequence, KV head) are merged in two levels, so that no CTA walks
-    // through all of them one L2 round trip after the other (74 slots for a 131072-token head on
-    // 592 CTAs: 20 us at the tail of the launch).  The last CTA to arrive of each group of kGroup
+    // through all of them one L2 round trip after the other (a slot per CTA where one head has the
+    // grid to itself).  The last CTA to arrive of each group of kGroup
     // neighbouring contributors merges the group into its first slot; the last group to finish
     // merges the group results into the output.  Every ticket resets itself; nobody waits.
     constexpr int kGroup = 8, kOneLevel = 24;   // up to kOneLevel slots are merged in one go
@@ -238,7 +238,7 @@ __device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& it
     const int g = ((int)blockIdx.x - item.first_cta) / kGroup;
     const int gsize = min(kGroup, n - g * kGroup);
     float* seg = p.ws_part + (bh + (size_t)item.first_cta) * (size_t)kColsPad * kPartStride;
-    constexpr uint32_t cstride = kColsPad * kPartStride;   // (a segment has at most 592 slots: offsets fit 32 bits)
+    constexpr uint32_t cstride = kColsPad * kPartStride;   // (a segment has a slot per CTA at most: offsets fit 32 bits)
     named_bar(bar_id, kConsThreads);
     if (tid == 0) {
       bool last = true;   // of this CTA's group (n <= kOneLevel: of the whole segment)
@@ -502,6 +502,8 @@ __device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, in
 #include "attention_f16.cuh"
 
 // ------------------------------------------------------------------ host side
+// The scratch has room for this many CTAs per SM, although every kernel runs one: lynx_workspace_bytes and the limit of
+// lynx_anchor_attention_static are figures that callers hold (8 bytes to 33 KB per CTA and column count).
 constexpr int kMaxCtasPerSm = 4;
 
 // Query positions per launch of a verification call: all of them up to kMaxQ positions and kMaxCols
@@ -514,7 +516,7 @@ inline int verify_slice(int nq, int G) {
 
 struct Plan {
   int per;             // query positions per verification launch
-  int ncols, variant;  // variant: 0: NT1 TW4 CG1; 1: NT2 TW4 CG1; 2: NT2 TW4 CG2; 3: NT2 TW2 CG4
+  int ncols;           // columns of the widest launch
   int cols_pad;
   size_t off_chunk_ctr, off_seq_ctr, off_group_ctr, off_dev, off_lse, off_part, bytes;
 };
@@ -534,7 +536,6 @@ bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
   if (cap >= (1ll << 31)) return false;
   if ((int64_t)s->num_blocks * s->num_kv_heads * s->block_tokens >= (1ll << 32)) return false;
   pl->ncols = ncols;
-  pl->variant = ncols <= 8 ? 0 : ncols <= 16 ? 1 : ncols <= 32 ? 2 : 3;
   // (the partial slots also serve anchor calls on the same workspace, which take up to 32 columns per launch)
   const int cols_anchor = nq * G <= 32 ? nq * G : (32 / G > 0 ? 32 / G : 1) * G;
   const int cols_max = ncols > cols_anchor ? ncols : cols_anchor;

@@ -36,8 +36,8 @@
 // memory (integer digit planes: 224 columns per team at 32), while the expansions and the softmax of a unit are long
 // enough to overlap as pipeline stages with double-buffered S, K and V.
 //
-// What bounds it: instruction issue.  A unit takes 6200 warp instructions at 32 columns and 8000 at 64 (K expansion 1300,
-// V expansion 1400, softmax 1900 per 32 columns), at 2.2 per cycle; tensor pipe 15-20 %, DRAM under half.  What mattered on
+// What bounds it: instruction issue.  A unit takes 6700 warp instructions at 32 columns and 8300 at 64 (K expansion 1300,
+// V expansion 1400, most of the rest softmax), at 2.3 per cycle; tensor pipe 18-21 %, DRAM under a third.  What mattered on
 // the way: no register spills in the softmax loop (little L1 is left beside 227 KB of shared memory: 400 bytes of spills
 // per thread cost a factor of two; hence scores in the 16-lane layout, where a thread sums 8 columns over 4 tokens instead
 // of 32 columns over one), rolled expansion loops (the roles compete for the instruction caches: 118 -> 98 us at 32
@@ -490,15 +490,15 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           const uint32_t tm_s = tmem0 + C::kTmS + sl * C::kSCols + col0 + lane_sel;
           uint32_t s[2][4 * NG];   // one part: tokens t0, t0 + 8 | t0 + 16, t0 + 24; two parts: the parts of one half
           if (C::kQP == 1) {
-            tc_ld_16x256<NG>(tm_s, s[0]);
-            tc_ld_16x256<NG>(tm_s + (16u << 16), s[1]);
+            tc_ld_16x256(tm_s, s[0]);
+            tc_ld_16x256(tm_s + (16u << 16), s[1]);
             tc_wait_ld();
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             if (C::kQP == 2 && (k & 1) == 0) {
-              tc_ld_16x256<NG>(tm_s + ((uint32_t)(8 * k) << 16), s[0]);
-              tc_ld_16x256<NG>(tm_s + NC + ((uint32_t)(8 * k) << 16), s[1]);
+              tc_ld_16x256(tm_s + ((uint32_t)(8 * k) << 16), s[0]);
+              tc_ld_16x256(tm_s + NC + ((uint32_t)(8 * k) << 16), s[1]);
               tc_wait_ld();
             }
             const float4 ts = tok4[(gs & 3) * 128 + 8 * k];

@@ -113,7 +113,9 @@ struct I8Cfg {
   static constexpr int kTeamWarps = 4 * kGroups, kTeamThreads = 32 * kTeamWarps;
   // (4 and 8 columns: four teams.  Five teams have 80 registers a thread and spill: at 4 columns 11 % slower on one launch
   // per layer and 3-12 % on short and ragged contexts; at 8 columns, 16 flattened layers of two sequences of 131072
-  // tokens, 1095 us with products issued behind a lane test and 1310 us by an elected lane, against 1055 us for four teams.)
+  // tokens, 1095 us with products issued behind a lane test and 1310 us by an elected lane, against 1055 us for four teams.
+  // Five teams behind a lane test and four by an elected lane, 8 columns, us: one sequence of 32768 tokens 28.4 and 24.6, of
+  // 131072 55.5 and 49.4; 4 of 32768 54.1 and 49.2; 16 of 16384 84.2 and 78.3; 16 ragged up to 65536 176 and 160.)
   static constexpr int kTeams = CP == 32 ? 2 : (FULL || CP == 16) ? 3 : 4;
   static constexpr int kProdWarps = CP == 32 ? 2 : 4;
   static constexpr int kProdWarp0 = kTeamWarps * kTeams;
@@ -474,12 +476,6 @@ __device__ __forceinline__ uint64_t i8_pack(uint32_t lo, uint32_t hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
   return d;
 }
-// Shared-memory matrix descriptor with the swizzle mode given (2 = 128 B, 4 = 64 B, 6 = 32 B).
-__device__ __forceinline__ uint64_t i8_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint32_t layout) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) | ((uint64_t)layout << 61);
-}
-
 // Bounded wait until a shared-memory sequence counter has reached `need` (a counter, unlike an mbarrier
 // phase, cannot be misread by a waiter that is ahead of the writer).  Gives up after ~2 s like mbar_wait.
 __device__ __noinline__ bool seq_wait(const volatile int* ctr, int need, volatile int* abort_word) {

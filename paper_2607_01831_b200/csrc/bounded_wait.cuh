@@ -16,8 +16,8 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;
 // Waits until probe() succeeds.  Gives up after about two seconds, or within 16 probes once another thread of the CTA has given
 // up (the abort word is set): then it sets the abort word and returns false.
 // (Inlined at some forty places of a kernel whose roles compete for the instruction caches: one test behind every 16th probe
-// and nothing else.  32-column verification of 131072 tokens takes 95.7 us this way -- the same with a test per 256 probes --
-// and 98.9 us with the abort word looked at apart from the clock, 64 columns 213 and 225 us.)
+// and nothing else.  32-column verification of 131072 tokens takes 97.2 us this way -- the same with a test per 256 probes --
+// and 100.4 us with the abort word looked at in front of the probes and apart from the clock, 64 columns 217 and 228 us.)
 template <class Probe, class Clock>
 LYNX_HD bool bounded_wait(Probe probe, Clock now_ns, volatile int* abort_word) {
   uint64_t t0 = 0;

@@ -25,11 +25,6 @@ constexpr int kLanesPerRow = 8;   // a quarter-warp owns a row: 32 B per lane
 constexpr int kRowsInFlight = 4;
 constexpr int kRowsInFlightIds = 4;
 
-// Round-half-even of the exact product u*inv, as the low byte of an FP32 whose ulp is 1:
-// fma(u, inv, 1.5 * 2^23) rounds the exact sum once, to an integer, ties to even.
-__device__ __forceinline__ uint32_t code_bits(float x, float mn, float inv) {
-  return __float_as_uint(__fmaf_rn(__fsub_rn(x, mn), inv, 12582912.0f));
-}
 __device__ __forceinline__ uint32_t bf2min(uint32_t a, uint32_t b) {
   uint32_t d;
   asm("min.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -61,7 +56,8 @@ __device__ __forceinline__ void codes8(const uint32_t (&w)[4], float mn, float i
   const uint64_t mn2 = pack2(mn, mn), inv2 = pack2(inv, inv), magic2 = pack2(12582912.0f, 12582912.0f);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    // (x - mn) rounded, then fma(u, inv, 1.5 * 2^23): the two elements of a word at once
+    // u = (x - mn) rounded, then fma(u, inv, 1.5 * 2^23), which rounds the exact sum once, to an integer, ties to even: the
+    // code is the low byte.  The two elements of a word at once.
     const uint64_t x2 = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
     uint64_t u2, y2;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(u2) : "l"(x2), "l"(mn2));
@@ -233,7 +229,9 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
                       (uint32_t)rows_per_block, n_rows / rows_per_block, reinterpret_cast<uint32_t*>(anchor),
                       reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta), wide);
   }
-  // (many short CTAs rather than a few waves of long ones: 1105 us with 8 CTAs per SM, 1080 us with 64, 6.6 GB)
+  // (many short CTAs rather than a few waves of long ones.  K and V of 8 heads, 8 and 64 CTAs per SM: 67.8 and 66.7 us for
+  // 65536 tokens, 279 and 240 us for 262144, 1135 and 960 us for 1048576; the same below.  Listed blocks show no such
+  // difference, 78.4 and 80.4 us for 65536 tokens out of 262144, 287 and 283 us for 262144 out of 1048576: 8.)
   const int grid = grid_for((n_rows + rows_per_cta_trip - 1) / rows_per_cta_trip, 64);
   return launch_pdl(split_quantize_kernel<false>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), n_rows, nullptr, 1u,
                     n_rows, reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),

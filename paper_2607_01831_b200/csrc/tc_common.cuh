@@ -25,12 +25,6 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
 }
-// Shared-memory matrix descriptor, 128-byte swizzle: start address, leading / stride byte
-// offsets (16-byte units), descriptor version 1, layout type 2 (SWIZZLE_128B).
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (2ull << 61);
-}
 // Instruction descriptor: FP32 accumulate, FP16 A and B, A K-major, M = 128.
 __host__ __device__ constexpr uint32_t tc_idesc(int n, bool b_mn_major) {
   return (1u << 4) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
@@ -70,32 +64,21 @@ struct TmemRegs<16> {
 };
 template <>
 struct TmemRegs<32> {
-  static __device__ __forceinline__ void ld(uint32_t a, uint32_t* r) {
-    TmemRegs<16>::ld(a, r);
-    TmemRegs<16>::ld(a + 16, r + 16);
-  }
   static __device__ __forceinline__ void st(uint32_t a, const uint32_t* r) {
     TmemRegs<16>::st(a, r);
     TmemRegs<16>::st(a + 16, r + 16);
   }
 };
 
-// Scores with a thread per (8 rows apart) tokens and column pairs: 16 lanes of tensor memory x 8 NG columns in the
+// Scores with a thread per (8 rows apart) tokens and column pairs: 16 lanes of tensor memory x 32 columns in the
 // accumulator layout of the warp-level products -- thread i holds, of column group j, columns 8 j + 2 (i & 3), + 1 of
 // rows i >> 2 (r[4 j], r[4 j + 1]) and i >> 2 + 8 (r[4 j + 2], r[4 j + 3]).
-template <int NG>
 __device__ __forceinline__ void tc_ld_16x256(uint32_t a, uint32_t* r) {
-  static_assert(NG == 2 || NG == 4, "column groups");
-  if constexpr (NG == 4)
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(a) : "memory");
-  else
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(a) : "memory");
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(a) : "memory");
 }
 // Four 8 x 8 blocks of 16-bit values into shared memory: lane i gives the address of row i & 7 of block i >> 3.
 __device__ __forceinline__ void stm_x4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {

@@ -1,8 +1,7 @@
 """GPU parity of the log-sum-exps the attention calls leave in their workspaces, and of decode attention over a
 quantised prefix followed by a BF16 tail (prefix call + BF16-page call + lynx_lse_merge), against the binary64
 oracle (oracle/tail.py).  Outputs within |gpu - ref| <= 2e-3 + 1e-2 |ref| as for every attention call; the
-log-sum-exps within 2e-4 (integer kernels, BF16 kernel) or 3e-3 (FP16 kernel, 33..64 columns): a relative
-error e of a softmax sum moves its logarithm by e."""
+log-sum-exps within 2e-4 whatever the kernel: a relative error e of a softmax sum moves its logarithm by e."""
 import numpy as np
 import pytest
 import torch
@@ -62,8 +61,8 @@ def _oracle(c, full, causal_tail, lens=None, tlens=None):
                                       causal_tail=causal_tail)
 
 
-# columns = n_q * G: 4 / 8 / 16 / 32 (integer kernels; verification takes 32 as two passes), 64 (FP16 kernel for
-# verification, two slices for anchor); a 40000-token sequence spans many CTAs (partial slots, two-level merge)
+# columns = n_q * G: 3 / 4 / 8 / 16 (integer kernels), 32 (FP16 kernel for verification), 64 (likewise; two slices for
+# anchor); a 40000-token sequence spans many CTAs (partial slots, two-level merge)
 @pytest.mark.parametrize("G,n_q,lens", [(4, 1, (700, 0, 33)), (4, 2, (40000, 5)), (8, 2, (130, 2100)), (4, 8, (3000, 3)),
                                         (8, 8, (900, 70)), (1, 3, (1, 257))])
 def test_log_sum_exps_of_the_plane_attention(lynx, G, n_q, lens):
@@ -87,7 +86,7 @@ def test_log_sum_exps_of_the_plane_attention(lynx, G, n_q, lens):
                 r = _oracle(cj, full, False, lens=seen.to(torch.int32))
                 ref_lse[:, j], ref_out[:, j] = r["lse_prefix"][:, 0], r["out"][:, 0]
             _close(got.cpu().numpy().astype(np.float64), ref_out, f"out full={full} causal={causal}")
-            _lse_close(lse, ref_lse, 3e-3 if full and n_q * G > 32 else 2e-4, f"G={G} n_q={n_q} full={full} causal={causal}")
+            _lse_close(lse, ref_lse, 2e-4, f"G={G} n_q={n_q} full={full} causal={causal}")
 
 
 @pytest.mark.parametrize("G,n_q,lens,tail_lens,bt_t", [(4, 1, (5000, 300, 0, 0), (37, 0, 260, 0), 16),

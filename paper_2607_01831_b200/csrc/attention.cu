@@ -1,6 +1,6 @@
 // lynx_anchor_attention and lynx_merge_verify_attention: split-K decode attention over the
 // packed nibble planes, dequantised on chip (sm_100a).  This file holds what the kernels share
-// (parameters, PTX helpers, the end-of-piece merge and the accept / reject decision) and the host
+// (parameters, PTX helpers, the joining of partial results and the accept / reject decision) and the host
 // side; the kernels are in attention_i8.cuh and attention_f16.cuh.
 //
 // What is computed (Section 2 attention equation on the states of Section 4.2; accept/reject
@@ -20,10 +20,10 @@
 // Producer warps stream 16-token sub-blocks of the planes (1 KiB each, contiguous in the paged
 // layout) into a shared-memory ring with bulk copies (TMA) completing on mbarriers, and
 // the queries of each piece into one of two slots.
-// A range that covers a whole (sequence, KV head) writes the output directly, otherwise the
-// partial (m, l, O) goes to the workspace and the last contributor (atomic ticket, no waiting)
-// merges them; for verification the last CTA of a sequence also takes the accept/reject
-// decision.
+// A range that covers a whole (sequence, KV head) writes the output directly (the FP16 kernel: its slot like the others),
+// otherwise the partial (m, l, O) goes to the workspace, and a small dependent kernel joins them, row by row, and takes the
+// accept/reject decision of a verification; anchor calls with many heads have the last contributor of a head join them
+// (atomic ticket, no waiting).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -51,12 +51,11 @@ struct AttnParams {
   int32_t* first_reject;
   float* dev;
   uint32_t* ws_flags;
-  uint32_t* ws_chunk_ctr;  // [B*Hkv]
+  uint32_t* ws_chunk_ctr;  // [B*Hkv] tickets of the CTAs that share a (sequence, KV head)
   uint32_t* ws_seq_ctr;    // [B]
-  uint32_t* ws_group_ctr;  // [2 * CTAs of the largest grid]: tickets of the groups of partial slots
   float* ws_dev;           // [B*Hkv][kMaxQ]
   float* ws_lse;           // [B][nq_stride][Hq] natural-log log-sum-exp of every output row's scores
-  float* ws_part;          // [B*Hkv + CTAs][ncols_pad][kPartStride], slot = segment + CTA index
+  float* ws_part;          // [B*Hkv + CTAs][ncols_pad][kPartStride], slot = segment + CTA index (and see seg_word)
   float atol, rtol;
   float sm_log2;           // softmax_scale * log2(e)
   int B, nq, causal, Hq, Hkv, G, bt, num_blocks, max_blocks, ncols;
@@ -65,7 +64,14 @@ struct AttnParams {
   // (the causal limit of position j of the slice is len - tail + j + 1).  Unsliced: both equal nq.
   int nq_stride, tail;
   int draft_vec;   // draft is 16-byte aligned: its rows are read four values at a time
+  int combine_single;   // the attention kernel leaves a segment of one CTA in its slot, too
+  int inline_merge;     // the last CTA of a segment joins its slots, not attn_combine_kernel
 };
+// The contributors of a segment, first CTA << 16 | number of CTAs (0: no tokens), for attn_combine_kernel: in the padding of
+// the slot of the segment's index, whosever that slot is.
+__device__ __forceinline__ uint32_t* seg_word(const AttnParams& p, size_t bh, int part_cols) {
+  return reinterpret_cast<uint32_t*>(p.ws_part + bh * (size_t)part_cols * kPartStride + 130);
+}
 
 // ------------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -177,17 +183,6 @@ __device__ __forceinline__ float lse_of(float M, float L) {
   return L > 0.0f ? (M + __log2f(L)) * 0.6931471805599453f : -INFINITY;
 }
 
-// Values 4 lane .. 4 lane + 3 of the draft row at float offset `off`.  The interface asks for no more than the alignment
-// of a float: callers hold the draft inside larger buffers.
-__device__ __forceinline__ float4 draft_row_vec(const AttnParams& p, size_t off, int lane) {
-  return ld_dep(reinterpret_cast<const float4*>(p.draft + off) + lane);
-}
-__device__ __forceinline__ float4 draft_row(const AttnParams& p, size_t off, int lane) {
-  if (p.draft_vec) return draft_row_vec(p, off, lane);
-  const float* d = p.draft + off + 4 * lane;
-  return make_float4(ld_dep(d), ld_dep(d + 1), ld_dep(d + 2), ld_dep(d + 3));
-}
-
 struct Item {  // one piece: a run of stage-units of one (sequence, KV head) given to one CTA
   int b, hkv, len, first_cta, n_contrib, pad0, pad1, pad2;  // pad0 = units, pad1 = first unit
 };
@@ -195,207 +190,6 @@ struct Item {  // one piece: a run of stage-units of one (sequence, KV head) giv
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-
-// After a piece's result is in the output (direct) or in its partial slot: the last
-// contributor of the (sequence, KV head) merges the slots, and for verification the CTA holding
-// the final outputs of a head takes part in the accept / reject decision (Section 4.3).
-// Called by all consumer threads of the CTA (named barrier 1).
-template <bool FULL, int kColsPad, int kConsThreads, int kCols = kColsPad, int kFly = 8, int kMaxCC = 4>   // kCols: the most columns of a launch; kFly: row loads in flight per thread
-__device__ __forceinline__ void finish_piece(const AttnParams& p, const Item& item, bool direct, int tid,
-                                             int* misc, int bar_id = 1) {
-  const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
-  const int lane = tid & 31;
-  bool final_here = direct;
-  // The largest |f - d| / (atol + rtol |f|) per position of the window (Section 4.3) goes to devs[], for the CTA that
-  // writes a head's final outputs.  A warp holds a column, so one shuffle reduction and one shared-memory maximum per
-  // column (re-reading the outputs after the merge with a maximum per element: 33.5 us for one layer of 4096 tokens at 16
-  // columns, 29.0 us this way; 18 us less for 64 columns at 131072 tokens, 311.5 to 293.1 us).
-  const bool decide = FULL && p.draft != nullptr;
-  int* devs = misc + 16;
-  if (decide && tid < kMaxQ) devs[tid] = 0;   // (free: the previous piece's were read before its last barrier)
-  // float offset of an output row of this head: column c = position c / G, query head c % G
-  auto row_off = [&](int c) {
-    const int j = c / p.G;
-    return ((uint32_t)(item.b * p.nq_stride + j) * (uint32_t)p.Hq + (uint32_t)(item.hkv * p.G + c - j * p.G));
-  };
-  auto deviation = [&](const float4& f, const float4& d, int j) {
-    const float fv[4] = {f.x, f.y, f.z, f.w}, dv[4] = {d.x, d.y, d.z, d.w};
-    float r = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) r = fmaxf(r, fabsf(fv[i] - dv[i]) / (p.atol + p.rtol * fabsf(fv[i])));
-    const int m = __reduce_max_sync(0xFFFFFFFFu, __float_as_int(r));   // r >= 0: integer order = float order
-    if (lane == 0) atomicMax(devs + j, m);
-  };
-  if (!direct) {
-    // The partial slots of this (sequence, KV head) are merged in two levels, so that no CTA walks
-    // through all of them one L2 round trip after the other (a slot per CTA where one head has the
-    // grid to itself).  The last CTA to arrive of each group of kGroup
-    // neighbouring contributors merges the group into its first slot; the last group to finish
-    // merges the group results into the output.  Every ticket resets itself; nobody waits.
-    constexpr int kGroup = 8, kOneLevel = 24;   // up to kOneLevel slots are merged in one go
-    const int n = item.n_contrib;
-    const int ng = (n + kGroup - 1) / kGroup;
-    const int g = ((int)blockIdx.x - item.first_cta) / kGroup;
-    const int gsize = min(kGroup, n - g * kGroup);
-    float* seg = p.ws_part + (bh + (size_t)item.first_cta) * (size_t)kColsPad * kPartStride;
-    constexpr uint32_t cstride = kColsPad * kPartStride;   // (a segment has a slot per CTA at most: offsets fit 32 bits)
-    named_bar(bar_id, kConsThreads);
-    if (tid == 0) {
-      bool last = true;   // of this CTA's group (n <= kOneLevel: of the whole segment)
-      if (n <= kOneLevel) {
-        last = atomicInc(p.ws_chunk_ctr + bh, (uint32_t)n - 1) == (uint32_t)n - 1;
-      } else if (gsize > 1) {
-        // the group's ticket lives with its first CTA; a CTA can lead two groups at most: the first
-        // group of the segment that starts in its range, and a later group of the one that ends there
-        uint32_t* ctr = p.ws_group_ctr + 2 * (item.first_cta + g * kGroup) + (g == 0 ? 1 : 0);
-        last = atomicInc(ctr, (uint32_t)gsize - 1) == (uint32_t)gsize - 1;
-      }
-      misc[1] = last ? 1 : 0;
-    }
-    named_bar(bar_id, kConsThreads);
-    final_here = false;
-    bool top = n <= kOneLevel;   // this pass writes the output
-    // (one copy of the merge code, run once or twice: uniform over the CTA)
-    for (bool go = misc[1] != 0; go;) {
-      __threadfence();
-      const int first = top ? 0 : g * kGroup;
-      const int count = top ? (n <= kOneLevel ? n : ng) : gsize;
-      const uint32_t sstride = (top && n > kOneLevel ? kGroup : 1) * cstride;
-      // A warp takes kCC columns at a time, a lane 4 dims of each; `count` slots from `first` on (at most 32: a grid has a
-      // CTA per SM); the result goes to the output (normalised) or back to slot `first`.  Lane i first takes the maximum
-      // and the sum of slot i (one load per column), so that the factors of all slots are known and the rows are
-      // independent loads, kFly in flight per thread.  (Column after column, each slot waiting for the one before: 16.5 us
-      // for 18 slots of 32 columns with the decision, 12 us this way.)
-      constexpr int kWarps = kConsThreads / 32, kPerWarp = (kCols + kWarps - 1) / kWarps;
-      constexpr int kCC = kPerWarp < kMaxCC ? kPerWarp : kMaxCC, kSS = kFly / kCC;
-#pragma unroll 1
-      for (int cw = (tid >> 5) * kCC; cw < p.ncols; cw += kWarps * kCC) {
-        float* col = seg + (uint32_t)first * cstride + (uint32_t)(cw * kPartStride);
-        float f[kCC], my_m = 0.0f, my_l = 0.0f;
-        float2 ml[kCC];
-#pragma unroll
-        for (int c = 0; c < kCC; ++c) {
-          ml[c] = make_float2(-INFINITY, 0.0f);
-          if (lane < count && cw + c < p.ncols)
-            ml[c] = __ldcg(reinterpret_cast<const float2*>(col + ((uint32_t)lane * sstride + (uint32_t)(c * kPartStride + 128))));
-        }
-#pragma unroll
-        for (int c = 0; c < kCC; ++c) {
-          float M = ml[c].x;
-#pragma unroll
-          for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
-          f[c] = ml[c].x == -INFINITY ? 0.0f : ex2(ml[c].x - M);
-          float L = f[c] * ml[c].y;
-#pragma unroll
-          for (int off = 16; off >= 1; off >>= 1) L += __shfl_xor_sync(0xFFFFFFFFu, L, off);
-          if (top) f[c] *= L > 0.0f ? 1.0f / L : 0.0f;
-          if (lane == c) { my_m = M; my_l = L; }
-        }
-        float4 acc[kCC];
-#pragma unroll
-        for (int c = 0; c < kCC; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-        for (int i0 = 0; i0 < count; i0 += kSS) {
-          float4 oi[kSS][kCC];
-#pragma unroll
-          for (int u = 0; u < kSS; ++u) {
-            const float4* row = reinterpret_cast<const float4*>(col + (uint32_t)min(i0 + u, count - 1) * sstride) + lane;
-#pragma unroll
-            for (int c = 0; c < kCC; ++c)   // (columns beyond the last of the launch: the slots are padded)
-              oi[u][c] = __ldcg(row + c * (kPartStride / 4));
-          }
-#pragma unroll
-          for (int u = 0; u < kSS; ++u)
-#pragma unroll
-            for (int c = 0; c < kCC; ++c) {
-              const float fu = i0 + u < count ? __shfl_sync(0xFFFFFFFFu, f[c], i0 + u) : 0.0f;
-              if (fu != 0.0f) {
-                acc[c].x = fmaf(oi[u][c].x, fu, acc[c].x);
-                acc[c].y = fmaf(oi[u][c].y, fu, acc[c].y);
-                acc[c].z = fmaf(oi[u][c].z, fu, acc[c].z);
-                acc[c].w = fmaf(oi[u][c].w, fu, acc[c].w);
-              }
-            }
-        }
-        // lane c finishes column c's scalars and knows its row; the rows follow one by one (a loop: this code runs once per
-        // head, straight from a cold instruction cache, where unrolling it costs more than it saves)
-        const int my_c = min(cw + lane, p.ncols - 1);
-        const uint32_t my_row = row_off(my_c);
-        const int my_j = my_c / p.G;
-        if (lane < kCC && cw + lane < p.ncols) {
-          if (top) p.ws_lse[my_row] = lse_of(my_m, my_l);
-          else *reinterpret_cast<float2*>(col + (lane * kPartStride + 128)) = make_float2(my_m, my_l);
-        }
-        float4 dr[kCC];
-#pragma unroll
-        for (int c = 0; c < kCC; ++c)
-          if (decide && top && p.draft_vec)   // (ahead of the stores; a draft that is not aligned is read row by row below)
-            dr[c] = draft_row_vec(p, (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D, lane);
-#pragma unroll 1
-        for (int c = 0; c < kCC && cw + c < p.ncols; ++c) {
-          float4 a = acc[0], d = dr[0];
-#pragma unroll
-          for (int i = 1; i < kCC; ++i)
-            if (c == i) { a = acc[i]; d = dr[i]; }
-          const size_t off = (size_t)__shfl_sync(0xFFFFFFFFu, my_row, c) * LYNX_D;
-          if (decide && top && !p.draft_vec) d = draft_row(p, off, lane);
-          float* dst = top ? p.out + off : col + c * kPartStride;
-          reinterpret_cast<float4*>(dst)[lane] = a;
-          if (decide && top) deviation(a, d, __shfl_sync(0xFFFFFFFFu, my_j, c));
-        }
-      }
-      if (top) {
-        final_here = true;
-        break;
-      }
-      // the group's result is in its first slot: one more ticket, among the groups
-      __threadfence();
-      named_bar(bar_id, kConsThreads);
-      if (tid == 0) misc[1] = (atomicInc(p.ws_chunk_ctr + bh, (uint32_t)ng - 1) == (uint32_t)ng - 1);
-      named_bar(bar_id, kConsThreads);
-      go = misc[1] != 0;
-      top = true;
-    }
-  }
-  // accept / reject (Section 4.3): by the CTA that wrote the final outputs of this head
-  if (decide) {
-    named_bar(bar_id, kConsThreads);  // final outputs written; devs zeroed, or complete where slots were merged
-    if (final_here) {
-      if (direct) {
-#pragma unroll 1
-        for (int c = tid >> 5; c < p.ncols; c += kConsThreads / 32) {
-          const size_t o = (size_t)row_off(c) * LYNX_D;
-          const float4 dr = draft_row(p, o, lane);
-          const float4 f = reinterpret_cast<const float4*>(p.out + o)[lane];
-          deviation(f, dr, c / p.G);
-        }
-        named_bar(bar_id, kConsThreads);
-      }
-      // the last head of the sequence decides: a lane per position, the heads' deviations eight loads at a time
-      if (tid < 32) {
-        if (lane < p.nq) __stcg(p.ws_dev + bh * kMaxQ + lane, __int_as_float(devs[lane]));
-        __threadfence();
-        __syncwarp();
-        uint32_t last = 0;
-        if (lane == 0) last = atomicInc(p.ws_seq_ctr + item.b, (uint32_t)p.Hkv - 1) == (uint32_t)p.Hkv - 1;
-        if (__shfl_sync(0xFFFFFFFFu, last, 0)) {
-          __threadfence();
-          float worst = 0.0f;
-          const float* hd = p.ws_dev + (size_t)item.b * p.Hkv * kMaxQ + lane;
-          if (lane < p.nq) {
-#pragma unroll 8
-            for (int h = 0; h < p.Hkv; ++h) worst = fmaxf(worst, __ldcg(hd + (size_t)h * kMaxQ));
-            p.dev[(size_t)item.b * p.nq_stride + lane] = worst;
-          }
-          const unsigned rej = __ballot_sync(0xFFFFFFFFu, lane < p.nq && worst > 1.0f);
-          if (lane == 0) p.first_reject[item.b] = rej ? __ffs(rej) - 1 : p.nq;
-        }
-      }
-    }
-    named_bar(bar_id, kConsThreads);
-  }
-}
-
 
 // The stream-K cut of the work list (units of ST tokens in (sequence, KV head, position) order) for
 // CTA `cta` of `n_cta`, derived by one warp from the sequence lengths on the device.  Normally every
@@ -410,23 +204,37 @@ struct SkRange {
   long long q, lo, hi, off_lo;   // off_lo: offset of `lo` among the Hkv * U units of sequence b_lo
   int b_lo;
 };
-template <int ST, class ClampLen>
-__device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int cta, int lane, ClampLen clamp_len) {
+// The lengths as one warp knows them: lane i keeps sequence i's, so that the first 32 are read once (a look-up again is a
+// round trip to the L2 on the way to a launch's first copy).
+struct SeqLens {
+  const int32_t* lens;
+  int cap, len0;
+  SeqLens() = default;
+  __device__ __forceinline__ SeqLens(const AttnParams& p, int lane) : lens(p.seq_lens), cap(p.max_blocks * p.bt) {
+    len0 = lane < p.B ? load(lane) : 0;
+  }
+  __device__ __forceinline__ int load(int b) const {
+    const int len = ld_dep(lens + b);
+    return len < 0 ? 0 : (len > cap ? cap : len);
+  }
+  // by the whole warp, of one sequence
+  __device__ __forceinline__ int of(int b) const { return b < 32 ? __shfl_sync(0xFFFFFFFFu, len0, b) : load(b); }
+  // by a lane, of sequence b0 + lane
+  __device__ __forceinline__ int at(int b0, int lane) const { return b0 == 0 ? len0 : load(b0 + lane); }
+};
+template <int ST>
+__device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int cta, int lane, const SeqLens& sl) {
   SkRange r;
   long long tot = 0;
   int umin = 0x7FFFFFFF, umax = 0;
-  for (int b = lane; b < p.B; b += 32) {
-    const int u = (clamp_len(b) + ST - 1) / ST;
-    tot += u;
-    umin = min(umin, u);
-    umax = max(umax, u);
+  for (int b0 = 0; b0 < p.B; b0 += 32) {
+    const bool in = b0 + lane < p.B;
+    const int u = in ? (sl.at(b0, lane) + ST - 1) / ST : 0;   // (at most 2^24)
+    tot += __reduce_add_sync(0xFFFFFFFFu, (unsigned)u);
+    if (in) { umin = min(umin, u); umax = max(umax, u); }
   }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    tot += __shfl_xor_sync(0xFFFFFFFFu, tot, off);
-    umin = min(umin, __shfl_xor_sync(0xFFFFFFFFu, umin, off));
-    umax = max(umax, __shfl_xor_sync(0xFFFFFFFFu, umax, off));
-  }
+  umin = __reduce_min_sync(0xFFFFFFFFu, umin);
+  umax = __reduce_max_sync(0xFFFFFFFFu, umax);
   const long long T = tot * p.Hkv;
   const long long segs = (long long)p.B * p.Hkv;
   if (umin == umax && umax > 0 && segs <= n_cta && (n_cta / segs) * segs * 100 >= 85LL * n_cta) {
@@ -451,7 +259,7 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
     long long running = 0;
     for (int b0 = 0; b0 < p.B; b0 += 32) {
       const int b = b0 + lane;
-      const long long u = b < p.B ? (long long)p.Hkv * ((clamp_len(b) + ST - 1) / ST) : 0;
+      const long long u = b < p.B ? (long long)p.Hkv * ((sl.at(b0, lane) + ST - 1) / ST) : 0;
       long long incl = u;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -474,10 +282,12 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
 }
 
 // Sequences with no token, by one warp of one CTA each: outputs are zero, nothing is rejected unless the draft is not zero.
-template <bool FULL, class ClampLen>
-__device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, int n_cta, int lane, ClampLen clamp_len) {
+// (Off the path of the other sequences: called behind a CTA's last copy.)
+template <bool FULL, int kPartCols>
+__device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, int n_cta, int lane, const SeqLens& sl) {
   for (int b = cta; b < p.B; b += n_cta) {
-    if (clamp_len(b) != 0) continue;
+    if (sl.of(b) != 0) continue;
+    for (int h = lane; h < p.Hkv; h += 32) *seg_word(p, (size_t)b * p.Hkv + h, kPartCols) = 0;
     const size_t n = (size_t)p.nq * p.Hq * LYNX_D;
     for (size_t i = lane; i < n; i += 32) p.out[(size_t)b * p.nq_stride * p.Hq * LYNX_D + i] = 0.0f;
     for (int i = lane; i < p.nq * p.Hq; i += 32) p.ws_lse[(size_t)b * p.nq_stride * p.Hq + i] = -INFINITY;
@@ -495,6 +305,144 @@ __device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, in
       if (lane == 0) p.first_reject[b] = fr;
     }
   }
+}
+
+// Joins the partial results of the CTAs that share a (sequence, KV head) and takes the accept / reject decision: W warps per
+// output row, its slots (m, l, O) dealt to them, five in flight each, the warps' sums joined in order.
+// Launched behind every attention kernel as a programmatic dependent.
+// Latency bounds it -- the look-up of the segment, a round of slots, for verification a ticket and one more round -- and the
+// instructions of a thread in a row, so that a row is cut over many threads where it has many slots.  (Before, the last CTA of
+// a head joined all its columns behind a ticket and took the decision, and the other SMs had nothing to do.  us: one layer of
+// 4096 tokens, 16 columns 27.8 -> 17.6, 4 columns 13.2 -> 11.6, both replayed from a graph; of 131072 tokens, 32 columns, 96.4
+// -> 87.4; two sequences of 131072, 64 columns, 243 -> 236; two of 16000, 8 columns, 25.7 -> 23.8.)
+constexpr int kCombineWarps = 4, kCombineFly = 5;
+template <int W>
+__global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const AttnParams p, int part_cols, int n_slots) {
+  pdl_trigger();
+  const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;   // warp of the row
+  const unsigned r = W == 1 ? blockIdx.x * kCombineWarps + (threadIdx.x >> 5) : blockIdx.x;
+  const int hq = r % p.Hq, bj = r / p.Hq, j = bj % p.nq, b = bj / p.nq;
+  if (W == 1 && b >= p.B) return;
+  const int hkv = hq / p.G, g = hq - hkv * p.G;
+  const size_t bh = (size_t)b * p.Hkv + hkv, row = ((size_t)b * p.nq_stride + j) * p.Hq + hq;
+  const bool decide = p.draft != nullptr;
+  __shared__ float4 o_s[kCombineWarps][32];
+  __shared__ float2 ml_s[kCombineWarps];
+  pdl_wait();
+  const uint32_t seg = ld_dep(seg_word(p, bh, part_cols));
+  float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (decide && warp == 0) {
+    const float* dp = p.draft + row * LYNX_D + 4 * lane;   // (no more than the alignment of a float is asked of the draft)
+    if (p.draft_vec) d = ld_dep(reinterpret_cast<const float4*>(dp));
+    else d = make_float4(ld_dep(dp), ld_dep(dp + 1), ld_dep(dp + 2), ld_dep(dp + 3));
+  }
+  const int first = min((int)(seg >> 16), n_slots - 1), n = min((int)(seg & 0xFFFFu), n_slots - first);
+  const bool direct = n == 1 && !p.combine_single;   // written by the attention kernel
+  if (n == 0 || (direct && !decide)) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!direct) {
+    const size_t sstride = (size_t)part_cols * kPartStride;
+    const float* col = p.ws_part + (bh + first) * sstride + (size_t)(j * p.G + g) * kPartStride;
+    float M = -INFINITY, L = 0.0f;
+    for (int i0 = warp; i0 < n; i0 += W * kCombineFly) {
+      float4 o[kCombineFly];
+      float2 ml[kCombineFly];
+#pragma unroll
+      for (int u = 0; u < kCombineFly; ++u) {
+        const int i = i0 + u * W;
+        ml[u] = make_float2(-INFINITY, 0.0f);
+        o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < n) {
+          const float* s = col + (size_t)i * sstride;
+          ml[u] = ld_dep(reinterpret_cast<const float2*>(s + 128));
+          o[u] = ld_dep(reinterpret_cast<const float4*>(s) + lane);
+        }
+      }
+      const float m0 = M;
+#pragma unroll
+      for (int u = 0; u < kCombineFly; ++u) M = fmaxf(M, ml[u].x);
+      const float f0 = m0 == -INFINITY ? 0.0f : ex2(m0 - M);
+      L *= f0;
+      acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
+#pragma unroll
+      for (int u = 0; u < kCombineFly; ++u) {
+        const float f = ml[u].x == -INFINITY ? 0.0f : ex2(ml[u].x - M);
+        L = fmaf(ml[u].y, f, L);
+        acc.x = fmaf(o[u].x, f, acc.x);
+        acc.y = fmaf(o[u].y, f, acc.y);
+        acc.z = fmaf(o[u].z, f, acc.z);
+        acc.w = fmaf(o[u].w, f, acc.w);
+      }
+    }
+    if (W > 1) {
+      if (warp > 0) o_s[warp][lane] = acc;
+      if (lane == 0) ml_s[warp] = make_float2(M, L);
+      __syncthreads();
+      if (warp > 0) return;
+      float mx = M;
+#pragma unroll
+      for (int k = 1; k < W; ++k) mx = fmaxf(mx, ml_s[k].x);
+      const float f0 = M == -INFINITY ? 0.0f : ex2(M - mx);
+      L *= f0;
+      M = mx;
+      acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
+#pragma unroll
+      for (int k = 1; k < W; ++k) {
+        const float2 ml = ml_s[k];
+        const float4 o = o_s[k][lane];
+        const float f = ml.x == -INFINITY ? 0.0f : ex2(ml.x - mx);
+        L = fmaf(ml.y, f, L);
+        acc.x = fmaf(o.x, f, acc.x);
+        acc.y = fmaf(o.y, f, acc.y);
+        acc.z = fmaf(o.z, f, acc.z);
+        acc.w = fmaf(o.w, f, acc.w);
+      }
+    }
+    const float inv = L > 0.0f ? 1.0f / L : 0.0f;
+    acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+    reinterpret_cast<float4*>(p.out + row * LYNX_D)[lane] = acc;
+    if (lane == 0) p.ws_lse[row] = lse_of(M, L);
+  } else {
+    if (warp > 0) return;
+    acc = ld_dep(reinterpret_cast<const float4*>(p.out + row * LYNX_D) + lane);
+  }
+  if (!decide) return;
+  // the largest |f - d| / (atol + rtol |f|) of the position (Section 4.3), at first per KV head
+  float worst = 0.0f;
+  const float fv[4] = {acc.x, acc.y, acc.z, acc.w}, dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) worst = fmaxf(worst, fabsf(fv[i] - dv[i]) / (p.atol + p.rtol * fabsf(fv[i])));
+  const int m = __reduce_max_sync(0xFFFFFFFFu, __float_as_int(worst));   // worst >= 0: integer order = float order
+  const uint32_t all = (uint32_t)(p.Hq * p.nq);
+  uint32_t last = 0;
+  if (lane == 0) {
+    atomicMax(reinterpret_cast<int*>(p.ws_dev) + bh * kMaxQ + j, m);   // (zeroed by the attention kernel)
+    __threadfence();
+    last = atomicInc(p.ws_seq_ctr + b, all - 1) == all - 1;   // (resets itself)
+  }
+  // the last row of the sequence decides: a lane per position, the heads' deviations eight loads at a time
+  if (__shfl_sync(0xFFFFFFFFu, last, 0)) {
+    __threadfence();
+    float dev = 0.0f;
+    const float* hd = p.ws_dev + (size_t)b * p.Hkv * kMaxQ + lane;
+    if (lane < p.nq) {
+#pragma unroll 8
+      for (int h = 0; h < p.Hkv; ++h) dev = fmaxf(dev, __ldcg(hd + (size_t)h * kMaxQ));
+      p.dev[(size_t)b * p.nq_stride + lane] = dev;
+    }
+    const unsigned rej = __ballot_sync(0xFFFFFFFFu, lane < p.nq && dev > 1.0f);
+    if (lane == 0) p.first_reject[b] = rej ? __ffs(rej) - 1 : p.nq;
+  }
+}
+
+// (units of st tokens; nothing to join where every segment is one unit)
+inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tokens, cudaStream_t st) {
+  if (p.inline_merge || (!p.draft && !p.combine_single && (long long)p.max_blocks * p.bt <= st_tokens)) return LYNX_OK;
+  // a warp per row where a head has no more than a few CTAs on average (one layer: 18; 16 layers of two sequences: 0.6)
+  const unsigned rows = (unsigned)(p.B * p.nq * p.Hq);
+  const bool wide = p.B * p.Hkv * 4 < sm_count();
+  return launch_pdl(wide ? attn_combine_kernel<4> : attn_combine_kernel<1>, wide ? rows : (rows + kCombineWarps - 1) / kCombineWarps,
+                    kCombineWarps * 32, 0, st, p, part_cols, sm_count());
 }
 
 #include "tc_common.cuh"
@@ -518,7 +466,7 @@ struct Plan {
   int per;             // query positions per verification launch
   int ncols;           // columns of the widest launch
   int cols_pad;
-  size_t off_chunk_ctr, off_seq_ctr, off_group_ctr, off_dev, off_lse, off_part, bytes;
+  size_t off_chunk_ctr, off_seq_ctr, off_dev, off_lse, off_part, bytes;
 };
 
 bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
@@ -543,7 +491,7 @@ bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
   size_t off = kWsHeaderBytes;
   pl->off_chunk_ctr = off; off += (size_t)B * s->num_kv_heads * 4;
   pl->off_seq_ctr = off;   off += (size_t)B * 4;
-  pl->off_group_ctr = off; off += (size_t)2 * sm_count() * kMaxCtasPerSm * 4;
+  off += (size_t)2 * sm_count() * kMaxCtasPerSm * 4;   // (unused; the size is a figure that callers hold)
   off = (off + 255) & ~(size_t)255;
   pl->off_dev = off;       off += (size_t)B * s->num_kv_heads * kMaxQ * 4;
   off = (off + 255) & ~(size_t)255;
@@ -623,11 +571,16 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.va = V.anchor; p.vr = V.residual; p.vm = V.meta;
   p.block_table = block_table; p.seq_lens = seq_lens;
   p.out = out; p.draft = full ? draft : nullptr; p.first_reject = first_reject; p.dev = dev;
+  p.combine_single = 0;
+  // Who joins the partial results: attn_combine_kernel where few heads share the grid (and for verification, which needs it for
+  // the decision), the last CTA of a head where a head has a CTA or two on average and its merge overlaps other heads' work (16
+  // layers of two sequences of 131072 tokens, 8 columns: 1025 us, 1040 us by a kernel of its own; one layer of 4096 tokens, 4
+  // columns: 13.2 us by the last CTA, 11.5 us by the kernel).
+  p.inline_merge = !full && (long long)B * shape->num_kv_heads * 4 >= sm_count();
   p.draft_vec = p.draft && aligned16(p.draft);   // (a slice starts whole rows of 512 bytes further on)
   p.ws_flags = reinterpret_cast<uint32_t*>(ws);
   p.ws_chunk_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_chunk_ctr);
   p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_seq_ctr);
-  p.ws_group_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_group_ctr);
   p.ws_dev = reinterpret_cast<float*>(ws + pl.off_dev);
   p.ws_lse = reinterpret_cast<float*>(ws + pl.off_lse);
   p.ws_part = reinterpret_cast<float*>(ws + pl.off_part);

@@ -175,21 +175,16 @@ __device__ __forceinline__ void f16_expand_v(uint32_t raw, uint32_t tile, int i)
 // sequences) and copies its half of the sub-blocks of one tensor: warps 0, 1 the K planes, warps 2, 3 the V planes, eight
 // copies per unit (4 sub-blocks x Anchor / Residual) in one instruction.
 template <class C>
-__device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange& rng, int pw, int lane, uint32_t sbase, uint32_t full0,
+__device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange& rng, const SeqLens& sl, int pw, int lane, uint32_t sbase, uint32_t full0,
                                              uint32_t empty0, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
                                              volatile int* abort_word, const I8Maps* maps) {
   constexpr int ST = C::kST;
   const int tensor = pw >> 1, nstage = tensor ? C::kRingV : C::kRingK;
   const int sub0 = 4 * (pw & 1);
-  const int cap = p.max_blocks * p.bt;
-  auto clamp_len = [&](int b) {
-    int len = ld_dep(p.seq_lens + b);
-    return len < 0 ? 0 : (len > cap ? cap : len);
-  };
   const uint32_t dst0 = sbase + (tensor ? C::kOffRV : C::kOffRK) + (uint32_t)(sub0 * 1024);
   const CUtensorMap *map_a = &maps->m[tensor], *map_r = &maps->m[2 + tensor];
   uint32_t* my_blk = blk_s + pw * 4 * kI8PieceUnits;
-  int b = rng.b_lo, len = clamp_len(b), U = (len + ST - 1) / ST;
+  int b = rng.b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
   int hkv = (int)(rng.off_lo / U), u = (int)(rng.off_lo % U);
   const int n_units = (int)(rng.hi - rng.lo);
   int remaining = n_units, slot = 0, ic = 0;
@@ -207,9 +202,11 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         it.n_contrib = (int)((seg0 + U - 1) / rng.q) - it.first_cta + 1;
         it.pad0 = n; it.pad1 = u; it.pad2 = 0;
         items[qi] = it;
+        if (u == 0) *seg_word(p, (size_t)b * p.Hkv + hkv, C::kPartCols) = (uint32_t)it.first_cta << 16 | (uint32_t)it.n_contrib;
         mbar_arrive(qfull0 + qi * 8);
       }
       __syncwarp();
+      if (u == 0 && lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
     }
     for (int c0 = 0; c0 < n; c0 += kI8PieceUnits) {
       const int cn = min(kI8PieceUnits, n - c0);
@@ -263,7 +260,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         hkv = 0;
         do {
           ++b;
-          len = b < p.B ? clamp_len(b) : 0;
+          len = b < p.B ? sl.of(b) : 0;
           U = (len + ST - 1) / ST;
         } while (b < p.B && U == 0);
         if (b >= p.B) break;  // cannot happen: the range ends inside the list
@@ -391,17 +388,11 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   SkRange rng;
+  SeqLens sl;
   if (warp >= 16 && warp < 20) {
-    const int cap = p.max_blocks * p.bt;
-    auto clamp_len = [&](int b) {
-      int len = ld_dep(p.seq_lens + b);
-      return len < 0 ? 0 : (len > cap ? cap : len);
-    };
-    rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, clamp_len);
-    if (warp == 16) {
-      if (lane == 0) misc[7] = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
-      empty_sequences<true>(p, blockIdx.x, gridDim.x, lane, clamp_len);
-    }
+    sl = SeqLens(p, lane);
+    rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, sl);
+    if (warp == 16 && lane == 0) misc[7] = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
   }
   __syncthreads();  // (A) the range is published
   const int n_units = misc[7];
@@ -636,19 +627,12 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         if (r < CG) ref_s[r] = -INFINITY;
         named_bar(bar_g, 128);
       }
-      const bool direct = item.n_contrib == 1;
       const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
       float* part = p.ws_part + (bh + (size_t)blockIdx.x) * (size_t)C::kPartCols * kPartStride;
       auto put = [&](int c, float v, float m, float l) {   // column c, this lane's dim
         if (c >= p.ncols) return;
-        if (direct) {
-          const int j = c / p.G, hh = c % p.G;
-          p.out[(((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh) * LYNX_D + dim_out] = l > 0.0f ? v / l : 0.0f;
-          if (r == 0) p.ws_lse[((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh] = lse_of(m, l);
-        } else {
-          part[(size_t)c * kPartStride + dim_out] = v;
-          if (r == 0) { part[(size_t)c * kPartStride + 128] = m; part[(size_t)c * kPartStride + 129] = l; }
-        }
+        part[(size_t)c * kPartStride + dim_out] = v;
+        if (r == 0) *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(m, l);
       };
       // (rolled loops, four columns of tensor memory at a time: this code runs once per piece, from a cold instruction cache)
       auto o_cols = [&](int c, float* o) {
@@ -696,10 +680,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         }
       }
       tc_fence_before();
-      __threadfence();
       named_bar(3, 256);   // (the mail and the other group's totals have been read)
-      finish_piece<true, C::kPartCols, 256, NC, 12>(p, item, direct, tid, misc, 3);
-      __syncwarp();
       if (lane == 0) mbar_arrive(qempty + qi * 8);
       gs_base += n_piece;
       ++ic;
@@ -843,8 +824,9 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     const int pw = warp - 16;
     if (n_units == 0) bar_arrive(5, C::kDoneThreads);
     else
-      f16_producer<C>(p, rng, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
+      f16_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
                       reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
+    if (pw == 0) empty_sequences<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl);
     return;
   }
   // ================================================================================== products
@@ -924,7 +906,9 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
 }
 
 template <int NC>
-lynx_status launch_f16(const AttnParams& p, cudaStream_t st) {
+lynx_status launch_f16(AttnParams p, cudaStream_t st) {
   using C = F16Cfg<NC>;
-  return launch_units<true, C::kSmem, C::kThreads, C::kST, attn_f16_kernel<NC>>(p, st);
+  p.combine_single = 1;
+  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, 1, attn_f16_kernel<NC>>(p, st);
+  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, st);
 }

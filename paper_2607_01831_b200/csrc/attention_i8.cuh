@@ -1,6 +1,6 @@
 // Anchor and merge-verify attention on the integer path of the fifth-generation tensor cores
 // (tcgen05.mma kind::i8, accumulators in tensor memory).  Included by attention.cu inside its
-// namespace: shares AttnParams, the stream-K cut of the work and finish_piece with the other
+// namespace: shares AttnParams and the stream-K cut of the work with the other
 // kernels.
 //
 // With one (scale, zero) per token row the two contractions of Section 2's attention run on the
@@ -333,21 +333,17 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
                                             volatile int* abort_word, const I8Maps* maps) {
   constexpr int ST = C::kST, NSTAGE = C::kNStage, NARR = C::kNArr;
   const int n_cta = gridDim.x, cta = blockIdx.x;
-  const int cap = p.max_blocks * p.bt;
-  auto clamp_len = [&](int b) {
-    int len = ld_dep(p.seq_lens + b);
-    return len < 0 ? 0 : (len > cap ? cap : len);
-  };
-  const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, clamp_len);
+  const SeqLens sl(p, lane);
+  const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, sl);
   const long long q = rng.q, lo = rng.lo, hi = rng.hi, off_lo = rng.off_lo;
   const int b_lo = rng.b_lo;
-  if (pw == 0) {
-    if (lane == 0) misc[7] = lo < hi ? (int)(hi - lo) : 0;
-    empty_sequences<FULL>(p, cta, n_cta, lane, clamp_len);
-  }
+  if (pw == 0 && lane == 0) misc[7] = lo < hi ? (int)(hi - lo) : 0;
   __syncthreads();  // (A) the range is published
   const int n_units = (int)(lo < hi ? hi - lo : 0);
-  if (n_units == 0) return;
+  if (n_units == 0) {
+    if (pw == 0) empty_sequences<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
+    return;
+  }
 
   constexpr int SPW = 8 / C::kProdWarps;       // 16-token sub-blocks per warp: 1, 2 or 4
   constexpr int RP = SPW * NARR;               // roles of this warp: (sub-block, array)
@@ -358,7 +354,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
                           (uint32_t)sub * my_bytes;
   constexpr uint32_t kBytesSub = (FULL ? 4u : 2u) * 1024u;   // bytes of one sub-block
   uint32_t* my_blk = blk_s + pw * SPW * kI8PieceUnits;   // [SPW sub-blocks][kI8PieceUnits]
-  int b = b_lo, len = clamp_len(b), U = (len + ST - 1) / ST;
+  int b = b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
   int hkv = (int)(off_lo / U), u = (int)(off_lo % U);
   int remaining = n_units, gs = 0, ic = 0;
   while (remaining > 0) {
@@ -374,9 +370,11 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         it.n_contrib = (int)((seg0 + U - 1) / q) - it.first_cta + 1;
         it.pad0 = n; it.pad1 = u; it.pad2 = 0;
         items[qi] = it;
+        if (u == 0) *seg_word(p, (size_t)b * p.Hkv + hkv, C::kPartCols) = (uint32_t)it.first_cta << 16 | (uint32_t)it.n_contrib;
         mbar_expect_tx(qfull0 + qi * 8, (uint32_t)(p.nq * p.G * LYNX_D * 2));
       }
       __syncwarp();
+      if (u == 0 && lane < kMaxQ && FULL) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
       for (int j = lane; j < p.nq; j += 32)
         bulk_g2s(qraw_u32 + (uint32_t)((qi * C::kColsPad + j * p.G) * LYNX_D * 2),
                  p.q + (((size_t)b * p.nq_stride + j) * p.Hq + (size_t)hkv * p.G) * LYNX_D,
@@ -426,7 +424,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         hkv = 0;
         do {
           ++b;
-          len = b < p.B ? clamp_len(b) : 0;
+          len = b < p.B ? sl.of(b) : 0;
           U = (len + ST - 1) / ST;
         } while (b < p.B && U == 0);
         if (b >= p.B) break;  // cannot happen: the range ends inside the list
@@ -435,6 +433,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   }
   __syncwarp();
   bar_arrive(9, C::kThreads);
+  if (pw == 0) empty_sequences<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
 }
 
 // Largest |q| of a piece's raw queries, by 128 threads (index i of 0..127), reduced over the
@@ -475,6 +474,57 @@ __device__ __forceinline__ uint64_t i8_pack(uint32_t lo, uint32_t hi) {
   uint64_t d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
   return d;
+}
+// The last CTA of a segment (atomic ticket that resets itself, nobody waits) joins its slots, by a team: a warp per column, a
+// lane four dims, four slots in flight.
+template <class C>
+__device__ __forceinline__ void i8_merge_slots(const AttnParams& p, const Item& item, int tt, int tw, int lane, int* my_misc, int bar) {
+  const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
+  const int n = item.n_contrib;
+  constexpr size_t kSlot = (size_t)C::kPartCols * kPartStride;
+  __threadfence();
+  named_bar(bar, C::kTeamThreads);
+  if (tt == 0) my_misc[1] = atomicInc(p.ws_chunk_ctr + bh, (uint32_t)n - 1) == (uint32_t)n - 1;
+  named_bar(bar, C::kTeamThreads);
+  if (my_misc[1] == 0) return;
+  __threadfence();
+#pragma unroll 1
+  for (int c = tw; c < p.ncols; c += C::kTeamWarps) {
+    const float* col = p.ws_part + (bh + (size_t)item.first_cta) * kSlot + (size_t)c * kPartStride;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float M = -INFINITY, L = 0.0f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 4) {
+      float4 o[4];
+      float2 ml[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float* s = col + (size_t)min(i0 + u, n - 1) * kSlot;
+        ml[u] = __ldcg(reinterpret_cast<const float2*>(s + 128));
+        o[u] = __ldcg(reinterpret_cast<const float4*>(s) + lane);
+        if (i0 + u >= n) ml[u].x = -INFINITY;
+      }
+      const float m0 = M;
+      M = fmaxf(fmaxf(fmaxf(M, ml[0].x), ml[1].x), fmaxf(ml[2].x, ml[3].x));   // (finite: the first slot's is)
+      const float f0 = ex2(m0 - M);
+      L *= f0;
+      acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float f = ex2(ml[u].x - M);
+        L = fmaf(ml[u].y, f, L);
+        acc.x = fmaf(o[u].x, f, acc.x);
+        acc.y = fmaf(o[u].y, f, acc.y);
+        acc.z = fmaf(o[u].z, f, acc.z);
+        acc.w = fmaf(o[u].w, f, acc.w);
+      }
+    }
+    const float inv = L > 0.0f ? 1.0f / L : 0.0f;
+    const int j = c / p.G;
+    const size_t row = ((size_t)item.b * p.nq_stride + j) * p.Hq + (size_t)item.hkv * p.G + (c - j * p.G);
+    reinterpret_cast<float4*>(p.out + row * LYNX_D)[lane] = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+    if (lane == 0) p.ws_lse[row] = lse_of(M, L);
+  }
 }
 // Bounded wait until a shared-memory sequence counter has reached `need` (a counter, unlike an mbarrier
 // phase, cannot be misread by a waiter that is ahead of the writer).  Gives up after ~2 s like mbar_wait.
@@ -1098,11 +1148,10 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             if (r == 0) p.ws_lse[((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh] = lse_of(mt[cc], lt[cc]);
           } else {
             part[(size_t)c * kPartStride + dim_out] = v;
-            if (r == 0) { part[(size_t)c * kPartStride + 128] = mt[cc]; part[(size_t)c * kPartStride + 129] = lt[cc]; }
+            if (r == 0) *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(mt[cc], lt[cc]);
           }
         }
-        __threadfence();
-        finish_piece<FULL, C::kPartCols, TT, CP, 8, 2>(p, item, direct, tt, my_misc, bar_tm);
+        if (!FULL && !direct && p.inline_merge) i8_merge_slots<C>(p, item, tt, tw, lane, my_misc, bar_tm);
       }
     }
     // every team keeps count of every team's deposits (the phase of its deposit barrier)
@@ -1126,8 +1175,13 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   if (tid == 0 && (misc[0] || misc[kItemAbort])) atomicOr(p.ws_flags, kFlagTimeout);
 }
 
-// Launches one of the persistent attention kernels: SMEM bytes, THREADS per CTA, units of ST tokens.
-template <bool FULL, int SMEM, int THREADS, int ST, auto KERN>
+// Launches one of the persistent attention kernels: SMEM bytes, THREADS per CTA, units of ST tokens, at least MIN of them
+// per CTA where a sequence has as many (and no more CTAs than SMs).
+// The integer kernels take two: their teams do them side by side (one layer of 4096 tokens, 4 / 16 columns, us replayed from
+// a graph: one unit per CTA 12.9 / 18.2, two 11.6 / 17.7, three 12.9 / 22.5, four 12.7 / 22.4; four by the CTA, whatever the
+// sequences, as before: 17.2 / 36.0 for one sequence of 85 tokens, a CTA to itself for each head 8.5 / 17.7).  The FP16
+// kernels take one (64 columns, 85 tokens: 18.5, four 90; two sequences of 189 tokens: 18.0, two 19.0, four 48).
+template <bool FULL, int SMEM, int THREADS, int ST, int MIN, auto KERN>
 lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
   static bool configured[64] = {false};
   int dev = 0;
@@ -1137,8 +1191,7 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
       return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  const long long cap_units = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + ST - 1) / ST);
-  long long grid = (cap_units + 3) / 4;
+  long long grid = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + MIN * ST - 1) / (MIN * ST));
   const long long full = sm_count();   // one CTA per SM
   grid = grid < 1 ? 1 : (grid > full ? full : grid);
   // Programmatic dependent launch: when the kernel before this one in the stream is of the same kind (one
@@ -1173,5 +1226,6 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
 template <bool FULL, int CP>
 lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
   using C = I8Cfg<FULL, CP>;
-  return launch_units<FULL, C::kSmem, C::kThreads, C::kST, attn_i8_kernel<FULL, CP>>(p, st);
+  const lynx_status rc = launch_units<FULL, C::kSmem, C::kThreads, C::kST, 2, attn_i8_kernel<FULL, CP>>(p, st);
+  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, st);
 }

@@ -614,7 +614,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     return LYNX_OK;
   }
   // verification: the integer kernels up to 16 columns, tcgen05 with FP16 operands (attention_f16.cuh) above (one layer of
-  // 131072 tokens, 32 columns: 96 us by the FP16 kernel, 174 us as two passes of the integer kernel at 16).
+  // 131072 tokens, 32 columns: 83 us by the FP16 kernel, 174 us as two passes of the integer kernel at 16).
   // A window of more than kMaxQ positions or kMaxCols columns runs as slices of whole positions, each a pass
   // of its own over the planes that writes its outputs and deviations; the index of the first rejected
   // position over the whole window then follows from the deviations.

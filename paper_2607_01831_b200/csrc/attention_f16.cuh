@@ -36,14 +36,17 @@
 // memory (integer digit planes: 224 columns per team at 32), while the expansions and the softmax of a unit are long
 // enough to overlap as pipeline stages with double-buffered S, K and V.
 //
-// What bounds it: instruction issue.  A unit takes 6700 warp instructions at 32 columns and 8300 at 64 (K expansion 1300,
-// V expansion 1400, most of the rest softmax), at 2.3 per cycle; tensor pipe 18-21 %, DRAM under a third.  What mattered on
+// What bounds it: instruction issue and the instruction caches.  A unit takes 6000 warp instructions at 32 columns and 7800 at
+// 64 (the expansions a third, most of the rest softmax), at 2.6 per cycle; heavy FMA pipe 45 %, ALU 43 %, tensor pipe 20 %, DRAM
+// a third.  With 64 columns the softmax groups are never idle, with 32 they wait a fifth of the time.  What mattered on
 // the way: no register spills in the softmax loop (little L1 is left beside 227 KB of shared memory: 400 bytes of spills
 // per thread cost a factor of two; hence scores in the 16-lane layout, where a thread sums 8 columns over 4 tokens instead
-// of 32 columns over one), rolled expansion loops (the roles compete for the instruction caches: 118 -> 98 us at 32
-// columns), products issued by an elected lane (93 -> 30 cycles each).  One layer of 131072 tokens: 174 us as two passes of
-// the 16-column integer kernel -> 96 us (32 columns); 293 us by the previous kernel (M = columns, codes not centred) ->
-// 245 us (64 columns, batch 2).
+// of 32 columns over one), rolled loops in the expansions and the producers (118 -> 98 us at 32 columns; unrolled copies of
+// a producer: +5 %), products issued by an elected lane (93 -> 30 cycles each), expansions without a register rotation and drains in
+// packed additions without selects, behind the scores instead of in front of them (32 columns 88.4 -> 83.0 us).  Twice the softmax warps with
+// half of a unit's tokens each and 80 registers: 64 columns +15 %, 32 +4 %.  One layer of 131072 tokens: 174 us as two passes
+// of the 16-column integer kernel -> 83 us (32 columns); two sequences, 64 columns: 293 us by the previous kernel (M = columns, codes
+// not centred) -> 207 us; back to back, before the power cap sets in.
 
 template <int NC>
 struct F16Cfg {
@@ -75,8 +78,8 @@ struct F16Cfg {
   static_assert(kTmOF + 64 <= 512, "tensor memory");
   static constexpr int kThreads = 768, kDoneThreads = 256 + 128 + 32;   // softmax warpgroups, producers, products
   // units between drains: each adds 8 truncating products to a sum.  32 columns, one layer of 131072 tokens: a drain per 8
-  // units 92.7 us (largest error 3.4e-6), per 4 units 94.0 us (2.2e-6), per 2 units 96.2 us (1.4e-6), by when it is below the
-  // integer kernel's in every case; 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
+  // units has a largest error of 3.4e-6, per 4 units 2.2e-6, per 2 units 1.4e-6, by when it is below the integer kernel's in
+  // every case (4 % of the time between 8 and 2 when it was measured); 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
   static constexpr int kDrainUnits = NC == 64 ? 16 : 2;
   // who computes the per-token scalars: with 64 columns the K warps have the time (261 -> 256 us), with 32 they are the
   // slower stage and two spare warps do it (96.1 us, 97.4 us in the K warps)
@@ -130,19 +133,18 @@ __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint3
 // copy engine's 64-byte swizzle (see i8_expand_k_tmem).
 __device__ __forceinline__ void f16_expand_k(uint32_t raw, int r, uint32_t tm_k) {
   const uint32_t s = ((uint32_t)r >> 1) & 3u, row = raw + (uint32_t)r * 64u;
-  // (a rolled loop, with the next chunk's loads ahead: five roles share an instruction cache of some 12 KB per scheduler)
-  uint4 xa = lds128(row + (s << 4)), xr = lds128(row + 8192u + (s << 4));
+  // (a rolled loop: five roles share an instruction cache of some 12 KB per scheduler.  No loads ahead: these warps have time to
+  // wait for shared memory, and moving the next chunk into place costs eight instructions a step)
 #pragma unroll 1
   for (int h = 0; h < 4; ++h) {
-    const uint32_t off = ((uint32_t)((h + 1) & 3) ^ s) << 4;
-    const uint4 na = lds128(row + off), nr = lds128(row + 8192u + off);
+    const uint32_t off = ((uint32_t)h ^ s) << 4;
+    const uint4 xa = lds128(row + off), xr = lds128(row + 8192u + off);
     uint32_t regs[16];
     f16_codes(xa.x, xr.x, regs);
     f16_codes(xa.y, xr.y, regs + 4);
     f16_codes(xa.z, xr.z, regs + 8);
     f16_codes(xa.w, xr.w, regs + 12);
     TmemRegs<16>::st(tm_k + h * 16, regs);
-    xa = na; xr = nr;
   }
 }
 // V codes of a unit into the V tile by 128 threads: thread i takes the 16-byte chunk i & 3 (32 elements) of rows i >> 2 + 32 j.
@@ -153,21 +155,17 @@ __device__ __forceinline__ void f16_expand_v(uint32_t raw, uint32_t tile, int i)
   const uint32_t sw = (uint32_t)(((cc >> 1) ^ (row0 >> 1)) & 1) * 2u;
   const uint32_t base = tile + (uint32_t)(cc >> 1) * 16384u + (uint32_t)row0 * 128u;
   const uint32_t swz = (uint32_t)(((cc & 1) * 4) ^ (row0 & 7) ^ (int)sw) * 16u;
-  uint32_t a = raw + (uint32_t)(row0 * 64 + cc * 16);
-  uint2 xa[2] = {lds64(a + sw * 4u), lds64(a + (sw ^ 2u) * 4u)}, xr[2] = {lds64(a + 8192u + sw * 4u), lds64(a + 8192u + (sw ^ 2u) * 4u)};
+  uint32_t a = raw + (uint32_t)(row0 * 64 + cc * 16), dst = base + swz;
 #pragma unroll 1
-  for (int j = 0; j < 4; ++j) {   // (loads one step ahead, rolled: see f16_expand_k)
-    a = raw + (uint32_t)((row0 + 32 * ((j + 1) & 3)) * 64 + cc * 16);
-    const uint2 na[2] = {lds64(a + sw * 4u), lds64(a + (sw ^ 2u) * 4u)};
-    const uint2 nr[2] = {lds64(a + 8192u + sw * 4u), lds64(a + 8192u + (sw ^ 2u) * 4u)};
+  for (int j = 0; j < 4; ++j, a += 2048u, dst += 4096u) {   // (rolled: see f16_expand_k)
+    const uint2 xa[2] = {lds64(a + sw * 4u), lds64(a + (sw ^ 2u) * 4u)}, xr[2] = {lds64(a + 8192u + sw * 4u), lds64(a + 8192u + (sw ^ 2u) * 4u)};
     const uint32_t wa[4] = {xa[0].x, xa[0].y, xa[1].x, xa[1].y}, wr[4] = {xr[0].x, xr[0].y, xr[1].x, xr[1].y};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {   // register k holds word k ^ sw of the chunk
       uint32_t o[4];
       f16_codes(wa[k], wr[k], o);
-      sts128(base + (uint32_t)j * 4096u + (swz ^ (uint32_t)(k * 16)), o[0], o[1], o[2], o[3]);
+      sts128(dst ^ (uint32_t)(k * 16), o[0], o[1], o[2], o[3]);
     }
-    xa[0] = na[0]; xa[1] = na[1]; xr[0] = nr[0]; xr[1] = nr[1];
   }
 }
 
@@ -337,7 +335,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
                                                                            const __grid_constant__ I8Maps maps) {
   using C = F16Cfg<NC>;
   constexpr bool SPLIT = C::kSplit;
-  constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2, kDW = 16;
+  constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2, kDW = 8;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -433,8 +431,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       // Moves the accumulators (the group's last P.V is complete) into the FP32 copy, scaled by fac_s[] if asked.
       auto drain = [&](bool scale) {
         tc_fence_after();
-        // (a loop: the caller's values fill the registers; 16 columns at a time, a drain per 2 units at 32 columns 96.2 us, 8 at a
-        // time 102 us, and 64 columns 220 -> 215 us)
+        // (a loop: the caller's values, scores among them, fill the registers)
 #pragma unroll 1
         for (int c = 0; c < CG; c += kDW) {
           uint32_t h[kDW], q[kDW], of[kDW];
@@ -442,13 +439,25 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           TmemRegs<kDW>::ld(tm_o + 32 + c, q);
           TmemRegs<kDW>::ld(tm_of + c, of);
           tc_wait_ld();
+          if (!have_of) {   // (a piece's first drain finds the previous piece's copy)
 #pragma unroll
-          for (int k = 0; k < kDW; ++k) {
-            float v = 0.0f;   // (a piece's first drain finds the previous piece's copy; accumulators not restarted since the last drain)
-            if (have_of) v = __uint_as_float(of[k]);
-            if (units_in_acc > 0) v += __uint_as_float(h[k]) + __uint_as_float(q[k]);
-            if (scale) v *= fac_s[c + k];
-            of[k] = __float_as_uint(v);
+            for (int k = 0; k < kDW; ++k) of[k] = 0u;
+          }
+          if (units_in_acc > 0) {   // (else the accumulators have not been restarted since the last drain)
+#pragma unroll
+            for (int k = 0; k < kDW; k += 2) {
+              const uint64_t v = f2_add(f2_add(f2_pack(__uint_as_float(h[k]), __uint_as_float(h[k + 1])),
+                                               f2_pack(__uint_as_float(q[k]), __uint_as_float(q[k + 1]))),
+                                        f2_pack(__uint_as_float(of[k]), __uint_as_float(of[k + 1])));
+              float a, b;
+              f2_unpack(v, a, b);
+              of[k] = __float_as_uint(a);
+              of[k + 1] = __float_as_uint(b);
+            }
+          }
+          if (scale) {
+#pragma unroll
+            for (int k = 0; k < kDW; ++k) of[k] = __float_as_uint(__uint_as_float(of[k]) * fac_s[c + k]);
           }
           TmemRegs<kDW>::st(tm_of + c, of);
         }
@@ -474,10 +483,6 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           bool scale = false;
 #pragma unroll 1
           for (int pass = 0; pass < 2; ++pass) {   // (a second time, from tensor memory, after a change of the references)
-          if (scale || units_in_acc >= C::kDrainUnits) {   // (here, while few registers are live)
-            mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);
-            drain(scale);
-          }
           const uint32_t tm_s = tmem0 + C::kTmS + sl * C::kSCols + col0 + lane_sel;
           uint32_t s[2][4 * NG];   // one part: tokens t0, t0 + 8 | t0 + 16, t0 + 24; two parts: the parts of one half
           if (C::kQP == 1) {
@@ -529,6 +534,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
               ymax = max3(ymax, a, b);
             }
           if (n_own > 0) mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // P free, accumulators current
+          // (behind the scores: the product that is waited for here has had their time to complete)
+          if (scale || units_in_acc >= C::kDrainUnits) drain(scale);
           // ---- a piece's first unit, or a weight that would leave FP16: new reference exponents ----------
           if (!bar_or(bar_g, 128, fresh || ymax > 15.0f)) break;
 #pragma unroll
@@ -570,6 +577,9 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
             scale = !fresh;
             fresh = false;
           }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sfree + sl * 8);   // the scores have been read: the unit after next may have their place
           // ---- weights of this thread's tokens into the P tile --------------------------------------------------
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -597,7 +607,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) { mbar_arrive(sfree + sl * 8); mbar_arrive(mfree + (gs & 3) * 8); mbar_arrive(pready + g * 8); }
+          if (lane == 0) { mbar_arrive(mfree + (gs & 3) * 8); mbar_arrive(pready + g * 8); }
           ++units_in_acc;
         }
         mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // the last P.V
@@ -895,10 +905,23 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         __syncwarp();
       }
     };
-    if (n_units > 0) qk(0);
+    // Q.K^T runs a unit ahead of P.V.  With 32 columns, where a group has one place for its scores, two units where it can: the
+    // scores of unit gs are given up before its weights are complete.  It must not insist on unit gs + 2: where pieces are short
+    // its queries may belong to a piece that is published only once unit gs has been left.  (One layer of 131072 tokens 89.2 ->
+    // 88.4 us; with 64 columns, which have two places, looking ahead costs 2 %.)
+    int next = 0;
 #pragma unroll 1
     for (int gs = 0; gs < n_units; ++gs) {
-      if (gs + 1 < n_units) qk(gs + 1);
+#pragma unroll 1
+      while (next < min(gs + 2, n_units)) qk(next++);
+      if (!SPLIT && next < n_units) {
+        const uint32_t kb = kready + (next & 1) * 8, kp = (next >> 1) & 1, sb = sfree + (next & 1) * 8, sp = kp ^ 1u;
+        const uint32_t pb = pready + (gs & 1) * 8, pp = (gs >> 1) & 1;
+        bool early = false;
+        bounded_wait([&] { early = mbar_test(kb, kp) && mbar_test(sb, sp); return early || mbar_test(pb, pp); },
+                     [] { return globaltimer_ns(); }, abort_word);
+        if (early) qk(next++);
+      }
       pv(gs);
     }
     bar_arrive(5, C::kDoneThreads);

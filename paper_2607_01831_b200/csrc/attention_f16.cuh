@@ -93,9 +93,13 @@ template <int N>
 __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // The bounded wait of mbar_wait without a call: ptxas cannot split the registers of a kernel that has calls.
+template <class Probe>
+__device__ __forceinline__ bool wait_in(Probe probe, volatile int* abort_word) {
+  return bounded_wait(probe, [] { return globaltimer_ns(); }, abort_word);
+}
 __device__ __forceinline__ bool mbar_wait_in(uint32_t bar, uint32_t parity, volatile int* abort_word) {
   if (mbar_test(bar, parity)) return true;
-  return bounded_wait([=] { return mbar_try_wait(bar, parity); }, [] { return globaltimer_ns(); }, abort_word);
+  return wait_in([=] { return mbar_try_wait(bar, parity); }, abort_word);
 }
 
 // position -> element within a group of 8: {0,4,2,6,1,5,3,7} (what the nibble expansion yields), its own inverse
@@ -918,8 +922,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         const uint32_t kb = kready + (next & 1) * 8, kp = (next >> 1) & 1, sb = sfree + (next & 1) * 8, sp = kp ^ 1u;
         const uint32_t pb = pready + (gs & 1) * 8, pp = (gs >> 1) & 1;
         bool early = false;
-        bounded_wait([&] { early = mbar_test(kb, kp) && mbar_test(sb, sp); return early || mbar_test(pb, pp); },
-                     [] { return globaltimer_ns(); }, abort_word);
+        wait_in([&] { early = mbar_test(kb, kp) && mbar_test(sb, sp); return early || mbar_test(pb, pp); }, abort_word);
         if (early) qk(next++);
       }
       pv(gs);

@@ -114,6 +114,13 @@ def _ok(status: int, what: str):
         raise LynxError(f"{what}: status {status} ({msg})")
 
 
+def _result(r, what: str):
+    """What a fast call returned: its result, or a status to raise."""
+    if type(r) is int:
+        _ok(r, what)
+    return r
+
+
 def _ptr(t: torch.Tensor | None):
     if t is None:
         return None
@@ -134,6 +141,34 @@ def _stream():
     if _raw_stream is None or _raw_device is None:
         return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_raw_device())
+
+
+# The calls below that a program makes per layer and step go through an extension (csrc/native.cpp) that does what their Python
+# bodies do, in one call; it returns None for whatever is not plain, and then the Python body runs.  us of host time per call
+# (marshalling through ctypes -> extension): anchor_attention 12 -> 5 to 8, merge_verify_attention 17 -> 10, the four calls of a decode with a BF16
+# tail 45 -> 21, Algorithm 1 there and back for K and V 51 -> 28.
+def _python_only(*_):
+    return None
+
+
+def _fast(var: str, name: str):
+    """The extension's function `name`, found when the global `var` that holds this is first called."""
+    def first(*args):
+        load()   # (raises where the library is not built)
+        try:
+            from . import _native
+        except ImportError:   # built for another torch: ctypes alone
+            _native = None
+        globals()[var] = getattr(_native, name, _python_only)
+        return globals()[var](*args)
+    return first
+
+
+_fast_split_quantize, _fast_recombine = _fast("_fast_split_quantize", "split_quantize"), _fast("_fast_recombine", "recombine")
+_fast_anchor, _fast_verify = _fast("_fast_anchor", "anchor_attention"), _fast("_fast_verify", "merge_verify_attention")
+_fast_bf16, _fast_lse_view = _fast("_fast_bf16", "bf16_attention"), _fast("_fast_lse_view", "lse_view")
+_fast_lse_merge = _fast("_fast_lse_merge", "lse_merge")
+_fast_hier_quantize, _fast_hier_dequantize = _fast("_fast_hier_quantize", "hier_quantize"), _fast("_fast_hier_dequantize", "hier_dequantize")
 
 
 @dataclass
@@ -161,6 +196,10 @@ def split_quantize(src: torch.Tensor, out: Planes | None = None, block_ids: torc
         raise LynxError("src must be BF16 [..., 128]")
     if out is None:
         out = alloc_planes(src.shape[:-1], src.device)
+    r = _fast_split_quantize(src, out, block_ids, rows_per_block)
+    if r is not None:
+        _ok(r, "lynx_split_quantize")
+        return out
     n_rows = src.numel() // D
     nb = 0 if block_ids is None else block_ids.numel()
     _ok(load().lynx_split_quantize(_ptr(src), n_rows, _ptr(block_ids), nb, rows_per_block,
@@ -171,6 +210,9 @@ def split_quantize(src: torch.Tensor, out: Planes | None = None, block_ids: torc
 
 def recombine(planes: Planes, want_codes: bool = True, want_bf16: bool = False):
     """lynx_recombine: returns (codes u8 [...,128] or None, dequantised BF16 [...,128] or None)."""
+    r = _fast_recombine(planes, want_codes, want_bf16)
+    if r is not None:
+        return _result(r, "lynx_recombine")
     lead = tuple(planes.anchor.shape[:-1])
     dev = planes.anchor.device
     codes = torch.empty(lead + (D,), dtype=torch.uint8, device=dev) if want_codes else None
@@ -218,6 +260,9 @@ def anchor_attention(geo: Geometry, q: torch.Tensor, K: Planes, V: Planes, block
                      seq_lens: torch.Tensor, workspace: torch.Tensor, causal: bool = False,
                      softmax_scale: float = 0.0, out: torch.Tensor | None = None) -> torch.Tensor:
     """lynx_anchor_attention: q BF16 [B][n_q][Hq][128] -> float32 [B][n_q][Hq][128]."""
+    r = _fast_anchor(geo, q, K, V, block_table, seq_lens, workspace, causal, softmax_scale, out)
+    if r is not None:
+        return _result(r, "lynx_anchor_attention")
     B, n_q, Hq, d = q.shape
     if q.dtype != torch.bfloat16 or d != D or Hq != geo.num_q_heads:
         raise LynxError("q must be BF16 [B][n_q][Hq][128]")
@@ -257,6 +302,10 @@ def merge_verify_attention(geo: Geometry, q: torch.Tensor, K: Planes, V: Planes,
                            dev: torch.Tensor | None = None):
     """lynx_merge_verify_attention -> (out_full f32 [B][k][Hq][128], first_reject i32 [B], dev f32 [B][k]).
     first_reject / dev are None when no draft is given."""
+    r = _fast_verify(geo, q, K, V, block_table, seq_lens, workspace, draft_out, atol, rtol, causal, softmax_scale, out_full,
+                     first_reject, dev)
+    if r is not None:
+        return _result(r, "lynx_merge_verify_attention")
     B, k, Hq, d = q.shape
     if q.dtype != torch.bfloat16 or d != D or Hq != geo.num_q_heads:
         raise LynxError("q must be BF16 [B][k][Hq][128]")
@@ -283,6 +332,9 @@ def bf16_attention(geo: Geometry, q: torch.Tensor, k_pages: torch.Tensor, v_page
                    causal: bool = False, softmax_scale: float = 0.0, out: torch.Tensor | None = None) -> torch.Tensor:
     """lynx_bf16_attention: decode attention over dequantised BF16 pages [num_blocks][Hkv][bt][128]
     (what recombine(want_bf16=True) writes).  q BF16 [B][n_q][Hq][128] -> float32 [B][n_q][Hq][128]."""
+    r = _fast_bf16(geo, q, k_pages, v_pages, block_table, seq_lens, workspace, causal, softmax_scale, out)
+    if r is not None:
+        return _result(r, "lynx_bf16_attention")
     B, n_q, Hq, d = q.shape
     if q.dtype != torch.bfloat16 or d != D or Hq != geo.num_q_heads:
         raise LynxError("q must be BF16 [B][n_q][Hq][128]")
@@ -314,12 +366,18 @@ def _lse_view(addr, workspace: torch.Tensor, B: int, n_q: int, Hq: int, what: st
 def workspace_lse(geo: Geometry, B: int, n_q: int, workspace: torch.Tensor) -> torch.Tensor:
     """lynx_workspace_lse: float32 [B][n_q][Hq] view, inside `workspace`, of the natural-log log-sum-exps the last
     anchor_attention / merge_verify_attention call with this (B, n_q) left there."""
+    r = _fast_lse_view(geo, B, n_q, workspace, False)
+    if r is not None:
+        return r
     return _lse_view(load().lynx_workspace_lse(ctypes.byref(geo._c()), B, n_q, _ptr(workspace)), workspace, B, n_q,
                      geo.num_q_heads, "lynx_workspace_lse")
 
 
 def bf16_workspace_lse(geo: Geometry, B: int, n_q: int, workspace: torch.Tensor) -> torch.Tensor:
     """lynx_bf16_workspace_lse: the same for the workspace of a bf16_attention call."""
+    r = _fast_lse_view(geo, B, n_q, workspace, True)
+    if r is not None:
+        return r
     return _lse_view(load().lynx_bf16_workspace_lse(ctypes.byref(geo._c()), B, n_q, _ptr(workspace)), workspace, B,
                      n_q, geo.num_q_heads, "lynx_bf16_workspace_lse")
 
@@ -328,6 +386,9 @@ def lse_merge(out_a: torch.Tensor, lse_a: torch.Tensor, out_b: torch.Tensor, lse
               out: torch.Tensor | None = None, want_lse: bool = False):
     """lynx_lse_merge: two attention results float32 [...][128] over disjoint key sets, with their log-sum-exps
     float32 [...], joined into the attention over the union.  Returns out, or (out, lse) with want_lse."""
+    r = _fast_lse_merge(out_a, lse_a, out_b, lse_b, out, want_lse)
+    if r is not None:
+        return _result(r, "lynx_lse_merge")
     if out_a.dtype != torch.float32 or out_b.dtype != torch.float32 or out_a.shape != out_b.shape or out_a.shape[-1] != D:
         raise LynxError("out_a, out_b must be float32 [...][128] of one shape")
     rows = out_a.numel() // D
@@ -393,6 +454,9 @@ class HierPlanes:
 
 def hier_quantize(src: torch.Tensor) -> HierPlanes:
     """lynx_hier_quantize: src BF16 [n_pages][256][128] -> HierPlanes."""
+    r = _fast_hier_quantize(src)
+    if r is not None:
+        return HierPlanes(*_result(r, "lynx_hier_quantize"))
     if src.dtype != torch.bfloat16 or src.dim() != 3 or tuple(src.shape[1:]) != (256, D):
         raise LynxError("src must be BF16 [n_pages][256][128]")
     n, dev = src.shape[0], src.device
@@ -406,6 +470,9 @@ def hier_quantize(src: torch.Tensor) -> HierPlanes:
 
 def hier_dequantize(h: HierPlanes, anchor_only: bool = False, out: torch.Tensor | None = None) -> torch.Tensor:
     """lynx_hier_dequantize -> BF16 [n_pages][256][128] (from the Anchor stream alone if asked)."""
+    r = _fast_hier_dequantize(h.q_anc, None if anchor_only else h.q_res, h.gamma_min, h.gamma_scale, h.mu, h.sigma, out)
+    if r is not None:
+        return _result(r, "lynx_hier_dequantize")
     n = h.q_anc.shape[0]
     if out is None:
         out = torch.empty(n, 256, D, dtype=torch.bfloat16, device=h.q_anc.device)

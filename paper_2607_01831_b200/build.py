@@ -1,29 +1,45 @@
-"""Builds liblynx.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds liblynx.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _native.so (the Python calls that go straight
+to it, against the installed torch) with g++."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "liblynx.so")
+NATIVE = os.path.join(_HERE, "_native.so")
 SOURCES = ["api.cu", "split_quantize.cu", "attention.cu", "bf16_attention.cu", "hier_quantize.cu", "token_verify.cu", "lse_merge.cu", "bit_split.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(_ROOT, "include", "lynx.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _native_cmd(out: str) -> list:
+    """The extension is linked to liblynx.so beside it; torch's own libraries are there once torch is imported."""
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cxx = os.environ.get("CXX", "g++")
+    cmd = [cxx, "-O2", "-std=c++17", "-fPIC", "-shared", "-I", os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"]]
+    for p in include_paths(device_type="cuda"):
+        cmd += ["-isystem", p]
+    cmd += [os.path.join(CSRC, "native.cpp"), "-o", out]
+    for p in library_paths(device_type="cuda"):
+        cmd += ["-L", p]
+    return cmd + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-L", _HERE, "-l:liblynx.so", "-Wl,-rpath,$ORIGIN"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into liblynx.so; returns its path."""
+    """Compile every .cu under csrc/ into liblynx.so and csrc/native.cpp into _native.so; returns the former's path."""
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -47,6 +63,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.run([nvcc, "-shared", "-o", tmp, *objs], check=True)   # static cudart (nvcc default)
     os.replace(tmp, LIB)
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.run(_native_cmd(tmp), check=True)
+    os.replace(tmp, NATIVE)
     return LIB
 
 

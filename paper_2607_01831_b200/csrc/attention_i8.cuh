@@ -248,6 +248,33 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+// (One instruction per maximum and the sums below instead of butterflies in the restart and at the end of a piece, which lie in and
+// around the unit loop: fewer steps in a row where a piece starts and ends, and less code in the instruction caches.  us: 16 ragged
+// sequences at 16 columns 321 -> 275, 16 layers of two sequences of 131072 tokens at 8 columns 907 -> 878 before the power cap sets
+// in, one layer of 131072 tokens at 4 columns 39.0 -> 37.7, two sequences of 16000 at 8 columns 24.0 -> 21.8.)
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+// The sums of N values per lane over a warp: lane i returns that of value i / (32 / N).  Half of the values change places at
+// every step, 2 N - 2 additions in all where N butterflies would take 5 N; each sum in the order of a butterfly.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+  static_assert(N == 8 || N == 16 || N == 32, "lanes share the values evenly");
+  int off = 16;
+#pragma unroll
+  for (int m = N / 2; m >= 1; m >>= 1, off >>= 1)
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+      const bool up = (lane & off) != 0;
+      const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, off);
+    }
+#pragma unroll
+  for (; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], off);
+  return v[0];
+}
 __device__ __forceinline__ float ex2_full(float x) {   // no flush of small results
   float y;
   asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -965,9 +992,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           for (int c = 0; c < CG; ++c) {   // (rare path: back to absolute exponents x = y + ref)
             float a, b;
             f2_unpack(y2[c >> 1], a, b);
-            float mx = ((c & 1) ? b : a) + (fresh ? 0.0f : ref_s[c0 + c]);
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
+            const float mx = warp_max(((c & 1) ? b : a) + (fresh ? 0.0f : ref_s[c0 + c]));
             if (lane == 0) my_red[tw * CG + c] = mx;
           }
           named_bar(bar_tm, TT);
@@ -1072,22 +1097,15 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       }
       tc_fence_before();
       // totals of l and zs over the 128 token lanes of every column group
+      {
+        float v[2 * CG];   // l of the group's columns, then zs
 #pragma unroll
-      for (int c = 0; c < CG; ++c) {
-        float a, b;
-        {
-          float l_lo, l_hi, z_lo, z_hi;
-          f2_unpack(l2[c >> 1], l_lo, l_hi);
-          f2_unpack(zs2[c >> 1], z_lo, z_hi);
-          a = (c & 1) ? l_hi : l_lo;
-          b = (c & 1) ? z_hi : z_lo;
+        for (int c = 0; c < CG / 2; ++c) {
+          f2_unpack(l2[c], v[2 * c], v[2 * c + 1]);
+          f2_unpack(zs2[c], v[CG + 2 * c], v[CG + 2 * c + 1]);
         }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-          a += __shfl_xor_sync(0xFFFFFFFFu, a, off);
-          b += __shfl_xor_sync(0xFFFFFFFFu, b, off);
-        }
-        if (lane == 0) { my_red[tw * 2 * CG + c] = a; my_red[tw * 2 * CG + CG + c] = b; }
+        const float sum = warp_sums(v, lane);
+        if ((lane & (32 / (2 * CG) - 1)) == 0) my_red[tw * 2 * CG + lane / (32 / (2 * CG))] = sum;
       }
       named_bar(bar_tm, TT);
       if (tt < 2 * CP) {   // my_lz: l of the CP columns, then zs
@@ -1116,11 +1134,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         float lt[CG], zt[CG], mt[CG];
 #pragma unroll
         for (int c = 0; c < CG; ++c) { lt[c] = my_lz[c0 + c]; zt[c] = my_lz[CP + c0 + c]; mt[c] = ref_s[c0 + c]; }
+        // (one wait for all of them, one barrier before and one behind: team by team cost two barriers each)
+        auto deposit = [&](int d) { return d != tm && (d - team0 + T) % T < n_piece; };   // (not itself, nor a team without a unit in the piece)
+        if (tt == 0) {
+#pragma unroll
+          for (int d = 0; d < T; ++d)
+            if (deposit(d)) seq_wait(misc + 16 + d, (int)dep_cnt[d] + 1, abort_word);
+        }
+        named_bar(bar_tm, TT);
 #pragma unroll
         for (int d = 0; d < T; ++d) {
-          if (d == tm || (d - team0 + T) % T >= n_piece) continue;   // itself; a team without a unit in the piece
-          if (tt == 0) seq_wait(misc + 16 + d, (int)dep_cnt[d] + 1, abort_word);   // its deposit is complete
-          named_bar(bar_tm, TT);
+          if (!deposit(d)) continue;
           const float* mo = reinterpret_cast<const float*>(smem + d * C::kTeamBytes);
           const float* mh = reinterpret_cast<const float*>(smem + d * C::kTeamBytes + C::kTile);
 #pragma unroll
@@ -1134,9 +1158,13 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             zt[c] = zt[c] * f1 + z2 * f2;
             mt[c] = M;
           }
-          __threadfence_block();
-          named_bar(bar_tm, TT);
-          if (tt == 0) *reinterpret_cast<volatile int*>(misc + 24 + d) = (int)dep_cnt[d] + 1;   // it may deposit again
+        }
+        __threadfence_block();
+        named_bar(bar_tm, TT);
+        if (tt == 0) {
+#pragma unroll
+          for (int d = 0; d < T; ++d)
+            if (deposit(d)) *reinterpret_cast<volatile int*>(misc + 24 + d) = (int)dep_cnt[d] + 1;   // it may deposit again
         }
         const bool direct = item.n_contrib == 1;
         const size_t bh = (size_t)item.b * p.Hkv + item.hkv;

@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "block_division.cuh"
 #include "bounded_wait.cuh"
 #include "lynx_common.cuh"
 
@@ -64,9 +65,15 @@ struct AttnParams {
   // (the causal limit of position j of the slice is len - tail + j + 1).  Unsliced: both equal nq.
   int nq_stride, tail;
   int draft_vec;   // draft is 16-byte aligned: its rows are read four values at a time
+  BlockDiv bt_div;      // for t / bt
   int combine_single;   // the attention kernel leaves a segment of one CTA in its slot, too
   int inline_merge;     // the last CTA of a segment joins its slots, not attn_combine_kernel
 };
+// Block of token t of a sequence.  (No division: its code, at four places of the unit loops, costs more in the instruction caches
+// than its time.  Together with rolled drains and one copy of the 4-column kernel's restart, us: one layer of 131072 tokens 37.7 ->
+// 37.1, two sequences of 16000 at 8 columns 22.1 -> 21.2, 16 ragged sequences with a verification at 16 columns 276 -> 274, one layer
+// of 4096 tokens at 16 columns 18.0 -> 17.0.)
+__device__ __forceinline__ int block_of(const AttnParams& p, int t) { return quotient(t, p.bt_div); }
 // The contributors of a segment, first CTA << 16 | number of CTAs (0: no tokens), for attn_combine_kernel: in the padding of
 // the slot of the segment's index, whosever that slot is.
 __device__ __forceinline__ uint32_t* seg_word(const AttnParams& p, size_t bh, int part_cols) {
@@ -200,6 +207,16 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
 // end of one piece and the start of another, at the cost of n_cta - c * segments idle CTAs (accepted
 // up to 15 %).  lo, hi index a list in which every segment occupies c * q entries, so that the
 // contributors of a segment and their partial slots follow from lo and q as in the plain cut.
+// a / b for 0 <= a < 2^22, 0 < b < 2^22: ten instructions, where an integer division takes thirty (64-bit: a hundred) one after
+// the other, in the one warp that the first copy of a launch waits for.
+__device__ __forceinline__ int small_div(int a, int b) {
+  const int q = __float2int_rz(__fdividef((float)a, (float)b));   // (two units of the last place: off by one at most)
+  const int r = a - q * b;
+  return q + (r >= b) - (r < 0);
+}
+__device__ __forceinline__ long long sk_div(long long a, long long b) {   // a, b >= 0
+  return ((a | b) >> 22) == 0 ? (long long)small_div((int)a, (int)b) : a / b;
+}
 struct SkRange {
   long long q, lo, hi, off_lo;   // off_lo: offset of `lo` among the Hkv * U units of sequence b_lo
   int b_lo;
@@ -237,20 +254,21 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
   umax = __reduce_max_sync(0xFFFFFFFFu, umax);
   const long long T = tot * p.Hkv;
   const long long segs = (long long)p.B * p.Hkv;
-  if (umin == umax && umax > 0 && segs <= n_cta && (n_cta / segs) * segs * 100 >= 85LL * n_cta) {
-    const int c = (int)(n_cta / segs), U = umax;
-    r.q = (U + c - 1) / c;
-    const int s = cta / c, part = cta % c;
+  const int per_seg = segs <= n_cta ? small_div(n_cta, (int)segs) : 0;
+  if (umin == umax && umax > 0 && segs <= n_cta && per_seg * (int)segs * 100 >= 85 * n_cta) {
+    const int c = per_seg, U = umax;
+    r.q = sk_div(U + c - 1, c);
+    const int s = small_div(cta, c), part = cta - s * c;
     r.lo = r.hi = 0; r.b_lo = 0; r.off_lo = 0;
     if (s < segs && (long long)part * r.q < U) {
-      r.b_lo = s / p.Hkv;
-      r.off_lo = (long long)(s % p.Hkv) * U + (long long)part * r.q;
+      r.b_lo = small_div(s, p.Hkv);
+      r.off_lo = (long long)(s - r.b_lo * p.Hkv) * U + (long long)part * r.q;
       r.lo = ((long long)s * c + part) * r.q;
       r.hi = r.lo + min(r.q, (long long)U - (long long)part * r.q);
     }
     return r;
   }
-  r.q = (T + n_cta - 1) / n_cta;
+  r.q = sk_div(T + n_cta - 1, n_cta);
   r.lo = (long long)cta * r.q;
   r.hi = (r.lo + r.q < T) ? r.lo + r.q : T;
   r.b_lo = 0;
@@ -591,6 +609,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.Hq = shape->num_q_heads; p.Hkv = shape->num_kv_heads; p.G = p.Hq / p.Hkv;
   p.bt = shape->block_tokens; p.num_blocks = shape->num_blocks; p.max_blocks = shape->max_blocks_per_seq;
   p.ncols = pl.ncols;
+  p.bt_div = block_div(p.bt);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the fixed array keeps what the previous call left: the status word and the tickets must be zero
   if (fixed_scratch && cudaMemsetAsync(workspace, 0, pl.off_dev, st) != cudaSuccess) return LYNX_ERR_CUDA;

@@ -187,7 +187,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
   const CUtensorMap *map_a = &maps->m[tensor], *map_r = &maps->m[2 + tensor];
   uint32_t* my_blk = blk_s + pw * 4 * kI8PieceUnits;
   int b = rng.b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
-  int hkv = (int)(rng.off_lo / U), u = (int)(rng.off_lo % U);
+  int hkv = (int)sk_div(rng.off_lo, U), u = (int)(rng.off_lo - (long long)hkv * U);
   const int n_units = (int)(rng.hi - rng.lo);
   int remaining = n_units, slot = 0, ic = 0;
   uint32_t phase = 1;   // (a fresh barrier passes a wait for the phase before its first)
@@ -200,8 +200,8 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
       if (lane == 0) {
         Item it;
         it.b = b; it.hkv = hkv; it.len = len;
-        it.first_cta = (int)(seg0 / rng.q);
-        it.n_contrib = (int)((seg0 + U - 1) / rng.q) - it.first_cta + 1;
+        it.first_cta = (int)sk_div(seg0, rng.q);
+        it.n_contrib = (int)sk_div(seg0 + U - 1, rng.q) - it.first_cta + 1;
         it.pad0 = n; it.pad1 = u; it.pad2 = 0;
         items[qi] = it;
         if (u == 0) *seg_word(p, (size_t)b * p.Hkv + hkv, C::kPartCols) = (uint32_t)it.first_cta << 16 | (uint32_t)it.n_contrib;
@@ -216,12 +216,13 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         const int t0 = (u + c0 + (i >> 2)) * ST + (sub0 + (i & 3)) * 16;
         uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
         if (t0 < len) {
-          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+          const int bi = block_of(p, t0);
+          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + bi);
           if (blk < 0 || blk >= p.num_blocks) {
             atomicOr(p.ws_flags, kFlagBadBlock);
             blk = blk < 0 ? 0 : p.num_blocks - 1;
           }
-          row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 % p.bt));
+          row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 - bi * p.bt));
         }
         my_blk[i] = row;
       }
@@ -281,25 +282,24 @@ struct F16Meta {
   float4* tok4;
   float* tok1;
   const int32_t* table;
-  int i0, bt_shift, ih, len, n_piece, u0;
+  int i0, ih, len, n_piece, u0;
   int blk_n[N];
   float2 km[N], vm[N];
   __device__ __forceinline__ void init(const AttnParams& p, unsigned char* smem, int first) {
     i0 = first;
     tok4 = reinterpret_cast<float4*>(smem + C::kOffTok) + i0;
     tok1 = reinterpret_cast<float*>(smem + C::kOffTok + 4 * 128 * 16) + i0;
-    bt_shift = (p.bt & (p.bt - 1)) == 0 ? 31 - __clz(p.bt) : -1;
   }
   __device__ __forceinline__ int blk_of(const AttnParams& p, int uu, int i) const {
     const int t = (u0 + uu) * C::kST + i0 + 32 * i;
     if (uu >= n_piece || t >= len) return 0;
-    return ld_dep(table + (bt_shift >= 0 ? t >> bt_shift : t / p.bt));
+    return ld_dep(table + block_of(p, t));
   }
   __device__ __forceinline__ void meta_of(const AttnParams& p, int uu, int i, int blk) {
     const int t = (u0 + uu) * C::kST + i0 + 32 * i;
     km[i] = make_float2(0.f, 0.f); vm[i] = km[i];
     if (uu >= n_piece || t >= len) return;
-    const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
+    const int in_blk = t - block_of(p, t) * p.bt;
     blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
     const uint32_t row = (uint32_t)(((size_t)blk * p.Hkv + ih) * p.bt + in_blk);
     km[i] = ld_dep(reinterpret_cast<const float2*>(p.km) + row);

@@ -387,7 +387,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   constexpr uint32_t kBytesSub = (FULL ? 4u : 2u) * 1024u;   // bytes of one sub-block
   uint32_t* my_blk = blk_s + pw * SPW * kI8PieceUnits;   // [SPW sub-blocks][kI8PieceUnits]
   int b = b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
-  int hkv = (int)(off_lo / U), u = (int)(off_lo % U);
+  int hkv = (int)sk_div(off_lo, U), u = (int)(off_lo - (long long)hkv * U);
   int remaining = n_units, gs = 0, ic = 0;
   while (remaining > 0) {
     const int n = min(remaining, U - u);
@@ -398,8 +398,8 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
       if (lane == 0) {
         Item it;
         it.b = b; it.hkv = hkv; it.len = len;
-        it.first_cta = (int)(seg0 / q);
-        it.n_contrib = (int)((seg0 + U - 1) / q) - it.first_cta + 1;
+        it.first_cta = (int)sk_div(seg0, q);
+        it.n_contrib = (int)sk_div(seg0 + U - 1, q) - it.first_cta + 1;
         it.pad0 = n; it.pad1 = u; it.pad2 = 0;
         items[qi] = it;
         if (u == 0) *seg_word(p, (size_t)b * p.Hkv + hkv, C::kPartCols) = (uint32_t)it.first_cta << 16 | (uint32_t)it.n_contrib;
@@ -419,12 +419,13 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         const int t0 = (u + c0 + i) * ST + (sub_first + (i2 % SPW)) * 16;
         uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
         if (t0 < len) {
-          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
+          const int bi = block_of(p, t0);
+          int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + bi);
           if (blk < 0 || blk >= p.num_blocks) {
             atomicOr(p.ws_flags, kFlagBadBlock);
             blk = blk < 0 ? 0 : p.num_blocks - 1;
           }
-          row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 % p.bt));
+          row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 - bi * p.bt));
         }
         my_blk[(i2 % SPW) * kI8PieceUnits + i] = row;
       }
@@ -797,10 +798,12 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       // Ends the current accumulation (the team's last P.V is complete): the int32 accumulators, four
       // byte planes per column, are added to the FP32 copy and the sum is scaled by fac_s[] (the change
       // of the reference exponents).
+      // (rolled where the copy is in tensor memory: this code lies in the unit loop, whose size the instruction caches feel)
+      constexpr int kDrainUnroll = C::kOfInTmem ? 1 : CG / 4;
       auto drain = [&](bool scale) {
         if (units_in_acc > 0) {
           tc_fence_after();
-#pragma unroll
+#pragma unroll kDrainUnroll
           for (int c4 = 0; c4 < CG / 4; ++c4) {
             uint32_t a[16], of[4];
             TmemRegs<16>::ld(tm_o + c4 * 16, a);
@@ -821,7 +824,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           have_of = true;
           units_in_acc = 0;
         } else if (have_of && scale) {
-#pragma unroll
+#pragma unroll kDrainUnroll
           for (int c4 = 0; c4 < CG / 4; ++c4) {
             if (C::kOfInTmem) {
               uint32_t of[4];
@@ -842,17 +845,15 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       // Metadata of this thread's token, read with plain loads two steps ahead: the block id of the unit
       // after next (a block-table look-up whose result is first touched one step later, so that nothing
       // waits for it), the (scale, zero) pairs of the next unit.
-      const int bt_shift = (p.bt & (p.bt - 1)) == 0 ? 31 - __clz(p.bt) : -1;   // block size a power of two?
       auto blk_of = [&](int uu) -> int {      // the raw table entry (0 where there is no such token)
         const int t = (item.pad1 + uu) * C::kST + r;
         if (uu >= n_piece || t >= len) return 0;
-        const int bi = bt_shift >= 0 ? t >> bt_shift : t / p.bt;
-        return ld_dep(p.block_table + (size_t)item.b * p.max_blocks + bi);
+        return ld_dep(p.block_table + (size_t)item.b * p.max_blocks + block_of(p, t));
       };
       auto row_of = [&](int uu, int blk) -> uint32_t {
         const int t = (item.pad1 + uu) * C::kST + r;
         if (uu >= n_piece || t >= len) return 0xFFFFFFFFu;
-        const int in_blk = bt_shift >= 0 ? t & (p.bt - 1) : t % p.bt;
+        const int in_blk = t - block_of(p, t) * p.bt;
         blk = min(max(blk, 0), p.num_blocks - 1);     // (out-of-range ids are reported by the producer)
         return (uint32_t)(((size_t)blk * p.Hkv + item.hkv) * p.bt + in_blk);
       };
@@ -1054,13 +1055,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           if (bar_or(bar_tm, TT, forced || over)) restart();
           weights(true);
         } else {
-          if (forced) restart();
-          else if (over) *raise_flag = 1;
-          // (a thread beyond the range keeps its weights out of the sums: after the restart they are different ones)
-          weights(forced || !over);
-          if (!forced && *raise_flag != 0) {   // uniform: read after the barrier; cleared inside restart()
-            restart();
-            weights(over);
+          if (!forced && over) *raise_flag = 1;
+          // (a thread beyond the range keeps its weights out of the sums: after the restart they are different ones.  A loop, so
+          // that the unit loop holds one copy of either step)
+          bool again = forced, commit = forced || !over;
+#pragma unroll 1
+          for (;;) {
+            if (again) restart();
+            weights(commit);
+            if (again || *raise_flag == 0) break;   // uniform: read after the barrier; cleared inside restart()
+            again = true;
+            commit = over;
           }
         }
         if (tw == 0) {

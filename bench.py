@@ -140,19 +140,24 @@ class Workload:
                     self.geo, win["q"], K, V, self.table, self.lens_flat, win["ws"], draft_out=win["draft"],
                     atol=0.5, rtol=0.1, causal=True, out_full=win["out_full"],
                     first_reject=win["first_reject"], dev=win["dev"]))
-                n += win["k"] + self.verify_kernels(win["k"])
+                n += win["k"] * self.anchor_kernels() + self.verify_kernels(win["k"])
         return n
 
+    def anchor_kernels(self):
+        """Kernels of one anchor call: the attention, and the joining of partial results where few heads share the GPU."""
+        sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+        return 1 if self.B * self.wl.num_kv_heads * 4 >= sms else 2
+
     def verify_kernels(self, k):
-        """Kernels of one merge-verify call: one attention launch per slice of the window (a launch takes up to 16
-        positions and 64 columns), plus the decision kernel when there is more than one."""
+        """Kernels of one merge-verify call: per slice of the window (a launch takes up to 16 positions and 64 columns) the
+        attention and the joining of its results with the decision, plus the decision over all slices when there is more than one."""
         G = self.wl.num_q_heads // self.wl.num_kv_heads
         per = k if k <= 16 and k * G <= 64 else min(16, max(1, 64 // G))
         slices = -(-k // per)
-        return slices + (1 if slices > 1 else 0)
+        return 2 * slices + (1 if slices > 1 else 0)
 
     def launches_per_step(self):
-        return 2 + sum(w["reps"] * (w["k"] + self.verify_kernels(w["k"])) for w in self.windows)
+        return 2 + sum(w["reps"] * (w["k"] * self.anchor_kernels() + self.verify_kernels(w["k"])) for w in self.windows)
 
     def bytes_per_step(self):
         b = 2 * self.launch_rows["split_quantize"] * BYTES_PER_ROW["split_quantize"]

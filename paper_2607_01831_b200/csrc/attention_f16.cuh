@@ -648,42 +648,42 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         part[(size_t)c * kPartStride + dim_out] = v;
         if (r == 0) *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(m, l);
       };
-      // (rolled loops, four columns of tensor memory at a time: this code runs once per piece, from a cold instruction cache)
+      // (rolled loops, eight columns of tensor memory at a time: this code runs once per piece)
       auto o_cols = [&](int c, float* o) {
-        uint32_t t[4];
-        TmemRegs<4>::ld(tm_of + c, t);
+        uint32_t t[8];
+        TmemRegs<8>::ld(tm_of + c, t);
         tc_wait_ld();
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = have ? __uint_as_float(t[k]) : 0.0f;
+        for (int k = 0; k < 8; ++k) o[k] = have ? __uint_as_float(t[k]) : 0.0f;
       };
       if (SPLIT) {
 #pragma unroll 1
-        for (int c = 0; c < CG; c += 4) {
-          float o[4];
+        for (int c = 0; c < CG; c += 8) {
+          float o[8];
           o_cols(c, o);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) put(col0 + c + k, o[k] + lz_s[32 + c + k], ref_s[c + k], lz_s[c + k]);
+          for (int k = 0; k < 8; ++k) put(col0 + c + k, o[k] + lz_s[32 + c + k], ref_s[c + k], lz_s[c + k]);
         }
       } else {
         // each group hands the other one half of its columns through its idle P tile, and merges and writes the other half
         float* mail = reinterpret_cast<float*>(smem + C::kOffP + g * C::kPTile);
         const int g0 = 16 * g;   // first column of this group's half
 #pragma unroll 1
-        for (int c = 0; c < 16; c += 4) {
-          float o[4];
+        for (int c = 0; c < 16; c += 8) {
+          float o[8];
           o_cols(16 - g0 + c, o);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) mail[(c + k) * 128 + r] = o[k];
+          for (int k = 0; k < 8; ++k) mail[(c + k) * 128 + r] = o[k];
         }
         named_bar(3, 256);
         const float* omail = reinterpret_cast<const float*>(smem + C::kOffP + (g ^ 1) * C::kPTile);
         const float* ogrp = reinterpret_cast<const float*>(smem + C::kOffGrp) + (g ^ 1) * C::kGrpScal;
 #pragma unroll 1
-        for (int c = 0; c < 16; c += 4) {
-          float o[4];
+        for (int c = 0; c < 16; c += 8) {
+          float o[8];
           o_cols(g0 + c, o);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
+          for (int k = 0; k < 8; ++k) {
             const int cc = g0 + c + k;
             const float m1 = ref_s[cc], m2 = ogrp[cc], M = fmaxf(m1, m2);
             const float f1 = ex2_full(m1 - M), f2 = ex2_full(m2 - M);
@@ -727,30 +727,49 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       const int ib = items[qi].b, ih = items[qi].hkv, len = items[qi].len, n_piece = items[qi].pad0;
       // ---- the piece's queries: thread = 16-byte chunk kt & 15 of columns kt >> 4, + 8, ... ---------------------
       {
+        // (read once and kept, maxima on packed pairs, sums by exchanging halves, no division per chunk: with the
+        // results written eight columns at a time, 64 columns of 85 tokens 18.8 -> 15.0 us, 32 columns of 4 x 7056 34.8 -> 32.6 us)
         constexpr int NI = NC / 8;
-        auto chunk_of = [&](int c) {
-          if (c >= p.ncols) return make_uint4(0u, 0u, 0u, 0u);
-          const int j = c / p.G, hh = c % p.G;
-          return ld_dep(reinterpret_cast<const uint4*>(p.q + (((size_t)ib * p.nq_stride + j) * p.Hq + (size_t)ih * p.G + hh) * LYNX_D) + (kt & 15));
-        };
-        float amax = 0.0f;
-#pragma unroll 4
+        const uint32_t g_inv = 65536u / (uint32_t)p.G + 1u;   // c / G = c * g_inv >> 16 for c < 64, G <= 16
+        uint4 qv[NI];
+#pragma unroll
         for (int i = 0; i < NI; ++i) {
-          const uint4 v = chunk_of(i * 8 + (kt >> 4));
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-          float sum = 0.0f;
+          const uint32_t c = (uint32_t)(i * 8 + (kt >> 4)), j = c * g_inv >> 16, hh = c - j * (uint32_t)p.G;
+          qv[i] = make_uint4(0u, 0u, 0u, 0u);
+          if ((int)c < p.ncols)
+            qv[i] = ld_dep(reinterpret_cast<const uint4*>(p.q + (((size_t)ib * p.nq_stride + j) * p.Hq + (size_t)ih * p.G + hh) * LYNX_D) + (kt & 15));
+        }
+        uint32_t amax2 = 0u;
+        float sums[NI];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const uint32_t w[4] = {qv[i].x, qv[i].y, qv[i].z, qv[i].w};
+          uint64_t s2 = 0ull;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xFFFF0000u);
-            amax = fmaxf(amax, fmaxf(fabsf(lo), fabsf(hi)));
-            sum += lo + hi;
+            asm("max.bf16x2 %0, %0, %1;" : "+r"(amax2) : "r"(w[k] & 0x7FFF7FFFu));
+            s2 = f2_add(s2, f2_pack(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xFFFF0000u)));
           }
-#pragma unroll
-          for (int off = 8; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-          if ((kt & 15) == 0) scal[qi * NC + i * 8 + (kt >> 4)] = sum;
+          float lo, hi;
+          f2_unpack(s2, lo, hi);
+          sums[i] = lo + hi;
         }
+        float amax = fmaxf(__uint_as_float(amax2 << 16), __uint_as_float(amax2 & 0xFFFF0000u));
+        {   // the sums of the 16 lanes of a column: lane i of them returns that of chunk i / (16 / NI)
+          int off = 8;
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, off));
+          for (int m = NI / 2; m >= 1; m >>= 1, off >>= 1)
+#pragma unroll
+            for (int i = 0; i < m; ++i) {
+              const bool up = (lane & off) != 0;
+              const float give = up ? sums[i] : sums[i + m], keep = up ? sums[i + m] : sums[i];
+              sums[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, off);
+            }
+#pragma unroll
+          for (; off >= 1; off >>= 1) sums[0] += __shfl_xor_sync(0xFFFFFFFFu, sums[0], off);
+          if ((lane & (16 / NI - 1)) == 0) scal[qi * NC + ((kt & 15) / (16 / NI)) * 8 + (kt >> 4)] = sums[0];
+        }
+        amax = warp_max(amax);
         if (lane == 0) amax_s[w4] = amax;
         named_bar(4, 128);
         amax = fmaxf(fmaxf(amax_s[0], amax_s[1]), fmaxf(amax_s[2], amax_s[3]));
@@ -764,11 +783,10 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         if (kt < NC) reinterpret_cast<int*>(scal)[2 * NC + qi * NC + kt] =
             kt < p.ncols ? (p.causal ? len - p.tail + kt / p.G + 1 : len) : 0;
         if (gs > 0) mbar_wait_in(sfull + ((gs - 1) & 1) * 8, ((gs - 1) >> 1) & 1, abort_word);   // the previous piece's last Q.K^T
-#pragma unroll 4
-        for (int i = 0; i < NI; ++i) {   // (read again, from the cache: 64 columns do not fit the registers)
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
           const int c = i * 8 + (kt >> 4), ch = kt & 15;
-          const uint4 v = chunk_of(c);
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          const uint32_t w[4] = {qv[i].x, qv[i].y, qv[i].z, qv[i].w};
           float f[8];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {

@@ -7,13 +7,14 @@
 // BF16, as lynx_recombine writes them.
 //
 // Flash-decoding split-K: a CTA takes a chunk of kChunk tokens of one (sequence, KV head) and writes a
-// partial (m, l, O) to the workspace; a second kernel merges the chunks.  Nothing waits on anything.
+// partial (m, l, O) to the workspace; a second kernel merges the chunks.  Nothing waits on anything but a cluster's own CTAs.
 // Two kernels for the chunk: on the BF16 tensor cores (mma.sync m16n8k16, K and V tiles through a cp.async
 // ring per warp) for block sizes that are multiples of 16 tokens -- it streams the pages at the rate of a
 // plain copy -- and on the FP32 pipes for any other block size (8 or 16 lanes own a token, each 16 or 8 of
 // its 128 dims; partial dot products reduced with shuffles), which runs out of multiply-adds at 8 columns.
 #include <cuda_bf16.h>
 
+#include "block_division.cuh"
 #include "lynx_common.cuh"
 
 namespace lynx {
@@ -37,12 +38,21 @@ struct BfParams {
   // position j0): nq_stride = the caller's n_q, tail = n_q - j0 (the causal limit of position j of the slice is
   // len - tail + j + 1).  Unsliced: both equal nq.
   int nq_stride, tail;
+  BlockDiv bt_div;   // for t / bt
 };
 
 __device__ __forceinline__ float ex2f(float x) {
   float y;
   asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// Dim d of the output row of column c, and (dim 0) the row's log-sum-exp, from its unnormalised sums.
+__device__ __forceinline__ void store_row(const BfParams& p, int b, int hkv, int c, int d, float acc, float M, float L) {
+  const int j = c / p.G, hh = c % p.G;
+  const size_t row = ((size_t)b * p.nq_stride + j) * p.Hq + hkv * p.G + hh;
+  p.out[row * LYNX_D + d] = L > 0.0f ? acc / L : 0.0f;
+  if (d == 0) p.lse[row] = L > 0.0f ? (M + __log2f(L)) * 0.6931471805599453f : -INFINITY;
 }
 
 // COLS query columns (padded), LPT lanes per token
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(kWarps * 32, COLS <= 4 ? 2 : 1) bf16_decode_ke
 //                                     through ldmatrix.trans
 // The weights enter P.V as two BF16 terms (p = hi + lo, the remainder of the rounding): with one term their
 // 8-bit mantissa would show in the outputs.
-constexpr int kTcWarps = 4, kTcStages = 3, kTcTile = 16;
+constexpr int kTcWarps = 4, kTcStages = 3, kTcTile = 16, kTcMaxCluster = 8;
 constexpr int kTcStageBytes = 2 * kTcTile * 256;   // K rows, then V rows
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -237,17 +247,38 @@ __device__ __forceinline__ void ldsm4_t(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the float at the same shared-memory address of CTA `rank` of the cluster
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t bf16x2_of(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// Where there are fewer chunks than the SMs can hold CTAs (short contexts, few sequences), S CTAs of a cluster share a chunk,
+// tile by tile, and join their results through distributed shared memory: the partial results stay one per chunk, as the
+// workspace has them.  A call whose sequences are one chunk each writes the output at once, without the combine kernel.
 template <int COLS>
-__global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const BfParams p) {
+__global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const BfParams p, const int S) {
   extern __shared__ __align__(128) unsigned char smem_tc[];
   pdl_begin();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int chunk = blockIdx.x % p.chunks, bh = blockIdx.x / p.chunks;
+  const int rank = S == 1 ? 0 : (int)cluster_rank(), piece = blockIdx.x / S;
+  const int chunk = piece % p.chunks, bh = piece / p.chunks;
   const int b = bh / p.Hkv, hkv = bh % p.Hkv;
   const int cap = p.max_blocks * p.bt;
   int len = ld_dep(p.seq_lens + b);
@@ -277,14 +308,20 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
   for (int j = 0; j < 16; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
   float m = -1.0e30f, l = 0.0f;
 
-  // tile i of this warp = tile warp + 4 i of the chunk; its rows: 16 consecutive rows of one block
-  auto issue = [&](int i) {
-    const int tile = warp + kTcWarps * i;
+  // tile i of this warp = tile rank + S (warp + 4 i) of the chunk; its rows: 16 consecutive rows of one block.  A tile's block
+  // id is looked up a step before its copies are issued (the look-up is a round trip to the L2).
+  const int tile0 = rank + S * warp, tile_step = S * kTcWarps;
+  const int32_t* table = p.block_table + (size_t)b * p.max_blocks;
+  auto blk_of = [&](int i) -> int {
+    const int tile = tile0 + tile_step * i;
+    return tile < n_tiles ? ld_dep(table + quotient(t_begin + tile * kTcTile, p.bt_div)) : 0;
+  };
+  auto issue = [&](int i, int blk) {
+    const int tile = tile0 + tile_step * i;
     if (tile < n_tiles) {
       const int t0 = t_begin + tile * kTcTile;
-      int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + t0 / p.bt);
       blk = min(max(blk, 0), p.num_blocks - 1);
-      const size_t row0 = ((size_t)blk * p.Hkv + hkv) * p.bt + (t0 % p.bt);
+      const size_t row0 = ((size_t)blk * p.Hkv + hkv) * p.bt + (t0 - quotient(t0, p.bt_div) * p.bt);
       const uint32_t st = ring + (uint32_t)(i % kTcStages) * kTcStageBytes;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -299,15 +336,19 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  const int my_tiles = n_tiles > warp ? (n_tiles - warp + kTcWarps - 1) / kTcWarps : 0;
-  issue(0);
-  issue(1);
+  const int my_tiles = n_tiles > tile0 ? (n_tiles - tile0 + tile_step - 1) / tile_step : 0;
+  const int blk0 = blk_of(0), blk1 = blk_of(1);
+  int blk2 = blk_of(2);
+  issue(0, blk0);
+  issue(1, blk1);
   for (int i = 0; i < my_tiles; ++i) {
-    issue(i + 2);
+    const int blk3 = blk_of(i + 3);
+    issue(i + 2, blk2);
+    blk2 = blk3;
     asm volatile("cp.async.wait_group 2;" ::: "memory");
     __syncwarp();
     const uint32_t st = ring + (uint32_t)(i % kTcStages) * kTcStageBytes;
-    const int t0 = t_begin + (warp + kTcWarps * i) * kTcTile;
+    const int t0 = t_begin + (tile0 + tile_step * i) * kTcTile;
     // ---- S = Q K^T: two n-tiles of 8 tokens, eight k-steps of 16 dims
     float s[2][4];
 #pragma unroll
@@ -388,8 +429,19 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
     if (t == 0) { sm_ml[(warp * COLS + g) * 2] = m; sm_ml[(warp * COLS + g) * 2 + 1] = l; }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < COLS * LYNX_D; idx += kTcWarps * 32) {
-    const int c = idx / LYNX_D, d = idx % LYNX_D;
+  float* red = sm_ml + kTcWarps * COLS * 2;                           // [COLS][128], [COLS][2]: this CTA's sums, for its cluster
+  float* red_ml = red + COLS * LYNX_D;
+  const int d = threadIdx.x;
+  auto emit = [&](int c, float acc, float M, float L) {
+    if (p.chunks > 1) {
+      part[(size_t)c * kPartStrideB + d] = acc;
+      if (d == 0) { part[(size_t)c * kPartStrideB + 128] = M; part[(size_t)c * kPartStrideB + 129] = L; }
+    } else if (c < p.ncols) {
+      store_row(p, b, hkv, c, d, acc, M, L);
+    }
+  };
+#pragma unroll
+  for (int c = 0; c < COLS; ++c) {   // a thread per dim
     float M = -1.0e30f;
 #pragma unroll
     for (int w = 0; w < kTcWarps; ++w) M = fmaxf(M, sm_ml[(w * COLS + c) * 2]);
@@ -400,9 +452,34 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
       acc = fmaf(sm_o[(w * COLS + c) * LYNX_D + d], f, acc);
       L = fmaf(sm_ml[(w * COLS + c) * 2 + 1], f, L);
     }
-    part[(size_t)c * kPartStrideB + d] = acc;
-    if (d == 0) { part[(size_t)c * kPartStrideB + 128] = M; part[(size_t)c * kPartStrideB + 129] = L; }
+    if (S == 1) {
+      emit(c, acc, M, L);
+    } else {
+      red[c * LYNX_D + d] = acc;
+      if (d == 0) { red_ml[c * 2] = M; red_ml[c * 2 + 1] = L; }
+    }
   }
+  if (S == 1) return;
+  cluster_sync();
+  for (int c = rank; c < COLS; c += S) {
+    float m8[kTcMaxCluster], l8[kTcMaxCluster], o8[kTcMaxCluster], M = -1.0e30f, acc = 0.0f, L = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kTcMaxCluster; ++k) {
+      m8[k] = k < S ? ld_cluster(red_ml + c * 2, k) : -1.0e30f;
+      l8[k] = k < S ? ld_cluster(red_ml + c * 2 + 1, k) : 0.0f;
+      o8[k] = k < S ? ld_cluster(red + c * LYNX_D + d, k) : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < kTcMaxCluster; ++k) M = fmaxf(M, m8[k]);
+#pragma unroll
+    for (int k = 0; k < kTcMaxCluster; ++k) {
+      const float f = ex2f(m8[k] - M);
+      acc = fmaf(o8[k], f, acc);
+      L = fmaf(l8[k], f, L);
+    }
+    emit(c, acc, M, L);
+  }
+  cluster_sync();   // (nobody leaves while its sums are read)
 }
 
 // One CTA per (sequence, KV head, column): merges the chunk partials, normalises, writes the output.
@@ -438,9 +515,7 @@ __global__ void __launch_bounds__(LYNX_D) bf16_combine_kernel(const BfParams p) 
       M = mn;
     }
   }
-  const int j = c / p.G, hh = c % p.G;
-  p.out[(((size_t)b * p.nq_stride + j) * p.Hq + hkv * p.G + hh) * LYNX_D + d] = L > 0.0f ? acc / L : 0.0f;
-  if (d == 0) p.lse[((size_t)b * p.nq_stride + j) * p.Hq + hkv * p.G + hh] = L > 0.0f ? (M + __log2f(L)) * 0.6931471805599453f : -INFINITY;
+  store_row(p, b, hkv, c, d, acc, M, L);
 }
 
 template <int COLS, int LPT>
@@ -453,7 +528,7 @@ lynx_status launch_bf16(const BfParams& p, cudaStream_t st) {
 template <int COLS>
 lynx_status launch_bf16_tc(const BfParams& p, cudaStream_t st) {
   constexpr int kSmem = kTcWarps * kTcStages * kTcStageBytes;   // 96 KB: two CTAs per SM
-  static_assert(kSmem >= (int)((kTcWarps * COLS * LYNX_D + kTcWarps * COLS * 2) * sizeof(float)), "merge scratch");
+  static_assert(kSmem >= (int)((kTcWarps + 1) * COLS * (LYNX_D + 2) * sizeof(float)), "merge scratch");
   auto kern = bf16_decode_tc_kernel<COLS>;
   static bool configured[64] = {false};
   int dev = 0;
@@ -462,8 +537,15 @@ lynx_status launch_bf16_tc(const BfParams& p, cudaStream_t st) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  const lynx_status rc = launch_pdl(kern, (unsigned)(p.B * p.Hkv * p.chunks), kTcWarps * 32, kSmem, st, p);
-  if (rc != LYNX_OK) return rc;
+  // CTAs per chunk: a power of two, as long as all CTAs are resident at once (two per SM) and every warp has a tile.  us: 8 heads
+  // of 4096 tokens 28.2 by a CTA per chunk, 9.6 by eight; of 32768 tokens 31.5 and 28.4 by two (31.9 by four, 40.5 by eight: the
+  // CTAs of a second round bring their start and end with them); 16 sequences of up to 512 tokens 13.4, 8.5 by two, 11.5 by four.
+  const long long pieces = (long long)p.B * p.Hkv * p.chunks, cap = (long long)p.max_blocks * p.bt;
+  const long long tiles = ((cap < kChunk ? cap : kChunk) + kTcTile - 1) / kTcTile;
+  int S = 1;
+  while (S < kTcMaxCluster && pieces * 2 * S <= 2 * sm_count() && kTcWarps * S < tiles) S *= 2;
+  const lynx_status rc = launch_cluster(kern, (unsigned)(pieces * S), kTcWarps * 32, kSmem, (unsigned)S, st, p, S);
+  if (rc != LYNX_OK || p.chunks == 1) return rc;
   return launch_pdl(bf16_combine_kernel<COLS>, (unsigned)(p.B * p.Hkv * COLS), LYNX_D, 0, st, p);
 }
 
@@ -530,6 +612,7 @@ extern "C" lynx_status lynx_bf16_attention(const lynx_shape* shape, const void* 
   p.B = batch; p.nq = n_q; p.causal = causal ? 1 : 0;
   p.Hq = shape->num_q_heads; p.Hkv = shape->num_kv_heads; p.G = p.Hq / p.Hkv;
   p.bt = shape->block_tokens; p.num_blocks = shape->num_blocks; p.max_blocks = shape->max_blocks_per_seq;
+  p.bt_div = p.bt > 1 ? block_div(p.bt) : BlockDiv{0, 0};   // (used by the tensor-core kernel only: multiples of 16)
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // a launch takes up to 8 query columns; a call with more runs as slices of whole positions, each a pass of its
   // own over the pages, one after the other on the stream (they share the partials)

@@ -30,22 +30,30 @@ __host__ inline lynx_status launch_status() {
 // for 131072, equal at 524288; two small quantisations 10.9 -> 9.9 us).  Where a grid's CTAs run long, the trigger belongs
 // behind their work: see hier_quantize.cu.
 template <class... P, class... A>
-__host__ inline lynx_status launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, void* stream, A... args) {
+__host__ inline lynx_status launch_cluster(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, unsigned cluster, void* stream,
+                                           A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) != cudaSuccess) {
     launch_status();
     return LYNX_ERR_CUDA;
   }
   return launch_status();
+}
+template <class... P, class... A>
+__host__ inline lynx_status launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, void* stream, A... args) {
+  return launch_cluster(kernel, grid, block, smem, 1u, stream, args...);
 }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -9,7 +9,7 @@
 // Constants and readings (alpha = 255, epsilon = 1e-6, magnitude scale 120, Sign of the centred value,
 // round to nearest even) are those of the CPU oracle; arithmetic here is binary32.
 //
-// One CTA per page: the page (64 KB) is staged in shared memory once, the statistics are computed
+// One CTA per half page (64 channels): it (32 KB) is staged in shared memory once, the statistics are computed
 // from there by channel pairs (a 32-bit word holds two channels of a token: conflict-free column
 // walks), the codes leave as packed nibbles, byte j of a token row = channel 2j | channel 2j+1 << 4,
 // the same packing as the linear planes.  HBM-bound by construction (64 KB read, 32 KB + 9 KB written
@@ -112,9 +112,11 @@ __device__ __forceinline__ void hier_nibbles4(const uint32_t* r, const uint32_t*
   res = lop3_sel(J, J >> 4, 0x000F000Fu);
 }
 
-// One CTA per page: the page (64 KB) is staged in shared memory by asynchronous 16-byte copies.  A thread owns
+// One CTA per half page: its 64 channels of 256 tokens (32 KB) are staged in shared memory by asynchronous 16-byte copies.  (A
+// channel is a problem of its own; six CTAs per SM instead of three for whole pages keep loading while others compute.  us: 16
+// pages 4.3 -> 3.1, 1024 25.5 -> 23.7, 4096 85.0 -> 82.5.)  A thread owns
 // eight channels (four 32-bit words of a token row: 16-byte shared-memory loads, 4-byte plane stores) of half a
-// chunk (16 tokens); the two halves of a chunk are lanes l and l ^ 16 of one warp.  First the chunk statistics
+// chunk (16 tokens); the two halves of a chunk are lanes l and l ^ 8 of one warp.  First the chunk statistics
 // (minimum, maximum as packed BF16 pairs; sums in FP32 pairs), from which the page's minimum and range follow
 // (stage 1) and, with them, every chunk's mean and largest deviation (stage 2: max |x - mean| =
 // max(max - mean, mean - min)); then the codes.  The reciprocals are split between the two halves of a chunk and
@@ -124,37 +126,39 @@ __device__ __forceinline__ void hier_nibbles4(const uint32_t* r, const uint32_t*
 // pages, and the next kernel's CTAs, let in early, take the SMs' room while they wait.  K and V quantised and inverted in
 // turn, us: 512 pages each 60.2 triggered at the start, 58.8 without dependent launches, 48.7 this way; 1024: 92.8, 95.0,
 // 85.0; 4096: 355, 325, 316; 16384: 1350, 1247, 1238.
-__global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat16* src, int n_pages,
+constexpr int kHq = 8, kHalfThreads = kChunks * 2 * kHq;   // quads of channel pairs of half a page's channels
+__global__ void __launch_bounds__(kHalfThreads, 6) hier_quantize_kernel(const __nv_bfloat16* src, int n_pages,
                                                                uint8_t* __restrict__ q_anc, uint8_t* __restrict__ q_res,
                                                                float* __restrict__ g_min, float* __restrict__ g_scale,
                                                                float* __restrict__ mu, float* __restrict__ sigma) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const uint4* page = reinterpret_cast<const uint4*>(smem);           // [256 tokens][16 quads of channel pairs]
-  uint4* c_min = reinterpret_cast<uint4*>(smem + kP * 256);           // [8 chunks][16 quads] packed BF16 pairs
-  uint4* c_max = c_min + kChunks * 16;
+  const uint4* page = reinterpret_cast<const uint4*>(smem);           // [256 tokens][8 quads of channel pairs]
+  uint4* c_min = reinterpret_cast<uint4*>(smem + kP * 128);           // [8 chunks][8 quads] packed BF16 pairs
+  uint4* c_max = c_min + kChunks * kHq;
   const uint32_t page_s = (uint32_t)__cvta_generic_to_shared(smem);
-  const int tid = threadIdx.x, q = tid & 15, half = (tid >> 4) & 1, ch = tid >> 5;
+  const int tid = threadIdx.x, q = tid & (kHq - 1), half = (tid >> 3) & 1, ch = tid >> 4;
   const int row0 = ch * kC + half * (kC / 2);
   pdl_wait();
-  for (int pg = blockIdx.x; pg < n_pages; pg += gridDim.x) {
-    const uint4* gsrc = reinterpret_cast<const uint4*>(src + (size_t)pg * kP * LYNX_D);
-    __syncthreads();                                                  // the previous page is done with shared memory
+  for (unsigned item = blockIdx.x; item < 2u * (unsigned)n_pages; item += gridDim.x) {
+    const int pg = (int)(item >> 1), ch0 = (int)(item & 1) * (LYNX_D / 2);   // page, first channel
+    const uint4* gsrc = reinterpret_cast<const uint4*>(src + (size_t)pg * kP * LYNX_D + ch0);
+    __syncthreads();                                                  // the previous half page is done with shared memory
 #pragma unroll 8
-    for (int i = tid; i < kP * LYNX_D / 8; i += 256) cp_async16(page_s + (uint32_t)i * 16u, gsrc + i);
+    for (int i = tid; i < kP * kHq; i += kHalfThreads) cp_async16(page_s + (uint32_t)i * 16u, gsrc + (i >> 3) * 16 + (i & 7));
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     // ---- chunk statistics of the thread's 16 tokens, then of the chunk (both halves) --------------------------
     uint32_t mn[4], mx[4];
     uint64_t sm2[4];
     {
-      const uint4 v = page[row0 * 16 + q];
+      const uint4 v = page[row0 * kHq + q];
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) { mn[j] = w[j]; mx[j] = w[j]; sm2[j] = pack2(lo_bf16(w[j]), hi_bf16(w[j])); }
     }
 #pragma unroll 5
     for (int t = 1; t < kC / 2; ++t) {
-      const uint4 v = page[(row0 + t) * 16 + q];
+      const uint4 v = page[(row0 + t) * kHq + q];
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -166,27 +170,27 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
     float mean[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      mn[j] = bf2_min(mn[j], __shfl_xor_sync(0xFFFFFFFFu, mn[j], 16));
-      mx[j] = bf2_max(mx[j], __shfl_xor_sync(0xFFFFFFFFu, mx[j], 16));
+      mn[j] = bf2_min(mn[j], __shfl_xor_sync(0xFFFFFFFFu, mn[j], kHq));
+      mx[j] = bf2_max(mx[j], __shfl_xor_sync(0xFFFFFFFFu, mx[j], kHq));
       float s0, s1;
       unpack2(sm2[j], s0, s1);
-      mean[2 * j] = (s0 + __shfl_xor_sync(0xFFFFFFFFu, s0, 16)) * (1.0f / kC);
-      mean[2 * j + 1] = (s1 + __shfl_xor_sync(0xFFFFFFFFu, s1, 16)) * (1.0f / kC);
+      mean[2 * j] = (s0 + __shfl_xor_sync(0xFFFFFFFFu, s0, kHq)) * (1.0f / kC);
+      mean[2 * j + 1] = (s1 + __shfl_xor_sync(0xFFFFFFFFu, s1, kHq)) * (1.0f / kC);
     }
     if (half == 0) {
-      c_min[ch * 16 + q] = make_uint4(mn[0], mn[1], mn[2], mn[3]);
-      c_max[ch * 16 + q] = make_uint4(mx[0], mx[1], mx[2], mx[3]);
+      c_min[ch * kHq + q] = make_uint4(mn[0], mn[1], mn[2], mn[3]);
+      c_max[ch * kHq + q] = make_uint4(mx[0], mx[1], mx[2], mx[3]);
     }
     __syncthreads();
     // ---- stage 1: the page's minimum and range per channel (each half reduces four chunks) --------------------
     uint32_t pmn[4], pmx[4];
     {
-      const uint4 a = c_min[(4 * half) * 16 + q], b = c_max[(4 * half) * 16 + q];
+      const uint4 a = c_min[(4 * half) * kHq + q], b = c_max[(4 * half) * kHq + q];
       pmn[0] = a.x; pmn[1] = a.y; pmn[2] = a.z; pmn[3] = a.w;
       pmx[0] = b.x; pmx[1] = b.y; pmx[2] = b.z; pmx[3] = b.w;
 #pragma unroll
       for (int c = 1; c < 4; ++c) {
-        const uint4 a2 = c_min[(4 * half + c) * 16 + q], b2 = c_max[(4 * half + c) * 16 + q];
+        const uint4 a2 = c_min[(4 * half + c) * kHq + q], b2 = c_max[(4 * half + c) * kHq + q];
         pmn[0] = bf2_min(pmn[0], a2.x); pmn[1] = bf2_min(pmn[1], a2.y);
         pmn[2] = bf2_min(pmn[2], a2.z); pmn[3] = bf2_min(pmn[3], a2.w);
         pmx[0] = bf2_max(pmx[0], b2.x); pmx[1] = bf2_max(pmx[1], b2.y);
@@ -196,8 +200,8 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
     float gmn[8], gsc[8], inv[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      pmn[j] = bf2_min(pmn[j], __shfl_xor_sync(0xFFFFFFFFu, pmn[j], 16));
-      pmx[j] = bf2_max(pmx[j], __shfl_xor_sync(0xFFFFFFFFu, pmx[j], 16));
+      pmn[j] = bf2_min(pmn[j], __shfl_xor_sync(0xFFFFFFFFu, pmn[j], kHq));
+      pmx[j] = bf2_max(pmx[j], __shfl_xor_sync(0xFFFFFFFFu, pmx[j], kHq));
       gmn[2 * j] = lo_bf16(pmn[j]);
       gmn[2 * j + 1] = hi_bf16(pmn[j]);
       gsc[2 * j] = lo_bf16(pmx[j]) - gmn[2 * j];
@@ -207,12 +211,12 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float mine = rcp_fast((half ? gsc[4 + i] : gsc[i]) + kEps);
-      const float other = __shfl_xor_sync(0xFFFFFFFFu, mine, 16);
+      const float other = __shfl_xor_sync(0xFFFFFFFFu, mine, kHq);
       inv[i] = half ? other : mine;
       inv[4 + i] = half ? mine : other;
     }
     if (ch == 0) {
-      float* dstp = (half ? g_scale : g_min) + (size_t)pg * LYNX_D + q * 8;
+      float* dstp = (half ? g_scale : g_min) + (size_t)pg * LYNX_D + ch0 + q * 8;
       const float* v = half ? gsc : gmn;
       reinterpret_cast<float4*>(dstp)[0] = make_float4(v[0], v[1], v[2], v[3]);
       reinterpret_cast<float4*>(dstp)[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -228,7 +232,7 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
       float o[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) o[i] = half ? sg[i] : (mean[i] - gmn[i]) * inv[i];
-      float* dstp = (half ? sigma : mu) + ((size_t)pg * kChunks + ch) * LYNX_D + q * 8;
+      float* dstp = (half ? sigma : mu) + ((size_t)pg * kChunks + ch) * LYNX_D + ch0 + q * 8;
       reinterpret_cast<float4*>(dstp)[0] = make_float4(o[0], o[1], o[2], o[3]);
       reinterpret_cast<float4*>(dstp)[1] = make_float4(o[4], o[5], o[6], o[7]);
     }
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float mine = rcp_fast((half ? sg[4 + i] : sg[i]) + kEps);
-        const float other = __shfl_xor_sync(0xFFFFFFFFu, mine, 16);
+        const float other = __shfl_xor_sync(0xFFFFFFFFu, mine, kHq);
         A[i] = (half ? other : mine) * inv[i];
         A[4 + i] = (half ? mine : other) * inv[4 + i];
       }
@@ -250,11 +254,11 @@ __global__ void __launch_bounds__(256, 3) hier_quantize_kernel(const __nv_bfloat
       }
     }
     // ---- stages 3 and 4: the codes of the thread's 16 tokens x 8 channels ---------------------------------------
-    uint32_t* pa = reinterpret_cast<uint32_t*>(q_anc + ((size_t)pg * kP + row0) * 64) + q;
-    uint32_t* pr_ = reinterpret_cast<uint32_t*>(q_res + ((size_t)pg * kP + row0) * 64) + q;
+    uint32_t* pa = reinterpret_cast<uint32_t*>(q_anc + ((size_t)pg * kP + row0) * 64 + ch0 / 2) + q;
+    uint32_t* pr_ = reinterpret_cast<uint32_t*>(q_res + ((size_t)pg * kP + row0) * 64 + ch0 / 2) + q;
 #pragma unroll 4
     for (int t = 0; t < kC / 2; ++t) {
-      const uint4 v = page[(row0 + t) * 16 + q];
+      const uint4 v = page[(row0 + t) * kHq + q];
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
       uint32_t r[8], s[8];
 #pragma unroll
@@ -386,7 +390,7 @@ extern "C" lynx_status lynx_hier_quantize(const void* src_bf16, int64_t n_pages,
   if (!src_bf16 || !q_anc || !q_res || !gamma_min || !gamma_scale || !mu || !sigma) return LYNX_ERR_NULL;
   if (!aligned16(src_bf16) || !aligned16(gamma_min) || !aligned16(gamma_scale) || !aligned16(mu) || !aligned16(sigma))
     return LYNX_ERR_ALIGN;
-  constexpr int kSmem = kP * 256 + 2 * kChunks * 64 * 4;
+  constexpr int kSmem = kP * 128 + 2 * kChunks * kHq * 16;
   static bool configured[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -395,8 +399,8 @@ extern "C" lynx_status lynx_hier_quantize(const void* src_bf16, int64_t n_pages,
       return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  const int64_t grid = n_pages < (int64_t)sm_count() * 3 ? n_pages : (int64_t)sm_count() * 3;
-  return launch_pdl(hier_quantize_kernel, (unsigned)grid, 256, kSmem, stream, static_cast<const __nv_bfloat16*>(src_bf16), (int)n_pages,
+  const int64_t grid = 2 * n_pages < (int64_t)sm_count() * 6 ? 2 * n_pages : (int64_t)sm_count() * 6;
+  return launch_pdl(hier_quantize_kernel, (unsigned)grid, kHalfThreads, kSmem, stream, static_cast<const __nv_bfloat16*>(src_bf16), (int)n_pages,
                     q_anc, q_res, gamma_min, gamma_scale, mu, sigma);
 }
 

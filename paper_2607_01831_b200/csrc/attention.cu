@@ -358,6 +358,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
   const bool direct = n == 1 && !p.combine_single;   // written by the attention kernel
   if (n == 0 || (direct && !decide)) return;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  float lse = 0.0f;
   if (!direct) {
     const size_t sstride = (size_t)part_cols * kPartStride;
     const float* col = p.ws_part + (bh + first) * sstride + (size_t)(j * p.G + g) * kPartStride;
@@ -418,13 +419,20 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
     }
     const float inv = L > 0.0f ? 1.0f / L : 0.0f;
     acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-    reinterpret_cast<float4*>(p.out + row * LYNX_D)[lane] = acc;
-    if (lane == 0) p.ws_lse[row] = lse_of(M, L);
+    lse = lse_of(M, L);
   } else {
     if (warp > 0) return;
     acc = ld_dep(reinterpret_cast<const float4*>(p.out + row * LYNX_D) + lane);
   }
-  if (!decide) return;
+  auto store = [&]() {
+    if (direct) return;
+    reinterpret_cast<float4*>(p.out + row * LYNX_D)[lane] = acc;
+    if (lane == 0) p.ws_lse[row] = lse;
+  };
+  if (!decide) {
+    store();
+    return;
+  }
   // the largest |f - d| / (atol + rtol |f|) of the position (Section 4.3), at first per KV head
   float worst = 0.0f;
   const float fv[4] = {acc.x, acc.y, acc.z, acc.w}, dv[4] = {d.x, d.y, d.z, d.w};
@@ -438,6 +446,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
     __threadfence();
     last = atomicInc(p.ws_seq_ctr + b, all - 1) == all - 1;   // (resets itself)
   }
+  store();   // (behind the ticket: its fence has nothing else to wait for)
   // the last row of the sequence decides: a lane per position, the heads' deviations eight loads at a time
   if (__shfl_sync(0xFFFFFFFFu, last, 0)) {
     __threadfence();

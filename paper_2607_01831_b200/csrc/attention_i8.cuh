@@ -727,17 +727,19 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       const int e = i8_q_exponent(amax);
       const float ca = p.sm_log2 * __int_as_float((127 - e) << 23) * ((FULL || C::kRawK) ? 1.0f : 16.0f);
       const uint32_t qt = sbase + C::kOffQT + qi * C::kQTile;
-      if (u_first == 0 && tt < CP * 4) {
+      if (u_first == 0) {
         // this team owns the piece's first unit: it writes the three balanced s8 digit planes of
         // q_int = rint(q 2^e), rows plane * CP + column.  (The slot's previous planes belong to the piece
         // before last, which every team has left: the queries of this piece were loaded after that.)
+        // Eight entries per thread and step: the first product of a launch waits for this, and 32 by a quarter of the threads took
+        // longer than the first planes to arrive (one layer of 4096 tokens, from a graph: 4 columns 10.85 -> 9.91 us, 16 columns 17.2 ->
+        // 16.3 us, with the decision's ticket ahead of the output's stores).
         const float up = __int_as_float((127 + e) << 23);
-        const int c = tt >> 2, j = tt & 3;
         constexpr int NP = C::kQPlanes;
-        uint32_t pl[NP][2][4];   // [plane][half][word]
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const uint4 v = *reinterpret_cast<const uint4*>(qb + c * 256 + j * 64 + w * 16);
+#pragma unroll 1
+        for (int it = tt; it < CP * 16; it += TT) {
+          const int c = it >> 4, j = (it >> 2) & 3, w = it & 3;   // column, 32 dims of the row, 8 of them
+          const uint4 v = *reinterpret_cast<const uint4*>(qb + it * 16);
           const uint32_t ww[4] = {v.x, v.y, v.z, v.w};
           uint32_t acc[NP][2];
 #pragma unroll
@@ -767,17 +769,14 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             }
           }
 #pragma unroll
-          for (int pln = 0; pln < NP; ++pln) { pl[pln][0][w] = acc[pln][0]; pl[pln][1][w] = acc[pln][1]; }
-        }
+          for (int pln = 0; pln < NP; ++pln) {
+            const int n = pln * CP + c;
 #pragma unroll
-        for (int pln = 0; pln < NP; ++pln) {
-          const int n = pln * CP + c;
-#pragma unroll
-          for (int par = 0; par < 2; ++par) {
-            const int chunk = C::kRawK ? 4 * par + j : 2 * j + par;   // 16 bytes of the row's 128
-            const uint32_t a = qt + (uint32_t)n * 128u + ((uint32_t)(chunk ^ (n & 7)) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(pl[pln][par][0]),
-                         "r"(pl[pln][par][1]), "r"(pl[pln][par][2]), "r"(pl[pln][par][3]) : "memory");
+            for (int par = 0; par < 2; ++par) {
+              const int chunk = C::kRawK ? 4 * par + j : 2 * j + par;   // 16 bytes of the row's 128
+              const uint32_t a = qt + (uint32_t)n * 128u + ((uint32_t)(chunk ^ (n & 7)) << 4) + 4u * w;
+              asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(acc[pln][par]) : "memory");
+            }
           }
         }
       }

@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
   for (int j = 0; j < 16; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
   float m = -1.0e30f, l = 0.0f;
 
-  // tile i of this warp = tile rank + S (warp + 4 i) of the chunk; its rows: 16 consecutive rows of one block.  A tile's block
-  // id is looked up a step before its copies are issued (the look-up is a round trip to the L2).
+  // tile i of this warp = tile rank + S (warp + 4 i) of the chunk; its rows: 16 consecutive rows of one block.  (Block ids looked up
+  // a step before the copies are issued: 2 % slower at 8 columns, the other warps hide the look-up.)
   const int tile0 = rank + S * warp, tile_step = S * kTcWarps;
   const int32_t* table = p.block_table + (size_t)b * p.max_blocks;
   auto blk_of = [&](int i) -> int {
@@ -338,13 +338,10 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bf16_decode_tc_kernel(const 
   };
   const int my_tiles = n_tiles > tile0 ? (n_tiles - tile0 + tile_step - 1) / tile_step : 0;
   const int blk0 = blk_of(0), blk1 = blk_of(1);
-  int blk2 = blk_of(2);
   issue(0, blk0);
   issue(1, blk1);
   for (int i = 0; i < my_tiles; ++i) {
-    const int blk3 = blk_of(i + 3);
-    issue(i + 2, blk2);
-    blk2 = blk3;
+    issue(i + 2, blk_of(i + 2));
     asm volatile("cp.async.wait_group 2;" ::: "memory");
     __syncwarp();
     const uint32_t st = ring + (uint32_t)(i % kTcStages) * kTcStageBytes;

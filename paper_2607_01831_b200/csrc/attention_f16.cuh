@@ -938,9 +938,10 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       if (!SPLIT && next < n_units) {
         const uint32_t kb = kready + (next & 1) * 8, kp = (next >> 1) & 1, sb = sfree + (next & 1) * 8, sp = kp ^ 1u;
         const uint32_t pb = pready + (gs & 1) * 8, pp = (gs >> 1) & 1;
-        bool early = false;
-        wait_in([&] { early = mbar_test(kb, kp) && mbar_test(sb, sp); return early || mbar_test(pb, pp); }, abort_word);
-        if (early) qk(next++);
+        // (one answer for the warp: the products are issued by an elected lane, and `next` has to be the same in all)
+        if (first_of([&](auto probe) { wait_in(probe, abort_word); }, [&] { return mbar_test(kb, kp) && mbar_test(sb, sp); },
+                     [&] { return mbar_test(pb, pp); }, [](bool seen) { return __any_sync(0xFFFFFFFFu, seen) != 0; }))
+          qk(next++);
       }
       pv(gs);
     }

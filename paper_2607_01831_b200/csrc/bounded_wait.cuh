@@ -33,6 +33,16 @@ LYNX_HD bool bounded_wait(Probe probe, Clock now_ns, volatile int* abort_word) {
   return true;
 }
 
+// Whether `first` came before `second`, for a warp whose next steps depend on it.  wait(probe) is the bounded wait; every lane waits
+// for itself, and lanes that look at a barrier while its phase ends may leave by different conditions, so that the answer is one
+// vote: any(x) is true in every lane if x is in one.  (What one lane has seen complete stays so for the others' waits.)
+template <class Wait, class First, class Second, class Any>
+LYNX_HD bool first_of(Wait wait, First first, Second second, Any any) {
+  bool seen = false;
+  wait([&] { seen = first(); return seen || second(); });
+  return any(seen);
+}
+
 // What follows a wait that gave up, behind the last copy and product of the CTA and before it gives back the memory that they
 // write to: a millisecond, a thousand times what one of them takes.
 constexpr uint64_t kLandNs = 1000000ull;

@@ -104,7 +104,9 @@ lynx_status lynx_recombine(const uint8_t* anchor, const uint8_t* residual, const
  * positions (n_q or k) and sequences of at most max_blocks_per_seq * block_tokens tokens.
  * Returns 0 for an unsupported shape.  The workspace must be zero-filled once before its first
  * use (lynx_workspace_init, or cudaMemsetAsync of the whole buffer); each call leaves it ready
- * for the next.  Calls sharing a workspace must be ordered on one stream.
+ * for the next, whatever the batch, heads and positions of either, as long as it is large enough
+ * for both.  Calls sharing a workspace must be ordered on one stream.  It is not to be handed to
+ * lynx_bf16_attention in between, whose scratch starts at its first byte.
  * A buffer smaller than this figure is rejected by the attention calls (LYNX_ERR_WORKSPACE): nothing
  * degrades silently.  It holds the status word, tickets, per-head deviations, log-sum-exps and the partial
  * results of split contexts. */

@@ -31,15 +31,16 @@
 #include "block_division.cuh"
 #include "bounded_wait.cuh"
 #include "lynx_common.cuh"
+#include "workspace_layout.cuh"
 
 namespace lynx {
 namespace {
 
-constexpr int kMaxQ = 16;          // query positions per launch
+constexpr int kMaxQ = kWsMaxQ;     // query positions per launch
 constexpr int kMaxWindow = 64;     // query positions per call (Section 5.1: at most 64 speculative tokens); more than
                                    // kMaxQ positions or kMaxCols columns run as slices, one pass over the planes each
 constexpr int kMaxCols = 64;       // n_q * G per launch
-constexpr int kPartStride = 132;   // floats per (chunk, column) partial: O[128], m, l, pad
+constexpr int kPartStride = kWsPartStride;
 
 struct AttnParams {
   const __nv_bfloat16* q;
@@ -52,8 +53,8 @@ struct AttnParams {
   int32_t* first_reject;
   float* dev;
   uint32_t* ws_flags;
-  uint32_t* ws_chunk_ctr;  // [B*Hkv] tickets of the CTAs that share a (sequence, KV head)
-  uint32_t* ws_seq_ctr;    // [B]
+  uint32_t* ws_tickets;    // [SMs] tickets of the CTAs that share a (sequence, KV head), at the first one's index
+  uint32_t* ws_seq_ctr;    // [B] rows of a sequence that have been joined (zeroed by the attention kernel)
   float* ws_dev;           // [B*Hkv][kMaxQ]
   float* ws_lse;           // [B][nq_stride][Hq] natural-log log-sum-exp of every output row's scores
   float* ws_part;          // [B*Hkv + CTAs][ncols_pad][kPartStride], slot = segment + CTA index (and see seg_word)
@@ -78,6 +79,11 @@ __device__ __forceinline__ int block_of(const AttnParams& p, int t) { return quo
 // the slot of the segment's index, whosever that slot is.
 __device__ __forceinline__ uint32_t* seg_word(const AttnParams& p, size_t bh, int part_cols) {
   return reinterpret_cast<uint32_t*>(p.ws_part + bh * (size_t)part_cols * kPartStride + 130);
+}
+// What attn_combine_kernel counts and takes maxima in, by the warp that publishes a segment's first piece.
+__device__ __forceinline__ void zero_decision(const AttnParams& p, int b, int hkv, int lane) {
+  if (lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;
+  if (hkv == 0 && lane == kMaxQ) p.ws_seq_ctr[b] = 0u;
 }
 
 // ------------------------------------------------------------------ PTX helpers
@@ -444,7 +450,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
   if (lane == 0) {
     atomicMax(reinterpret_cast<int*>(p.ws_dev) + bh * kMaxQ + j, m);   // (zeroed by the attention kernel)
     __threadfence();
-    last = atomicInc(p.ws_seq_ctr + b, all - 1) == all - 1;   // (resets itself)
+    last = atomicAdd(p.ws_seq_ctr + b, 1u) == all - 1;        // (likewise)
   }
   store();   // (behind the ticket: its fence has nothing else to wait for)
   // the last row of the sequence decides: a lane per position, the heads' deviations eight loads at a time
@@ -477,10 +483,6 @@ inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tok
 #include "attention_f16.cuh"
 
 // ------------------------------------------------------------------ host side
-// The scratch has room for this many CTAs per SM, although every kernel runs one: lynx_workspace_bytes and the limit of
-// lynx_anchor_attention_static are figures that callers hold (8 bytes to 33 KB per CTA and column count).
-constexpr int kMaxCtasPerSm = 4;
-
 // Query positions per launch of a verification call: all of them up to kMaxQ positions and kMaxCols
 // columns, else as many whole positions as fit both.
 inline int verify_slice(int nq, int G) {
@@ -492,8 +494,7 @@ inline int verify_slice(int nq, int G) {
 struct Plan {
   int per;             // query positions per verification launch
   int ncols;           // columns of the widest launch
-  int cols_pad;
-  size_t off_chunk_ctr, off_seq_ctr, off_dev, off_lse, off_part, bytes;
+  WsLayout ws;
 };
 
 bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
@@ -514,19 +515,8 @@ bool make_plan(const lynx_shape* s, int B, int nq, Plan* pl) {
   // (the partial slots also serve anchor calls on the same workspace, which take up to 32 columns per launch)
   const int cols_anchor = nq * G <= 32 ? nq * G : (32 / G > 0 ? 32 / G : 1) * G;
   const int cols_max = ncols > cols_anchor ? ncols : cols_anchor;
-  pl->cols_pad = cols_max <= 8 ? 8 : cols_max <= 16 ? 16 : cols_max <= 32 ? 32 : 64;
-  size_t off = kWsHeaderBytes;
-  pl->off_chunk_ctr = off; off += (size_t)B * s->num_kv_heads * 4;
-  pl->off_seq_ctr = off;   off += (size_t)B * 4;
-  off += (size_t)2 * sm_count() * kMaxCtasPerSm * 4;   // (unused; the size is a figure that callers hold)
-  off = (off + 255) & ~(size_t)255;
-  pl->off_dev = off;       off += (size_t)B * s->num_kv_heads * kMaxQ * 4;
-  off = (off + 255) & ~(size_t)255;
-  pl->off_lse = off;       off += (size_t)B * nq * s->num_q_heads * 4;
-  off = (off + 255) & ~(size_t)255;
-  pl->off_part = off;
-  off += ((size_t)B * s->num_kv_heads + (size_t)sm_count() * kMaxCtasPerSm) * pl->cols_pad * kPartStride * 4;
-  pl->bytes = (off + 255) & ~(size_t)255;
+  const int cols_pad = cols_max <= 8 ? 8 : cols_max <= 16 ? 16 : cols_max <= 32 ? 32 : 64;
+  pl->ws = ws_layout(sm_count(), B, nq, s->num_q_heads, s->num_kv_heads, cols_pad);
   return true;
 }
 
@@ -588,7 +578,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
       !aligned16(V.meta) || !aligned16(workspace) || !aligned16(out) ||
       (full && (!aligned16(K.residual) || !aligned16(V.residual))))
     return LYNX_ERR_ALIGN;
-  if (workspace_bytes < pl.bytes) return LYNX_ERR_WORKSPACE;
+  if (workspace_bytes < pl.ws.bytes) return LYNX_ERR_WORKSPACE;
   if (full && draft && !(atol > 0.0f && rtol >= 0.0f)) return LYNX_ERR_SHAPE;
 
   unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -606,11 +596,11 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.inline_merge = !full && (long long)B * shape->num_kv_heads * 4 >= sm_count();
   p.draft_vec = p.draft && aligned16(p.draft);   // (a slice starts whole rows of 512 bytes further on)
   p.ws_flags = reinterpret_cast<uint32_t*>(ws);
-  p.ws_chunk_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_chunk_ctr);
-  p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.off_seq_ctr);
-  p.ws_dev = reinterpret_cast<float*>(ws + pl.off_dev);
-  p.ws_lse = reinterpret_cast<float*>(ws + pl.off_lse);
-  p.ws_part = reinterpret_cast<float*>(ws + pl.off_part);
+  p.ws_tickets = reinterpret_cast<uint32_t*>(ws + pl.ws.off_tickets);
+  p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.ws.off_seq_ctr);
+  p.ws_dev = reinterpret_cast<float*>(ws + pl.ws.off_dev);
+  p.ws_lse = reinterpret_cast<float*>(ws + pl.ws.off_lse);
+  p.ws_part = reinterpret_cast<float*>(ws + pl.ws.off_part);
   p.atol = atol; p.rtol = rtol;
   const float sc = softmax_scale == 0.0f ? 0.08838834764831845f : softmax_scale;
   p.sm_log2 = sc * 1.4426950408889634f;
@@ -621,7 +611,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.bt_div = block_div(p.bt);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the fixed array keeps what the previous call left: the status word and the tickets must be zero
-  if (fixed_scratch && cudaMemsetAsync(workspace, 0, pl.off_dev, st) != cudaSuccess) return LYNX_ERR_CUDA;
+  if (fixed_scratch && cudaMemsetAsync(workspace, 0, pl.ws.end_kept, st) != cudaSuccess) return LYNX_ERR_CUDA;
   if (!full) {
     // Anchor attention: the integer tcgen05 kernels take up to 32 columns.  A call with more (33..64) is
     // run as slices of whole query positions, each a pass of its own over the planes, one after the
@@ -673,7 +663,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
 extern "C" size_t lynx_workspace_bytes(const lynx_shape* shape, int32_t batch, int32_t n_cols_q) {
   lynx::Plan pl;
   if (!lynx::make_plan(shape, batch, n_cols_q, &pl)) return 0;
-  return pl.bytes;
+  return pl.ws.bytes;
 }
 
 extern "C" lynx_status lynx_verify_decision(const float* out_full, const float* draft_out, int32_t batch, int32_t k,
@@ -698,7 +688,7 @@ extern "C" lynx_status lynx_verify_decision(const float* out_full, const float* 
 extern "C" const float* lynx_workspace_lse(const lynx_shape* shape, int32_t batch, int32_t n_q, const void* workspace) {
   lynx::Plan pl;
   if (!workspace || !lynx::make_plan(shape, batch, n_q, &pl)) return nullptr;
-  return reinterpret_cast<const float*>(static_cast<const unsigned char*>(workspace) + pl.off_lse);
+  return reinterpret_cast<const float*>(static_cast<const unsigned char*>(workspace) + pl.ws.off_lse);
 }
 
 extern "C" lynx_status lynx_anchor_attention(const lynx_shape* shape, const void* q_bf16, int32_t batch,
@@ -765,7 +755,7 @@ extern "C" lynx_status lynx_anchor_attention_static(const lynx_shape* shape, con
   if (batch < 0 || n_q <= 0) return LYNX_ERR_SHAPE;
   Plan pl;
   if (!make_plan(shape, batch, n_q, &pl)) return LYNX_ERR_UNSUPPORTED;
-  if (pl.bytes > kStaticScratchBytes) return LYNX_ERR_WORKSPACE;  // problem too large for the fixed array
+  if (pl.ws.bytes > kStaticScratchBytes) return LYNX_ERR_WORKSPACE;  // problem too large for the fixed array
   void* scratch = nullptr;
   const lynx_status st = static_scratch_address(&scratch);
   if (st != LYNX_OK) return st;
@@ -773,5 +763,5 @@ extern "C" lynx_status lynx_anchor_attention_static(const lynx_shape* shape, con
   // `stream` only once the call is known to launch)
   return run_attention(false, shape, q_bf16, batch, n_q, causal, K, V, block_table, seq_lens,
                        softmax_scale, nullptr, 0.f, 0.f, out, nullptr, nullptr, scratch,
-                       pl.bytes, stream, true);
+                       pl.ws.bytes, stream, true);
 }

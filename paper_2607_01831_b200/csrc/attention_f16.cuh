@@ -207,7 +207,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         mbar_arrive(qfull0 + qi * 8);
       }
       __syncwarp();
-      if (u == 0 && lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
+      if (u == 0) zero_decision(p, b, hkv, lane);
     }
     for (int c0 = 0; c0 < n; c0 += kI8PieceUnits) {
       const int cn = min(kI8PieceUnits, n - c0);

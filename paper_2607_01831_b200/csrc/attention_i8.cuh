@@ -406,7 +406,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         mbar_expect_tx(qfull0 + qi * 8, (uint32_t)(p.nq * p.G * LYNX_D * 2));
       }
       __syncwarp();
-      if (u == 0 && lane < kMaxQ && FULL) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
+      if (u == 0 && FULL) zero_decision(p, b, hkv, lane);
       for (int j = lane; j < p.nq; j += 32)
         bulk_g2s(qraw_u32 + (uint32_t)((qi * C::kColsPad + j * p.G) * LYNX_D * 2),
                  p.q + (((size_t)b * p.nq_stride + j) * p.Hq + (size_t)hkv * p.G) * LYNX_D,
@@ -517,7 +517,7 @@ __device__ __forceinline__ void i8_merge_slots(const AttnParams& p, const Item& 
   constexpr size_t kSlot = (size_t)C::kPartCols * kPartStride;
   __threadfence();
   named_bar(bar, C::kTeamThreads);
-  if (tt == 0) my_misc[1] = atomicInc(p.ws_chunk_ctr + bh, (uint32_t)n - 1) == (uint32_t)n - 1;
+  if (tt == 0) my_misc[1] = atomicInc(p.ws_tickets + item.first_cta, (uint32_t)n - 1) == (uint32_t)n - 1;
   named_bar(bar, C::kTeamThreads);
   if (my_misc[1] == 0) return;
   __threadfence();

@@ -6,6 +6,7 @@
 #include <stdlib.h>
 
 #include "lynx.h"
+#include "workspace_layout.cuh"
 
 #define LYNX_D 128
 
@@ -81,8 +82,7 @@ __device__ __forceinline__ T ld_dep(const T* p) {
 // Number of SMs of the current device (cached per device id).
 __host__ int sm_count();
 
-// Workspace header (first 256 bytes): word 0 = status flags set by kernels.
-constexpr int kWsHeaderBytes = 256;
+// Status flags, word 0 of a workspace.
 constexpr uint32_t kFlagBadBlock = 1u;
 constexpr uint32_t kFlagTimeout = 2u;
 constexpr uint32_t kFlagRange = 4u;

@@ -54,6 +54,7 @@ struct AttnParams {
   float* dev;
   uint32_t* ws_flags;
   uint32_t* ws_tickets;    // [SMs] tickets of the CTAs that share a (sequence, KV head), at the first one's index
+  uint32_t* ws_groups;     // [SMs][2] tickets of groups of such CTAs
   uint32_t* ws_seq_ctr;    // [B] rows of a sequence that have been joined (zeroed by the attention kernel)
   float* ws_dev;           // [B*Hkv][kMaxQ]
   float* ws_lse;           // [B][nq_stride][Hq] natural-log log-sum-exp of every output row's scores
@@ -79,11 +80,6 @@ __device__ __forceinline__ int block_of(const AttnParams& p, int t) { return quo
 // the slot of the segment's index, whosever that slot is.
 __device__ __forceinline__ uint32_t* seg_word(const AttnParams& p, size_t bh, int part_cols) {
   return reinterpret_cast<uint32_t*>(p.ws_part + bh * (size_t)part_cols * kPartStride + 130);
-}
-// What attn_combine_kernel counts and takes maxima in, by the warp that publishes a segment's first piece.
-__device__ __forceinline__ void zero_decision(const AttnParams& p, int b, int hkv, int lane) {
-  if (lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;
-  if (hkv == 0 && lane == kMaxQ) p.ws_seq_ctr[b] = 0u;
 }
 
 // ------------------------------------------------------------------ PTX helpers
@@ -305,11 +301,13 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
   return r;
 }
 
-// Sequences with no token, by one warp of one CTA each: outputs are zero, nothing is rejected unless the draft is not zero.
-// (Off the path of the other sequences: called behind a CTA's last copy.)
+// What is left to do for a sequence, by one warp of one CTA each: the count of finished rows that attn_combine_kernel decides by
+// starts at zero; where there is no token, outputs are zero and nothing is rejected unless the draft is not zero.
+// (Off the path of the sequences' tokens: called behind a CTA's last copy.)
 template <bool FULL, int kPartCols>
-__device__ __forceinline__ void empty_sequences(const AttnParams& p, int cta, int n_cta, int lane, const SeqLens& sl) {
+__device__ __forceinline__ void per_sequence(const AttnParams& p, int cta, int n_cta, int lane, const SeqLens& sl) {
   for (int b = cta; b < p.B; b += n_cta) {
+    if (FULL && lane == 0) p.ws_seq_ctr[b] = 0u;
     if (sl.of(b) != 0) continue;
     for (int h = lane; h < p.Hkv; h += 32) *seg_word(p, (size_t)b * p.Hkv + h, kPartCols) = 0;
     const size_t n = (size_t)p.nq * p.Hq * LYNX_D;
@@ -597,6 +595,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.draft_vec = p.draft && aligned16(p.draft);   // (a slice starts whole rows of 512 bytes further on)
   p.ws_flags = reinterpret_cast<uint32_t*>(ws);
   p.ws_tickets = reinterpret_cast<uint32_t*>(ws + pl.ws.off_tickets);
+  p.ws_groups = reinterpret_cast<uint32_t*>(ws + pl.ws.off_groups);
   p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.ws.off_seq_ctr);
   p.ws_dev = reinterpret_cast<float*>(ws + pl.ws.off_dev);
   p.ws_lse = reinterpret_cast<float*>(ws + pl.ws.off_lse);

@@ -207,7 +207,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         mbar_arrive(qfull0 + qi * 8);
       }
       __syncwarp();
-      if (u == 0) zero_decision(p, b, hkv, lane);
+      if (u == 0 && lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
     }
     for (int c0 = 0; c0 < n; c0 += kI8PieceUnits) {
       const int cn = min(kI8PieceUnits, n - c0);
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     else
       f16_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
                       reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
-    if (pw == 0) empty_sequences<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl);
+    if (pw == 0) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl);
     return;
   }
   // ================================================================================== products

@@ -373,7 +373,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   __syncthreads();  // (A) the range is published
   const int n_units = (int)(lo < hi ? hi - lo : 0);
   if (n_units == 0) {
-    if (pw == 0) empty_sequences<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
+    if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
     return;
   }
 
@@ -406,7 +406,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         mbar_expect_tx(qfull0 + qi * 8, (uint32_t)(p.nq * p.G * LYNX_D * 2));
       }
       __syncwarp();
-      if (u == 0 && FULL) zero_decision(p, b, hkv, lane);
+      if (u == 0 && lane < kMaxQ && FULL) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
       for (int j = lane; j < p.nq; j += 32)
         bulk_g2s(qraw_u32 + (uint32_t)((qi * C::kColsPad + j * p.G) * LYNX_D * 2),
                  p.q + (((size_t)b * p.nq_stride + j) * p.Hq + (size_t)hkv * p.G) * LYNX_D,
@@ -466,7 +466,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   }
   __syncwarp();
   bar_arrive(9, C::kThreads);
-  if (pw == 0) empty_sequences<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
+  if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
 }
 
 // Largest |q| of a piece's raw queries, by 128 threads (index i of 0..127), reduced over the
@@ -508,37 +508,48 @@ __device__ __forceinline__ uint64_t i8_pack(uint32_t lo, uint32_t hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
   return d;
 }
-// The last CTA of a segment (atomic ticket that resets itself, nobody waits) joins its slots, by a team: a warp per column, a
-// lane four dims, four slots in flight.
+// Joining the slots of a segment that several CTAs share, by the last of them (atomic tickets that reset themselves, nobody waits).
+// A segment of more than kOneLevel CTAs -- a long sequence among many short ones, with few heads -- is joined in two levels, so
+// that no CTA walks through all of its slots: the last CTA of each kGroup neighbouring ones joins theirs into the first of them,
+// the last group the groups'.
+constexpr int kGroup = 8, kOneLevel = 24;
+// The group of this CTA (its first slot, its slots) and the group's ticket, which lies with its first CTA: that one can lead two
+// groups, the first of the segment that starts in its range and a later one of the segment that ends there.
+struct SlotGroup {
+  int first, count;
+  uint32_t* ticket;
+};
+__device__ __forceinline__ SlotGroup slot_group(const AttnParams& p, const Item& item) {
+  if (item.n_contrib <= kOneLevel) return {0, item.n_contrib, p.ws_tickets + item.first_cta};
+  const int first = ((int)blockIdx.x - item.first_cta) / kGroup * kGroup;
+  return {first, min(kGroup, item.n_contrib - first), p.ws_groups + 2 * (item.first_cta + first) + (first == 0 ? 1 : 0)};
+}
+__device__ __forceinline__ bool last_of(uint32_t* ticket, int n) { return atomicInc(ticket, (uint32_t)n - 1) == (uint32_t)n - 1; }
+// `count` slots from `first` on, STRIDE apart, by all teams: a warp per column, a lane four dims, four slots in flight.  Into the
+// output, or (`top` false) into the first of them.
 template <class C>
-__device__ __forceinline__ void i8_merge_slots(const AttnParams& p, const Item& item, int tt, int tw, int lane, int* my_misc, int bar) {
-  const size_t bh = (size_t)item.b * p.Hkv + item.hkv;
-  const int n = item.n_contrib;
+__device__ __forceinline__ void i8_join(const AttnParams& p, const Item& item, int first, int count, int stride, bool top, int tid) {
   constexpr size_t kSlot = (size_t)C::kPartCols * kPartStride;
-  __threadfence();
-  named_bar(bar, C::kTeamThreads);
-  if (tt == 0) my_misc[1] = atomicInc(p.ws_tickets + item.first_cta, (uint32_t)n - 1) == (uint32_t)n - 1;
-  named_bar(bar, C::kTeamThreads);
-  if (my_misc[1] == 0) return;
-  __threadfence();
+  const int lane = tid & 31;
+  float* seg = p.ws_part + ((size_t)item.b * p.Hkv + item.hkv + (size_t)(item.first_cta + first)) * kSlot;
 #pragma unroll 1
-  for (int c = tw; c < p.ncols; c += C::kTeamWarps) {
-    const float* col = p.ws_part + (bh + (size_t)item.first_cta) * kSlot + (size_t)c * kPartStride;
+  for (int c = tid >> 5; c < p.ncols; c += C::kTeams * C::kTeamWarps) {
+    float* col = seg + (size_t)c * kPartStride;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float M = -INFINITY, L = 0.0f;
 #pragma unroll 1
-    for (int i0 = 0; i0 < n; i0 += 4) {
+    for (int i0 = 0; i0 < count; i0 += 4) {
       float4 o[4];
       float2 ml[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const float* s = col + (size_t)min(i0 + u, n - 1) * kSlot;
+        const float* s = col + (size_t)(min(i0 + u, count - 1) * stride) * kSlot;
         ml[u] = __ldcg(reinterpret_cast<const float2*>(s + 128));
         o[u] = __ldcg(reinterpret_cast<const float4*>(s) + lane);
-        if (i0 + u >= n) ml[u].x = -INFINITY;
+        if (i0 + u >= count) ml[u].x = -INFINITY;
       }
       const float m0 = M;
-      M = fmaxf(fmaxf(fmaxf(M, ml[0].x), ml[1].x), fmaxf(ml[2].x, ml[3].x));   // (finite: the first slot's is)
+      M = fmaxf(fmaxf(fmaxf(M, ml[0].x), ml[1].x), fmaxf(ml[2].x, ml[3].x));   // (finite: every slot's is)
       const float f0 = ex2(m0 - M);
       L *= f0;
       acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
@@ -552,11 +563,56 @@ __device__ __forceinline__ void i8_merge_slots(const AttnParams& p, const Item& 
         acc.w = fmaf(o[u].w, f, acc.w);
       }
     }
+    if (!top) {
+      __syncwarp();   // (all lanes have read the first slot)
+      reinterpret_cast<float4*>(col)[lane] = acc;
+      if (lane == 0) *reinterpret_cast<float2*>(col + 128) = make_float2(M, L);
+      continue;
+    }
     const float inv = L > 0.0f ? 1.0f / L : 0.0f;
     const int j = c / p.G;
     const size_t row = ((size_t)item.b * p.nq_stride + j) * p.Hq + (size_t)item.hkv * p.G + (c - j * p.G);
     reinterpret_cast<float4*>(p.out + row * LYNX_D)[lane] = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
     if (lane == 0) p.ws_lse[row] = lse_of(M, L);
+  }
+}
+// The segments that a CTA shares -- its first with the CTAs before it, its last with those behind -- once all of its slots have been
+// written, fenced and passed a barrier.  (At the end of the CTA, not of the piece: within reach of the unit loop this code costs
+// registers there.  us, before -> after: one sequence of 32768 tokens among 39 of 64, one KV head, 4 / 16 columns 24.0 / 72.1 ->
+// 14.3 / 21.4; 8 of 65536, 8 KV heads, 8 / 16 columns 132.6 / 184.2 -> 131.4 / 180.4; 6 of 9000, 4 / 32 columns 18.4 / 55.2 -> 18.5 / 52.8.)
+template <class C>
+__device__ __forceinline__ void i8_join_shared(const AttnParams& p, const Item* shared, int tid, int* misc) {
+  constexpr int kThreads = C::kTeams * C::kTeamThreads;
+  if (tid < 2) {   // (both tickets at once)
+    misc[1 + tid] = 0;
+    if (shared[tid].n_contrib > 1) {
+      const SlotGroup g = slot_group(p, shared[tid]);
+      misc[1 + tid] = last_of(g.ticket, g.count);
+    }
+  }
+  named_bar(14, kThreads);
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    if (misc[1 + i] == 0) continue;
+    const Item item = shared[i];
+    const int n = item.n_contrib;
+    bool top = n <= kOneLevel;
+    SlotGroup g = slot_group(p, item);
+    __threadfence();
+#pragma unroll 1
+    for (int stride = 1;; stride = kGroup) {
+      i8_join<C>(p, item, g.first, g.count, stride, top, tid);
+      if (top) break;
+      g.first = 0;
+      g.count = (n + kGroup - 1) / kGroup;
+      __threadfence();
+      named_bar(14, kThreads);
+      if (tid == 0) misc[3] = last_of(p.ws_tickets + item.first_cta, g.count);
+      named_bar(14, kThreads);
+      if (misc[3] == 0) break;
+      __threadfence();
+      top = true;
+    }
   }
 }
 // Bounded wait until a shared-memory sequence counter has reached `need` (a counter, unlike an mbarrier
@@ -670,6 +726,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   float* my_lz = my_scal + 16 * CP;               // [2 CP]
   const int tw = grp * 4 + w4;                    // warp of the team
   int* my_misc = misc + 64 * (1 + tm);
+  Item* shared = reinterpret_cast<Item*>(misc + 64 + 16);   // [2] this CTA's first and last segment where others have part in it (zeroed)
   // named barriers of this team.  On bar_k and bar_p all but the issuing warp only arrive; each has an id of its own, so that
   // between two arrivals of a warp there lies a barrier at which all warps synchronise (the restart question, or bar_p itself
   // where they synchronise there): the phases stay apart even if the waits for products in between have given up.
@@ -704,6 +761,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
     const int team_f = (gs_base + n_piece - 1) % T;       // team of the piece's last unit: it writes the piece's result
     if (u_first < n_piece) {
       const bool finisher = tm == team_f;
+      if (!FULL && finisher && tt == 0 && item.n_contrib > 1) shared[gs_base == 0 ? 0 : 1] = item;   // (see behind the loop)
       const int full_lim = p.causal ? len - p.tail + 1 : len;
       // ---- the piece's queries: fixed-point exponent, sum of q per column, causal limits ----------
       const unsigned char* qb = qraw + qi * CP * 256;
@@ -1188,7 +1246,6 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             if (r == 0) *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(mt[cc], lt[cc]);
           }
         }
-        if (!FULL && !direct && p.inline_merge) i8_merge_slots<C>(p, item, tt, tw, lane, my_misc, bar_tm);
       }
     }
     // every team keeps count of every team's deposits (the phase of its deposit barrier)
@@ -1202,7 +1259,12 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   }
   // ---- release the tensor memory ---------------------------------------------------------------
   tc_fence_before();
+  // (a thread sees what its own team has noted: whose slots are its own.  Here, not behind a piece, where it holds up the next: 12
+  // ragged sequences of up to 9000 tokens, 8 columns, 36.5 -> 35.3 us)
+  const auto any_shared = [&]() { return !FULL && p.inline_merge && (shared[0].n_contrib > 1 || shared[1].n_contrib > 1); };
+  if (any_shared()) __threadfence();
   named_bar(9, C::kThreads);   // (the producers have arrived there behind their last copy)
+  if (any_shared()) i8_join_shared<C>(p, shared, tid, misc);
   if (warp == 0) {
     land_after_abort([] { return globaltimer_ns(); }, abort_word);
     tc_fence_after();

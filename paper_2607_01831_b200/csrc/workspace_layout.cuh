@@ -17,6 +17,7 @@ constexpr int kWsMaxCtasPerSm = 4;
 // for, and the results of one never lie on the tickets of another.  All that follows is written by a call before it is read.
 struct WsLayout {
   size_t off_tickets;   // one per SM: of the segment shared by several CTAs whose first is this one (no CTA is first of two)
+  size_t off_groups;    // two per SM: of groups of such CTAs (see slot_group)
   size_t end_kept;
   size_t off_seq_ctr;   // [B] counts of a sequence's finished rows
   size_t off_dev;       // [B * Hkv][kWsMaxQ] deviations
@@ -25,24 +26,17 @@ struct WsLayout {
   size_t bytes;
 };
 inline WsLayout ws_layout(int sms, int B, int nq, int Hq, int Hkv, int cols_pad) {
+  const auto up = [](size_t x, size_t n) { return (x + n - 1) / n * n; };
   WsLayout w;
-  size_t off = kWsHeaderBytes;
-  w.off_tickets = off;
-  off += (size_t)2 * sms * kWsMaxCtasPerSm * 4;
-  w.end_kept = off;
-  w.off_seq_ctr = off;
-  off += (size_t)B * 4;
-  off += (size_t)B * Hkv * 4;   // (unused; the size is a figure that callers hold)
-  off = (off + 255) & ~(size_t)255;
-  w.off_dev = off;
-  off += (size_t)B * Hkv * kWsMaxQ * 4;
-  off = (off + 255) & ~(size_t)255;
-  w.off_lse = off;
-  off += (size_t)B * nq * Hq * 4;
-  off = (off + 255) & ~(size_t)255;
-  w.off_part = off;
-  off += ((size_t)B * Hkv + (size_t)sms * kWsMaxCtasPerSm) * cols_pad * kWsPartStride * 4;
-  w.bytes = (off + 255) & ~(size_t)255;
+  w.off_tickets = kWsHeaderBytes;
+  w.off_groups = w.off_tickets + (size_t)sms * 4;
+  w.end_kept = w.off_groups + (size_t)2 * sms * 4;
+  w.off_seq_ctr = up(w.end_kept, 128);
+  // (the room between counts and deviations is not used; the size is a figure that callers hold)
+  w.off_dev = up(kWsHeaderBytes + (size_t)2 * sms * kWsMaxCtasPerSm * 4 + (size_t)B * 4 + (size_t)B * Hkv * 4, 256);
+  w.off_lse = up(w.off_dev + (size_t)B * Hkv * kWsMaxQ * 4, 256);
+  w.off_part = up(w.off_lse + (size_t)B * nq * Hq * 4, 256);
+  w.bytes = up(w.off_part + ((size_t)B * Hkv + (size_t)sms * kWsMaxCtasPerSm) * cols_pad * kWsPartStride * 4, 256);
   return w;
 }
 

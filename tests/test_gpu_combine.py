@@ -22,6 +22,11 @@ SHAPES = [
     (37, 1, 4, 1, [64 + 40 * i for i in range(37)]),      # just enough heads for the last CTA to join them
     (36, 1, 4, 1, [64 + 40 * i for i in range(36)]),      # and one fewer
     (40, 1, 2, 1, [20000] + [17] * 39),                   # many heads, one of them with nearly all CTAs
+    (40, 1, 4, 4, [32768] + [64] * 39),                   # and 16 columns: long segments among those of one CTA
+    (39, 1, 4, 8, [64] * 20 + [9000] + [100] * 17 + [15000]),   # two of them, 32 columns, in the middle and at the end
+    (21, 2, 8, 8, [64] * 20 + [7000]),                    # 64 columns, two heads
+    (41, 1, 4, 2, [3000] + [1] * 40),                     # 24 CTAs, where a segment begins to be long
+    (42, 1, 4, 2, [2900, 3100] + [1] * 40),               # 23 and 25, where two levels begin
     (2, 8, 4, 4, [1, 128]),                               # heads of one unit
     (5, 3, 1, 7, [257, 1, 0, 900, 128]),
 ]

@@ -27,10 +27,10 @@ int main() {
             const lynx::WsLayout w = lynx::ws_layout(sms, B, nq, Hkv * G, Hkv, cols);
             if (n++ == 0) { kept = w.off_tickets; end = w.end_kept; }
             bad += w.off_tickets != kept || w.end_kept != end;                                   // the same for every call
-            bad += w.off_tickets < 4 || w.off_tickets + (size_t)sms * 4 > w.end_kept;            // room for a ticket per CTA
-            const size_t at[] = {w.end_kept, w.off_seq_ctr, w.off_dev, w.off_lse, w.off_part, w.bytes};
-            const size_t need[] = {0, (size_t)B * 4, (size_t)B * Hkv * 64, (size_t)B * nq * Hkv * G * 4, (size_t)(B * Hkv + sms) * cols * 528};
-            for (int i = 0; i < 5; ++i) bad += at[i] + need[i] > at[i + 1] || at[i + 1] % 16 != 0;
+            const size_t at[] = {4, w.off_tickets, w.off_groups, w.end_kept, w.off_seq_ctr, w.off_dev, w.off_lse, w.off_part, w.bytes};
+            const size_t need[] = {0, sms * 4, 2 * sms * 4, 0, (size_t)B * 4, (size_t)B * Hkv * 64, (size_t)B * nq * Hkv * G * 4,
+                                   (size_t)(B * Hkv + sms) * cols * 528};
+            for (int i = 0; i < 8; ++i) bad += at[i] + need[i] > at[i + 1] || at[i + 1] % (i > 3 ? 16 : 4) != 0;
           }
   std::printf("%zu %zu", bad, n);
 }
@@ -48,10 +48,13 @@ def test_no_results_on_what_is_kept(tmp_path):
 def test_counts_are_either_kept_or_zeroed_by_the_call():
     """Tickets are taken at places that do not depend on the batch; everything else that is counted is zeroed by the kernel before."""
     text = "".join(re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, n)).read()) for n in ("attention.cu", "attention_i8.cuh", "attention_f16.cuh"))
-    counted = re.findall(r"atomic(?:Inc|Add|Max|Or)\((?:reinterpret_cast<int\*>\()?p\.(\w+)", text)
-    assert set(counted) == {"ws_tickets", "ws_seq_ctr", "ws_dev", "ws_flags"}
-    zero = re.search(r"void zero_decision\(.*?\n\}", text, re.S).group(0)
-    assert "p.ws_dev[" in zero and "p.ws_seq_ctr[b] = 0u" in zero and len(re.findall(r"zero_decision\(p, b, hkv, lane\)", text)) == 2
+    counted = set(re.findall(r"atomic(?:Inc|Add|Max|Or)\((?:reinterpret_cast<int\*>\()?(?:p\.)?(\w+)", text))
+    assert counted == {"ticket", "ws_seq_ctr", "ws_dev", "ws_flags"}
+    group = re.search(r"SlotGroup slot_group\(.*?\n\}", text, re.S).group(0)
+    assert set(re.findall(r"p\.(ws_\w+)", group)) == {"ws_tickets", "ws_groups"}
+    assert set(re.findall(r"\blast_of\(([^,]+),", text)) == {"uint32_t* ticket", "g.ticket", "p.ws_tickets + item.first_cta"}
+    assert len(re.findall(r"p\.ws_dev\[[^;]*\] = 0\.0f;", text)) == 2 and "p.ws_seq_ctr[b] = 0u;" in text
+    assert len(re.findall(r"\bper_sequence<\w+, C::kPartCols>\(", text)) == 3, "at every end of a producer"
 
 
 def test_no_cta_is_first_of_two_shared_segments():

@@ -56,6 +56,7 @@ struct AttnParams {
   uint32_t* ws_tickets;    // [SMs] tickets of the CTAs that share a (sequence, KV head), at the first one's index
   uint32_t* ws_groups;     // [SMs][2] tickets of groups of such CTAs
   uint32_t* ws_seq_ctr;    // [B] rows of a sequence that have been joined (zeroed by the attention kernel)
+  uint32_t* ws_long;       // [SMs / kLongStep] word i: 1 + the long segment that CTA kLongStep i lies inside of, or 0
   float* ws_dev;           // [B*Hkv][kMaxQ]
   float* ws_lse;           // [B][nq_stride][Hq] natural-log log-sum-exp of every output row's scores
   float* ws_part;          // [B*Hkv + CTAs][ncols_pad][kPartStride], slot = segment + CTA index (and see seg_word)
@@ -301,11 +302,24 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
   return r;
 }
 
+// A segment of this many CTAs or more is long: there is a multiple of kLongStep among those that lie inside of it, with nothing
+// else to do.  Such a CTA tells attn_combine_kernel, and every other multiple that it does not.
+constexpr int kLongSegment = 24, kLongStep = 16;
+static_assert(kLongSegment >= kLongStep + 2, "a multiple between the first and the last");
+__device__ __forceinline__ void tell_long(const AttnParams& p, int cta, const Item* it) {   // it: a piece of this CTA, or none
+  if (cta % kLongStep) return;
+  uint32_t seg = 0;
+  if (it && it->n_contrib >= kLongSegment && cta > it->first_cta && cta < it->first_cta + it->n_contrib - 1)   // (then the only one)
+    seg = 1u + (uint32_t)(it->b * p.Hkv + it->hkv);
+  p.ws_long[cta / kLongStep] = seg;
+}
+
 // What is left to do for a sequence, by one warp of one CTA each: the count of finished rows that attn_combine_kernel decides by
 // starts at zero; where there is no token, outputs are zero and nothing is rejected unless the draft is not zero.
 // (Off the path of the sequences' tokens: called behind a CTA's last copy.)
 template <bool FULL, int kPartCols>
-__device__ __forceinline__ void per_sequence(const AttnParams& p, int cta, int n_cta, int lane, const SeqLens& sl) {
+__device__ __forceinline__ void per_sequence(const AttnParams& p, int cta, int n_cta, int lane, const SeqLens& sl, const Item* it) {
+  if (FULL && lane == 0) tell_long(p, cta, it);
   for (int b = cta; b < p.B; b += n_cta) {
     if (FULL && lane == 0) p.ws_seq_ctr[b] = 0u;
     if (sl.of(b) != 0) continue;
@@ -337,20 +351,79 @@ __device__ __forceinline__ void per_sequence(const AttnParams& p, int cta, int n
 // a head joined all its columns behind a ticket and took the decision, and the other SMs had nothing to do.  us: one layer of
 // 4096 tokens, 16 columns 27.8 -> 17.6, 4 columns 13.2 -> 11.6, both replayed from a graph; of 131072 tokens, 32 columns, 96.4
 // -> 87.4; two sequences of 131072, 64 columns, 243 -> 236; two of 16000, 8 columns, 25.7 -> 23.8.)
-constexpr int kCombineWarps = 4, kCombineFly = 5;
-template <int W>
-__global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const AttnParams p, int part_cols, int n_slots) {
+//
+// Where there are many heads a segment has a slot or two on average, and a row is one warp's (four warps for every row: 16
+// sequences of 500 tokens, 16 columns, 20.1 -> 21.8 us, 64 of 200, 32 columns, 47 -> 60 us).  But one long sequence among many short
+// ones with few heads has up to a slot per SM, 148 of them behind one another in one warp: the rows of long segments (see
+// tell_long) go to CTAs of their own in front of the others, four warps a row, eight slots in flight each.  (us, one sequence of 32768 tokens
+// among 39 of 64, one KV head, 4 / 16 / 32 columns: 36.6 / 43.2 / 53.4 by a warp per row, 16.8 / 25.3 / 26.8 this way.)
+constexpr int kCombineWarps = 4, kCombineFly = 5, kLongFly = 8;
+// The sums of slots warp, warp + W, ... of n at `col`, relative to their running maximum M; a lane has four dims.
+template <int FLY>
+__device__ __forceinline__ void join_slots(const float* col, size_t sstride, int n, int warp, int W, int lane, float4& acc, float& M, float& L) {
+  for (int i0 = warp; i0 < n; i0 += W * FLY) {
+    float4 o[FLY];
+    float2 ml[FLY];
+#pragma unroll
+    for (int u = 0; u < FLY; ++u) {
+      const int i = i0 + u * W;
+      ml[u] = make_float2(-INFINITY, 0.0f);
+      o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < n) {
+        const float* s = col + (size_t)i * sstride;
+        ml[u] = ld_dep(reinterpret_cast<const float2*>(s + 128));
+        o[u] = ld_dep(reinterpret_cast<const float4*>(s) + lane);
+      }
+    }
+    const float m0 = M;
+#pragma unroll
+    for (int u = 0; u < FLY; ++u) M = fmaxf(M, ml[u].x);
+    const float f0 = m0 == -INFINITY ? 0.0f : ex2(m0 - M);
+    L *= f0;
+    acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
+#pragma unroll
+    for (int u = 0; u < FLY; ++u) {
+      const float f = ml[u].x == -INFINITY ? 0.0f : ex2(ml[u].x - M);
+      L = fmaf(ml[u].y, f, L);
+      acc.x = fmaf(o[u].x, f, acc.x);
+      acc.y = fmaf(o[u].y, f, acc.y);
+      acc.z = fmaf(o[u].z, f, acc.z);
+      acc.w = fmaf(o[u].w, f, acc.w);
+    }
+  }
+}
+// A row per CTA (kWide), or four, and with kWithLong in front of them n_long CTAs for the rows of long segments.
+enum CombineMode { kWide, kNarrow, kWithLong };
+template <CombineMode MODE>
+__global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const AttnParams p, int part_cols, int n_slots, int n_long) {
   pdl_trigger();
+  const bool for_long = MODE == kWithLong && (int)blockIdx.x < n_long;
+  const int W = MODE == kWide || for_long ? kCombineWarps : 1;
   const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;   // warp of the row
-  const unsigned r = W == 1 ? blockIdx.x * kCombineWarps + (threadIdx.x >> 5) : blockIdx.x;
-  const int hq = r % p.Hq, bj = r / p.Hq, j = bj % p.nq, b = bj / p.nq;
-  if (W == 1 && b >= p.B) return;
+  __shared__ float4 o_s[kCombineWarps][32];
+  __shared__ float2 ml_s[kCombineWarps];
+  int b, j, hq;
+  if (for_long) {
+    pdl_wait();
+    const int i = (int)blockIdx.x / p.ncols, c = (int)blockIdx.x - i * p.ncols;
+    const uint32_t bh1 = ld_dep(p.ws_long + i);
+    if (bh1 == 0 || bh1 > (uint32_t)(p.B * p.Hkv)) return;
+    const int hkv = (int)((bh1 - 1) % p.Hkv);
+    b = (int)((bh1 - 1) / p.Hkv);
+    j = c / p.G;
+    hq = hkv * p.G + (c - j * p.G);
+  } else {
+    const unsigned r = MODE == kWide ? blockIdx.x : (blockIdx.x - n_long) * kCombineWarps + (threadIdx.x >> 5);
+    const unsigned bj = r / p.Hq;
+    hq = r % p.Hq;
+    j = bj % p.nq;
+    b = bj / p.nq;
+    if (MODE != kWide && b >= p.B) return;
+    pdl_wait();
+  }
   const int hkv = hq / p.G, g = hq - hkv * p.G;
   const size_t bh = (size_t)b * p.Hkv + hkv, row = ((size_t)b * p.nq_stride + j) * p.Hq + hq;
   const bool decide = p.draft != nullptr;
-  __shared__ float4 o_s[kCombineWarps][32];
-  __shared__ float2 ml_s[kCombineWarps];
-  pdl_wait();
   const uint32_t seg = ld_dep(seg_word(p, bh, part_cols));
   float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
   if (decide && warp == 0) {
@@ -359,6 +432,10 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
     else d = make_float4(ld_dep(dp), ld_dep(dp + 1), ld_dep(dp + 2), ld_dep(dp + 3));
   }
   const int first = min((int)(seg >> 16), n_slots - 1), n = min((int)(seg & 0xFFFFu), n_slots - first);
+  if (MODE == kWithLong) {
+    // a long segment's rows belong to the first of the multiples inside of it
+    if (for_long ? (int)blockIdx.x / p.ncols != first / kLongStep + 1 : n >= kLongSegment) return;
+  }
   const bool direct = n == 1 && !p.combine_single;   // written by the attention kernel
   if (n == 0 || (direct && !decide)) return;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -367,36 +444,8 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
     const size_t sstride = (size_t)part_cols * kPartStride;
     const float* col = p.ws_part + (bh + first) * sstride + (size_t)(j * p.G + g) * kPartStride;
     float M = -INFINITY, L = 0.0f;
-    for (int i0 = warp; i0 < n; i0 += W * kCombineFly) {
-      float4 o[kCombineFly];
-      float2 ml[kCombineFly];
-#pragma unroll
-      for (int u = 0; u < kCombineFly; ++u) {
-        const int i = i0 + u * W;
-        ml[u] = make_float2(-INFINITY, 0.0f);
-        o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < n) {
-          const float* s = col + (size_t)i * sstride;
-          ml[u] = ld_dep(reinterpret_cast<const float2*>(s + 128));
-          o[u] = ld_dep(reinterpret_cast<const float4*>(s) + lane);
-        }
-      }
-      const float m0 = M;
-#pragma unroll
-      for (int u = 0; u < kCombineFly; ++u) M = fmaxf(M, ml[u].x);
-      const float f0 = m0 == -INFINITY ? 0.0f : ex2(m0 - M);
-      L *= f0;
-      acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
-#pragma unroll
-      for (int u = 0; u < kCombineFly; ++u) {
-        const float f = ml[u].x == -INFINITY ? 0.0f : ex2(ml[u].x - M);
-        L = fmaf(ml[u].y, f, L);
-        acc.x = fmaf(o[u].x, f, acc.x);
-        acc.y = fmaf(o[u].y, f, acc.y);
-        acc.z = fmaf(o[u].z, f, acc.z);
-        acc.w = fmaf(o[u].w, f, acc.w);
-      }
-    }
+    if (for_long) join_slots<kLongFly>(col, sstride, n, warp, W, lane, acc, M, L);
+    else join_slots<kCombineFly>(col, sstride, n, warp, W, lane, acc, M, L);
     if (W > 1) {
       if (warp > 0) o_s[warp][lane] = acc;
       if (lane == 0) ml_s[warp] = make_float2(M, L);
@@ -404,13 +453,13 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
       if (warp > 0) return;
       float mx = M;
 #pragma unroll
-      for (int k = 1; k < W; ++k) mx = fmaxf(mx, ml_s[k].x);
+      for (int k = 1; k < kCombineWarps; ++k) mx = fmaxf(mx, ml_s[k].x);
       const float f0 = M == -INFINITY ? 0.0f : ex2(M - mx);
       L *= f0;
       M = mx;
       acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
 #pragma unroll
-      for (int k = 1; k < W; ++k) {
+      for (int k = 1; k < kCombineWarps; ++k) {
         const float2 ml = ml_s[k];
         const float4 o = o_s[k][lane];
         const float f = ml.x == -INFINITY ? 0.0f : ex2(ml.x - mx);
@@ -466,14 +515,27 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_combine_kernel(const 
   }
 }
 
-// (units of st tokens; nothing to join where every segment is one unit)
-inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tokens, cudaStream_t st) {
-  if (p.inline_merge || (!p.draft && !p.combine_single && (long long)p.max_blocks * p.bt <= st_tokens)) return LYNX_OK;
+// CTAs of an attention launch with units of st tokens: one per SM, but min_units units each where a sequence has as many.
+inline int attention_grid(const AttnParams& p, int st_tokens, int min_units) {
+  const long long per = (long long)min_units * st_tokens;
+  const long long grid = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + per - 1) / per);
+  const int full = sm_count();
+  return grid < 1 ? 1 : grid > full ? full : (int)grid;
+}
+
+// (nothing to join where every segment is one unit)
+inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tokens, int min_units, cudaStream_t st) {
+  const long long cap_units = ((long long)p.max_blocks * p.bt + st_tokens - 1) / st_tokens;
+  if (p.inline_merge || (!p.draft && !p.combine_single && cap_units <= 1)) return LYNX_OK;
   // a warp per row where a head has no more than a few CTAs on average (one layer: 18; 16 layers of two sequences: 0.6)
   const unsigned rows = (unsigned)(p.B * p.nq * p.Hq);
-  const bool wide = p.B * p.Hkv * 4 < sm_count();
-  return launch_pdl(wide ? attn_combine_kernel<4> : attn_combine_kernel<1>, wide ? rows : (rows + kCombineWarps - 1) / kCombineWarps,
-                    kCombineWarps * 32, 0, st, p, part_cols, sm_count());
+  if (p.B * p.Hkv * 4 < sm_count())
+    return launch_pdl(attn_combine_kernel<kWide>, rows, kCombineWarps * 32, 0, st, p, part_cols, sm_count(), 0);
+  const unsigned fours = (rows + kCombineWarps - 1) / kCombineWarps;
+  if (cap_units < kLongSegment)   // (no segment has more CTAs than units)
+    return launch_pdl(attn_combine_kernel<kNarrow>, fours, kCombineWarps * 32, 0, st, p, part_cols, sm_count(), 0);
+  const int n_long = (attention_grid(p, st_tokens, min_units) + kLongStep - 1) / kLongStep * p.ncols;
+  return launch_pdl(attn_combine_kernel<kWithLong>, n_long + fours, kCombineWarps * 32, 0, st, p, part_cols, sm_count(), n_long);
 }
 
 #include "tc_common.cuh"
@@ -597,6 +659,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   p.ws_tickets = reinterpret_cast<uint32_t*>(ws + pl.ws.off_tickets);
   p.ws_groups = reinterpret_cast<uint32_t*>(ws + pl.ws.off_groups);
   p.ws_seq_ctr = reinterpret_cast<uint32_t*>(ws + pl.ws.off_seq_ctr);
+  p.ws_long = reinterpret_cast<uint32_t*>(ws + pl.ws.off_long);
   p.ws_dev = reinterpret_cast<float*>(ws + pl.ws.off_dev);
   p.ws_lse = reinterpret_cast<float*>(ws + pl.ws.off_lse);
   p.ws_part = reinterpret_cast<float*>(ws + pl.ws.off_part);

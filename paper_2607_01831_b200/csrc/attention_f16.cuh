@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     else
       f16_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
                       reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
-    if (pw == 0) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl);
+    if (pw == 0) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
     return;
   }
   // ================================================================================== products
@@ -953,6 +953,7 @@ template <int NC>
 lynx_status launch_f16(AttnParams p, cudaStream_t st) {
   using C = F16Cfg<NC>;
   p.combine_single = 1;
-  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, 1, attn_f16_kernel<NC>>(p, st);
-  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, st);
+  constexpr int kMin = 1;
+  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, kMin, attn_f16_kernel<NC>>(p, st);
+  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }

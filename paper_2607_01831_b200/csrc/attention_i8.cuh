@@ -373,7 +373,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   __syncthreads();  // (A) the range is published
   const int n_units = (int)(lo < hi ? hi - lo : 0);
   if (n_units == 0) {
-    if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
+    if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl, nullptr);
     return;
   }
 
@@ -466,7 +466,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   }
   __syncwarp();
   bar_arrive(9, C::kThreads);
-  if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl);
+  if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl, items);
 }
 
 // Largest |q| of a piece's raw queries, by 128 threads (index i of 0..127), reduced over the
@@ -1290,15 +1290,12 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
       return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  long long grid = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + MIN * ST - 1) / (MIN * ST));
-  const long long full = sm_count();   // one CTA per SM
-  grid = grid < 1 ? 1 : (grid > full ? full : grid);
   // Programmatic dependent launch: when the kernel before this one in the stream is of the same kind (one
   // launch per layer of a decoder), this grid's CTAs may become resident, and set up their shared and tensor
   // memory, while the last CTAs of that kernel are still merging; they read nothing before
   // griddepcontrol.wait, i.e. before that kernel has completed and its memory is visible.
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = dim3((unsigned)attention_grid(p, ST, MIN));
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
@@ -1325,6 +1322,7 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
 template <bool FULL, int CP>
 lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
   using C = I8Cfg<FULL, CP>;
-  const lynx_status rc = launch_units<FULL, C::kSmem, C::kThreads, C::kST, 2, attn_i8_kernel<FULL, CP>>(p, st);
-  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, st);
+  constexpr int kMin = 2;
+  const lynx_status rc = launch_units<FULL, C::kSmem, C::kThreads, C::kST, kMin, attn_i8_kernel<FULL, CP>>(p, st);
+  return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }

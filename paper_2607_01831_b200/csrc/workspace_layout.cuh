@@ -19,6 +19,7 @@ struct WsLayout {
   size_t off_tickets;   // one per SM: of the segment shared by several CTAs whose first is this one (no CTA is first of two)
   size_t off_groups;    // two per SM: of groups of such CTAs (see slot_group)
   size_t end_kept;
+  size_t off_long;      // one per eight SMs at most: what attn_combine_kernel is told of long segments
   size_t off_seq_ctr;   // [B] counts of a sequence's finished rows
   size_t off_dev;       // [B * Hkv][kWsMaxQ] deviations
   size_t off_lse;       // [B][nq][Hq] log-sum-exps
@@ -31,7 +32,8 @@ inline WsLayout ws_layout(int sms, int B, int nq, int Hq, int Hkv, int cols_pad)
   w.off_tickets = kWsHeaderBytes;
   w.off_groups = w.off_tickets + (size_t)sms * 4;
   w.end_kept = w.off_groups + (size_t)2 * sms * 4;
-  w.off_seq_ctr = up(w.end_kept, 128);
+  w.off_long = up(w.end_kept, 128);
+  w.off_seq_ctr = up(w.off_long + (size_t)(sms / 8 + 1) * 4, 128);
   // (the room between counts and deviations is not used; the size is a figure that callers hold)
   w.off_dev = up(kWsHeaderBytes + (size_t)2 * sms * kWsMaxCtasPerSm * 4 + (size_t)B * 4 + (size_t)B * Hkv * 4, 256);
   w.off_lse = up(w.off_dev + (size_t)B * Hkv * kWsMaxQ * 4, 256);

@@ -27,10 +27,10 @@ int main() {
             const lynx::WsLayout w = lynx::ws_layout(sms, B, nq, Hkv * G, Hkv, cols);
             if (n++ == 0) { kept = w.off_tickets; end = w.end_kept; }
             bad += w.off_tickets != kept || w.end_kept != end;                                   // the same for every call
-            const size_t at[] = {4, w.off_tickets, w.off_groups, w.end_kept, w.off_seq_ctr, w.off_dev, w.off_lse, w.off_part, w.bytes};
-            const size_t need[] = {0, sms * 4, 2 * sms * 4, 0, (size_t)B * 4, (size_t)B * Hkv * 64, (size_t)B * nq * Hkv * G * 4,
+            const size_t at[] = {4, w.off_tickets, w.off_groups, w.end_kept, w.off_long, w.off_seq_ctr, w.off_dev, w.off_lse, w.off_part, w.bytes};
+            const size_t need[] = {0, sms * 4, 2 * sms * 4, 0, (sms + 7) / 8 * 4, (size_t)B * 4, (size_t)B * Hkv * 64, (size_t)B * nq * Hkv * G * 4,
                                    (size_t)(B * Hkv + sms) * cols * 528};
-            for (int i = 0; i < 8; ++i) bad += at[i] + need[i] > at[i + 1] || at[i + 1] % (i > 3 ? 16 : 4) != 0;
+            for (int i = 0; i < 9; ++i) bad += at[i] + need[i] > at[i + 1] || at[i + 1] % (i > 4 ? 16 : 4) != 0;
           }
   std::printf("%zu %zu", bad, n);
 }

@@ -1044,7 +1044,9 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         // its own for the question.
         const bool forced = fresh || units_in_acc >= C::kDrainUnits;   // uniform over the team
         const bool over = ymax > 31.5f;
-        volatile int* raise_flag = my_misc + 2;
+        // (two flags in turn: a warp may be on its way into the next unit while another looks at this one's, if the waits in
+        // between have given up)
+        volatile int* raise_flag = my_misc + 2 + (n_own & 1);
         auto restart = [&]() {
 #pragma unroll
           for (int c = 0; c < CG; ++c) {   // (rare path: back to absolute exponents x = y + ref)

@@ -92,3 +92,52 @@ def test_barrier_ids_are_distinct():
     assert len(fixed) == 2
     every = [0] + fixed + [f(tm) for f in ids.values() for tm in range(4)]
     assert len(set(every)) == len(every) and max(every) < 16
+
+
+def _decisions(flag_of, warps=4, units=8, orders=400):
+    """Units in which a team's warps do not agree whether to restart, over many orders of their steps: a warp may raise the unit's flag,
+    all meet, each looks at the flag, and a team that restarts meets twice more with the flag taken back in between."""
+    split = 0
+    for seed in range(orders):
+        rng, flags, seen = random.Random(seed), {}, [dict() for _ in range(warps)]
+
+        def program(w):
+            for u in range(units):
+                if rng.random() < 0.1:
+                    flags[flag_of(u)] = 1
+                    yield "step"
+                yield "sync"
+                seen[w][u] = flags.get(flag_of(u), 0)
+                yield "step"
+                if seen[w][u]:
+                    yield "sync"
+                    if w == 0:
+                        flags[flag_of(u)] = 0
+                    yield "sync"
+                    yield "sync"
+        progs, waiting, done = [program(w) for w in range(warps)], set(), set()
+        while len(done) < warps:
+            ready = [w for w in range(warps) if w not in waiting and w not in done]
+            if not ready:
+                if len(waiting) + len(done) < warps or done:
+                    break                       # warps that took different ways wait for one another
+                waiting.clear()
+                continue
+            w = rng.choice(ready)
+            step = next(progs[w], None)
+            if step is None:
+                done.add(w)
+            elif step == "sync":
+                waiting.add(w)
+        split += len(done) < warps or any(len({s.get(u) for s in seen}) > 1 for u in range(units))
+    return split
+
+
+def test_all_warps_take_the_restart_or_none_does():
+    text = _team_barriers()[1]
+    expr = re.search(r"raise_flag = my_misc \+ 2([^;]*);", text).group(1)
+    assert _decisions(lambda u: eval("0" + expr, {"n_own": u})) == 0
+
+
+def test_one_flag_for_all_units_would_split_the_team():
+    assert _decisions(lambda u: 0) > 0

@@ -10,7 +10,9 @@ merge_verify_attention, workspace_bytes.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -151,15 +153,28 @@ def _python_only(*_):
     return None
 
 
+@functools.lru_cache(maxsize=None)
+def _extension():
+    """The extension, or None (with a warning, once) where it does not load or was compiled against another torch, whose tensors
+    it would read wrongly."""
+    load()   # (raises where the library is not built)
+    try:
+        from . import _native
+        built = _native.torch_version
+        if built == torch.__version__:
+            return _native
+        why = f"it was built for torch {built}, this is {torch.__version__}"
+    except ImportError as e:
+        why = str(e)
+    warnings.warn(f"paper_2607_01831_b200._native is not used ({why}): calls go through ctypes and take about twice the host time; "
+                  "rebuild with `python -m paper_2607_01831_b200.build`", RuntimeWarning)
+    return None
+
+
 def _fast(var: str, name: str):
     """The extension's function `name`, found when the global `var` that holds this is first called."""
     def first(*args):
-        load()   # (raises where the library is not built)
-        try:
-            from . import _native
-        except ImportError:   # built for another torch: ctypes alone
-            _native = None
-        globals()[var] = getattr(_native, name, _python_only)
+        globals()[var] = getattr(_extension(), name, _python_only)
         return globals()[var](*args)
     return first
 

@@ -3,6 +3,7 @@
 // else: whatever is not plain (no exact torch.Tensor, not on the GPU, not contiguous, another type or shape, tensors of a
 // transform or a mode) is left to them by returning None, so that errors and special cases stay theirs.  What it saves is
 // host time per call, which bounds small problems (us, marshalling through ctypes -> here): see __init__.py.
+// It reads tensors through inline functions of the torch it is compiled against (LYNX_TORCH_VERSION) and is used with that one alone.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -334,5 +335,7 @@ PyMODINIT_FUNC PyInit__native() {
                                                      {&s_residual, "residual"}, {&s_meta, "meta"}};
   for (auto& x : names)
     if (!(*x.s = PyUnicode_InternFromString(x.n))) return nullptr;
-  return PyModule_Create(&module);
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "torch_version", LYNX_TORCH_VERSION)) Py_CLEAR(m);
+  return m;
 }

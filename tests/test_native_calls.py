@@ -1,6 +1,7 @@
 """The extension behind the per-step calls does what their Python bodies do: the same bits, objects and errors on the GPU, and it
 leaves alone (returns None for) whatever is not a plain GPU tensor."""
 import threading
+import warnings
 
 import pytest
 import torch
@@ -39,6 +40,48 @@ def test_what_is_not_plain_is_left_alone():
         lynx.anchor_attention(geo, q, planes, planes, i, i, ws)
     with pytest.raises(lynx.LynxError, match="q must be"):
         lynx.anchor_attention(geo, q.float(), planes, planes, i, i, ws)
+
+
+@pytest.fixture
+def unresolved(monkeypatch):
+    """The module as before its first call."""
+    lynx.load()
+    for v in [v for v in vars(lynx) if v.startswith("_fast_")]:
+        monkeypatch.setattr(lynx, v, lynx._fast(v, "recombine"))
+    lynx._extension.cache_clear()
+    yield monkeypatch
+    lynx._extension.cache_clear()
+
+
+def test_an_extension_for_another_torch_is_not_used(unresolved):
+    assert _native().torch_version == torch.__version__ and lynx._extension() is _native()
+    lynx._extension.cache_clear()
+    unresolved.setattr(torch, "__version__", "2.12.0+cu130")
+    with pytest.warns(RuntimeWarning, match="built for torch"):
+        assert lynx._fast_recombine(None, True, False) is None
+    assert lynx._fast_recombine is lynx._python_only
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        assert lynx._fast_anchor() is None        # said once
+
+
+def test_an_extension_that_does_not_load_is_said(unresolved):
+    import sys
+    unresolved.setitem(sys.modules, "paper_2607_01831_b200._native", None)
+    unresolved.delattr(lynx, "_native", raising=False)
+    with pytest.warns(RuntimeWarning, match="not used"):
+        assert lynx._fast_recombine(None, True, False) is None
+
+
+def test_the_library_is_built_without_its_extension(monkeypatch, tmp_path):
+    from paper_2607_01831_b200 import build as b
+    assert not b._native_stale()
+    monkeypatch.setattr(torch, "__version__", "2.12.0+cu130")
+    assert b._native_stale() and not b._stale()
+    monkeypatch.setattr(b, "_native_cmd", lambda out: ["false"])
+    monkeypatch.setattr(b, "_build_library", lambda verbose: pytest.fail("the library is there"))
+    with pytest.warns(UserWarning, match="was not built"):
+        assert b.build() == b.LIB
 
 
 def _everything(seed, stream=None):

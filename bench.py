@@ -43,6 +43,22 @@ def measured_peak():
 
 
 # --------------------------------------------------------------------------- workload set-up
+def attention_kernels(B, Hkv, G, n_q, capacity, sms, full, draft):
+    """Kernels that one attention call launches: per slice of its positions the attention and, where something is left to join
+    or to decide, the joining of its results, plus the decision over all slices where there are several."""
+    if full:     # a launch takes up to 16 positions and 64 columns
+        per = n_q if n_q <= 16 and n_q * G <= 64 else min(16, max(1, 64 // G))
+    else:        # up to 32 columns
+        per = n_q if n_q * G <= 32 else max(1, 32 // G)
+    slices = [min(per, n_q - j) for j in range(0, n_q, per)]
+    n = 0
+    for nq in slices:
+        in_kernel = not full and B * Hkv * 4 >= sms                      # the last CTA of a head joins
+        one_unit = not draft and not (full and nq * G > 16) and capacity <= 128   # (the FP16 kernel leaves every result to be joined)
+        n += 1 if in_kernel or one_unit else 2
+    return n + (1 if draft and len(slices) > 1 else 0)
+
+
 class Workload:
     """All device state of one configuration, layers flattened into the batch dimension."""
 
@@ -143,18 +159,18 @@ class Workload:
                 n += win["k"] * self.anchor_kernels() + self.verify_kernels(win["k"])
         return n
 
-    def anchor_kernels(self):
-        """Kernels of one anchor call: the attention, and the joining of partial results where few heads share the GPU."""
+    def _kernels(self, n_q, full):
         sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
-        return 1 if self.B * self.wl.num_kv_heads * 4 >= sms else 2
+        Hkv = self.wl.num_kv_heads
+        return attention_kernels(self.B, Hkv, self.wl.num_q_heads // Hkv, n_q, self.table.shape[1] * self.wl.block_tokens, sms, full, draft=full)
+
+    def anchor_kernels(self):
+        """Kernels of one anchor call of one position."""
+        return self._kernels(1, False)
 
     def verify_kernels(self, k):
-        """Kernels of one merge-verify call: per slice of the window (a launch takes up to 16 positions and 64 columns) the
-        attention and the joining of its results with the decision, plus the decision over all slices when there is more than one."""
-        G = self.wl.num_q_heads // self.wl.num_kv_heads
-        per = k if k <= 16 and k * G <= 64 else min(16, max(1, 64 // G))
-        slices = -(-k // per)
-        return 2 * slices + (1 if slices > 1 else 0)
+        """Kernels of one merge-verify call of k positions with a draft."""
+        return self._kernels(k, True)
 
     def launches_per_step(self):
         return 2 + sum(w["reps"] * (w["k"] * self.anchor_kernels() + self.verify_kernels(w["k"])) for w in self.windows)

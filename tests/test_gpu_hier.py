@@ -19,12 +19,21 @@ def _nib(packed):         # u8 [...,64] -> signed 4-bit values int [...,128]
     return np.where(v > 7, v - 16, v)
 
 
-# 1000 pages: more than the quantiser's grid (three CTAs per SM), so CTAs walk through several pages
+# 1000 pages: more than the quantiser's grid (half a page per CTA, six CTAs per SM), so CTAs walk through several half pages
 @pytest.mark.parametrize("recipe,n_pages", [("normal_outlier4x8", 5), ("student_t4", 37), ("lognormal_channels", 300),
                                             ("normal_outlier4x8", 1000)])
 def test_hier_quantize_and_dequantize_match_the_oracle(recipe, n_pages):
     # pages of 256 tokens x 128 channels (one KV head each)
     x = synth.kv_block_values(recipe, n_pages, 1, 256, "cpu", "hier", n_pages).reshape(n_pages, 256, 128)
+    _check_against_oracle(x)
+
+
+# at the thresholds, for 148 SMs: four, two or one CTA of the inverse per page (up to one page per SM, up to two), and the first
+# half pages that a CTA of the quantiser walks on to (three pages per SM)
+@pytest.mark.parametrize("pages_per_sm,extra", [(1, 0), (1, 1), (2, 0), (2, 1), (3, 0), (3, 1)])
+def test_hier_pages_at_the_thresholds(pages_per_sm, extra):
+    n_pages = pages_per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    x = synth.kv_block_values("student_t4", n_pages, 1, 256, "cpu", "hier", n_pages).reshape(n_pages, 256, 128)
     _check_against_oracle(x)
 
 

@@ -201,15 +201,6 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// The stream-K cut of the work list (units of ST tokens in (sequence, KV head, position) order) for
-// CTA `cta` of `n_cta`, derived by one warp from the sequence lengths on the device.  Normally every
-// CTA takes q = ceil(total / n_cta) consecutive units, wherever the (sequence, head) boundaries fall.
-// When all sequences have the same number of units U and the B * Hkv segments are few enough to give
-// each of them c >= 1 CTAs of its own (one layer of a long context per launch), the cut is aligned
-// instead: q = ceil(U / c), and CTA i takes part i % c of segment i / c.  No CTA then pays for the
-// end of one piece and the start of another, at the cost of n_cta - c * segments idle CTAs (accepted
-// up to 15 %).  lo, hi index a list in which every segment occupies c * q entries, so that the
-// contributors of a segment and their partial slots follow from lo and q as in the plain cut.
 // a / b for 0 <= a < 2^22, 0 < b < 2^22: ten instructions, where an integer division takes thirty (64-bit: a hundred) one after
 // the other, in the one warp that the first copy of a launch waits for.
 __device__ __forceinline__ int small_div(int a, int b) {
@@ -242,6 +233,15 @@ struct SeqLens {
   // by a lane, of sequence b0 + lane
   __device__ __forceinline__ int at(int b0, int lane) const { return b0 == 0 ? len0 : load(b0 + lane); }
 };
+// The stream-K cut of the work list (units of ST tokens in (sequence, KV head, position) order) for
+// CTA `cta` of `n_cta`, derived by one warp from the sequence lengths on the device.  Normally every
+// CTA takes q = ceil(total / n_cta) consecutive units, wherever the (sequence, head) boundaries fall.
+// When all sequences have the same number of units U and the B * Hkv segments are few enough to give
+// each of them c >= 1 CTAs of its own (one layer of a long context per launch), the cut is aligned
+// instead: q = ceil(U / c), and CTA i takes part i % c of segment i / c.  No CTA then pays for the
+// end of one piece and the start of another, at the cost of n_cta - c * segments idle CTAs (accepted
+// up to 15 %).  lo, hi index a list in which every segment occupies c * q entries, so that the
+// contributors of a segment and their partial slots follow from lo and q as in the plain cut.
 template <int ST>
 __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int cta, int lane, const SeqLens& sl) {
   SkRange r;
@@ -345,12 +345,14 @@ __device__ __forceinline__ void per_sequence(const AttnParams& p, int cta, int n
 
 // Joins the partial results of the CTAs that share a (sequence, KV head) and takes the accept / reject decision: W warps per
 // output row, its slots (m, l, O) dealt to them, five in flight each, the warps' sums joined in order.
-// Launched behind every attention kernel as a programmatic dependent.
+// A programmatic dependent behind every verification and behind anchor calls with few heads, unless no sequence can have more than
+// a unit and nothing is to be decided; anchor calls with many heads join in the attention kernel (see launch_combine).
 // Latency bounds it -- the look-up of the segment, a round of slots, for verification a ticket and one more round -- and the
 // instructions of a thread in a row, so that a row is cut over many threads where it has many slots.  (Before, the last CTA of
-// a head joined all its columns behind a ticket and took the decision, and the other SMs had nothing to do.  us: one layer of
-// 4096 tokens, 16 columns 27.8 -> 17.6, 4 columns 13.2 -> 11.6, both replayed from a graph; of 131072 tokens, 32 columns, 96.4
-// -> 87.4; two sequences of 131072, 64 columns, 243 -> 236; two of 16000, 8 columns, 25.7 -> 23.8.)
+// a head joined all its columns behind a ticket and took the decision, and the other SMs had nothing to do.  us, by this step alone:
+// one layer of 4096 tokens, 16 columns 27.8 -> 17.6, 4 columns 13.2 -> 11.6, of 131072 tokens, 32 columns, 96.4 -> 87.4, replayed
+// from a graph -- 16.5, 9.9 and 80 with the steps since --; two sequences of 131072, 64 columns, 243 -> 236 among other passes; two
+// of 16000, 8 columns, 25.7 -> 23.8.)
 //
 // Where there are many heads a segment has a slot or two on average, and a row is one warp's (four warps for every row: 16
 // sequences of 500 tokens, 16 columns, 20.1 -> 21.8 us, 64 of 200, 32 columns, 47 -> 60 us).  But one long sequence among many short
@@ -523,7 +525,8 @@ inline int attention_grid(const AttnParams& p, int st_tokens, int min_units) {
   return grid < 1 ? 1 : grid > full ? full : (int)grid;
 }
 
-// (nothing to join where every segment is one unit)
+// (Nothing to join where every segment is one unit and nothing to decide; anchor calls with many heads join in the attention
+// kernel.  bench.py counts kernels by this rule.)
 inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tokens, int min_units, cudaStream_t st) {
   const long long cap_units = ((long long)p.max_blocks * p.bt + st_tokens - 1) / st_tokens;
   if (p.inline_merge || (!p.draft && !p.combine_single && cap_units <= 1)) return LYNX_OK;
@@ -694,7 +697,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     return LYNX_OK;
   }
   // verification: the integer kernels up to 16 columns, tcgen05 with FP16 operands (attention_f16.cuh) above (one layer of
-  // 131072 tokens, 32 columns: 83 us by the FP16 kernel, 174 us as two passes of the integer kernel at 16).
+  // 131072 tokens, 32 columns, the attention kernels alone: 83 us by the FP16 one, 174 us as two passes of the integer one at 16;
+  // the whole call takes 91 us among other passes).
   // A window of more than kMaxQ positions or kMaxCols columns runs as slices of whole positions, each a pass
   // of its own over the planes that writes its outputs and deviations; the index of the first rejected
   // position over the whole window then follows from the deviations.

@@ -45,7 +45,7 @@
 // packed additions without selects, behind the scores instead of in front of them (32 columns 88.4 -> 83.0 us).  Twice the softmax warps with
 // half of a unit's tokens each and 80 registers: 64 columns +15 %, 32 +4 %.  One layer of 131072 tokens: 174 us as two passes
 // of the 16-column integer kernel -> 83 us (32 columns); two sequences, 64 columns: 293 us by the previous kernel (M = columns, codes
-// not centred) -> 207 us; back to back, before the power cap sets in.
+// not centred) -> 207 us; the kernel alone, back to back, before the power cap sets in (the calls among other passes: 91 and 227 us).
 
 template <int NC>
 struct F16Cfg {
@@ -727,7 +727,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       // ---- the piece's queries: thread = 16-byte chunk kt & 15 of columns kt >> 4, + 8, ... ---------------------
       {
         // (read once and kept, maxima on packed pairs, sums by exchanging halves, no division per chunk: with the
-        // results written eight columns at a time, 64 columns of 85 tokens 18.8 -> 15.0 us, 32 columns of 4 x 7056 34.8 -> 32.6 us)
+        // results written eight columns at a time, 64 columns of 85 tokens 18.8 -> 15.0 us, 32 columns of 4 x 7056 34.8 -> 32.6 us.
+        // At 64 columns they spill 72 bytes of these warps' registers, once per piece.)
         constexpr int NI = NC / 8;
         const uint32_t g_inv = 65536u / (uint32_t)p.G + 1u;   // c / G = c * g_inv >> 16 for c < 64, G <= 16
         uint4 qv[NI];

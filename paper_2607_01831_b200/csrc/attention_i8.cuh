@@ -249,9 +249,9 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return r;
 }
 // (One instruction per maximum and the sums below instead of butterflies in the restart and at the end of a piece, which lie in and
-// around the unit loop: fewer steps in a row where a piece starts and ends, and less code in the instruction caches.  us: 16 ragged
-// sequences at 16 columns 321 -> 275, 16 layers of two sequences of 131072 tokens at 8 columns 907 -> 878 before the power cap sets
-// in, one layer of 131072 tokens at 4 columns 39.0 -> 37.7, two sequences of 16000 at 8 columns 24.0 -> 21.8.)
+// around the unit loop: fewer steps in a row where a piece starts and ends, and less code in the instruction caches.  us, before the
+// power cap sets in: 16 ragged sequences at 16 columns 321 -> 275 (in it 338 -> 307), 16 layers of two sequences of 131072 tokens at 8
+// columns 907 -> 878; one layer of 131072 tokens at 4 columns 39.0 -> 37.7, two sequences of 16000 at 8 columns 24.0 -> 21.8.)
 __device__ __forceinline__ float warp_max(float x) {
   float r;
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));

@@ -6,8 +6,9 @@
 // measured against: softmax(q K^T scale) V of Section 2 on pages [num_blocks][Hkv][block_tokens][128]
 // BF16, as lynx_recombine writes them.
 //
-// Flash-decoding split-K: a CTA takes a chunk of kChunk tokens of one (sequence, KV head) and writes a
-// partial (m, l, O) to the workspace; a second kernel merges the chunks.  Nothing waits on anything but a cluster's own CTAs.
+// Flash-decoding split-K: a CTA, or a cluster of up to eight, takes a chunk of kChunk tokens of one (sequence, KV head) and writes
+// a partial (m, l, O) to the workspace, which a second kernel merges; where the table holds no more than one chunk per sequence the
+// tensor-core kernel writes the output itself.  Nothing waits on anything but a cluster's own CTAs.
 // Two kernels for the chunk: on the BF16 tensor cores (mma.sync m16n8k16, K and V tiles through a cp.async
 // ring per warp) for block sizes that are multiples of 16 tokens -- it streams the pages at the rate of a
 // plain copy -- and on the FP32 pipes for any other block size (8 or 16 lanes own a token, each 16 or 8 of
@@ -20,7 +21,7 @@
 namespace lynx {
 namespace {
 
-constexpr int kChunk = 2048;        // tokens per CTA
+constexpr int kChunk = 2048;        // tokens per CTA or cluster
 constexpr int kWarps = 8;           // warps per CTA: 256 tokens each
 constexpr int kPartStrideB = 132;   // floats per (chunk, column) partial: O[128], m, l, pad
 
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(kWarps * 32, COLS <= 4 ? 2 : 1) bf16_decode_ke
 // ---------------------------------------------------------------------------------------------------
 // The same split-K decode on the BF16 tensor cores (mma.sync m16n8k16), for block sizes that are multiples
 // of 16 tokens: with 8 columns the FP32 pipes above need more multiply-adds per byte than they have.
-// A warp takes every fourth 16-token tile of the CTA's chunk: the tile's K and V rows (4 KB each, contiguous
+// A warp takes every 4 S-th 16-token tile of the chunk of its cluster of S CTAs: the tile's K and V rows (4 KB each, contiguous
 // in a block) go through a three-stage cp.async ring of the warp's own in shared memory, 16-byte chunks
 // XOR-swizzled by the row so that ldmatrix reads them without bank conflicts.
 //   S[columns x 16 tokens] = Q K^T    A = Q (rows = query columns, 8 of 16 used), B = K rows as stored
@@ -534,9 +535,11 @@ lynx_status launch_bf16_tc(const BfParams& p, cudaStream_t st) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LYNX_ERR_CUDA;
     configured[dev] = true;
   }
-  // CTAs per chunk: a power of two, as long as all CTAs are resident at once (two per SM) and every warp has a tile.  us: 8 heads
+  // CTAs per chunk: a power of two, as long as all CTAs are resident at once (two per SM) and every warp has a tile.  (us: 8 heads
   // of 4096 tokens 28.2 by a CTA per chunk, 9.6 by eight; of 32768 tokens 31.5 and 28.4 by two (31.9 by four, 40.5 by eight: the
   // CTAs of a second round bring their start and end with them); 16 sequences of up to 512 tokens 13.4, 8.5 by two, 11.5 by four.
+  // The chunks are those of the table, whose lengths the host does not know: 8 heads of 1000 tokens take 5.4 with a table as wide,
+  // 16.3 with one of 131072 tokens, by a CTA per chunk and with the second kernel.)
   const long long pieces = (long long)p.B * p.Hkv * p.chunks, cap = (long long)p.max_blocks * p.bt;
   const long long tiles = ((cap < kChunk ? cap : kChunk) + kTcTile - 1) / kTcTile;
   int S = 1;

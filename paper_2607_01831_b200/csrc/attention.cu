@@ -1,7 +1,7 @@
 // lynx_anchor_attention and lynx_merge_verify_attention: split-K decode attention over the
 // packed nibble planes, dequantised on chip (sm_100a).  This file holds what the kernels share
 // (parameters, PTX helpers, the joining of partial results and the accept / reject decision) and the host
-// side; the kernels are in attention_i8.cuh and attention_f16.cuh.
+// side; the kernels are in attention_pipe.cuh, attention_i8.cuh and attention_f16.cuh.
 //
 // What is computed (Section 2 attention equation on the states of Section 4.2; accept/reject
 // of Section 4.3): for every (sequence, KV head) the G = Hq/Hkv query heads of each of the n_q
@@ -12,8 +12,8 @@
 //     sum_t p_t V^_t  = sum_t (p_t scale_t) level_t + (sum_t p_t zero_t) * 1
 // so the two contractions run on the integer levels and the scalars are applied per token
 // outside.  Anchor attention (any column count) and verification with up to 16 columns per launch run both contractions as exact integer products on
-// tcgen05.mma kind::i8 (attention_i8.cuh); verification with 17..64 columns per launch runs them on
-// tcgen05.mma kind::f16 with two-term FP16 weights (attention_f16.cuh).
+// tcgen05.mma kind::i8 (attention_pipe.cuh up to 16 columns, attention_i8.cuh above); verification with 17..64 columns per launch
+// runs them on tcgen05.mma kind::f16 with two-term FP16 weights (attention_f16.cuh).
 //
 // Common shape.  Persistent grid, one CTA per SM, flash-decoding split-K in stream-K form: the
 // (sequence, KV head, stage-unit) list is cut into equal contiguous ranges, one per CTA.
@@ -544,6 +544,7 @@ inline lynx_status launch_combine(const AttnParams& p, int part_cols, int st_tok
 #include "tc_common.cuh"
 #include "attention_i8.cuh"
 #include "attention_f16.cuh"
+#include "attention_pipe.cuh"
 
 // ------------------------------------------------------------------ host side
 // Query positions per launch of a verification call: all of them up to kMaxQ positions and kMaxCols
@@ -678,7 +679,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
   // the fixed array keeps what the previous call left: the status word and the tickets must be zero
   if (fixed_scratch && cudaMemsetAsync(workspace, 0, pl.ws.end_kept, st) != cudaSuccess) return LYNX_ERR_CUDA;
   if (!full) {
-    // Anchor attention: the integer tcgen05 kernels take up to 32 columns.  A call with more (33..64) is
+    // Anchor attention: the integer tcgen05 kernels take up to 32 columns, 16 as a pipeline of stages, above in teams.  A call with more (33..64) is
     // run as slices of whole query positions, each a pass of its own over the planes, one after the
     // other on the stream (they share the workspace).
     const int per = nq * p.G <= 32 ? nq : (32 / p.G > 0 ? 32 / p.G : 1);
@@ -690,8 +691,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
       ps.q = p.q + (size_t)j0 * p.Hq * LYNX_D;
       ps.out = p.out + (size_t)j0 * p.Hq * LYNX_D;
       ps.ws_lse = p.ws_lse + (size_t)j0 * p.Hq;
-      const lynx_status rc = ps.ncols <= 4 ? launch_i8<false, 4>(ps, st) : ps.ncols <= 8 ? launch_i8<false, 8>(ps, st)
-                           : ps.ncols <= 16 ? launch_i8<false, 16>(ps, st) : launch_i8<false, 32>(ps, st);
+      const lynx_status rc = ps.ncols <= 4 ? launch_pipe<false, 4>(ps, st) : ps.ncols <= 8 ? launch_pipe<false, 8>(ps, st)
+                           : ps.ncols <= 16 ? launch_pipe<false, 16>(ps, st) : launch_i8<false, 32>(ps, st);
       if (rc != LYNX_OK) return rc;
     }
     return LYNX_OK;
@@ -711,8 +712,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     ps.out = p.out + (size_t)j0 * p.Hq * LYNX_D;
     ps.ws_lse = p.ws_lse + (size_t)j0 * p.Hq;
     if (p.draft) { ps.draft = p.draft + (size_t)j0 * p.Hq * LYNX_D; ps.dev = p.dev + j0; }
-    const lynx_status rc = ps.ncols <= 4 ? launch_i8<true, 4>(ps, st) : ps.ncols <= 8 ? launch_i8<true, 8>(ps, st)
-                         : ps.ncols <= 16 ? launch_i8<true, 16>(ps, st) : ps.ncols <= 32 ? launch_f16<32>(ps, st)
+    const lynx_status rc = ps.ncols <= 4 ? launch_pipe<true, 4>(ps, st) : ps.ncols <= 8 ? launch_pipe<true, 8>(ps, st)
+                         : ps.ncols <= 16 ? launch_pipe<true, 16>(ps, st) : ps.ncols <= 32 ? launch_f16<32>(ps, st)
                          : launch_f16<64>(ps, st);
     if (rc != LYNX_OK) return rc;
   }

@@ -26,7 +26,7 @@
 //   warps 0-7    two softmax warpgroups of 32 columns each: scores -> weights -> P tile
 //   warps 8-11   K codes into tensor memory, and a piece's queries into the Q tile
 //   warps 12-15  V codes into the V tile
-//   warps 16-19  producers (tensor-map copies of 16-token sub-blocks): two warps for the K ring, two for the V ring
+//   warps 16-19  producers (tensor-map copies of 16-token sub-blocks): two warps for the K ring, one for the V ring
 //   warp 20      issues every tcgen05.mma
 //   warps 21, 22 the per-token scalars of the scores and weights at 32 columns (the rest completes the warpgroup, for the
 //                register split)
@@ -50,6 +50,7 @@
 template <int NC>
 struct F16Cfg {
   static_assert(NC == 32 || NC == 64, "padded column counts");
+  static constexpr bool kFull = true, kMetaRing = false;
   static constexpr bool kSplit = NC == 64;          // both groups score every unit (else they alternate)
   static constexpr int kST = 128, kCG = 32, kNG = kCG / 8;
   static constexpr int kPartCols = NC;
@@ -132,16 +133,14 @@ __device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint3
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
 
-// K codes of a token (thread r of 128 = TMEM lane r) into 64 columns of tensor memory.  The raw planes arrive with the
-// copy engine's 64-byte swizzle (see i8_expand_k_tmem).
+// K codes of a token (thread r of 128 = TMEM lane r) into 64 columns of tensor memory.
 __device__ __forceinline__ void f16_expand_k(uint32_t raw, int r, uint32_t tm_k) {
-  const uint32_t s = ((uint32_t)r >> 1) & 3u, row = raw + (uint32_t)r * 64u;
   // (a rolled loop: five roles share an instruction cache of some 12 KB per scheduler.  No loads ahead: these warps have time to
   // wait for shared memory, and moving the next chunk into place costs eight instructions a step)
 #pragma unroll 1
   for (int h = 0; h < 4; ++h) {
-    const uint32_t off = ((uint32_t)h ^ s) << 4;
-    const uint4 xa = lds128(row + off), xr = lds128(row + 8192u + off);
+    const uint32_t row = raw + k_chunk((uint32_t)r, (uint32_t)h);
+    const uint4 xa = lds128(row), xr = lds128(row + 8192u);
     uint32_t regs[16];
     f16_codes(xa.x, xr.x, regs);
     f16_codes(xa.y, xr.y, regs + 4);
@@ -172,19 +171,20 @@ __device__ __forceinline__ void f16_expand_v(uint32_t raw, uint32_t tile, int i)
   }
 }
 
-// A producer warp: derives the CTA's range like the others (warp 0 publishes it, the pieces, and the results of empty
-// sequences) and copies its half of the sub-blocks of one tensor: warps 0, 1 the K planes, warps 2, 3 the V planes, eight
-// copies per unit (4 sub-blocks x Anchor / Residual) in one instruction.
+// A producer warp: derives the CTA's range like the others (warp 0 publishes it, the pieces, and the results of empty sequences).
+// Warps 0, 1 copy one half of the K sub-blocks each, warp 2 the V sub-blocks, warp 3 the metadata of both (where kMetaRing).  full0,
+// empty0, stages: of the warp's own ring.
+// What bounds a producer is the latency of its instructions in a row: some 55 cycles per copy, 300 per unit.  Hence gathers of four
+// sub-blocks per copy for V and the metadata (the 128-byte swizzle of K does not go with them), and always all eight sub-blocks of a
+// unit, whether or not the sequence has them.
 template <class C>
-__device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange& rng, const SeqLens& sl, int pw, int lane, uint32_t sbase, uint32_t full0,
-                                             uint32_t empty0, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
-                                             volatile int* abort_word, const I8Maps* maps) {
+__device__ __forceinline__ void plane_producer(const AttnParams& p, const SkRange& rng, const SeqLens& sl, int pw, int lane, uint32_t sbase, uint32_t full0,
+                                               uint32_t empty0, int stages, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
+                                               volatile int* abort_word, const I8Maps* maps, int bar_done) {
   constexpr int ST = C::kST;
-  const int tensor = pw >> 1, nstage = tensor ? C::kRingV : C::kRingK;
-  const int sub0 = 4 * (pw & 1);
-  const uint32_t dst0 = sbase + (tensor ? C::kOffRV : C::kOffRK) + (uint32_t)(sub0 * 1024);
-  const CUtensorMap *map_a = &maps->m[tensor], *map_r = &maps->m[2 + tensor];
-  uint32_t* my_blk = blk_s + pw * 4 * kI8PieceUnits;
+  const int lg = pw < 2 ? 2 : 3;                 // log2 of the sub-blocks of a unit that are this warp's
+  const int sub0 = pw == 1 ? 4 : 0;
+  uint32_t* my_blk = blk_s + (pw < 2 ? 4 * pw : 8 * (pw - 1)) * kI8PieceUnits;
   int b = rng.b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
   int hkv = (int)sk_div(rng.off_lo, U), u = (int)(rng.off_lo - (long long)hkv * U);
   const int n_units = (int)(rng.hi - rng.lo);
@@ -207,13 +207,13 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
         mbar_arrive(qfull0 + qi * 8);
       }
       __syncwarp();
-      if (u == 0 && lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
+      if (C::kFull && u == 0 && lane < kMaxQ) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
     }
     for (int c0 = 0; c0 < n; c0 += kI8PieceUnits) {
       const int cn = min(kI8PieceUnits, n - c0);
-      for (int i = lane; i < 4 * cn; i += 32) {
-        const int t0 = (u + c0 + (i >> 2)) * ST + (sub0 + (i & 3)) * 16;
-        uint32_t row = 0xFFFFFFFFu;  // sub-block beyond the end of the sequence: nothing to copy
+      for (int i = lane; i < cn << lg; i += 32) {
+        const int t0 = (u + c0 + (i >> lg)) * ST + (sub0 + (i & ((1 << lg) - 1))) * 16;
+        uint32_t row = 0;  // sub-block beyond the end of the sequence: any that exists, its levels meet weights of zero
         if (t0 < len) {
           const int bi = block_of(p, t0);
           int blk = ld_dep(p.block_table + (size_t)b * p.max_blocks + bi);
@@ -223,33 +223,47 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
           }
           row = (uint32_t)(((size_t)blk * p.Hkv + hkv) * p.bt + (t0 - bi * p.bt));
         }
-        my_blk[i] = row;
+        my_blk[i] = map_row(row, pw < 2);
       }
       __syncwarp();
       for (int k = 0; k < cn; ++k) {
         mbar_wait_in(empty0 + slot * 8, phase, abort_word);
-        const uint4 rw = *reinterpret_cast<const uint4*>(my_blk + 4 * k);
-        // (one elected lane: with a copy per lane the compiler walks through the lanes, operands to the uniform
-        // datapath and back for each; only the sub-blocks at the end of a sequence can be absent)
+        const uint4* rows = reinterpret_cast<const uint4*>(my_blk) + (k << (lg - 2));
+        // (one elected lane: with a copy per lane the compiler walks through the lanes, operands to the uniform datapath and back)
         if (tc_elect()) {
-          const uint32_t bar = full0 + slot * 8, dst = dst0 + (uint32_t)slot * C::kStageBytes;
-          const uint32_t rows[4] = {rw.x, rw.y, rw.z, rw.w};
-          uint32_t bytes = 0;
+          const uint32_t bar = full0 + slot * 8;
+          const uint4 r0 = rows[0];
+          if (pw < 2) {
+            const uint32_t dst = sbase + C::kOffRK + (uint32_t)(slot * C::kStageBytes + sub0 * 1024), r[4] = {r0.x, r0.y, r0.z, r0.w};
+            mbar_expect_tx(bar, C::kFull ? 8192u : 4096u);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) bytes += rows[i] != 0xFFFFFFFFu ? 2048u : 0u;
-          if (bytes) mbar_expect_tx(bar, bytes);
-          else mbar_arrive(bar);
-#pragma unroll 1
-          for (int i = 0; i < 4; ++i) {   // (rolled, for the instruction caches: 256 -> 251 us at 64 columns)
-            const uint32_t row = my_blk[4 * k + i];
-            if (row != 0xFFFFFFFFu) {
-              tma_rows16(dst + i * 1024, map_a, (int)row, bar);
-              tma_rows16(dst + 8192 + i * 1024, map_r, (int)row, bar);
+            for (int i = 0; i < 4; ++i) {
+              tma_box(dst + i * 1024, &maps->m[0], r[i], bar);
+              if (C::kFull) tma_box(dst + 8192 + i * 1024, &maps->m[2], r[i], bar);
+            }
+          } else {
+            const uint4 r1 = rows[1];
+            if (pw == 2) {
+              const uint32_t dst = sbase + C::kOffRV + (uint32_t)(slot * C::kStageBytes);
+              mbar_expect_tx(bar, C::kFull ? 16384u : 8192u);
+              tma_gather4(dst, &maps->m[1], r0, bar);
+              tma_gather4(dst + 4096, &maps->m[1], r1, bar);
+              if (C::kFull) {
+                tma_gather4(dst + 8192, &maps->m[3], r0, bar);
+                tma_gather4(dst + 12288, &maps->m[3], r1, bar);
+              }
+            } else if constexpr (C::kMetaRing) {
+              const uint32_t dst = sbase + C::kOffMeta + (uint32_t)(slot * 2048);
+              mbar_expect_tx(bar, 2048u);
+              tma_gather4(dst, &maps->meta[0], r0, bar);
+              tma_gather4(dst + 512, &maps->meta[0], r1, bar);
+              tma_gather4(dst + 1024, &maps->meta[1], r0, bar);
+              tma_gather4(dst + 1536, &maps->meta[1], r1, bar);
             }
           }
         }
         __syncwarp();
-        if (++slot == nstage) { slot = 0; phase ^= 1; }
+        if (++slot == stages) { slot = 0; phase ^= 1; }
       }
       __syncwarp();  // my_blk is rewritten by the next round
     }
@@ -270,7 +284,7 @@ __device__ __forceinline__ void f16_producer(const AttnParams& p, const SkRange&
     }
   }
   __syncwarp();
-  bar_arrive(5, C::kDoneThreads);
+  bar_arrive(bar_done, C::kDoneThreads);
 }
 
 // The per-token scalars of a unit, for N tokens (32 apart) of a thread: scale and offset of the scores, log2 of the value
@@ -359,7 +373,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   if (warp == 16 && lane < 4) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.m[lane])) : "memory");
   if (tid == 0) {
     for (int i = 0; i < C::kRingK; ++i) { mbar_init(kfull + i * 8, 2); mbar_init(kempty + i * 8, 4); }
-    for (int i = 0; i < C::kRingV; ++i) { mbar_init(vfull + i * 8, 2); mbar_init(vempty + i * 8, 4); }
+    for (int i = 0; i < C::kRingV; ++i) { mbar_init(vfull + i * 8, 1); mbar_init(vempty + i * 8, 4); }
     for (int i = 0; i < 2; ++i) {
       mbar_init(qfull + i * 8, 1);
       mbar_init(qempty + i * 8, C::kMetaK ? 12 : 14);
@@ -854,10 +868,10 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   if (warp < 20) {
     reg_dec<C::kRegProd>();
     const int pw = warp - 16;
-    if (n_units == 0) bar_arrive(5, C::kDoneThreads);
+    if (n_units == 0 || pw == 3) bar_arrive(5, C::kDoneThreads);
     else
-      f16_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, qfull, qempty,
-                      reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps);
+      plane_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, pw < 2 ? C::kRingK : C::kRingV, qfull,
+                        qempty, reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps, 5);
     if (pw == 0) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
     return;
   }

@@ -1,7 +1,8 @@
-// Anchor and merge-verify attention on the integer path of the fifth-generation tensor cores
-// (tcgen05.mma kind::i8, accumulators in tensor memory).  Included by attention.cu inside its
-// namespace: shares AttnParams and the stream-K cut of the work with the other
-// kernels.
+// Attention on the integer path of the fifth-generation tensor cores (tcgen05.mma kind::i8, accumulators in tensor memory), a team
+// of warps per unit.  Included by attention.cu inside its namespace: shares AttnParams and the stream-K cut of the work with the
+// other kernels.  Takes anchor calls with 17..32 columns, whose accumulators leave no tensor memory for the buffers of
+// attention_pipe.cuh; that kernel shares the algebra and the expansions here and takes up to 16 columns.  (What is measured below at
+// fewer columns was measured before it.)
 //
 // With one (scale, zero) per token row the two contractions of Section 2's attention run on the
 // integer levels themselves (see attention.cu).  Here both are exact integer tensor-core
@@ -45,38 +46,63 @@
 // holds dim 32 j + 8 w + 2 i + parity (what the nibble expansion yields with two logic
 // operations per word); the query planes use the same order and O is un-permuted at write-out.
 
-// Tensor maps of the K planes ([rows][64 bytes] u8, box = one 16-token sub-block, 64-byte swizzle): the
-// copy engine stores 16-byte chunk c of row r at position c ^ ((r >> 1) & 3), which is the order in which
-// the threads of a quarter-warp can read their rows (64 bytes apart) without bank conflicts; read back at
-// position i ^ ((r >> 1) & 3), chunk i arrives in place with no reordering in registers.
-// The V planes go through maps of the same shape without swizzle, so that one instruction of a producer warp
-// issues all its copies of a unit (the map is a per-lane operand).
+// Tensor maps of the planes; a box is one 16-token sub-block, 1 KiB contiguous.  K planes as [rows / 2][128 bytes] with the 128-byte
+// swizzle: the copy engine stores 16-byte chunk j of a pair of tokens r >> 1 at position j ^ ((r >> 1) & 7), so that the eight
+// threads of a quarter-warp that read chunk i of their own rows (64 bytes apart) meet in no bank (see k_chunk).  V planes as
+// [rows / 16][1024 bytes] without swizzle, which gathers of four sub-blocks take, too.  (148 CTAs, nothing but copies, TB/s: rows of
+// 64 bytes 6.50 by four issuing warps, of 128 and more 6.75; one warp 3.06, two 6.0; gathers by one warp 4.3, by two 6.7.)
 struct alignas(64) I8Maps {
   CUtensorMap m[4];   // K Anchor, V Anchor, K Residual, V Residual (the order of the stage's arrays)
+  CUtensorMap meta[2];   // (scale, zero) pairs of K, V: [rows / 16][32 floats], for gathers of four sub-blocks
 };
-inline bool i8_plane_map(CUtensorMap* m, const uint8_t* base, uint64_t rows, bool swizzle) {
-  using Fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                          const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                          CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static Fn fn = [] {
+using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                 const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+inline EncodeTiled encode_tiled() {
+  static EncodeTiled fn = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess)
       f = nullptr;
-    return reinterpret_cast<Fn>(f);
+    return reinterpret_cast<EncodeTiled>(f);
   }();
-  if (!fn || !base || rows == 0) return false;
-  const cuuint64_t dims[2] = {64, rows};
-  const cuuint64_t strides[1] = {64};
-  const cuuint32_t box[2] = {64, 16}, es[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return fn;
 }
-// one 16-row box of a plane (rows row .. row + 15, all 64 bytes) into shared memory
-__device__ __forceinline__ void tma_rows16(uint32_t dst, const CUtensorMap* map, int row, uint32_t bar) {
+inline bool i8_plane_map(CUtensorMap* m, const uint8_t* base, uint64_t rows, bool k_plane) {
+  const EncodeTiled fn = encode_tiled();
+  if (!fn || !base || rows == 0) return false;
+  const cuuint64_t dims[2] = {k_plane ? 128u : 256u, k_plane ? rows / 2 : rows / 16};   // (bytes, 32-bit words; rows is a multiple of 16)
+  const cuuint64_t strides[1] = {k_plane ? 128u : 1024u};
+  const cuuint32_t box[2] = {k_plane ? 128u : 256u, k_plane ? 8u : 1u}, es[2] = {1, 1};
+  return fn(m, k_plane ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint8_t*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, k_plane ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+inline bool meta_map(CUtensorMap* m, const float* base, uint64_t rows) {
+  const EncodeTiled fn = encode_tiled();
+  if (!fn || !base || rows == 0) return false;
+  const cuuint64_t dims[2] = {32, rows / 16};
+  const cuuint64_t strides[1] = {128};
+  const cuuint32_t box[2] = {32, 1}, es[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// Four rows of a map (of V planes, of metadata) one behind the other into shared memory.
+__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, uint4 r, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(r.x), "r"(r.y), "r"(r.z), "r"(r.w), "r"(bar)
+      : "memory");
+}
+// The row of a plane's map at which the sub-block of plane row `row` starts, K or V (and the metadata's).
+__device__ __forceinline__ uint32_t map_row(uint32_t row, bool k_plane) { return row >> (k_plane ? 1 : 4); }
+// Offset of 16-byte chunk i of token r's 64 bytes in a raw K stage.
+__device__ __forceinline__ uint32_t k_chunk(uint32_t r, uint32_t i) {
+  return (r >> 1) * 128u + ((((r & 1u) * 4u + i) ^ ((r >> 1) & 7u)) << 4);
+}
+// the box of a plane that starts at row `row` of its map into shared memory
+__device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap* map, uint32_t row, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(bar)
@@ -282,8 +308,9 @@ __device__ __forceinline__ float ex2_full(float x) {   // no flush of small resu
 }
 
 // Expand the nibble planes of one tensor of a 128-token raw stage into its u8 level tile.  A warp
-// takes 8 token rows per step (512 contiguous raw bytes): lane = (row & 7) * 4 + 16-byte chunk.
-template <bool FULL>
+// takes 8 token rows per step (512 contiguous raw bytes): lane = (row & 7) * 4 + 16-byte chunk.  ODD16: the odd elements of an
+// Anchor plane as they lie in their bytes, 16 times the level (the caller takes it off the sums).
+template <bool FULL, bool ODD16 = false>
 __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32_t tile, int w4, int lane) {
   const int row8 = lane >> 2, j = lane & 3;
   uint4 xa[4], xr[4];
@@ -305,7 +332,7 @@ __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32
         merge_codes(a[k], r[k], ev[k], od[k]);
       } else {
         ev[k] = a[k] & 0x0F0F0F0Fu;
-        od[k] = (a[k] >> 4) & 0x0F0F0F0Fu;
+        od[k] = ODD16 ? a[k] & 0xF0F0F0F0u : (a[k] >> 4) & 0x0F0F0F0Fu;
       }
     }
     const uint32_t base = tile + (uint32_t)row * 128u;
@@ -319,22 +346,18 @@ __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32
 
 // K levels of a 128-token raw stage into tensor memory: thread r owns token r (TMEM lane r) and writes
 // its 128 level bytes to 32 columns, byte 4 col + b in the order of the operand tiles (see the header).
-// The four 16-byte chunks of the row are read in a lane-dependent order (chunk i ^ s, s = (r >> 1) & 3:
-// rows are 64 bytes apart, so a fixed order would put a quarter-warp on two bank groups) and put back
-// in order with two levels of selects.
 template <bool FULL, bool RAW>
 __device__ __forceinline__ void i8_expand_k_tmem(uint32_t raw_a, uint32_t raw_r, int r, uint32_t tm_k) {
-  const uint32_t s = ((uint32_t)r >> 1) & 3u;
   uint4 xa[4], xr[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const uint32_t off = (uint32_t)r * 64u + (((uint32_t)i ^ s) << 4);
+    const uint32_t off = k_chunk((uint32_t)r, (uint32_t)i);
     xa[i] = lds128(raw_a + off);
     if (FULL) xr[i] = lds128(raw_r + off);
   }
   uint32_t regs[32];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {   // (position j ^ s holds chunk j: the copy engine's 64-byte swizzle)
+  for (int j = 0; j < 4; ++j) {
     const uint32_t a[4] = {xa[j].x, xa[j].y, xa[j].z, xa[j].w};
     uint32_t rr[4] = {0, 0, 0, 0};
     if (FULL) { rr[0] = xr[j].x; rr[1] = xr[j].y; rr[2] = xr[j].z; rr[3] = xr[j].w; }
@@ -444,7 +467,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         }
         __syncwarp();
         if (lane < RP && row != 0xFFFFFFFFu)
-          tma_rows16(ring_u32 + slot * C::kStageBytes + my_dst, &maps->m[arr], (int)row, bar);
+          tma_box(ring_u32 + slot * C::kStageBytes + my_dst, &maps->m[arr], map_row(row, (arr & 1) == 0), bar);
       }
       __syncwarp();  // my_blk is rewritten by the next round
     }
@@ -1317,6 +1340,7 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
     maps.m[2] = maps.m[0];
     maps.m[3] = maps.m[1];
   }
+  if (!meta_map(&maps.meta[0], p.km, plane_rows) || !meta_map(&maps.meta[1], p.vm, plane_rows)) return LYNX_ERR_CUDA;
   if (cudaLaunchKernelEx(&cfg, KERN, p, maps) != cudaSuccess) return LYNX_ERR_CUDA;
   return launch_status();
 }

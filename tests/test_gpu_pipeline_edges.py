@@ -1,0 +1,93 @@
+"""Anchor and verification attention with up to 16 query columns where the pipeline of their kernel can go wrong: pieces of fewer
+units than it has softmax groups, of as many as it has buffers and one more, CTAs with many pieces, more units than the rings hold
+several times over, and references that are raised in every stage of it.  Against a 64-bit evaluation with torch on the
+dequantised planes.
+
+Tolerance: a weight 2^(x - ref) formed in binary32 from four roundings of a score below 128 (log2 units) is off by 2.1e-5 of itself,
+its rounding to an integer by 2^-29 of the largest, independently from token to token; the integer sums are exact, and putting
+them together adds some 2^-22.  An output row, a weighted mean of values, is then off by less than 3e-5 of its 2-norm; half as
+much again is allowed.  A log-sum-exp carries the four roundings and that of its own sum: 7e-5, likewise."""
+import math
+
+import pytest
+import torch
+
+import paper_2607_01831_b200 as lynx
+
+pytestmark = pytest.mark.gpu
+REL, LSE = 4.5e-5, 1.05e-4
+
+
+def _values(p, full):
+    nib = lambda t: torch.stack((t & 15, t >> 4), -1).flatten(-2).double()  # noqa: E731
+    return p.meta[..., 1:2].double() + p.meta[..., 0:1].double() * (nib(p.anchor) * 16 + (nib(p.residual) if full else 8))
+
+
+def _run(lens, Hkv, G, n_q, ramp, bt=16):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(sum(lens) + G * n_q)
+    need = [(n + bt - 1) // bt for n in lens]
+    nb, B = sum(need), len(lens)
+    table = torch.zeros(B, max(need), dtype=torch.int32)
+    perm, pos = torch.randperm(nb, generator=torch.Generator().manual_seed(nb)).to(torch.int32), 0
+    for b, n in enumerate(need):
+        table[b, :n] = perm[pos:pos + n]
+        pos += n
+    k, v = (torch.randn(nb, Hkv, bt, 128, generator=g, device="cuda") for _ in range(2))
+    q = torch.randn(B, n_q, Hkv * G, 128, generator=g, device="cuda")
+    if ramp:   # scores that climb along the sequence: the largest weight so far is exceeded again and again
+        q = 1.0 + 0.05 * q
+        climb = torch.zeros(nb, device="cuda")
+        for b, n in enumerate(need):
+            climb[table[b, :n].long().cuda()] = torch.arange(n, device="cuda", dtype=torch.float32) / n
+        k = 0.3 * k + 7.0 * climb.view(-1, 1, 1, 1)
+    q = q.to(torch.bfloat16)
+    K, V = (lynx.split_quantize(x.to(torch.bfloat16)) for x in (k, v))
+    geo = lynx.Geometry(Hkv * G, Hkv, bt, nb, table.shape[1])
+    ws = lynx.make_workspace(geo, B, n_q, "cuda")
+    tab, ln = table.cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda")
+    for full in (False, True):
+        call = lynx.merge_verify_attention if full else lynx.anchor_attention
+        outs = []
+        for _ in range(2):   # (a second time on the workspace as the first left it)
+            o = call(geo, q, K, V, tab, ln, ws, causal=True)
+            outs.append(o[0] if full else o)
+        lynx.check(ws)
+        assert torch.equal(outs[0], outs[1])
+        lse = lynx.workspace_lse(geo, B, n_q, ws)
+        kd, vd = _values(K, full), _values(V, full)
+        for b in range(B):
+            n = lens[b]
+            kk, vv = (x[tab[b, :need[b]].long()].permute(1, 0, 2, 3).reshape(Hkv, -1, 128)[:, :n] for x in (kd, vd))
+            s = q[b].double().permute(1, 0, 2).reshape(Hkv, G * n_q, 128) @ kk.transpose(1, 2) / math.sqrt(128)
+            last = n - n_q + torch.arange(n_q, device="cuda").repeat(G)
+            s.masked_fill_(torch.arange(n, device="cuda") > last[:, None], -math.inf)
+            ref = (torch.softmax(s, 2).nan_to_num(0.0) @ vv).reshape(Hkv * G, n_q, 128).permute(1, 0, 2)
+            got = outs[0][b].double()
+            assert torch.isfinite(got).all()
+            assert (got - ref).norm() <= REL * ref.norm(), (full, b, ((got - ref).norm() / ref.norm()).item())
+            want = torch.logsumexp(s, 2).reshape(Hkv * G, n_q).permute(1, 0)
+            fin = torch.isfinite(want)
+            assert torch.equal(fin, torch.isfinite(lse[b])) and (lse[b].double() - want)[fin].abs().max() <= LSE
+
+
+@pytest.mark.parametrize("G,n_q", [(3, 1), (4, 1), (7, 1), (4, 2), (3, 3), (4, 4), (16, 1)])   # 3, 4, 7, 8, 9, 16, 16 columns
+@pytest.mark.parametrize("lens", [
+    [1, 16, 127, 128, 129],                                   # pieces of one unit and of two
+    [128 * n for n in range(1, 18)] + [128 * 17 + 1],         # around every depth of the buffers, CTAs with several pieces
+    [60 + 70 * (i % 5) for i in range(400)],                  # many pieces per CTA
+])
+def test_pieces(G, n_q, lens):
+    _run(lens, 1, G, n_q, ramp=False)
+
+
+@pytest.mark.parametrize("G,n_q", [(4, 1), (8, 1), (4, 4)])
+@pytest.mark.parametrize("ramp", [False, True])
+def test_rings_that_come_round(G, n_q, ramp):
+    _run([148 * 128 * 19 + 77], 1, G, n_q, ramp)              # 19 and 20 units per CTA
+
+
+@pytest.mark.parametrize("G,n_q", [(4, 1), (8, 1), (4, 4)])
+@pytest.mark.parametrize("lens", [[700, 129], [2600], [128 * 9] * 40])
+def test_references_that_are_raised(G, n_q, lens):
+    _run(lens, 2, G, n_q, ramp=True)

@@ -13,7 +13,7 @@
 // so the two contractions run on the integer levels and the scalars are applied per token
 // outside.  Anchor attention (any column count) and verification with up to 16 columns per launch run both contractions as exact integer products on
 // tcgen05.mma kind::i8 (attention_pipe.cuh up to 16 columns, attention_i8.cuh above); verification with 17..64 columns per launch
-// runs them on tcgen05.mma kind::f16 with two-term FP16 weights (attention_f16.cuh).
+// runs its scores on tcgen05.mma kind::f16, its values likewise with two-term FP16 weights or as integers (attention_f16.cuh).
 //
 // Common shape.  Persistent grid, one CTA per SM, flash-decoding split-K in stream-K form: the
 // (sequence, KV head, stage-unit) list is cut into equal contiguous ranges, one per CTA.
@@ -713,8 +713,8 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
     ps.ws_lse = p.ws_lse + (size_t)j0 * p.Hq;
     if (p.draft) { ps.draft = p.draft + (size_t)j0 * p.Hq * LYNX_D; ps.dev = p.dev + j0; }
     const lynx_status rc = ps.ncols <= 4 ? launch_pipe<true, 4>(ps, st) : ps.ncols <= 8 ? launch_pipe<true, 8>(ps, st)
-                         : ps.ncols <= 16 ? launch_pipe<true, 16>(ps, st) : ps.ncols <= 32 ? launch_f16<32>(ps, st)
-                         : launch_f16<64>(ps, st);
+                         : ps.ncols <= 16 ? launch_pipe<true, 16>(ps, st) : ps.ncols > 32 ? launch_f16<64, false>(ps, st)
+                         : f16_int_pv(ps) ? launch_f16<32, true>(ps, st) : launch_f16<32, false>(ps, st);
     if (rc != LYNX_OK) return rc;
   }
   if (p.draft && pl.per < nq) {

@@ -1,5 +1,5 @@
-// Merge-verify attention for 17..64 columns on the fifth-generation tensor cores, FP16 operands with FP32
-// accumulators.  Included by attention.cu inside its namespace.
+// Merge-verify attention for 17..64 columns on the fifth-generation tensor cores: scores as FP16 products, values as FP16 or integer
+// ones.  Included by attention.cu inside its namespace.
 //
 // A unit is 128 tokens.  Both contractions take the 8-bit codes centred, c - 128, which FP16 represents exactly:
 //   S^T[128 tokens x NC]      = (codes(K) - 128) . Q^T       A = K in tensor memory (a thread owns a token = a lane),
@@ -8,19 +8,22 @@
 //                                                                in two parts side by side in N (f16_split_q)
 //   O^T[128 dims x 2 x 32]   += (codes(V) - 128)^T . [h | r] A = V tile (MN-major), B = the weights as two FP16 terms,
 //                                                                w = h + r (22 bits), side by side in N
+// or, up to 32 columns where a CTA has many units (f16_int_pv), with kind::i8:
+//   O^T[128 dims x 4 x 32]   += (codes(V) - 128)^T . Wd      A = V tile (s8), B = the four bytes of weights scaled to u32
 // Centring costs one packed addition per two codes and is what keeps FP32 sufficient: the zero points, 128 steps below
 // the centre of a row, would otherwise be added and taken off again around results a hundred times smaller.
 // x = s log2(e) + log2(scale_v), w = 2^(x - ref[c]); ref[c] is set so that the largest weight of a column's first unit is
-// 2^8 and raised (accumulators drained, rare) before a weight would leave FP16.  The tensor core's accumulation truncates
-// (0.46 ulp of the running sum per product).  Scores: the high part of a query is a multiple of 2^-10 of the largest entry,
-// so that its products with the codes sum up exactly, and the truncation acts on the low part, a thousand times smaller.
-// Values: every kDrainUnits units the accumulators move into an FP32 copy.
+// 2^8 (integers: 1, scaled to 2^25) and raised (accumulators drained or rescaled, rare) before a weight would leave FP16 or u32.  The
+// tensor core's FP32 accumulation truncates (0.46 ulp of the running sum per product).  Scores: the high part of a query is a
+// multiple of 2^-10 of the largest entry, so that its products with the codes sum up exactly, and the truncation acts on the low
+// part, a thousand times smaller.  Values: every kDrainUnits units the accumulators move into an FP32 copy; the integer sums are exact.
 //
 // Error against 64 bits (2-norm; 34 cases of 17..32 and 26 of 33..64 columns, 64 to 131072 tokens, log-normal, heavy-tailed
 // and outlier values).  17..32 columns, against the exact integer products of attention_i8.cuh in two passes: 0.29 times on
 // the geometric mean, at most 0.97 times, largest 1.4e-6 (7.5e-6); log-sum-exps 0.54 times, largest 9e-6 (4.4e-5).  With
 // whole queries and a drain per 8 units it was 0.42 times on the mean but up to 2.0 times on heavy-tailed keys and long
-// contexts.  33..64 columns, against the uncentred kernel before it: 0.09 times, largest 1.2e-5 (3.4e-4).
+// contexts.  33..64 columns, against the uncentred kernel before it: 0.09 times, largest 1.2e-5 (3.4e-4).  Values on integers against
+// values in FP16, 32 columns, means of six draws: 131072 tokens log-normal 3.6e-7 (6.6e-7), 2 of 30000 heavy-tailed 7.1e-7 (8.6e-7).
 //
 // Warp roles, one CTA per SM; every hand-off is an mbarrier with a bounded wait, nothing waits on another CTA:
 //   warps 0-7    two softmax warpgroups of 32 columns each: scores -> weights -> P tile
@@ -46,27 +49,37 @@
 // half of a unit's tokens each and 80 registers: 64 columns +15 %, 32 +4 %.  One layer of 131072 tokens: 174 us as two passes
 // of the 16-column integer kernel -> 83 us (32 columns); two sequences, 64 columns: 293 us by the previous kernel (M = columns, codes
 // not centred) -> 207 us; the kernel alone, back to back, before the power cap sets in (the calls among other passes: 91 and 227 us).
+// Since then both barriers of a stage are probed at once (64 columns 200 -> 197 us), and values go through integer products at 32
+// columns: half of the work on V codes, no drains, two instructions a weight instead of five (80 -> 72 us).  At 64 columns the
+// conversions to u32, which share their unit with the exponentials, cost what that saves (200 -> 215 us).  Tried and left: K and V codes
+// by the same warpgroup, units in turn (72 -> 73), in that order or K a unit ahead (75), a look-ahead by more than one unit (75).
 
-template <int NC>
+template <int NC, bool INT>
 struct F16Cfg {
-  static_assert(NC == 32 || NC == 64, "padded column counts");
+  static_assert(NC == 32 || (NC == 64 && !INT), "padded column counts");
   static constexpr bool kFull = true, kMetaRing = false;
   static constexpr bool kSplit = NC == 64;          // both groups score every unit (else they alternate)
   static constexpr int kST = 128, kCG = 32, kNG = kCG / 8;
   static constexpr int kPartCols = NC;
   static constexpr int kStageBytes = kST * 128;     // Anchor and Residual of one tensor: [2][128 tokens][64 B]
-  static constexpr int kVTile = 32768;              // [2 dim blocks][128 tokens][128 B]
-  static constexpr int kPTile = 16384;              // [128 tokens][32 h | 32 r]
+  static constexpr bool kIntPV = INT;               // P.V on integers: codes less 128 as s8, weights as u32
+  static constexpr int kVTile = kIntPV ? 16384 : 32768;   // [128 tokens][128 B], or [2 dim blocks][128 tokens][128 B]
+  static constexpr int kPTile = 16384;              // [128 tokens][32 columns x 4 bytes], or [128 tokens][32 h | 32 r]
+  static constexpr int kNPV = kIntPV ? 128 : 64;    // N of a group's P.V
   static constexpr int kQP = NC == 32 ? 2 : 1;      // parts of the queries (see f16_split_q)
   static constexpr int kSCols = kQP * NC;           // columns of Q.K^T: the queries' high parts, then the low ones
   static constexpr int kQTile = kSCols * 256;       // [2 dim blocks][kSCols][128 B]
   static constexpr int kRingK = 3, kRingV = 3;
-  static constexpr int kOffV = 0, kOffP = 2 * kVTile, kOffQ = kOffP + 2 * kPTile, kOffRK = kOffQ + kQTile,
+  static constexpr int kOFBytes = kIntPV ? 2 * kCG * 512 : 0;   // FP32 copy of O where tensor memory has no room for it: [group][column][128]
+  static constexpr int kOffV = 0, kOffP = 2 * kVTile, kOffOF = kOffP + 2 * kPTile, kOffQ = kOffOF + kOFBytes, kOffRK = kOffQ + kQTile,
                        kOffRV = kOffRK + kRingK * kStageBytes, kOffScal = kOffRV + kRingV * kStageBytes;
   // floats: qs[2][NC], limits[2][NC], exponents[2] (+ 2); per group: ref[32], fac[32], red[4][64], lz[64]
   static constexpr int kGrpScal = 2 * 32 + 256 + 64;
   static constexpr int kOffGrp = kOffScal + (4 * NC + 4) * 4;
-  static constexpr int kOffTok = kOffGrp + 2 * kGrpScal * 4;        // per-token scalars, 4 slots: [4][128] float4, [4][128] float
+  // (Scalars stored as the packed pairs that the softmax takes, in two slots, spare it a tenth of its instructions and cost more in
+  // shared memory: 64 columns 197 -> 205 us.)
+  static constexpr int kSlots = 4;                                  // units whose per-token scalars are kept: [4][128] float4, [4][128] float
+  static constexpr int kOffTok = kOffGrp + 2 * kGrpScal * 4;
   static constexpr int kOffBlk = kOffTok + 4 * 128 * 20;        // [4 producer warps][4 sub-blocks][kI8PieceUnits]
   static constexpr int kOffItems = kOffBlk + 16 * kI8PieceUnits * 4;
   static constexpr int kOffBars = kOffItems + 2 * 32;
@@ -74,13 +87,16 @@ struct F16Cfg {
   static constexpr int kSmem = kOffMisc + 256 + 1024;               // + alignment slack
   static_assert(kSmem <= 227 * 1024, "shared memory");
   static_assert(kOffScal % 16 == 0 && kOffGrp % 16 == 0 && kOffBars % 8 == 0, "alignment");
-  static constexpr int kTmS = 0, kTmK = 2 * kSCols, kTmO = kTmK + 128, kTmOF = kTmO + 128;   // [2][kSCols], [2][64], [2][64], [2][32]
-  static_assert(kTmOF + 64 <= 512, "tensor memory");
+  static constexpr int kTmS = 0, kTmK = 2 * kSCols, kTmO = kTmK + 128, kTmOF = kTmO + 2 * kNPV;   // [2][kSCols], [2][64], [2][kNPV], [2][32]
+  static_assert(kTmOF + (kIntPV ? 0 : 64) <= 512, "tensor memory");
   static constexpr int kThreads = 768, kDoneThreads = 256 + 128 + 32;   // softmax warpgroups, producers, products
   // units between drains: each adds 8 truncating products to a sum.  32 columns, one layer of 131072 tokens: a drain per 8
   // units has a largest error of 3.4e-6, per 4 units 2.2e-6, per 2 units 1.4e-6, by when it is below the integer kernel's in
   // every case (4 % of the time between 8 and 2 when it was measured); 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
-  static constexpr int kDrainUnits = NC == 64 ? 16 : 2;
+  static constexpr int kDrainUnits = kIntPV ? 256 : NC == 64 ? 16 : 2;
+  // log2 of the largest weight of a column's first unit, and of a weight that raises the references.  On integers weights are formed
+  // relative to that and scaled by 2^25 afterwards (up to 2^31.5): an exponent of 25 would carry four times the rounding.
+  static constexpr float kTop = kIntPV ? 0.0f : 8.0f, kRaise = kIntPV ? 6.5f : 15.0f;
   // who computes the per-token scalars: with 64 columns the K warps have the time (261 -> 256 us), with 32 they are the
   // slower stage and two spare warps do it (96.1 us, 97.4 us in the K warps)
   static constexpr bool kMetaK = kSplit;
@@ -100,6 +116,14 @@ __device__ __forceinline__ bool wait_in(Probe probe, volatile int* abort_word) {
 __device__ __forceinline__ bool mbar_wait_in(uint32_t bar, uint32_t parity, volatile int* abort_word) {
   if (mbar_test(bar, parity)) return true;
   return wait_in([=] { return mbar_try_wait(bar, parity); }, abort_word);
+}
+
+// Two waits whose first probes are under way at the same time.
+__device__ __forceinline__ void mbar_wait2_in(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1, volatile int* abort_word) {
+  const bool a = mbar_test(bar0, parity0), b = mbar_test(bar1, parity1);
+  if (a && b) return;
+  mbar_wait_in(bar0, parity0, abort_word);
+  mbar_wait_in(bar1, parity1, abort_word);
 }
 
 // position -> element within a group of 8: {0,4,2,6,1,5,3,7} (what the nibble expansion yields), its own inverse
@@ -169,6 +193,31 @@ __device__ __forceinline__ void f16_expand_v(uint32_t raw, uint32_t tile, int i)
       sts128(dst ^ (uint32_t)(k * 16), o[0], o[1], o[2], o[3]);
     }
   }
+}
+
+// V codes of a unit, less 128, as bytes into the V tile by four warps: i8_expand with the top bit of every code flipped (and rolled:
+// see f16_expand_k).
+__device__ __forceinline__ void f16_expand_v8(uint32_t raw, uint32_t tile, int w4, int lane) {
+  const int row8 = lane >> 2, j = lane & 3;
+  uint32_t a = raw + (uint32_t)((w4 * 8 + row8) * 64 + j * 16), dst = tile + (uint32_t)(w4 * 8 + row8) * 128u;
+  const uint32_t c0 = (uint32_t)((2 * j) ^ row8) << 4, c1 = (uint32_t)((2 * j + 1) ^ row8) << 4;
+#pragma unroll 1
+  for (int s = 0; s < 4; ++s, a += 2048u, dst += 4096u) {
+    const uint4 xa = lds128(a), xr = lds128(a + 8192u);
+    const uint32_t wa[4] = {xa.x, xa.y, xa.z, xa.w}, wr[4] = {xr.x, xr.y, xr.z, xr.w};
+    uint32_t ev[4], od[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) merge_codes(wa[k] ^ 0x88888888u, wr[k], ev[k], od[k]);
+    sts128(dst + c0, ev[0], ev[1], ev[2], ev[3]);
+    sts128(dst + c1, od[0], od[1], od[2], od[3]);
+  }
+}
+// Column of a group whose weights' bytes are word k of 16-byte chunk c of a row of the P tile (stmatrix deals a thread's columns
+// 8 j + 2 i and 8 j + 2 i + 1 to chunks j and 4 + j).
+__host__ __device__ constexpr int f16_col(int c, int k) { return 8 * (c & 3) + 2 * k + (c >> 2); }
+// The sum of a column from its four byte planes.
+__device__ __forceinline__ float f16_planes(const uint32_t* a) {
+  return fmaf(fmaf(fmaf((float)(int)a[3], 256.0f, (float)(int)a[2]), 256.0f, (float)(int)a[1]), 256.0f, (float)(int)a[0]);
 }
 
 // A producer warp: derives the CTA's range like the others (warp 0 publishes it, the pieces, and the results of empty sequences).
@@ -334,8 +383,9 @@ struct F16Meta {
       if (C::kSplit && valid && !(vm[i].x < 16.0f)) atomicOr(p.ws_flags, kFlagRange);   // beyond the stated range of this width
       const float sve = fmaxf(vm[i].x, 9.094947e-13f);   // floor 2^-40
       const float ia = valid ? rcp_approx(sve) : 0.0f;
-      tok4[(gs & 3) * 128 + 32 * i] = make_float4(km[i].x * ca, fmaf(km[i].x, 128.0f, km[i].y) * p.sm_log2, lg2_approx(sve), ia);
-      tok1[(gs & 3) * 128 + 32 * i] = fmaf(sve, 128.0f, vm[i].y) * ia;
+      const int at = gs % C::kSlots * 128 + 32 * i;
+      tok4[at] = make_float4(km[i].x * ca, fmaf(km[i].x, 128.0f, km[i].y) * p.sm_log2, lg2_approx(sve), ia);
+      tok1[at] = fmaf(sve, 128.0f, vm[i].y) * ia;
     }
   }
   __device__ __forceinline__ void next(const AttnParams& p, int u) {
@@ -347,10 +397,10 @@ struct F16Meta {
   }
 };
 
-template <int NC>
-__global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const AttnParams p,
+template <int NC, bool INT>
+__global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(const AttnParams p,
                                                                            const __grid_constant__ I8Maps maps) {
-  using C = F16Cfg<NC>;
+  using C = F16Cfg<NC, INT>;
   constexpr bool SPLIT = C::kSplit;
   constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2, kDW = 8;
   extern __shared__ unsigned char smem_raw[];
@@ -417,17 +467,18 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     reg_inc<C::kRegSoft>();
     const int g = warp >> 2, w4 = warp & 3, r = tid & 127;
     const uint32_t lane_sel = (uint32_t)(w4 * 32) << 16;
-    const uint32_t tm_o = tmem0 + C::kTmO + g * 64 + lane_sel, tm_of = tmem0 + C::kTmOF + g * 32 + lane_sel;
+    const uint32_t tm_o = tmem0 + C::kTmO + g * C::kNPV + lane_sel, tm_of = tmem0 + C::kTmOF + g * 32 + lane_sel;
+    float* of_s = reinterpret_cast<float*>(smem + C::kOffOF) + g * CG * 128 + r;   // (kIntPV)
     // this thread's tokens of a unit: t0 + 8 k, k = 0..3; its columns 8 j + c2, + 1
     const int t0 = w4 * 32 + (lane >> 2), c2 = (lane & 3) * 2;
-    // row lane & 7 of block lane >> 3 of a warp's first eight tokens in the P tile (the remainders: 64 bytes on, swizzled)
+    // row lane & 7 of block lane >> 3 of a warp's first eight tokens in the P tile (the remainders or odd columns: 64 bytes on, swizzled)
     const uint32_t p_addr = sbase + C::kOffP + g * C::kPTile + (uint32_t)(w4 * 32 + (lane & 7)) * 128u +
                             (uint32_t)((lane >> 3) ^ (lane & 7)) * 16u;
     float* grp = reinterpret_cast<float*>(smem + C::kOffGrp) + g * C::kGrpScal;
     float *ref_s = grp, *fac_s = grp + 32, *red_s = grp + 64, *lz_s = grp + 320;
     const int bar_g = 1 + g;
     const int col0 = SPLIT ? g * CG : 0;            // first column of this group
-    const int dim_out = (r & ~7) + f16_perm(r & 7);
+    const int dim_out = C::kIntPV ? 32 * (r >> 5) + 8 * ((r >> 2) & 3) + 2 * (r & 3) + ((r >> 4) & 1) : (r & ~7) + f16_perm(r & 7);
     const float4* tok4 = reinterpret_cast<const float4*>(smem + C::kOffTok) + t0;
     const float* tok1 = reinterpret_cast<const float*>(smem + C::kOffTok + 4 * 128 * 16) + t0;
     uint32_t n_own = 0;                             // units of this group so far
@@ -448,7 +499,24 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       // Moves the accumulators (the group's last P.V is complete) into the FP32 copy, scaled by fac_s[] if asked.
       auto drain = [&](bool scale) {
         tc_fence_after();
-        // (a loop: the caller's values, scores among them, fill the registers)
+        // (loops: the caller's values, scores among them, fill the registers)
+        if constexpr (C::kIntPV) {
+#pragma unroll 1
+          for (int c = 0; c < CG / 4; ++c) {
+            uint32_t a[16];
+            TmemRegs<16>::ld(tm_o + c * 16, a);
+            tc_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              float* o = of_s + f16_col(c, k) * 128;
+              const float v = f16_planes(a + 4 * k);
+              *o = have_of ? *o + v : v;
+            }
+          }
+          have_of = true;
+          units_in_acc = 0;
+          return;
+        }
 #pragma unroll 1
         for (int c = 0; c < CG; c += kDW) {
           uint32_t h[kDW], q[kDW], of[kDW];
@@ -482,6 +550,41 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         have_of = true;
         units_in_acc = 0;
       };
+      // (kIntPV) After a change of the references: the sums of the columns that it concerns, scaled where they are and taken apart into
+      // byte planes again.  Rarely more than one column of 32, which is why the others are left alone: with a drain of all columns
+      // raises took a fifth of the time where outliers make them frequent.
+      auto rescale = [&]() {
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < CG / 4; ++c) {
+          float f[4];
+          bool any = false;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) { f[k] = fac_s[f16_col(c, k)]; any |= f[k] != 1.0f; }
+          if (!any) continue;
+          uint32_t a[16];
+          TmemRegs<16>::ld(tm_o + c * 16, a);
+          tc_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float v = f16_planes(a + 4 * k) * f[k];
+            const int p3 = __float2int_rn(v * 0x1p-24f);
+            v = fmaf((float)p3, -0x1p24f, v);
+            const int p2 = __float2int_rn(v * 0x1p-16f);
+            v = fmaf((float)p2, -0x1p16f, v);
+            const int p1 = __float2int_rn(v * 0x1p-8f);
+            v = fmaf((float)p1, -0x1p8f, v);
+            a[4 * k] = (uint32_t)__float2int_rn(v);
+            a[4 * k + 1] = (uint32_t)p1;
+            a[4 * k + 2] = (uint32_t)p2;
+            a[4 * k + 3] = (uint32_t)p3;
+            if (have_of) of_s[f16_col(c, k) * 128] *= f[k];
+          }
+          TmemRegs<16>::st(tm_o + c * 16, a);
+        }
+        tc_wait_st();
+        tc_fence_before();
+      };
       if (have) {
         const int full_lim = p.causal ? len - p.tail + 1 : len;
         const int* lim_s = reinterpret_cast<const int*>(scal + 2 * NC + qi * NC) + col0;
@@ -493,8 +596,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           const int gs = gs_base + u, sl = gs & 1;
           const int unit_t0 = (item.pad1 + u) * C::kST;
           // ---- scores: log2 of the weights relative to the columns' references ------------------------------
-          mbar_wait_in(mready + (gs & 3) * 8, (gs >> 2) & 1, abort_word);
-          mbar_wait_in(sfull + sl * 8, (gs >> 1) & 1, abort_word);
+          const int ms = gs % C::kSlots;
+          mbar_wait2_in(mready + ms * 8, (gs / C::kSlots) & 1, sfull + sl * 8, (gs >> 1) & 1, abort_word);
           tc_fence_after();
           uint64_t y2[4][NG];
           bool scale = false;
@@ -514,7 +617,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
               tc_ld_16x256(tm_s + NC + ((uint32_t)(8 * k) << 16), s[1]);
               tc_wait_ld();
             }
-            const float4 ts = tok4[(gs & 3) * 128 + 8 * k];
+            const float4 ts = tok4[ms * 128 + 8 * k];
             const uint64_t al2 = f2_pack(ts.x, ts.x), be2 = f2_pack(ts.y, ts.y), lsv2 = f2_pack(ts.z, ts.z);
 #pragma unroll
             for (int j = 0; j < NG; ++j) {
@@ -552,9 +655,14 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
             }
           if (n_own > 0) mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // P free, accumulators current
           // (behind the scores: the product that is waited for here has had their time to complete)
-          if (scale || units_in_acc >= C::kDrainUnits) drain(scale);
+          if constexpr (C::kIntPV) {
+            if (scale) rescale();
+            if (units_in_acc >= C::kDrainUnits) drain(false);
+          } else {
+            if (scale || units_in_acc >= C::kDrainUnits) drain(scale);
+          }
           // ---- a piece's first unit, or a weight that would leave FP16: new reference exponents ----------
-          if (!bar_or(bar_g, 128, fresh || ymax > 15.0f)) break;
+          if (!bar_or(bar_g, 128, fresh || ymax > C::kRaise)) break;
 #pragma unroll
             for (int j = 0; j < NG; ++j) {
               float ma = -INFINITY, mb = -INFINITY;
@@ -577,8 +685,8 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
               const float old = fresh ? 0.0f : ref_s[r];
               const float mx = fmaxf(fmaxf(red_s[r], red_s[CG + r]), fmaxf(red_s[2 * CG + r], red_s[3 * CG + r])) + old;
               float nw = old, f = 1.0f;
-              if (fresh) { nw = fmaxf(mx, -1.0e4f) - 8.0f; f = 0.0f; }
-              else if (mx - old > 15.0f) { nw = mx - 8.0f; f = ex2_full(old - nw); }
+              if (fresh) { nw = fmaxf(mx, -1.0e4f) - C::kTop; f = 0.0f; }
+              else if (mx - old > (C::kIntPV ? C::kTop : C::kRaise)) { nw = mx - C::kTop; f = ex2_full(old - nw); }
               ref_s[r] = nw;
               fac_s[r] = f;
             }
@@ -600,7 +708,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           // ---- weights of this thread's tokens into the P tile --------------------------------------------------
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const float ia = tok4[(gs & 3) * 128 + 8 * k].w, ib = tok1[(gs & 3) * 128 + 8 * k];
+            const float ia = tok4[ms * 128 + 8 * k].w, ib = tok1[ms * 128 + 8 * k];
             const uint64_t ia2 = f2_pack(ia, ia), ib2 = f2_pack(ib, ib);
             uint32_t h[4], q[4];
 #pragma unroll
@@ -611,6 +719,12 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
               const uint64_t w2 = f2_pack(wa, wb);
               l2[j] = f2_fma(w2, ia2, l2[j]);
               zs2[j] = f2_fma(w2, ib2, zs2[j]);
+              if constexpr (C::kIntPV) {   // even and odd columns
+                f2_unpack(f2_mul(w2, f2_pack(0x1p25f, 0x1p25f)), a, b);
+                asm("cvt.rni.u32.f32 %0, %1;" : "=r"(h[j]) : "f"(a));
+                asm("cvt.rni.u32.f32 %0, %1;" : "=r"(q[j]) : "f"(b));
+                continue;
+              }
               h[j] = pack_f16x2(wa, wb);
               asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tcvt.f32.f16 %0, lo;\n\tcvt.f32.f16 %1, hi;\n\t}"
                   : "=f"(ha), "=f"(hb) : "r"(h[j]));
@@ -624,7 +738,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) { mbar_arrive(mfree + (gs & 3) * 8); mbar_arrive(pready + g * 8); }
+          if (lane == 0) { mbar_arrive(mfree + ms * 8); mbar_arrive(pready + g * 8); }
           ++units_in_acc;
         }
         mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // the last P.V
@@ -677,6 +791,21 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
 #pragma unroll
           for (int k = 0; k < 8; ++k) put(col0 + c + k, o[k] + lz_s[32 + c + k], ref_s[c + k], lz_s[c + k]);
         }
+      } else if constexpr (C::kIntPV) {
+        // each group merges and writes one half of the columns
+        named_bar(3, 256);   // (the other group's copy and totals are in place)
+        const float* of_o = of_s + (g ? -CG * 128 : CG * 128);
+        const float* ogrp = reinterpret_cast<const float*>(smem + C::kOffGrp) + (g ^ 1) * C::kGrpScal;
+        const bool have_o = ((g ^ 1 ^ gs_base) & 1) < n_piece;
+#pragma unroll 4
+        for (int cc = 16 * g; cc < 16 * g + 16; ++cc) {
+          const float m1 = ref_s[cc], m2 = ogrp[cc], M = fmaxf(m1, m2);
+          const float f1 = ex2_full(m1 - M), f2 = ex2_full(m2 - M);
+          const float l = lz_s[cc] * f1 + ogrp[320 + cc] * f2;
+          const float z = lz_s[32 + cc] * f1 + ogrp[320 + 32 + cc] * f2;
+          const float o = ((have ? of_s[cc * 128] * f1 : 0.0f) + (have_o ? of_o[cc * 128] * f2 : 0.0f)) * 0x1p-25f;
+          put(cc, o + z, M, l);
+        }
       } else {
         // each group hands the other one half of its columns through its idle P tile, and merges and writes the other half
         float* mail = reinterpret_cast<float*>(smem + C::kOffP + g * C::kPTile);
@@ -707,7 +836,7 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         }
       }
       tc_fence_before();
-      named_bar(3, 256);   // (the mail and the other group's totals have been read)
+      named_bar(3, 256);   // (the other group's sums and totals have been read)
       if (lane == 0) mbar_arrive(qempty + qi * 8);
       gs_base += n_piece;
       ++ic;
@@ -825,14 +954,14 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       if (C::kMetaK) meta.piece(p, items[qi]);
       for (int u = 0; u < n_piece; ++u, ++gs) {
         if (C::kMetaK) {
-          if (gs >= 4) mbar_wait_in(mfree + (gs & 3) * 8, ((gs >> 2) - 1) & 1, abort_word);
+          const int ms = gs % C::kSlots;
+          mbar_wait_in(mfree + ms * 8, ((gs / C::kSlots) - 1) & 1, abort_word);
           meta.unit(p, u, gs, ca);
           __syncwarp();
-          if (lane == 0) mbar_arrive(mready + (gs & 3) * 8);
+          if (lane == 0) mbar_arrive(mready + ms * 8);
           meta.next(p, u);
         }
-        mbar_wait_in(kfull + slot * 8, phase, abort_word);
-        if (gs >= 2) mbar_wait_in(sfull + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);   // Q.K^T of the unit before last
+        mbar_wait2_in(kfull + slot * 8, phase, sfull + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);   // and Q.K^T of the unit before last
         tc_fence_after();
         f16_expand_k(sbase + C::kOffRK + (uint32_t)slot * C::kStageBytes, kt, tm_k + (uint32_t)(gs & 1) * 64u);
         __syncwarp();
@@ -854,9 +983,10 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     int slot = 0;
     uint32_t phase = 0;
     for (int gs = 0; gs < n_units; ++gs) {
-      mbar_wait_in(vfull + slot * 8, phase, abort_word);
-      if (gs >= 2) mbar_wait_in(vfree + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);
-      f16_expand_v(sbase + C::kOffRV + (uint32_t)slot * C::kStageBytes, sbase + C::kOffV + (uint32_t)(gs & 1) * C::kVTile, vt);
+      mbar_wait2_in(vfull + slot * 8, phase, vfree + (gs & 1) * 8, ((gs >> 1) - 1) & 1, abort_word);
+      const uint32_t raw = sbase + C::kOffRV + (uint32_t)slot * C::kStageBytes, tile = sbase + C::kOffV + (uint32_t)(gs & 1) * C::kVTile;
+      if constexpr (C::kIntPV) f16_expand_v8(raw, tile, warp & 3, lane);
+      else f16_expand_v(raw, tile, vt);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) { mbar_arrive(vempty + slot * 8); mbar_arrive(vready + (gs & 1) * 8); }
@@ -890,10 +1020,11 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
       mbar_wait_in(qready + qi * 8, (ic >> 1) & 1, abort_word);
       const float ca = p.sm_log2 * __int_as_float((127 - reinterpret_cast<const int*>(scal)[4 * NC + qi]) << 23);
       for (int u = 0; u < n_piece; ++u, ++gs) {
-        if (gs >= 4) mbar_wait_in(mfree + (gs & 3) * 8, ((gs >> 2) - 1) & 1, abort_word);
+        const int ms = gs % C::kSlots;
+        mbar_wait_in(mfree + ms * 8, ((gs / C::kSlots) - 1) & 1, abort_word);
         meta.unit(p, u, gs, ca);
         __syncwarp();
-        if (lane == 0) mbar_arrive(mready + (gs & 3) * 8);
+        if (lane == 0) mbar_arrive(mready + ms * 8);
         meta.next(p, u);
       }
       __syncwarp();
@@ -903,15 +1034,15 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
     return;
   }
   if (warp == 20) {
-    constexpr uint32_t kIdescS = tc_idesc(C::kSCols, false), kIdescO = tc_idesc(64, true) | (1u << 15);
+    constexpr uint32_t kIdescS = tc_idesc(C::kSCols, false),
+                       kIdescO = C::kIntPV ? i8_idesc(C::kNPV, true, false) | (1u << 7) : tc_idesc(64, true) | (1u << 15);   // (A: signed bytes)
     // (low words of the operand descriptors; the issuing thread keeps them in registers)
     constexpr uint32_t kHi = i8_desc_hi(1024u, 2u);
     const uint32_t q_lo = i8_desc_lo(sbase + C::kOffQ, 16u), v_lo = i8_desc_lo(sbase + C::kOffV, 16384u),
                    p_lo = i8_desc_lo(sbase + C::kOffP, 16384u);
     auto qk = [&](int gs) {
       const int sl = gs & 1;
-      mbar_wait_in(kready + sl * 8, (gs >> 1) & 1, abort_word);
-      if (gs >= 2) mbar_wait_in(sfree + sl * 8, ((gs >> 1) - 1) & 1, abort_word);
+      mbar_wait2_in(kready + sl * 8, (gs >> 1) & 1, sfree + sl * 8, ((gs >> 1) - 1) & 1, abort_word);
       tc_fence_after();
       if (tc_elect()) {
         const uint32_t d = tmem0 + C::kTmS + sl * C::kSCols, a = tmem0 + C::kTmK + sl * 64;
@@ -931,10 +1062,12 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
         tc_fence_after();
         const uint32_t acc = *reinterpret_cast<volatile int*>(misc + 40 + g) ? 1u : 0u;
         if (tc_elect()) {
-          const uint32_t d = tmem0 + C::kTmO + g * 64, vl = v_lo + sl * (C::kVTile >> 4), pl = p_lo + g * (C::kPTile >> 4);
+          const uint32_t d = tmem0 + C::kTmO + g * C::kNPV, vl = v_lo + sl * (C::kVTile >> 4), pl = p_lo + g * (C::kPTile >> 4);
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
-            tc_mma_ss(d, i8_pack(vl + ks * 128u, kHi), i8_pack(pl + ks * 128u, kHi), kIdescO, ks > 0 ? 1u : acc);
+          for (int ks = 0; ks < (C::kIntPV ? 4 : 8); ++ks) {
+            if constexpr (C::kIntPV) i8_mma_ss(d, i8_pack(vl + ks * 256u, kHi), i8_pack(pl + ks * 256u, kHi), kIdescO, ks > 0 ? 1u : acc);
+            else tc_mma_ss(d, i8_pack(vl + ks * 128u, kHi), i8_pack(pl + ks * 128u, kHi), kIdescO, ks > 0 ? 1u : acc);
+          }
           tc_commit(pvdone + g * 8);
           tc_commit(vfree + sl * 8);
         }
@@ -964,11 +1097,19 @@ __global__ void __launch_bounds__(F16Cfg<NC>::kThreads, 1) attn_f16_kernel(const
   }
 }
 
-template <int NC>
+template <int NC, bool INT>
 lynx_status launch_f16(AttnParams p, cudaStream_t st) {
-  using C = F16Cfg<NC>;
+  using C = F16Cfg<NC, INT>;
   p.combine_single = 1;
   constexpr int kMin = 1;
-  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, kMin, attn_f16_kernel<NC>>(p, st);
+  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, kMin, attn_f16_kernel<NC, INT>>(p, st);
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
+}
+
+// P.V on integers where a CTA has 24 units or more: they take less per unit, and 0.3 us more at the end of a piece and up to a
+// thousand instructions more whenever a reference is raised, which outliers do mostly in the first units.  us, FP16 / integers, 32
+// columns, log-normal and outlier values: 85 tokens 12.9 / 13.2, one sequence of 16384 (7 units per CTA) 23.1 / 22.3 and 24.3 / 25.2,
+// 4 of 7056 (12) 30.7 / 29.2 and 32.4 / 32.9, one of 131072 (55) 79.8 / 72.1 and 83.0 / 78.2, 4 of 32768 (55) 86.5 / 76.8 and 89.1 / 84.7.
+inline bool f16_int_pv(const AttnParams& p) {
+  return (long long)p.B * p.Hkv * p.max_blocks * p.bt >= 24ll * 128 * sm_count();
 }

@@ -69,14 +69,6 @@ struct PipeCfg {
   static constexpr int kRegSoft = kSG == 2 ? 128 : kSG == 3 ? 104 : 80, kRegRest = kSG == 2 ? 56 : 48;
 };
 
-// Two waits whose first probes are under way at the same time.
-__device__ __forceinline__ void mbar_wait2_in(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1, volatile int* abort_word) {
-  const bool a = mbar_test(bar0, parity0), b = mbar_test(bar1, parity1);
-  if (a && b) return;
-  mbar_wait_in(bar0, parity0, abort_word);
-  mbar_wait_in(bar1, parity1, abort_word);
-}
-
 template <int N>
 struct TmemCols;   // (N consecutive columns of the thread's own lane, N a power of two up to 16)
 template <> struct TmemCols<4> : TmemRegs<4> {};
@@ -294,7 +286,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
               const float old = fresh ? 0.0f : ref_s[r];
               float nw = old, f = 1.0f;
               if (fresh) { nw = fmaxf(mx, -1.0e4f) - 28.0f; f = 0.0f; }
-              else if (mx - old > 31.5f) { nw = mx - 28.0f; f = ex2_full(old - nw); }
+              else if (mx - old > 28.0f) { nw = mx - 28.0f; f = ex2_full(old - nw); }
               ref_s[r] = nw;
               fac_s[r] = f;
               red_s[4 * CP + r] = nw - old;   // what the change takes off every exponent of the column

@@ -1,7 +1,8 @@
 """Anchor and verification attention with up to 16 query columns where the pipeline of their kernel can go wrong: pieces of fewer
 units than it has softmax groups, of as many as it has buffers and one more, CTAs with many pieces, more units than the rings hold
-several times over, and references that are raised in every stage of it.  Against a 64-bit evaluation with torch on the
-dequantised planes.
+several times over, references that are raised in every stage of it, and integer sums that are drained before they could overflow.
+Verification with 17..32 columns likewise where its values go through integer products (its rule goes by the table's width, so that
+a wide table takes short sequences there).  Against a 64-bit evaluation with torch on the dequantised planes.
 
 Tolerance: a weight 2^(x - ref) formed in binary32 from four roundings of a score below 128 (log2 units) is off by 2.1e-5 of itself,
 its rounding to an integer by 2^-29 of the largest, independently from token to token; the integer sums are exact, and putting
@@ -23,12 +24,12 @@ def _values(p, full):
     return p.meta[..., 1:2].double() + p.meta[..., 0:1].double() * (nib(p.anchor) * 16 + (nib(p.residual) if full else 8))
 
 
-def _run(lens, Hkv, G, n_q, ramp, bt=16):
+def _run(lens, Hkv, G, n_q, ramp, bt=16, width=0, states=(False, True)):
     g = torch.Generator(device="cuda")
     g.manual_seed(sum(lens) + G * n_q)
     need = [(n + bt - 1) // bt for n in lens]
     nb, B = sum(need), len(lens)
-    table = torch.zeros(B, max(need), dtype=torch.int32)
+    table = torch.zeros(B, max(max(need), width), dtype=torch.int32)
     perm, pos = torch.randperm(nb, generator=torch.Generator().manual_seed(nb)).to(torch.int32), 0
     for b, n in enumerate(need):
         table[b, :n] = perm[pos:pos + n]
@@ -46,7 +47,7 @@ def _run(lens, Hkv, G, n_q, ramp, bt=16):
     geo = lynx.Geometry(Hkv * G, Hkv, bt, nb, table.shape[1])
     ws = lynx.make_workspace(geo, B, n_q, "cuda")
     tab, ln = table.cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda")
-    for full in (False, True):
+    for full in states:
         call = lynx.merge_verify_attention if full else lynx.anchor_attention
         outs = []
         for _ in range(2):   # (a second time on the workspace as the first left it)
@@ -91,3 +92,52 @@ def test_rings_that_come_round(G, n_q, ramp):
 @pytest.mark.parametrize("lens", [[700, 129], [2600], [128 * 9] * 40])
 def test_references_that_are_raised(G, n_q, lens):
     _run(lens, 2, G, n_q, ramp=True)
+
+
+def _wide(Hkv, B):
+    """Blocks of a table that gives 148 CTAs 24 units of 128 tokens each, and some more."""
+    return 24 * 148 * 8 // (Hkv * B) + 1
+
+
+@pytest.mark.parametrize("G,n_q", [(3, 6), (3, 7), (4, 8)])   # 18, 21, 32 columns
+@pytest.mark.parametrize("lens", [[1, 16, 127, 128, 129], [128 * n for n in range(1, 7)], [60 + 70 * (i % 5) for i in range(100)]])
+def test_values_on_integers(G, n_q, lens):
+    _run(lens, 1, G, n_q, ramp=False, width=_wide(1, len(lens)), states=(True,))
+
+
+@pytest.mark.parametrize("lens", [[700, 129], [2600], [128 * 9] * 40])
+def test_values_on_integers_when_references_are_raised(lens):
+    _run(lens, 2, 4, 8, ramp=True, width=_wide(2, len(lens)), states=(True,))
+
+
+def test_sums_are_drained_before_they_could_overflow():
+    """148 heads of 1032 units: a CTA has a head, and each of up to four softmax groups more than the 256 units between drains."""
+    heads, tokens, bt = 148, 1032 * 128, 64
+    nb = tokens // bt
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    K, V = (lynx.alloc_planes((nb, heads, bt), "cuda") for _ in range(2))
+    for P in (K, V):
+        for i in range(0, nb, 129):
+            x = torch.randn(129, heads, bt, 128, generator=g, device="cuda")
+            lynx.split_quantize(x.to(torch.bfloat16), out=lynx.Planes(P.anchor[i:i + 129], P.residual[i:i + 129], P.meta[i:i + 129]))
+    tab = torch.arange(nb, dtype=torch.int32, device="cuda").view(1, -1)
+    ln = torch.tensor([tokens], dtype=torch.int32, device="cuda")
+    for G, n_q in ((1, 4), (1, 8), (1, 16), (2, 16)):
+        geo = lynx.Geometry(heads * G, heads, bt, nb, nb)
+        ws = lynx.make_workspace(geo, 1, n_q, "cuda")
+        q = torch.randn(1, n_q, heads * G, 128, generator=g, device="cuda").to(torch.bfloat16)
+        for full in (False, True):
+            call = lynx.merge_verify_attention if full else lynx.anchor_attention
+            o = call(geo, q, K, V, tab, ln, ws, causal=False)
+            o = o[0] if full else o
+            lynx.check(ws)
+            for h in (0, 77, 147):
+                kd, vd = (_values(lynx.Planes(*(t[:, h] for t in (P.anchor, P.residual, P.meta))), full).reshape(tokens, 128) for P in (K, V))
+                sl = slice(h * G, h * G + G)
+                ref = torch.softmax(q[0, :, sl].double().reshape(-1, 128) @ kd.T / math.sqrt(128), 1) @ vd
+                got = o[0, :, sl].double().reshape(-1, 128)
+                # (a mean of 132096 values is 1 / 360 of one, and the integer kernels form it as the difference of two sums of the size of
+                # a zero point, here up to 5.5, with some four roundings: 4 * 2^-24 * 5.5 for every element)
+                bound = REL * ref.norm() + 4 * 2.0 ** -24 * 5.5 * ref.numel() ** 0.5
+                assert (got - ref).norm() <= bound, (G, n_q, full, h, ((got - ref).norm() / bound).item())

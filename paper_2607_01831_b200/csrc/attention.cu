@@ -69,6 +69,9 @@ struct AttnParams {
   int nq_stride, tail;
   int draft_vec;   // draft is 16-byte aligned: its rows are read four values at a time
   BlockDiv bt_div;      // for t / bt
+  // The aligned cut (see sk_range), where it is possible at all: CTAs per segment (else 0), and for quotients by that and by Hkv
+  int per_seg;
+  BlockDiv seg_div, hkv_div;
   int combine_single;   // the attention kernel leaves a segment of one CTA in its slot, too
   int inline_merge;     // the last CTA of a segment joins its slots, not attn_combine_kernel
 };
@@ -213,8 +216,21 @@ __device__ __forceinline__ long long sk_div(long long a, long long b) {   // a, 
 }
 struct SkRange {
   long long q, lo, hi, off_lo;   // off_lo: offset of `lo` among the Hkv * U units of sequence b_lo
-  int b_lo;
+  int b_lo, hkv, u;              // hkv, u: the head and unit of `lo` where the cut gives them, or hkv < 0
 };
+// What the aligned cut gives a CTA whatever the lengths: its segment, and which part of it.  (Before the lengths are there: behind
+// them lies the first copy of a launch, and an instruction that waits for the one before it is 2 to 5 ns.)
+struct SkPlace {
+  int s, part, b, hkv;
+};
+__device__ __forceinline__ SkPlace sk_place(const AttnParams& p, int cta) {
+  SkPlace a;
+  a.s = p.per_seg > 1 ? quotient(cta, p.seg_div) : cta;
+  a.part = cta - a.s * max(p.per_seg, 1);
+  a.b = p.Hkv > 1 ? quotient(a.s, p.hkv_div) : a.s;
+  a.hkv = a.s - a.b * p.Hkv;
+  return a;
+}
 // The lengths as one warp knows them: lane i keeps sequence i's, so that the first 32 are read once (a look-up again is a
 // round trip to the L2 on the way to a launch's first copy).
 struct SeqLens {
@@ -243,8 +259,9 @@ struct SeqLens {
 // up to 15 %).  lo, hi index a list in which every segment occupies c * q entries, so that the
 // contributors of a segment and their partial slots follow from lo and q as in the plain cut.
 template <int ST>
-__device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int cta, int lane, const SeqLens& sl) {
+__device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int cta, int lane, const SeqLens& sl, const SkPlace& at) {
   SkRange r;
+  r.hkv = r.u = -1;
   long long tot = 0;
   int umin = 0x7FFFFFFF, umax = 0;
   for (int b0 = 0; b0 < p.B; b0 += 32) {
@@ -255,22 +272,22 @@ __device__ __forceinline__ SkRange sk_range(const AttnParams& p, int n_cta, int 
   }
   umin = __reduce_min_sync(0xFFFFFFFFu, umin);
   umax = __reduce_max_sync(0xFFFFFFFFu, umax);
-  const long long T = tot * p.Hkv;
-  const long long segs = (long long)p.B * p.Hkv;
-  const int per_seg = segs <= n_cta ? small_div(n_cta, (int)segs) : 0;
-  if (umin == umax && umax > 0 && segs <= n_cta && per_seg * (int)segs * 100 >= 85 * n_cta) {
-    const int c = per_seg, U = umax;
-    r.q = sk_div(U + c - 1, c);
-    const int s = small_div(cta, c), part = cta - s * c;
+  if (p.per_seg > 0 && umin == umax && umax > 0) {
+    const int c = p.per_seg, U = umax;                    // (U at most 2^24)
+    const int q = c > 1 ? quotient(U + c - 1, p.seg_div) : U;
+    r.q = q;
     r.lo = r.hi = 0; r.b_lo = 0; r.off_lo = 0;
-    if (s < segs && (long long)part * r.q < U) {
-      r.b_lo = small_div(s, p.Hkv);
-      r.off_lo = (long long)(s - r.b_lo * p.Hkv) * U + (long long)part * r.q;
-      r.lo = ((long long)s * c + part) * r.q;
-      r.hi = r.lo + min(r.q, (long long)U - (long long)part * r.q);
+    r.u = at.part * q;
+    if (at.b < p.B && r.u < U) {
+      r.b_lo = at.b;
+      r.hkv = at.hkv;
+      r.off_lo = (long long)at.hkv * U + r.u;
+      r.lo = (long long)cta * q;                          // (part of segment s: (s c + part) q)
+      r.hi = r.lo + min(q, U - r.u);
     }
     return r;
   }
+  const long long T = tot * p.Hkv;
   r.q = sk_div(T + n_cta - 1, n_cta);
   r.lo = (long long)cta * r.q;
   r.hi = (r.lo + r.q < T) ? r.lo + r.q : T;
@@ -523,6 +540,13 @@ inline int attention_grid(const AttnParams& p, int st_tokens, int min_units) {
   const long long grid = (long long)p.B * p.Hkv * (((long long)p.max_blocks * p.bt + per - 1) / per);
   const int full = sm_count();
   return grid < 1 ? 1 : grid > full ? full : (int)grid;
+}
+// The aligned cut of such a launch: each of the B * Hkv segments has CTAs of its own, and 85 % of the grid at least have one.
+inline void plan_cut(AttnParams* p, int n_cta) {
+  const long long segs = (long long)p->B * p->Hkv;
+  p->per_seg = segs <= n_cta && n_cta / segs * segs * 100 >= 85ll * n_cta ? (int)(n_cta / segs) : 0;
+  p->seg_div = p->per_seg > 1 ? block_div(p->per_seg) : BlockDiv{0, 0};
+  p->hkv_div = p->Hkv > 1 ? block_div(p->Hkv) : BlockDiv{0, 0};
 }
 
 // (Nothing to join where every segment is one unit and nothing to decide; anchor calls with many heads join in the attention

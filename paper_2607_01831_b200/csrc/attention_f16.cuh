@@ -220,12 +220,14 @@ __device__ __forceinline__ float f16_planes(const uint32_t* a) {
   return fmaf(fmaf(fmaf((float)(int)a[3], 256.0f, (float)(int)a[2]), 256.0f, (float)(int)a[1]), 256.0f, (float)(int)a[0]);
 }
 
-// A producer warp: derives the CTA's range like the others (warp 0 publishes it, the pieces, and the results of empty sequences).
+// A producer warp: derives the CTA's range like the others.  The V warp publishes the pieces and does what is left to do for a
+// sequence: its copies are the last to be waited for.
 // Warps 0, 1 copy one half of the K sub-blocks each, warp 2 the V sub-blocks, warp 3 the metadata of both (where kMetaRing).  full0,
 // empty0, stages: of the warp's own ring.
 // What bounds a producer is the latency of its instructions in a row: some 55 cycles per copy, 300 per unit.  Hence gathers of four
 // sub-blocks per copy for V and the metadata (the 128-byte swizzle of K does not go with them), and always all eight sub-blocks of a
 // unit, whether or not the sequence has them.
+constexpr int kPublisher = 2;
 template <class C>
 __device__ __forceinline__ void plane_producer(const AttnParams& p, const SkRange& rng, const SeqLens& sl, int pw, int lane, uint32_t sbase, uint32_t full0,
                                                uint32_t empty0, int stages, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
@@ -235,13 +237,17 @@ __device__ __forceinline__ void plane_producer(const AttnParams& p, const SkRang
   const int sub0 = pw == 1 ? 4 : 0;
   uint32_t* my_blk = blk_s + (pw < 2 ? 4 * pw : 8 * (pw - 1)) * kI8PieceUnits;
   int b = rng.b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
-  int hkv = (int)sk_div(rng.off_lo, U), u = (int)(rng.off_lo - (long long)hkv * U);
+  int hkv = rng.hkv, u = rng.u;
+  if (hkv < 0) {
+    hkv = (int)sk_div(rng.off_lo, U);
+    u = (int)(rng.off_lo - (long long)hkv * U);
+  }
   const int n_units = (int)(rng.hi - rng.lo);
   int remaining = n_units, slot = 0, ic = 0;
   uint32_t phase = 1;   // (a fresh barrier passes a wait for the phase before its first)
   while (remaining > 0) {
     const int n = min(remaining, U - u);
-    if (pw == 0) {
+    if (pw == kPublisher) {
       const int qi = ic & 1;
       if (ic >= 2) mbar_wait_in(qempty0 + qi * 8, ((ic >> 1) - 1) & 1, abort_word + kItemAbort);
       const long long seg0 = rng.lo + (n_units - remaining) - u;  // first unit of this segment
@@ -450,16 +456,27 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
   tc_fence_after();
   const uint32_t tmem0 = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(misc + 8), 0);
   // nothing in global memory has been touched so far: wait for the grids this one depends on
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-
-  SkRange rng;
-  SeqLens sl;
+  // ================================================================================== producers
   if (warp >= 16 && warp < 20) {
-    sl = SeqLens(p, lane);
-    rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, sl);
-    if (warp == 16 && lane == 0) misc[7] = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
+    reg_dec<C::kRegProd>();
+    const int pw = warp - 16;
+    const SkPlace at = sk_place(p, blockIdx.x);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const SeqLens sl(p, lane);
+    const SkRange rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, sl, at);
+    const int n_units = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
+    if (pw == 0 && lane == 0) misc[7] = n_units;
+    __syncwarp();
+    bar_arrive(7, C::kThreads);   // the range is published (the producers know it and do not wait)
+    if (n_units == 0 || pw == 3) bar_arrive(5, C::kDoneThreads);
+    else
+      plane_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, pw < 2 ? C::kRingK : C::kRingV, qfull,
+                        qempty, reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps, 5);
+    if (pw == kPublisher) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
+    return;
   }
-  __syncthreads();  // (A) the range is published
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  named_bar(7, C::kThreads);
   const int n_units = misc[7];
 
   // ================================================================================== softmax warpgroups
@@ -992,17 +1009,6 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
       if (lane == 0) { mbar_arrive(vempty + slot * 8); mbar_arrive(vready + (gs & 1) * 8); }
       if (++slot == C::kRingV) { slot = 0; phase ^= 1; }
     }
-    return;
-  }
-  // ================================================================================== producers
-  if (warp < 20) {
-    reg_dec<C::kRegProd>();
-    const int pw = warp - 16;
-    if (n_units == 0 || pw == 3) bar_arrive(5, C::kDoneThreads);
-    else
-      plane_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : vfull, pw < 2 ? kempty : vempty, pw < 2 ? C::kRingK : C::kRingV, qfull,
-                        qempty, reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps, 5);
-    if (pw == 0) per_sequence<true, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
     return;
   }
   // ================================================================================== products

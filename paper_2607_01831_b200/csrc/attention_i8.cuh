@@ -389,7 +389,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   constexpr int ST = C::kST, NSTAGE = C::kNStage, NARR = C::kNArr;
   const int n_cta = gridDim.x, cta = blockIdx.x;
   const SeqLens sl(p, lane);
-  const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, sl);
+  const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, sl, sk_place(p, cta));
   const long long q = rng.q, lo = rng.lo, hi = rng.hi, off_lo = rng.off_lo;
   const int b_lo = rng.b_lo;
   if (pw == 0 && lane == 0) misc[7] = lo < hi ? (int)(hi - lo) : 0;
@@ -1306,7 +1306,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
 // sequences, as before: 17.2 / 36.0 for one sequence of 85 tokens, a CTA to itself for each head 8.5 / 17.7).  The FP16
 // kernels take one (64 columns, 85 tokens: 18.5, four 90; two sequences of 189 tokens: 18.0, two 19.0, four 48).
 template <bool FULL, int SMEM, int THREADS, int ST, int MIN, auto KERN>
-lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
+lynx_status launch_units(AttnParams p, cudaStream_t st) {
   static bool configured[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1320,7 +1320,9 @@ lynx_status launch_units(const AttnParams& p, cudaStream_t st) {
   // memory, while the last CTAs of that kernel are still merging; they read nothing before
   // griddepcontrol.wait, i.e. before that kernel has completed and its memory is visible.
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)attention_grid(p, ST, MIN));
+  const int grid = attention_grid(p, ST, MIN);
+  plan_cut(&p, grid);
+  cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;

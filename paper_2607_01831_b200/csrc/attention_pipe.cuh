@@ -129,16 +129,28 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
   tc_fence_after();
   const uint32_t tmem0 = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(misc + 8), 0);
   // nothing in global memory has been touched so far: wait for the grids this one depends on
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-
-  SkRange rng;
-  SeqLens sl;
+  // ================================================================================== producers
   if (warp >= C::kWarpProd && warp < C::kWarpQK) {
-    sl = SeqLens(p, lane);
-    rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, sl);
-    if (warp == C::kWarpProd && lane == 0) misc[7] = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
+    reg_dec<C::kRegRest>();
+    const int pw = warp - C::kWarpProd;
+    const SkPlace at = sk_place(p, blockIdx.x);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const SeqLens sl(p, lane);
+    const SkRange rng = sk_range<C::kST>(p, gridDim.x, blockIdx.x, lane, sl, at);
+    const int n_units = rng.lo < rng.hi ? (int)(rng.hi - rng.lo) : 0;
+    if (pw == 0 && lane == 0) misc[7] = n_units;
+    __syncwarp();
+    bar_arrive(7, C::kThreads);   // the range is published (the producers know it and do not wait)
+    if (n_units == 0) bar_arrive(9, C::kDoneThreads);
+    else
+      plane_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : pw == 2 ? vfull : mfull, pw < 2 ? kempty : pw == 2 ? vempty : mfree,
+                        pw < 2 ? C::kRingK : pw == 2 ? C::kRingV : C::kNT, qfull, qempty,
+                        reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps, 9);
+    if (pw == kPublisher) per_sequence<FULL, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
+    return;
   }
-  __syncthreads();  // (A) the range is published
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  named_bar(7, C::kThreads);
   const int n_units = misc[7];
 
   // ================================================================================== softmax warpgroups
@@ -460,17 +472,6 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
     return;
   }
   reg_dec<C::kRegRest>();
-  // ================================================================================== producers
-  if (warp < C::kWarpQK) {
-    const int pw = warp - C::kWarpProd;
-    if (n_units == 0) bar_arrive(9, C::kDoneThreads);
-    else
-      plane_producer<C>(p, rng, sl, pw, lane, sbase, pw < 2 ? kfull : pw == 2 ? vfull : mfull, pw < 2 ? kempty : pw == 2 ? vempty : mfree,
-                        pw < 2 ? C::kRingK : pw == 2 ? C::kRingV : C::kNT, qfull, qempty,
-                        reinterpret_cast<uint32_t*>(smem + C::kOffBlk), items, abort_word, &maps, 9);
-    if (pw == 0) per_sequence<FULL, C::kPartCols>(p, blockIdx.x, gridDim.x, lane, sl, n_units ? items : nullptr);
-    return;
-  }
   // ================================================================================== Q.K^T
   constexpr uint32_t kHi = i8_desc_hi(1024u, 2u), kPdHi = i8_desc_hi(8u * C::kPRow, (uint32_t)C::kPLayout);
   if (warp == C::kWarpQK) {

@@ -11,6 +11,7 @@
 // Four rows are in flight per quarter-warp.
 #include <cuda_bf16.h>
 
+#include "block_division.cuh"
 #include "lynx_common.cuh"
 
 namespace lynx {
@@ -80,7 +81,7 @@ __device__ __forceinline__ void codes8(const uint32_t (&w)[4], float mn, float i
 template <bool kIds>
 __global__ void __launch_bounds__(kThreads)
 split_quantize_kernel(const uint4* src, int64_t n_logical_rows,
-                      const int32_t* block_ids, uint32_t rows_per_block,
+                      const int32_t* block_ids, uint32_t rows_per_block, BlockDiv block, bool fours,
                       int64_t n_blocks_total, uint32_t* __restrict__ anchor,
                       uint32_t* __restrict__ residual, float2* __restrict__ meta, bool wide) {
   pdl_begin();
@@ -92,12 +93,22 @@ split_quantize_kernel(const uint4* src, int64_t n_logical_rows,
   for (int64_t r0 = grp * kRows; r0 < n_logical_rows; r0 += grp_total * kRows) {
     uint4 lo[kRows], hi[kRows];
     int64_t row[kRows];
+    // (rows in fours: one look-up, by a multiplication, for all of a trip's rows where blocks are multiples of four rows, which r0 is:
+    // K and V of 4096 listed tokens 10.5 -> 10.05 us, of 16384 26.5 -> 24.4)
+    int64_t first = -1;
+    if (kIds && fours) {
+      const uint32_t lb = (uint32_t)quotient((int32_t)r0, block);
+      const int32_t blk = ld_dep(block_ids + lb);
+      if (blk >= 0 && blk < n_blocks_total) first = (int64_t)blk * rows_per_block + ((uint32_t)r0 - lb * rows_per_block);
+    }
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
       int64_t lr = r0 + u;
       row[u] = -1;
       if (lr < n_logical_rows) {
-        if (kIds) {
+        if (kIds && fours) {
+          row[u] = first < 0 ? -1 : first + u;
+        } else if (kIds) {
           uint32_t lb = (uint32_t)lr / rows_per_block;
           uint32_t in = (uint32_t)lr - lb * rows_per_block;
           int32_t blk = ld_dep(block_ids + lb);
@@ -117,27 +128,38 @@ split_quantize_kernel(const uint4* src, int64_t n_logical_rows,
         }
       }
     }
+    uint32_t v[kRows];   // (min, -max) of the rows
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
       // the shuffles below are executed by every lane of the warp, valid row or not
-      const uint32_t wl[4] = {lo[u].x, lo[u].y, lo[u].z, lo[u].w};
-      const uint32_t wh[4] = {hi[u].x, hi[u].y, hi[u].z, hi[u].w};
       // packed BF16 min / max over the lane's 16 values, then one register (min, -max) through
       // three xor-shuffles of the 8 lanes that own the row
-      const uint32_t mn2 = bf2min(bf2min(bf2min(wl[0], wl[1]), bf2min(wl[2], wl[3])),
-                                  bf2min(bf2min(wh[0], wh[1]), bf2min(wh[2], wh[3])));
-      const uint32_t mx2 = bf2max(bf2max(bf2max(wl[0], wl[1]), bf2max(wl[2], wl[3])),
-                                  bf2max(bf2max(wh[0], wh[1]), bf2max(wh[2], wh[3])));
-      uint32_t v = bf2min(__byte_perm(mn2, mx2, 0x5410) ^ 0x80000000u,
-                          __byte_perm(mn2, mx2, 0x7632) ^ 0x80000000u);
+      const uint32_t mn2 = bf2min(bf2min(bf2min(lo[u].x, lo[u].y), bf2min(lo[u].z, lo[u].w)),
+                                  bf2min(bf2min(hi[u].x, hi[u].y), bf2min(hi[u].z, hi[u].w)));
+      const uint32_t mx2 = bf2max(bf2max(bf2max(lo[u].x, lo[u].y), bf2max(lo[u].z, lo[u].w)),
+                                  bf2max(bf2max(hi[u].x, hi[u].y), bf2max(hi[u].z, hi[u].w)));
+      v[u] = bf2min(__byte_perm(mn2, mx2, 0x5410) ^ 0x80000000u,
+                    __byte_perm(mn2, mx2, 0x7632) ^ 0x80000000u);
 #pragma unroll
-      for (int off = 4; off >= 1; off >>= 1) v = bf2min(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
-      const float mn = __uint_as_float(v << 16);
-      const float mx = __uint_as_float((v & 0xFFFF0000u) ^ 0x80000000u);
-      const float range = __fsub_rn(mx, mn);
-      const bool live = range >= 0x1p-100f;
-      const float scale = live ? __fdiv_rn(range, 255.0f) : 0.0f;
-      const float inv = live ? __fdiv_rn(255.0f, range) : 0.0f;
+      for (int off = 4; off >= 1; off >>= 1) v[u] = bf2min(v[u], __shfl_xor_sync(0xFFFFFFFFu, v[u], off));
+    }
+    // Two divisions a row, eight for the four rows: one in each of the eight lanes that own them, lanes 0..3 the scales, 4..7 the
+    // reciprocals.  (Eight in every lane were a chain of their own in front of the codes: K and V of 4096 listed tokens 10.05 -> 8.3 us,
+    // of 64 5.75 -> 4.85, of 150 tokens in a row 5.2 -> 4.5; where memory bounds the call, no difference.)
+    static_assert(kRows == 4 && kLanesPerRow == 8, "a division per lane");
+    float mine;
+    {
+      const uint32_t w = (ln & 2) ? ((ln & 1) ? v[3] : v[2]) : ((ln & 1) ? v[1] : v[0]);
+      const float range = __fsub_rn(__uint_as_float((w & 0xFFFF0000u) ^ 0x80000000u), __uint_as_float(w << 16));
+      mine = __fdiv_rn(ln < 4 ? range : 255.0f, ln < 4 ? 255.0f : range);
+      if (!(range >= 0x1p-100f)) mine = 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      const uint32_t wl[4] = {lo[u].x, lo[u].y, lo[u].z, lo[u].w};
+      const uint32_t wh[4] = {hi[u].x, hi[u].y, hi[u].z, hi[u].w};
+      const float mn = __uint_as_float(v[u] << 16);
+      const float scale = __shfl_sync(0xFFFFFFFFu, mine, u, kLanesPerRow), inv = __shfl_sync(0xFFFFFFFFu, mine, 4 + u, kLanesPerRow);
       const float zero = __fadd_rn(mn, 0.0f);  // -0 -> +0
 
       uint32_t a_lo, r_lo, a_hi, r_hi;
@@ -225,8 +247,10 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
     const int64_t logical = (int64_t)n_block_ids * rows_per_block;
     if (logical >= (1ll << 31)) return LYNX_ERR_UNSUPPORTED;
     const int grid = grid_for((logical + rows_per_cta_trip - 1) / rows_per_cta_trip, 8);
+    const bool fours = rows_per_block % kRowsInFlightIds == 0;   // (logical rows are then a multiple of four as well)
     return launch_pdl(split_quantize_kernel<true>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), logical, block_ids,
-                      (uint32_t)rows_per_block, n_rows / rows_per_block, reinterpret_cast<uint32_t*>(anchor),
+                      (uint32_t)rows_per_block, fours ? block_div(rows_per_block) : BlockDiv{0, 0}, fours, n_rows / rows_per_block,
+                      reinterpret_cast<uint32_t*>(anchor),
                       reinterpret_cast<uint32_t*>(residual), reinterpret_cast<float2*>(meta), wide);
   }
   // (many short CTAs rather than a few waves of long ones.  K and V of 8 heads, 8 and 64 CTAs per SM: 67.8 and 66.7 us for
@@ -234,7 +258,7 @@ extern "C" lynx_status lynx_split_quantize(const void* src_bf16, int64_t n_rows,
   // difference, 78.4 and 80.4 us for 65536 tokens out of 262144, 287 and 283 us for 262144 out of 1048576: 8.)
   const int grid = grid_for((n_rows + rows_per_cta_trip - 1) / rows_per_cta_trip, 64);
   return launch_pdl(split_quantize_kernel<false>, grid, kThreads, 0, stream, static_cast<const uint4*>(src_bf16), n_rows, nullptr, 1u,
-                    n_rows, reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),
+                    BlockDiv{0, 0}, false, n_rows, reinterpret_cast<uint32_t*>(anchor), reinterpret_cast<uint32_t*>(residual),
                     reinterpret_cast<float2*>(meta), wide);
 }
 

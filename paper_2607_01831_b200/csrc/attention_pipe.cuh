@@ -572,30 +572,28 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
       for (int i = 0; i < NI; ++i) {
         const int c = i * 4 + (qt >> 4), j = (qt >> 2) & 3, w = qt & 3;   // column, 32 dims of the row, 8 of them
         const uint32_t ww[4] = {qv[i].x, qv[i].y, qv[i].z, qv[i].w};
-        uint32_t acc[NP][2];
-#pragma unroll
-        for (int pln = 0; pln < NP; ++pln) { acc[pln][0] = 0; acc[pln][1] = 0; }
+        // A balanced digit is a byte of the value plus 128 in every digit, less 128 again: the top bit flipped.  (Taken off digit by
+        // digit it was 200 instructions for eight entries, and a launch's first product waits for it: verification of 4096 tokens at 16
+        // columns 15.3 -> 14.8 us.)
+        constexpr int kBias = NP == 4 ? (int)0x80808080u : 0x808080;
+        uint32_t val[2][4];   // [even, odd dims][pair]
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          int qv2[2];
+          const int even = max(-4194303, min(4194303, __float2int_rn(__uint_as_float(ww[k] << 16) * up)));
+          const int odd = max(-4194303, min(4194303, __float2int_rn(__uint_as_float(ww[k] & 0xFFFF0000u) * up)));
+          // what multiplies the byte pair (odd value) and its low nibble (16 x even value - odd value), where K goes in as raw bytes
+          val[0][k] = (uint32_t)((C::kRawK ? odd : even) + kBias);
+          val[1][k] = (uint32_t)((C::kRawK ? 16 * even - odd : odd) + kBias);
+        }
+        uint32_t acc[NP][2];
 #pragma unroll
-          for (int par = 0; par < 2; ++par) {
-            const float f = par ? __uint_as_float(ww[k] & 0xFFFF0000u) : __uint_as_float(ww[k] << 16);
-            const int qn = __float2int_rn(f * up);
-            qv2[par] = max(-4194303, min(4194303, qn));
-          }
-          int val[2] = {qv2[0], qv2[1]};
-          if (C::kRawK) { val[0] = qv2[1]; val[1] = 16 * qv2[0] - qv2[1]; }
-#pragma unroll
-          for (int par = 0; par < 2; ++par) {
-            int qn = val[par];
-#pragma unroll
-            for (int pln = 0; pln < NP; ++pln) {
-              const int dgt = (int)(signed char)(qn & 0xFF);
-              acc[pln][par] |= (uint32_t)(dgt & 0xFF) << (8 * k);
-              qn = (qn - dgt) >> 8;
-            }
-          }
+        for (int par = 0; par < 2; ++par) {
+          const uint32_t l01 = prmt(val[par][0], val[par][1], 0x5140u), l23 = prmt(val[par][2], val[par][3], 0x5140u);
+          const uint32_t h01 = prmt(val[par][0], val[par][1], 0x7362u), h23 = prmt(val[par][2], val[par][3], 0x7362u);
+          acc[0][par] = prmt(l01, l23, 0x5410u) ^ 0x80808080u;
+          acc[1][par] = prmt(l01, l23, 0x7632u) ^ 0x80808080u;
+          acc[2][par] = prmt(h01, h23, 0x5410u) ^ 0x80808080u;
+          if (NP == 4) acc[NP - 1][par] = prmt(h01, h23, 0x7632u) ^ 0x80808080u;
         }
 #pragma unroll
         for (int pln = 0; pln < NP; ++pln) {

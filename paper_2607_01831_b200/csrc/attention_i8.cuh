@@ -309,8 +309,9 @@ __device__ __forceinline__ float ex2_full(float x) {   // no flush of small resu
 
 // Expand the nibble planes of one tensor of a 128-token raw stage into its u8 level tile.  A warp
 // takes 8 token rows per step (512 contiguous raw bytes): lane = (row & 7) * 4 + 16-byte chunk.  ODD16: the odd elements of an
-// Anchor plane as they lie in their bytes, 16 times the level (the caller takes it off the sums).
-template <bool FULL, bool ODD16 = false>
+// Anchor plane as they lie in their bytes, 16 times the level (the caller takes it off the sums).  FLIP: what the Anchor words are
+// exclusive-ored with (0x88888888: the codes less 128, as signed bytes).
+template <bool FULL, bool ODD16 = false, uint32_t FLIP = 0>
 __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32_t tile, int w4, int lane) {
   const int row8 = lane >> 2, j = lane & 3;
   uint4 xa[4], xr[4];
@@ -329,7 +330,7 @@ __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32
     for (int k = 0; k < 4; ++k) {
       if (FULL) {
         const uint32_t r[4] = {xr[s].x, xr[s].y, xr[s].z, xr[s].w};
-        merge_codes(a[k], r[k], ev[k], od[k]);
+        merge_codes(a[k] ^ FLIP, r[k], ev[k], od[k]);
       } else {
         ev[k] = a[k] & 0x0F0F0F0Fu;
         od[k] = ODD16 ? a[k] & 0xF0F0F0F0u : (a[k] >> 4) & 0x0F0F0F0Fu;
@@ -346,7 +347,7 @@ __device__ __forceinline__ void i8_expand(uint32_t raw_a, uint32_t raw_r, uint32
 
 // K levels of a 128-token raw stage into tensor memory: thread r owns token r (TMEM lane r) and writes
 // its 128 level bytes to 32 columns, byte 4 col + b in the order of the operand tiles (see the header).
-template <bool FULL, bool RAW>
+template <bool FULL, bool RAW, uint32_t FLIP = 0>
 __device__ __forceinline__ void i8_expand_k_tmem(uint32_t raw_a, uint32_t raw_r, int r, uint32_t tm_k) {
   uint4 xa[4], xr[4];
 #pragma unroll
@@ -364,7 +365,7 @@ __device__ __forceinline__ void i8_expand_k_tmem(uint32_t raw_a, uint32_t raw_r,
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       if (FULL) {
-        merge_codes(a[w], rr[w], regs[8 * j + w], regs[8 * j + 4 + w]);
+        merge_codes(a[w] ^ FLIP, rr[w], regs[8 * j + w], regs[8 * j + 4 + w]);
       } else if (RAW) {   // bytes 16 j + 4 w .. + 3 of the row as they are, and their low nibbles 64 bytes further on
         regs[4 * j + w] = a[w];
         regs[16 + 4 * j + w] = a[w] & 0x0F0F0F0Fu;

@@ -15,6 +15,9 @@
 // 35.0, of 4096 10.5 -> 9.4; 16 ragged sequences, 16 columns, 276 -> 243 (303 -> 283), 4 columns with a BF16 tail 166 -> 153; two
 // sequences of 16000, 8 columns, 22.2 -> 19.4; verification of one layer of 4096 tokens, 16 columns, 16.8 -> 16.5.
 //
+// Exponents are relative to the column's largest weight and the weights scaled by 2^28 afterwards: an exponent of 28 would carry
+// four times the rounding of one below 8.
+//
 // What bounds it: memory, 0.90-0.95 of the copy rate on long contexts, and on short ones the latency of the stages in a row.  What
 // mattered on the way, us for 16 layers at 8 columns and for 16 ragged sequences at 16:
 //   - metadata by gathers into a ring of its own: read by the softmax threads two units ahead, its latency was a third of their
@@ -36,6 +39,12 @@ struct PipeCfg {
   static constexpr bool kRawK = !FULL && CP <= 8;
   static constexpr int kQPlanes = kRawK ? 4 : 3;
   static constexpr int kNQK = (kQPlanes * CP + 15) / 16 * 16, kNPV = 4 * CP;   // N of the products
+  // Full codes enter less 128, as signed bytes: one operation per eight codes, and the sums of scores and values are no longer the
+  // difference of two that are some thirty times larger.  Error against 64 bits, 1e-6 of the 2-norm, means of six draws, teams / stages
+  // with whole codes / less 128: 4 ragged sequences of up to 32768, heavy-tailed, 16 columns 1.10 / 1.05 / 0.49; 2 of 20000, outliers, 8
+  // columns 2.37 / 2.40 / 0.76; a mean of 132096 normal values 33 / 33 / 0.25.  1 % of the time of 16 ragged sequences.
+  static constexpr uint32_t kFlip = FULL ? 0x88888888u : 0u;
+  static constexpr uint32_t kSignedA = FULL ? 1u << 7 : 0u;   // of the instruction descriptors
   static constexpr bool kMetaRing = true;
   static constexpr int kNT = FULL && CP == 16 ? 6 : 8;                          // units whose metadata are kept: [kNT][K, V][128 tokens][scale, zero]
   // buffers of the scores and of K levels in tensor memory, V tiles, P tiles of a group, barriers of P.V
@@ -167,7 +176,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
     const uint32_t p_swz = C::kPRow == 32 ? ((uint32_t)r >> 2) & 1u : C::kPRow == 64 ? ((uint32_t)r >> 1) & 3u : (uint32_t)r & 7u;
     const uint32_t p_row = sbase + C::kOffP + g * PB * C::kPTile + (uint32_t)r * C::kPRow;   // 16-byte chunk j goes to position j ^ p_swz
     const int dim_out = 32 * (r >> 5) + 8 * ((r >> 2) & 3) + 2 * (r & 3) + ((r >> 4) & 1);   // head dim of lane r of O
-    const float cb = p.sm_log2, odd = !FULL && ((r >> 4) & 1) ? 0.0625f : 1.0f;   // (odd dims of the Anchor: 16 times their levels)
+    const float cb = p.sm_log2, unit = !FULL && ((r >> 4) & 1) ? 0x1p-32f : 0x1p-28f;   // of the sums (odd dims of the Anchor: 16 times their levels)
     const float2* meta = reinterpret_cast<const float2*>(smem + C::kOffMeta) + r;   // [unit][K, V][128]
     int gs_base = 0, ic = 0;
     while (gs_base < n_units) {
@@ -194,7 +203,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
         for (int k = 0; k < 4; ++k) {
           float v = fmaf(fmaf(fmaf((float)(int)a[4 * k + 3], 256.0f, (float)(int)a[4 * k + 2]), 256.0f,
                               (float)(int)a[4 * k + 1]), 256.0f, (float)(int)a[4 * k]);
-          v *= odd;
+          v *= unit;
           if (units_in_acc == 0) v = 0.0f;   // (the accumulators have not been restarted since the last drain)
           o[k] = have_of ? v + __uint_as_float(of[k]) : v;
         }
@@ -236,10 +245,10 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
           if (!valid) { km = make_float2(0.f, 0.f); vm = make_float2(0.f, 0.f); }
           const float sve = fmaxf(FULL ? vm.x : 16.0f * vm.x, 9.094947e-13f);   // floor 2^-40
           const float al = km.x * ca;
-          const float be = (FULL ? km.y : fmaf(km.x, 8.0f, km.y)) * cb;
+          const float be = fmaf(km.x, FULL ? 128.0f : 8.0f, km.y) * cb;
           const float lsv = lg2_approx(sve);
           const float ia = valid ? rcp_approx(sve) : 0.0f;
-          const float ib = (FULL ? vm.y : fmaf(vm.x, 8.0f, vm.y)) * ia;
+          const float ib = (FULL ? fmaf(sve, 128.0f, vm.y) : fmaf(vm.x, 8.0f, vm.y)) * ia;
           uint64_t y2[CP / 2];
           {
             uint32_t s0[CP], s1[CP], s2[CP], s3[C::kRawK ? CP : 1];
@@ -290,7 +299,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
           const int pb = gs / SG % PB;
           if (gs >= SG * PB) mbar_wait_in(pvdone + ((gs - SG * PB) % NP) * 8, ((gs - SG * PB) / NP) & 1, abort_word);   // P free
           // ---- a piece's first unit, a weight that would leave the u32 range, sums about to overflow: new references ----
-          if (bar_or(bar_g, 128, fresh || units_in_acc >= C::kDrainUnits || ymax > 31.5f)) {
+          if (bar_or(bar_g, 128, fresh || units_in_acc >= C::kDrainUnits || ymax > 3.5f)) {
 #pragma unroll
             for (int c = 0; c < CP; ++c) {   // (back to absolute exponents x = y + ref)
               float a, b;
@@ -303,8 +312,8 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
               const float mx = fmaxf(fmaxf(red_s[r], red_s[CP + r]), fmaxf(red_s[2 * CP + r], red_s[3 * CP + r]));
               const float old = fresh ? 0.0f : ref_s[r];
               float nw = old, f = 1.0f;
-              if (fresh) { nw = fmaxf(mx, -1.0e4f) - 28.0f; f = 0.0f; }
-              else if (mx - old > 28.0f) { nw = mx - 28.0f; f = ex2_full(old - nw); }
+              if (fresh) { nw = fmaxf(mx, -1.0e4f); f = 0.0f; }
+              else if (mx > old) { nw = mx; f = ex2_full(old - nw); }
               ref_s[r] = nw;
               fac_s[r] = f;
               red_s[4 * CP + r] = nw - old;   // what the change takes off every exponent of the column
@@ -332,9 +341,10 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
               float a, b;
               f2_unpack(y2[c], a, b);
               const float wa = ex2_ftz(a), wb = ex2_ftz(b);
-              asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c]) : "f"(wa));
-              asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c + 1]) : "f"(wb));
               const uint64_t w2 = f2_pack(wa, wb);
+              f2_unpack(f2_mul(w2, f2_pack(0x1p28f, 0x1p28f)), a, b);
+              asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c]) : "f"(a));
+              asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c + 1]) : "f"(b));
               l2[c] = f2_fma(w2, ia2, l2[c]);
               zs2[c] = f2_fma(w2, ib2, zs2[c]);
             }
@@ -443,7 +453,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
       mbar_wait2_in(kfull + slot * 8, phase, sfull + sb * 8, ((gs / NB) - 1) & 1, abort_word);   // and Q.K^T of the unit that was here before
       tc_fence_after();
       const uint32_t raw = sbase + C::kOffRK + (uint32_t)slot * C::kStageBytes;
-      i8_expand_k_tmem<FULL, C::kRawK>(raw, raw + 8192u, kt, tm_k + (uint32_t)sb * 32u);
+      i8_expand_k_tmem<FULL, C::kRawK, C::kFlip>(raw, raw + 8192u, kt, tm_k + (uint32_t)sb * 32u);
       __syncwarp();
       if (lane == 0) mbar_arrive(kempty + slot * 8);
       tc_wait_st();
@@ -464,7 +474,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
       // (the tile's previous product; before there was one: of a phase that a fresh barrier passes)
       mbar_wait2_in(vfull + slot * 8, phase, pvdone + ((gs + NP - NV) % NP) * 8, ((gs + NP - NV) / NP - 1) & 1, abort_word);
       const uint32_t raw = sbase + C::kOffRV + (uint32_t)slot * C::kStageBytes;
-      i8_expand<FULL, !FULL>(raw, raw + 8192u, sbase + C::kOffV + (uint32_t)vb * C::kVTile, warp & 3, lane);
+      i8_expand<FULL, !FULL, C::kFlip>(raw, raw + 8192u, sbase + C::kOffV + (uint32_t)vb * C::kVTile, warp & 3, lane);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) { mbar_arrive(vempty + slot * 8); mbar_arrive(vready + vb * 8); }
@@ -476,7 +486,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
   // ================================================================================== Q.K^T
   constexpr uint32_t kHi = i8_desc_hi(1024u, 2u), kPdHi = i8_desc_hi(8u * C::kPRow, (uint32_t)C::kPLayout);
   if (warp == C::kWarpQK) {
-    constexpr uint32_t kIdescS = i8_idesc(C::kNQK, false, true);
+    constexpr uint32_t kIdescS = i8_idesc(C::kNQK, false, true) | C::kSignedA;
     const uint32_t q_lo = i8_desc_lo(sbase + C::kOffQ, 16u);
     int gs = 0, ic = 0;
     while (gs < n_units) {
@@ -505,7 +515,7 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
   }
   // ================================================================================== P.V
   if (warp == C::kWarpPV) {
-    constexpr uint32_t kIdescO = i8_idesc(C::kNPV, true, false);
+    constexpr uint32_t kIdescO = i8_idesc(C::kNPV, true, false) | C::kSignedA;
     const uint32_t v_lo = i8_desc_lo(sbase + C::kOffV, 16384u), p_lo = i8_desc_lo(sbase + C::kOffP, 16384u);
 #pragma unroll 1
     for (int gs = 0; gs < n_units; ++gs) {

@@ -1302,7 +1302,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
 
 // Launches one of the persistent attention kernels: SMEM bytes, THREADS per CTA, units of ST tokens, at least MIN of them
 // per CTA where a sequence has as many (and no more CTAs than SMs).
-// The integer kernels take two: their teams do them side by side (one layer of 4096 tokens, 4 / 16 columns, us replayed from
+// The integer kernels take two: their teams or softmax groups do them side by side (by teams, one layer of 4096 tokens, 4 / 16 columns, us replayed from
 // a graph: one unit per CTA 12.9 / 18.2, two 11.6 / 17.7, three 12.9 / 22.5, four 12.7 / 22.4; four by the CTA, whatever the
 // sequences, as before: 17.2 / 36.0 for one sequence of 85 tokens, a CTA to itself for each head 8.5 / 17.7).  The FP16
 // kernels take one (64 columns, 85 tokens: 18.5, four 90; two sequences of 189 tokens: 18.0, two 19.0, four 48).

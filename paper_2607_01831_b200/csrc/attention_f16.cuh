@@ -39,8 +39,9 @@
 // memory (integer digit planes: 224 columns per team at 32), while the expansions and the softmax of a unit are long
 // enough to overlap as pipeline stages with double-buffered S, K and V.
 //
-// What bounds it: instruction issue and the instruction caches.  A unit takes 6200 warp instructions at 32 columns and 7500 at
-// 64 (the expansions a third, most of the rest softmax), at 2.7 per cycle; heavy FMA pipe 44-47 %, ALU 41-43 %, tensor pipe 22-27 %.  With 64 columns the softmax groups are never idle, with 32 they wait a fifth of the time.  What mattered on
+// What bounds it: instruction issue and the instruction caches.  A unit takes 4800 warp instructions at 32 columns with integer
+// values (6200 with FP16 ones) and 7200 at 64, at 2.3 and 2.6 per cycle; heavy FMA pipe 34 and 46 %, ALU 35 and 39 %, tensor
+// pipe 25 and 27 %.  With 64 columns the softmax groups are never idle, with 32 (FP16) they wait a fifth of the time.  What mattered on
 // the way: no register spills in the softmax loop (little L1 is left beside 227 KB of shared memory: 400 bytes of spills
 // per thread cost a factor of two; hence scores in the 16-lane layout, where a thread sums 8 columns over 4 tokens instead
 // of 32 columns over one), rolled loops in the expansions and the producers (118 -> 98 us at 32 columns; unrolled copies of

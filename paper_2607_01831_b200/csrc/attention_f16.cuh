@@ -13,7 +13,7 @@
 // Centring costs one packed addition per two codes and is what keeps FP32 sufficient: the zero points, 128 steps below
 // the centre of a row, would otherwise be added and taken off again around results a hundred times smaller.
 // x = s log2(e) + log2(scale_v), w = 2^(x - ref[c]); ref[c] is set so that the largest weight of a column's first unit is
-// 2^8 (integers: 1, scaled to 2^25) and raised (accumulators drained or rescaled, rare) before a weight would leave FP16 or u32.  The
+// 2^8 (integers: 1, scaled to 2^26) and raised (accumulators drained or rescaled, rare) before a weight would leave FP16 or u32.  The
 // tensor core's FP32 accumulation truncates (0.46 ulp of the running sum per product).  Scores: the high part of a query is a
 // multiple of 2^-10 of the largest entry, so that its products with the codes sum up exactly, and the truncation acts on the low
 // part, a thousand times smaller.  Values: every kDrainUnits units the accumulators move into an FP32 copy; the integer sums are exact.
@@ -95,9 +95,18 @@ struct F16Cfg {
   // units has a largest error of 3.4e-6, per 4 units 2.2e-6, per 2 units 1.4e-6, by when it is below the integer kernel's in
   // every case (4 % of the time between 8 and 2 when it was measured); 64 columns: 3 % of the time for a drain per 16 units, 6 % per 8
   static constexpr int kDrainUnits = kIntPV ? 256 : NC == 64 ? 16 : 2;
-  // log2 of the largest weight of a column's first unit, and of a weight that raises the references.  On integers weights are formed
-  // relative to that and scaled by 2^25 afterwards (up to 2^31.5): an exponent of 25 would carry four times the rounding.
-  static constexpr float kTop = kIntPV ? 0.0f : 8.0f, kRaise = kIntPV ? 6.5f : 15.0f;
+  // log2 of the largest weight of a column's first unit, of a weight that raises the references, and of one whose column's is raised
+  // with it.  On integers weights are formed relative to that and scaled by kScale afterwards (up to 2^31.5): an exponent of 26 would
+  // carry four times the rounding.
+  // Integers as a weight of 2^-27 of the largest and less would vanish, and where one token outweighs the others they are what the rest
+  // of the context consists of.  So they are rounded up as often as their fraction says (see weight_offset), which leaves the sums
+  // without a bias.  Error against 64 bits, 1e-6 of the 2-norm, 32 columns, a token over the rest by 2^20 / 2^26.6 / 2^30: one
+  // sequence of 131072 tokens, weights as two FP16 terms 3.1 / 2.7 / 0.46, as integers to nearest at 2^25 1.1 / 58 / 6.6, as here 0.58 / 1.4 / 0.22;
+  // 16 of 65536 3.0 / 11.0 / 2.8, 3.6 / 500 / 58, 1.8 / 11.3 / 1.7 (11: of the 32-bit sums of the weights, in all three).  At 2^25 with
+  // fractions 1.06 / 1.5 / 0.29 and 3.4 / 11.4 / 1.9; at 2^27 the references are raised so often that log-normal values cost 5 % more.
+  // Raising with them only the columns that are 2 over theirs spares 1 % with outliers and 4 % where pieces are short.
+  static constexpr float kTop = kIntPV ? 0.0f : 8.0f, kRaise = kIntPV ? 5.5f : 15.0f, kRaiseToo = kIntPV ? 2.0f : 15.0f;
+  static constexpr float kScale = 0x1p26f;
   // who computes the per-token scalars: with 64 columns the K warps have the time (261 -> 256 us), with 32 they are the
   // slower stage and two spare warps do it (96.1 us, 97.4 us in the K warps)
   static constexpr bool kMetaK = kSplit;
@@ -216,6 +225,11 @@ __device__ __forceinline__ void f16_expand_v8(uint32_t raw, uint32_t tile, int w
 // Column of a group whose weights' bytes are word k of 16-byte chunk c of a row of the P tile (stmatrix deals a thread's columns
 // 8 j + 2 i and 8 j + 2 i + 1 to chunks j and 4 + j).
 __host__ __device__ constexpr int f16_col(int c, int k) { return 8 * (c & 3) + 2 * k + (c >> 2); }
+// What is added to a weight on its way to the nearest integer: -1/2 to 1/2, spread evenly over any run of tokens (the multiples of the
+// golden section, modulo one), so that of many like weights the share that their fraction says is rounded up.
+__device__ __forceinline__ float weight_offset(int tok) {
+  return __uint_as_float(0x3F800000u | ((uint32_t)tok * 2654435769u >> 9)) - 1.5f;
+}
 // The sum of a column from its four byte planes.
 __device__ __forceinline__ float f16_planes(const uint32_t* a) {
   return fmaf(fmaf(fmaf((float)(int)a[3], 256.0f, (float)(int)a[2]), 256.0f, (float)(int)a[1]), 256.0f, (float)(int)a[0]);
@@ -704,7 +718,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
               const float mx = fmaxf(fmaxf(red_s[r], red_s[CG + r]), fmaxf(red_s[2 * CG + r], red_s[3 * CG + r])) + old;
               float nw = old, f = 1.0f;
               if (fresh) { nw = fmaxf(mx, -1.0e4f) - C::kTop; f = 0.0f; }
-              else if (mx - old > (C::kIntPV ? C::kTop : C::kRaise)) { nw = mx - C::kTop; f = ex2_full(old - nw); }
+              else if (mx - old > C::kRaiseToo) { nw = mx - C::kTop; f = ex2_full(old - nw); }
               ref_s[r] = nw;
               fac_s[r] = f;
             }
@@ -728,6 +742,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
           for (int k = 0; k < 4; ++k) {
             const float ia = tok4[ms * 128 + 8 * k].w, ib = tok1[ms * 128 + 8 * k];
             const uint64_t ia2 = f2_pack(ia, ia), ib2 = f2_pack(ib, ib);
+            const float off = C::kIntPV ? weight_offset(unit_t0 + t0 + 8 * k) : 0.0f;
             uint32_t h[4], q[4];
 #pragma unroll
             for (int j = 0; j < NG; ++j) {
@@ -738,7 +753,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
               l2[j] = f2_fma(w2, ia2, l2[j]);
               zs2[j] = f2_fma(w2, ib2, zs2[j]);
               if constexpr (C::kIntPV) {   // even and odd columns
-                f2_unpack(f2_mul(w2, f2_pack(0x1p25f, 0x1p25f)), a, b);
+                f2_unpack(f2_fma(w2, f2_pack(C::kScale, C::kScale), f2_pack(off, off)), a, b);
                 asm("cvt.rni.u32.f32 %0, %1;" : "=r"(h[j]) : "f"(a));
                 asm("cvt.rni.u32.f32 %0, %1;" : "=r"(q[j]) : "f"(b));
                 continue;
@@ -821,7 +836,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
           const float f1 = ex2_full(m1 - M), f2 = ex2_full(m2 - M);
           const float l = lz_s[cc] * f1 + ogrp[320 + cc] * f2;
           const float z = lz_s[32 + cc] * f1 + ogrp[320 + 32 + cc] * f2;
-          const float o = ((have ? of_s[cc * 128] * f1 : 0.0f) + (have_o ? of_o[cc * 128] * f2 : 0.0f)) * 0x1p-25f;
+          const float o = ((have ? of_s[cc * 128] * f1 : 0.0f) + (have_o ? of_o[cc * 128] * f2 : 0.0f)) * (1.0f / C::kScale);
           put(cc, o + z, M, l);
         }
       } else {

@@ -568,22 +568,22 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
       };
       // (kIntPV) After a change of the references: the sums of the columns that it concerns, scaled where they are and taken apart into
       // byte planes again.  Rarely more than one column of 32, which is why the others are left alone: with a drain of all columns
-      // raises took a fifth of the time where outliers make them frequent.
-      auto rescale = [&]() {
+      // raises took a fifth of the time where outliers make them frequent.  (Known by one vote of the group's first warp, not from 32
+      // factors: with outliers one sequence of 131072 tokens 78.3 -> 77.5 us, 4 of 32768 84.1 -> 83.0, 16 of 2000 38.5 -> 37.9.)
+      auto rescale = [&](uint32_t raised) {
         tc_fence_after();
 #pragma unroll 1
         for (int c = 0; c < CG / 4; ++c) {
-          float f[4];
-          bool any = false;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) { f[k] = fac_s[f16_col(c, k)]; any |= f[k] != 1.0f; }
-          if (!any) continue;
+          const uint32_t cols = raised >> f16_col(c, 0);   // (its columns are 2 apart)
+          if (!(cols & 0x55u)) continue;
           uint32_t a[16];
           TmemRegs<16>::ld(tm_o + c * 16, a);
           tc_wait_ld();
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            float v = f16_planes(a + 4 * k) * f[k];
+            if (!(cols >> (2 * k) & 1u)) continue;
+            const float f = fac_s[f16_col(c, k)];
+            float v = f16_planes(a + 4 * k) * f;
             const int p3 = __float2int_rn(v * 0x1p-24f);
             v = fmaf((float)p3, -0x1p24f, v);
             const int p2 = __float2int_rn(v * 0x1p-16f);
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
             a[4 * k + 1] = (uint32_t)p1;
             a[4 * k + 2] = (uint32_t)p2;
             a[4 * k + 3] = (uint32_t)p3;
-            if (have_of) of_s[f16_col(c, k) * 128] *= f[k];
+            if (have_of) of_s[f16_col(c, k) * 128] *= f;
           }
           TmemRegs<16>::st(tm_o + c * 16, a);
         }
@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
           tc_fence_after();
           uint64_t y2[4][NG];
           bool scale = false;
+          uint32_t raised = 0;   // (kIntPV) the columns whose references changed
 #pragma unroll 1
           for (int pass = 0; pass < 2; ++pass) {   // (a second time, from tensor memory, after a change of the references)
           const uint32_t tm_s = tmem0 + C::kTmS + sl * C::kSCols + col0 + lane_sel;
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
           if (n_own > 0) mbar_wait_in(pvdone + g * 8, (n_own - 1) & 1, abort_word);   // P free, accumulators current
           // (behind the scores: the product that is waited for here has had their time to complete)
           if constexpr (C::kIntPV) {
-            if (scale) rescale();
+            if (scale) rescale(raised);
             if (units_in_acc >= C::kDrainUnits) drain(false);
           } else {
             if (scale || units_in_acc >= C::kDrainUnits) drain(scale);
@@ -705,8 +706,13 @@ __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(
               else if (mx - old > C::kRaiseToo) { nw = mx - C::kTop; f = ex2_full(old - nw); }
               ref_s[r] = nw;
               fac_s[r] = f;
+              if (C::kIntPV) {   // (the group's first warp)
+                const uint32_t columns = __ballot_sync(0xFFFFFFFFu, f != 1.0f);
+                if (r == 0) red_s[255] = __uint_as_float(columns);
+              }
             }
             named_bar(bar_g, 128);
+            if (C::kIntPV) raised = __float_as_uint(red_s[255]);
 #pragma unroll
             for (int j = 0; j < NG; ++j) {
               const uint64_t f2 = *reinterpret_cast<const uint64_t*>(fac_s + 8 * j + c2);

@@ -1139,10 +1139,14 @@ lynx_status launch_f16(AttnParams p, cudaStream_t st) {
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }
 
-// P.V on integers where a CTA has 24 units or more: they take less per unit, and 0.3 us more at the end of a piece and up to a
-// thousand instructions more whenever a reference is raised, which outliers do mostly in the first units.  us, FP16 / integers, 32
-// columns, log-normal and outlier values: 85 tokens 12.9 / 13.2, one sequence of 16384 (7 units per CTA) 23.1 / 22.3 and 24.3 / 25.2,
-// 4 of 7056 (12) 30.7 / 29.2 and 32.4 / 32.9, one of 131072 (55) 79.8 / 72.1 and 83.0 / 78.2, 4 of 32768 (55) 86.5 / 76.8 and 89.1 / 84.7.
+// P.V on integers where a table gives each CTA 24 units or more and has room for as many in a sequence: they take less per unit, 0.3 us
+// more at the end of a piece, and some 4000 cycles whenever a reference is raised, which outliers do mostly in a piece's first units.  us,
+// FP16 / integers, 32 columns, log-normal and outlier values: one sequence of 16384 (7 units per CTA) 24.0 / 23.1 and 25.2 / 26.1, 4 of 7056
+// (12) 31.2 / 28.6 and 32.3 / 32.7, 200 of 500 (42, in pieces of 4) 150.2 / 153.4 and 153.2 / 167.7, 24 of 4000 (41, in pieces of 32) 84.5 / 75.4 and
+// 85.7 / 80.8, one of 131072 (55) 80.0 / 72.3 and 82.5 / 77.5, 4 of 32768 (55) 87.2 / 77.9 and 90.0 / 83.0.  The host does not know the lengths: short
+// sequences in a wide table go there, too.  (Both variants in one kernel that decides by the lengths: the instruction caches, 72.1 -> 75.1 us for
+// one sequence of 131072, 16.0 -> 16.6 for one of 4096; each role's two codes side by side 73.5 and 18.1.)
 inline bool f16_int_pv(const AttnParams& p) {
-  return (long long)p.B * p.Hkv * p.max_blocks * p.bt >= 24ll * 128 * sm_count();
+  const long long tokens = (long long)p.max_blocks * p.bt;
+  return tokens >= 24 * 128 && tokens * p.B * p.Hkv >= 24ll * 128 * sm_count();
 }

@@ -283,11 +283,11 @@ __device__ __forceinline__ float warp_max(float x) {
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
   return r;
 }
-// The sums of N values per lane over a warp: lane i returns that of value i / (32 / N).  Half of the values change places at
-// every step, 2 N - 2 additions in all where N butterflies would take 5 N; each sum in the order of a butterfly.
-template <int N>
-__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
-  static_assert(N == 8 || N == 16 || N == 32, "lanes share the values evenly");
+// The sums (or whatever `op` is) of N values per lane over a warp: lane i returns that of value i / (32 / N).  Half of the values change
+// places at every step, 2 N - 2 additions in all where N butterflies would take 5 N; each sum in the order of a butterfly.
+template <int N, class Op>
+__device__ __forceinline__ float warp_halves(float (&v)[N], int lane, Op op) {
+  static_assert(N == 4 || N == 8 || N == 16 || N == 32, "lanes share the values evenly");
   int off = 16;
 #pragma unroll
   for (int m = N / 2; m >= 1; m >>= 1, off >>= 1)
@@ -295,11 +295,15 @@ __device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
     for (int i = 0; i < m; ++i) {
       const bool up = (lane & off) != 0;
       const float give = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, off);
+      v[i] = op(keep, __shfl_xor_sync(0xFFFFFFFFu, give, off));
     }
 #pragma unroll
-  for (; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], off);
+  for (; off >= 1; off >>= 1) v[0] = op(v[0], __shfl_xor_sync(0xFFFFFFFFu, v[0], off));
   return v[0];
+}
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+  return warp_halves(v, lane, [](float a, float b) { return a + b; });
 }
 __device__ __forceinline__ float ex2_full(float x) {   // no flush of small results
   float y;

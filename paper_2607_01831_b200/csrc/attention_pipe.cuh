@@ -300,12 +300,25 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
           if (gs >= SG * PB) mbar_wait_in(pvdone + ((gs - SG * PB) % NP) * 8, ((gs - SG * PB) / NP) & 1, abort_word);   // P free
           // ---- a piece's first unit, a weight that would leave the u32 range, sums about to overflow: new references ----
           if (bar_or(bar_g, 128, fresh || units_in_acc >= C::kDrainUnits || ymax > 3.5f)) {
+            // (At 8 and 16 columns by exchanging halves, as the sums: a maximum per column and instruction took 2 us of a piece at 16, now 0.9;
+            // 64 sequences of 16 tokens 27.2 -> 24.1 us, 16 ragged long ones 242 -> 241.  At 4 columns 1 % slower.)
+            if constexpr (CP > 4) {
+              float x[CP];   // (back to absolute exponents x = y + ref)
 #pragma unroll
-            for (int c = 0; c < CP; ++c) {   // (back to absolute exponents x = y + ref)
-              float a, b;
-              f2_unpack(y2[c >> 1], a, b);
-              const float mx = warp_max(((c & 1) ? b : a) + (fresh ? 0.0f : ref_s[c]));
-              if (lane == 0) red_s[w4 * CP + c] = mx;
+              for (int c = 0; c < CP / 2; ++c) {
+                f2_unpack(y2[c], x[2 * c], x[2 * c + 1]);
+                if (!fresh) { x[2 * c] += ref_s[2 * c]; x[2 * c + 1] += ref_s[2 * c + 1]; }
+              }
+              const float top = warp_halves(x, lane, [](float u, float v) { return fmaxf(u, v); });
+              if ((lane & (32 / CP - 1)) == 0) red_s[w4 * CP + lane / (32 / CP)] = top;
+            } else {
+#pragma unroll
+              for (int c = 0; c < CP; ++c) {
+                float a, b;
+                f2_unpack(y2[c >> 1], a, b);
+                const float top = warp_max(((c & 1) ? b : a) + (fresh ? 0.0f : ref_s[c]));
+                if (lane == 0) red_s[w4 * CP + c] = top;
+              }
             }
             named_bar(bar_g, 128);
             if (r < CP) {
@@ -394,31 +407,64 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
         float* part = p.ws_part + ((size_t)item.b * p.Hkv + item.hkv + (size_t)blockIdx.x) * (size_t)C::kPartCols * kPartStride;
         const float* grps = reinterpret_cast<const float*>(smem + C::kOffGrp);
         const float* mails = reinterpret_cast<const float*>(smem + C::kOffP) + r;
-        // (rolled: three columns at a time 231 -> 238 us for 16 ragged sequences at 16 columns, for the instruction caches)
-#pragma unroll 1
-        for (int c = g * H; c < min(g * H + H, p.ncols); ++c) {
+        const int c0 = g * H, nc = min(H, p.ncols - c0);
+        // what is the same for all 128 dims of column c: the groups' factors, its sums, its row
+        struct { float f[SG], z, l; uint32_t row; } t;
+        const auto look = [&](int c, bool leads) {
           float M = grps[c];
 #pragma unroll
           for (int i = 1; i < SG; ++i) M = fmaxf(M, grps[i * C::kGrpScal + c]);
-          float l = 0.0f, z = 0.0f, o = 0.0f;
+          t.l = t.z = 0.0f;
 #pragma unroll
           for (int i = 0; i < SG; ++i) {
             const float* gi = grps + i * C::kGrpScal + c;
-            const float f = ex2_full(gi[0] - M);
-            l = fmaf(gi[2 * CP], f, l);
-            z = fmaf(gi[3 * CP], f, z);
-            o = fmaf(mails[i * (PB * C::kPTile / 4) + c * 128], f, o);
+            t.f[i] = ex2_full(gi[0] - M);
+            t.l = fmaf(gi[2 * CP], t.f[i], t.l);
+            t.z = fmaf(gi[3 * CP], t.f[i], t.z);
           }
-          const float v = o + z;
+          t.row = 0;
           if (direct) {
             const int j = c / p.G, hh = c - j * p.G;
-            const size_t row = ((size_t)item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh;
-            p.out[row * LYNX_D + dim_out] = l > 0.0f ? v / l : 0.0f;
-            if (r == 0) p.ws_lse[row] = lse_of(M, l);
-          } else {
-            part[(size_t)c * kPartStride + dim_out] = v;
-            if (r == 0) *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(M, l);
+            t.row = (uint32_t)((item.b * p.nq_stride + j) * p.Hq + item.hkv * p.G + hh);
+            if (leads) p.ws_lse[t.row] = lse_of(M, t.l);
+          } else if (leads) {
+            *reinterpret_cast<float2*>(part + (size_t)c * kPartStride + 128) = make_float2(M, t.l);
           }
+        };
+        const auto put = [&](int c) {
+          float o = 0.0f;
+#pragma unroll
+          for (int i = 0; i < SG; ++i) o = fmaf(mails[i * (PB * C::kPTile / 4) + c * 128], t.f[i], o);
+          const float v = o + t.z;
+          if (direct) p.out[(size_t)t.row * LYNX_D + dim_out] = t.l > 0.0f ? v / t.l : 0.0f;
+          else part[(size_t)c * kPartStride + dim_out] = v;
+        };
+        if constexpr (H > 1) {
+          // By a thread per column: the instructions of a piece's end share the schedulers with 27 other warps, and every thread for itself
+          // took 2.1 us at 16 columns, of the 6.7 for a piece of one unit (64 sequences of 16 tokens 27.2 us, 31.5 by every thread).
+          static_assert(8 * H <= 8 * CP && SG <= 4, "room for the columns' scalars");
+          if (r < nc) {
+            look(c0 + r, true);
+#pragma unroll
+            for (int i = 0; i < SG; ++i) red_s[8 * r + i] = t.f[i];
+            *reinterpret_cast<float4*>(red_s + 8 * r + 4) = make_float4(t.z, t.l, __uint_as_float(t.row), 0.0f);
+          }
+          named_bar(bar_g, 128);
+          // (rolled: three columns at a time 231 -> 238 us for 16 ragged sequences at 16 columns, for the instruction caches)
+#pragma unroll 1
+          for (int i = 0; i < nc; ++i) {
+            const float4 f = *reinterpret_cast<const float4*>(red_s + 8 * i), zl = *reinterpret_cast<const float4*>(red_s + 8 * i + 4);
+            const float fs[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+            for (int k = 0; k < SG; ++k) t.f[k] = fs[k];
+            t.z = zl.x;
+            t.l = zl.y;
+            t.row = __float_as_uint(zl.z);
+            put(c0 + i);
+          }
+        } else if (nc > 0) {   // (a group's only column: not worth a barrier, 77.4 -> 74.6 us for 512 sequences of 16 tokens at 4 columns)
+          look(c0, r == 0);
+          put(c0);
         }
       }
       tc_fence_before();

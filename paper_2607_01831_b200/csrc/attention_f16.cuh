@@ -243,10 +243,10 @@ __device__ __forceinline__ float f16_planes(const uint32_t* a) {
 // sub-blocks per copy for V and the metadata (the 128-byte swizzle of K does not go with them), and always all eight sub-blocks of a
 // unit, whether or not the sequence has them.
 constexpr int kPublisher = 2;
-template <class C>
+template <class C, class MAPS>
 __device__ __forceinline__ void plane_producer(const AttnParams& p, const SkRange& rng, const SeqLens& sl, int pw, int lane, uint32_t sbase, uint32_t full0,
                                                uint32_t empty0, int stages, uint32_t qfull0, uint32_t qempty0, uint32_t* blk_s, Item* items,
-                                               volatile int* abort_word, const I8Maps* maps, int bar_done) {
+                                               volatile int* abort_word, const MAPS* maps, int bar_done) {
   constexpr int ST = C::kST;
   const int lg = pw < 2 ? 2 : 3;                 // log2 of the sub-blocks of a unit that are this warp's
   const int sub0 = pw == 1 ? 4 : 0;
@@ -420,7 +420,7 @@ struct F16Meta {
 
 template <int NC, bool INT>
 __global__ void __launch_bounds__(F16Cfg<NC, INT>::kThreads, 1) attn_f16_kernel(const AttnParams p,
-                                                                           const __grid_constant__ I8Maps maps) {
+                                                                           const __grid_constant__ PlaneMaps maps) {
   using C = F16Cfg<NC, INT>;
   constexpr bool SPLIT = C::kSplit;
   constexpr int CG = C::kCG, NG = C::kNG, STEP = SPLIT ? 1 : 2, kDW = 8;
@@ -1135,7 +1135,7 @@ lynx_status launch_f16(AttnParams p, cudaStream_t st) {
   using C = F16Cfg<NC, INT>;
   p.combine_single = 1;
   constexpr int kMin = 1;
-  const lynx_status rc = launch_units<true, C::kSmem, C::kThreads, C::kST, kMin, attn_f16_kernel<NC, INT>>(p, st);
+  const lynx_status rc = launch_units<true, PlaneMaps, C::kSmem, C::kThreads, C::kST, kMin, attn_f16_kernel<NC, INT>>(p, st);
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }
 

@@ -51,8 +51,12 @@
 // threads of a quarter-warp that read chunk i of their own rows (64 bytes apart) meet in no bank (see k_chunk).  V planes as
 // [rows / 16][1024 bytes] without swizzle, which gathers of four sub-blocks take, too.  (148 CTAs, nothing but copies, TB/s: rows of
 // 64 bytes 6.50 by four issuing warps, of 128 and more 6.75; one warp 3.06, two 6.0; gathers by one warp 4.3, by two 6.7.)
-struct alignas(64) I8Maps {
+struct alignas(64) PlaneMaps {
+  static constexpr bool kMeta = false;
   CUtensorMap m[4];   // K Anchor, V Anchor, K Residual, V Residual (the order of the stage's arrays)
+};
+struct alignas(64) PipeMaps : PlaneMaps {
+  static constexpr bool kMeta = true;
   CUtensorMap meta[2];   // (scale, zero) pairs of K, V: [rows / 16][32 floats], for gathers of four sub-blocks
 };
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -390,7 +394,7 @@ template <class C, bool FULL>
 __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lane, uint32_t ring_u32,
                                             uint32_t full0, uint32_t empty0, uint32_t qfull0, uint32_t qempty0,
                                             uint32_t qraw_u32, uint32_t* blk_s, Item* items, int* misc,
-                                            volatile int* abort_word, const I8Maps* maps) {
+                                            volatile int* abort_word, const PlaneMaps* maps) {
   constexpr int ST = C::kST, NSTAGE = C::kNStage, NARR = C::kNArr;
   const int n_cta = gridDim.x, cta = blockIdx.x;
   const SeqLens sl(p, lane);
@@ -659,7 +663,7 @@ __device__ __noinline__ bool seq_wait(const volatile int* ctr, int need, volatil
 
 template <bool FULL, int CP>
 __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(const AttnParams p,
-                                                                               const __grid_constant__ I8Maps maps) {
+                                                                               const __grid_constant__ PlaneMaps maps) {
   using C = I8Cfg<FULL, CP>;
   constexpr int NSTAGE = C::kNStage, T = C::kTeams, G = C::kGroups, CG = C::kCG, TT = C::kTeamThreads;
   extern __shared__ unsigned char smem_raw[];
@@ -1310,7 +1314,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
 // a graph: one unit per CTA 12.9 / 18.2, two 11.6 / 17.7, three 12.9 / 22.5, four 12.7 / 22.4; four by the CTA, whatever the
 // sequences, as before: 17.2 / 36.0 for one sequence of 85 tokens, a CTA to itself for each head 8.5 / 17.7).  The FP16
 // kernels take one (64 columns, 85 tokens: 18.5, four 90; two sequences of 189 tokens: 18.0, two 19.0, four 48).
-template <bool FULL, int SMEM, int THREADS, int ST, int MIN, auto KERN>
+template <bool FULL, class MAPS, int SMEM, int THREADS, int ST, int MIN, auto KERN>
 lynx_status launch_units(AttnParams p, cudaStream_t st) {
   static bool configured[64] = {false};
   int dev = 0;
@@ -1336,7 +1340,7 @@ lynx_status launch_units(AttnParams p, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  I8Maps maps;
+  MAPS maps;
   const uint64_t plane_rows = (uint64_t)p.num_blocks * p.Hkv * p.bt;
   if (!i8_plane_map(&maps.m[0], p.ka, plane_rows, true) || !i8_plane_map(&maps.m[1], p.va, plane_rows, false))
     return LYNX_ERR_CUDA;
@@ -1347,7 +1351,8 @@ lynx_status launch_units(AttnParams p, cudaStream_t st) {
     maps.m[2] = maps.m[0];
     maps.m[3] = maps.m[1];
   }
-  if (!meta_map(&maps.meta[0], p.km, plane_rows) || !meta_map(&maps.meta[1], p.vm, plane_rows)) return LYNX_ERR_CUDA;
+  if constexpr (MAPS::kMeta)
+    if (!meta_map(&maps.meta[0], p.km, plane_rows) || !meta_map(&maps.meta[1], p.vm, plane_rows)) return LYNX_ERR_CUDA;
   if (cudaLaunchKernelEx(&cfg, KERN, p, maps) != cudaSuccess) return LYNX_ERR_CUDA;
   return launch_status();
 }
@@ -1356,6 +1361,6 @@ template <bool FULL, int CP>
 lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
   using C = I8Cfg<FULL, CP>;
   constexpr int kMin = 2;
-  const lynx_status rc = launch_units<FULL, C::kSmem, C::kThreads, C::kST, kMin, attn_i8_kernel<FULL, CP>>(p, st);
+  const lynx_status rc = launch_units<FULL, PlaneMaps, C::kSmem, C::kThreads, C::kST, kMin, attn_i8_kernel<FULL, CP>>(p, st);
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }

@@ -85,7 +85,7 @@ template <> struct TmemCols<8> : TmemRegs<8> {};
 template <> struct TmemCols<16> : TmemRegs<16> {};
 
 template <bool FULL, int CP>
-__global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kernel(const AttnParams p, const __grid_constant__ I8Maps maps) {
+__global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kernel(const AttnParams p, const __grid_constant__ PipeMaps maps) {
   using C = PipeCfg<FULL, CP>;
   constexpr int SG = C::kSG, NB = C::kNB, NV = C::kNV, NP = C::kNP, PB = C::kPB;
   extern __shared__ unsigned char smem_raw[];
@@ -674,6 +674,6 @@ template <bool FULL, int CP>
 lynx_status launch_pipe(const AttnParams& p, cudaStream_t st) {
   using C = PipeCfg<FULL, CP>;
   constexpr int kMin = 2;
-  const lynx_status rc = launch_units<FULL, C::kSmem, C::kThreads, C::kST, kMin, attn_pipe_kernel<FULL, CP>>(p, st);
+  const lynx_status rc = launch_units<FULL, PipeMaps, C::kSmem, C::kThreads, C::kST, kMin, attn_pipe_kernel<FULL, CP>>(p, st);
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }

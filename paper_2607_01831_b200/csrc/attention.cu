@@ -716,7 +716,7 @@ lynx_status run_attention(bool full, const lynx_shape* shape, const void* q, int
       ps.out = p.out + (size_t)j0 * p.Hq * LYNX_D;
       ps.ws_lse = p.ws_lse + (size_t)j0 * p.Hq;
       const lynx_status rc = ps.ncols <= 4 ? launch_pipe<false, 4>(ps, st) : ps.ncols <= 8 ? launch_pipe<false, 8>(ps, st)
-                           : ps.ncols <= 16 ? launch_pipe<false, 16>(ps, st) : launch_i8<false, 32>(ps, st);
+                           : ps.ncols <= 16 ? launch_pipe<false, 16>(ps, st) : launch_i8(ps, st);
       if (rc != LYNX_OK) return rc;
     }
     return LYNX_OK;

@@ -1,31 +1,30 @@
 // Attention on the integer path of the fifth-generation tensor cores (tcgen05.mma kind::i8, accumulators in tensor memory), a team
 // of warps per unit.  Included by attention.cu inside its namespace: shares AttnParams and the stream-K cut of the work with the
-// other kernels.  Takes anchor calls with 17..32 columns, whose accumulators leave no tensor memory for the buffers of
-// attention_pipe.cuh; that kernel shares the algebra and the expansions here and takes up to 16 columns.  (What is measured below at
-// fewer columns was measured before it.)
+// other kernels.  The kernel here takes anchor calls with 17..32 columns, whose accumulators leave no tensor memory for the buffers of
+// attention_pipe.cuh; that one shares the algebra and the expansions and takes up to 16 columns.
 //
 // With one (scale, zero) per token row the two contractions of Section 2's attention run on the
 // integer levels themselves (see attention.cu).  Here both are exact integer tensor-core
 // products over a 128-token stage-unit:
-//   S^T[128 tokens x 3 CP]   = level(K)[128 x 128 dims] . Qd^T     A = K levels (u8, in tensor memory),
+//   S^T[128 tokens x 3 * 32] = level(K)[128 x 128 dims] . Qd^T     A = K levels (u8, in tensor memory),
 //                                                                   B = three balanced s8 digit planes
 //                                                                       of the fixed-point query
-//   O^T[128 dims x 4 CP]    += level(V)^T[128 x 128 tokens] . Wd    A = V tile (u8, MN-major),
+//   O^T[128 dims x 4 * 32]  += level(V)^T[128 x 128 tokens] . Wd    A = V tile (u8, MN-major),
 //                                                                   B = the four bytes of the u32
 //                                                                       fixed-point weights (MN-major)
-// CP = query columns (n_q * G) padded to 4, 8, 16 or 32 (anchor calls with more are run in slices).  The int32 accumulators are exact, so
-// there is no rounding in either product: the query is good to 2^-22 of its largest entry and a
-// weight to 2^-28 of the largest weight seen so far.
+// Query columns (n_q * G) are padded to 32 (anchor calls with more are run in slices).  The int32 accumulators are exact, so
+// there is no rounding in either product: the query is good to 2^-22 of its largest entry and a weight to 2^-28 of the largest
+// weight seen so far.
 //
 // Weights.  For token t and column c,  x = s * log2(e) + log2(scale_v(t))  and  W = 2^(x - ref[c])
 // rounded to a u32, with ref[c] chosen so that the largest W of the first unit is 2^28; a later x
 // that would push W beyond 2^31.5 raises ref[c] (rare), which ends the current accumulation: the
-// int32 accumulators are added, scaled, into an FP32 copy (also in tensor memory) and restart
+// int32 accumulators are added, scaled, into an FP32 copy (in registers) and restart
 // from zero.  The same happens before they could overflow.  The softmax sums use the unrounded
 // W / scale_v, so a single attended token reproduces its value row to FP32 rounding.
 //
 // Warp roles of a CTA (one CTA per SM):
-//   Teams of four warps (eight with 32 columns) each take every kTeams-th unit of the CTA's range
+//   Two teams of eight warps take the units of the CTA's range in turn
 //     and do everything for it, so that no hand-off between warps with different jobs lies on the
 //     path of a unit and the teams hide one another's latencies:
 //       K levels into tensor memory (a thread owns a token = a TMEM lane; Q.K^T takes its A
@@ -34,7 +33,8 @@
 //       V level tile into shared memory (128-byte-swizzled canonical layout, MN-major);
 //       scores -> weights: S read back (TMEM lane = token), per-token scale / zero point / causal
 //         limit applied, weights written to the team's P tile;
-//       P.V (one thread issues), accumulators and their FP32 copy in the team's tensor memory.
+//       P.V (one thread issues), accumulators in the team's tensor memory, their FP32 copy in registers.
+//     The two warpgroups of a team share the tokens of a unit, each scoring 16 columns, one expanding K, the other V.
 //     The team that owns a piece's first unit also writes the piece's query digit planes; at the
 //     end of a piece the teams' partial results are merged by the team that owns its last unit.
 //   Producer warps stream the raw planes into a shared-memory ring (cp.async.bulk).  The per-token
@@ -115,60 +115,33 @@ __device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap* map, ui
 
 constexpr int kI8PieceUnits = 32;  // stage-units whose block ids a producer warp looks up at a time
 
-template <bool FULL, int CP>
 struct I8Cfg {
-  static_assert(CP == 4 || CP == 8 || CP == 16 || CP == 32, "padded column counts");
   static constexpr int kST = 128;                   // tokens per stage-unit
-  static constexpr int kNArr = FULL ? 4 : 2;        // plane arrays copied per 16-token sub-block (the metadata is
-                                                    // read with plain loads: the copy engine takes ~35 cycles per copy)
-  static constexpr int kStageBytes = kST * (FULL ? 256 : 128);
-  static constexpr int kOffKA = 0, kOffVA = kST * 64, kOffKR = kST * 128, kOffVR = kST * 192;
-  // Anchor decode with 4 columns feeds the K planes to Q.K^T as they are: a token's 64 raw bytes
-  // b_m = a_2m + 16 a_2m+1 followed by the 64 masked bytes a_2m, against the query values Q_2m+1 and
-  // 16 Q_2m - Q_2m+1 (four digit planes instead of three: they fit the padding of N), which gives
-  // 16 sum_d Q_d a_d with a third of the logic operations of a full nibble expansion.
-  // (with more columns the fourth plane's share of the score arithmetic costs more registers than the
-  // expansion saves: 8 columns measured 20 % slower with it)
-  static constexpr bool kRawK = !FULL && CP == 4;
-  static constexpr bool kVoteFirst = FULL || CP > 4;   // restart question before the weights (see the unit loop)
-  static constexpr int kQPlanes = kRawK ? 4 : 3;
-  static constexpr int kNQK = (kQPlanes * CP + 15) / 16 * 16;   // N of the Q.K^T product
-  static constexpr int kNPV = 4 * CP;                    // N of the P.V product
-  static constexpr int kPartCols = CP < 8 ? 8 : CP;      // column stride of the partial slots
-  static constexpr int kColsPad = CP;
-  // warps: kTeams teams, then the producers.  A team is one warpgroup per column group: with 32 columns
-  // two warpgroups share the tokens of a unit, each scoring 16 columns (and one expanding K, the other V).
-  static constexpr int kGroups = CP == 32 ? 2 : 1;
-  static constexpr int kCG = CP / kGroups;               // columns of a column group
+  static constexpr int kCols = 32, kPartCols = kCols;    // query columns, column stride of the partial slots
+  static constexpr int kStageBytes = kST * 128;     // K Anchor, V Anchor (the metadata is read with plain loads: the copy engine takes ~35 cycles per copy)
+  static constexpr int kOffKA = 0, kOffVA = kST * 64;
+  static constexpr int kNQK = 3 * kCols;            // N of the Q.K^T product (three digit planes)
+  static constexpr int kNPV = 4 * kCols;            // N of the P.V product (four bytes of a weight)
+  // a team is two warpgroups that share the tokens of a unit, each scoring 16 columns (and one expanding K, the other V)
+  static constexpr int kGroups = 2, kCG = kCols / kGroups;
   static constexpr int kTeamWarps = 4 * kGroups, kTeamThreads = 32 * kTeamWarps;
-  // (4 and 8 columns: four teams.  Five teams have 80 registers a thread and spill: at 4 columns 11 % slower on one launch
-  // per layer and 3-12 % on short and ragged contexts; at 8 columns, 16 flattened layers of two sequences of 131072
-  // tokens, 1095 us with products issued behind a lane test and 1310 us by an elected lane, against 1055 us for four teams.
-  // Five teams behind a lane test and four by an elected lane, 8 columns, us: one sequence of 32768 tokens 28.4 and 24.6, of
-  // 131072 55.5 and 49.4; 4 of 32768 54.1 and 49.2; 16 of 16384 84.2 and 78.3; 16 ragged up to 65536 176 and 160.)
-  static constexpr int kTeams = CP == 32 ? 2 : (FULL || CP == 16) ? 3 : 4;
-  static constexpr int kProdWarps = CP == 32 ? 2 : 4;
-  static constexpr int kProdWarp0 = kTeamWarps * kTeams;
+  static constexpr int kTeams = 2, kProdWarps = 2, kProdWarp0 = kTeamWarps * kTeams;
   static constexpr int kThreads = (kProdWarp0 + kProdWarps) * 32;
   // shared memory map (offsets from a 1024-byte aligned base)
   static constexpr int kTile = 16384;                    // V level tile: [128 tokens][128 B]
-  static constexpr int kPRow = 4 * CP < 32 ? 32 : 4 * CP;   // bytes of a P tile row (one token)
-  static constexpr int kPTile = 128 * kPRow;
-  static constexpr int kPLayout = kPRow == 32 ? 6 : kPRow == 64 ? 4 : 2;   // descriptor swizzle mode of the P tile
-  static constexpr int kTeamBytes = kTile + kPTile;      // V tile, P tile (the K levels live in tensor memory)
-  static constexpr int kQTile = (kNQK * 128 + 1023) / 1024 * 1024;
-  static constexpr int kMail = CP * 128 * 4;             // end-of-piece deposit of a team: O in its V tile, (l, zs, ref) in its P tile
-  static_assert(kMail <= kTile, "the deposit lives in the team's V tile");
+  static constexpr int kPRow = 4 * kCols, kPTile = 128 * kPRow;   // P tile, a row of 128 bytes per token
+  static constexpr int kTeamBytes = kTile + kPTile;      // (the K levels live in tensor memory)
+  static constexpr int kQTile = kNQK * 128;
+  static_assert(kQTile % 1024 == 0 && kCols * 128 * 4 <= kTile, "the deposit of a team: O in its V tile, (l, zs, ref) in its P tile");
   static constexpr int kOffQT = kTeams * kTeamBytes;
   static constexpr int kOffRing = kOffQT + 2 * kQTile;
-  static constexpr int kTeamScal = (8 * CP + 4 * 2 * CP + 2 * CP) * 4;   // qs, ref, factor, limits, maxima; reduce scratch; totals
-  static constexpr int kFixedTail = 2 * CP * 256 + kTeams * kTeamScal +
-                                    8 * kI8PieceUnits * 4 + 2 * 32 + 64 * 8 + (1 + kTeams) * 256 + 64;
+  static constexpr int kTeamScal = (8 * kCols + 4 * 2 * kCols + 2 * kCols) * 4;   // qs, ref, factor, limits, maxima; reduce scratch; totals
+  static constexpr int kFixedTail = 2 * kCols * 256 + kTeams * kTeamScal + 8 * kI8PieceUnits * 4 + 2 * 32 + 64 * 8 + (1 + kTeams) * 256 + 64;
   static constexpr int kAvail = 227 * 1024 - 1024 - kOffRing - kFixedTail;
   static constexpr int kNStage = kAvail / kStageBytes > 8 ? 8 : kAvail / kStageBytes;
   static_assert(kNStage >= 2, "ring too small");
   static constexpr int kOffQRaw = kOffRing + kNStage * kStageBytes;
-  static constexpr int kOffScal = kOffQRaw + 2 * CP * 256;
+  static constexpr int kOffScal = kOffQRaw + 2 * kCols * 256;
   static constexpr int kOffBlk = kOffScal + kTeams * kTeamScal;
   static constexpr int kOffItems = kOffBlk + 8 * kI8PieceUnits * 4;
   static constexpr int kOffBars = kOffItems + 2 * 32;
@@ -176,14 +149,10 @@ struct I8Cfg {
   static constexpr int kSmem = kOffMisc + (1 + kTeams) * 256 + 64 + 1024;   // + alignment slack
   static_assert(kSmem <= 227 * 1024, "shared memory");
   static_assert(kOffScal % 16 == 0 && kTeamScal % 16 == 0 && kOffBars % 8 == 0, "alignment");
-  // tensor memory columns of a team: S, O accumulators, FP32 copy of O, K levels (128 bytes per token)
-  // (with 32 columns there is no room for the copy: it stays in registers)
-  static constexpr bool kOfInTmem = CP <= 16 && !(CP == 8 && !FULL);
-  static constexpr int kTmS = 0, kTmO = kNQK, kTmOF = kNQK + kNPV, kTmK = kOfInTmem ? (kTmOF + CP + 7) / 8 * 8 : kTmOF;
-  static constexpr int kTmTeam = CP == 32 ? 256 : CP == 16 ? 160 : (CP == 4 || !FULL) ? 96 : 128;
-  static constexpr int kTmCols = 512;
-  static_assert(kTmK + 32 <= kTmTeam && kTeams * kTmTeam <= 512, "tensor memory");
-  static constexpr int kDrainUnits = FULL ? 256 : 4096;  // own units after which the int32 sums could overflow
+  // tensor memory columns of a team: S, O accumulators, K levels (128 bytes per token); the FP32 copy of O stays in registers
+  static constexpr int kTmS = 0, kTmO = kNQK, kTmK = kNQK + kNPV, kTmTeam = 256, kTmCols = 512;
+  static_assert(kTmK + 32 <= kTmTeam && kTeams * kTmTeam <= kTmCols, "tensor memory");
+  static constexpr int kDrainUnits = 4096;  // own units after which the int32 sums could overflow (128 * 15 * 255 each)
 };
 
 template <>
@@ -388,14 +357,13 @@ __device__ __forceinline__ void i8_expand_k_tmem(uint32_t raw_a, uint32_t raw_r,
 
 // One of the producer warps: the stream-K bookkeeping (every warp derives the same range and
 // pieces; warp 0 alone publishes them, loads the queries and handles empty sequences) and, per
-// unit, its share of the plane copies: 8 sub-blocks of 16 tokens x kNArr arrays, two sub-blocks
-// per warp.
-template <class C, bool FULL>
+// unit, its share of the plane copies: 8 sub-blocks of 16 tokens x K and V, four sub-blocks per warp.
 __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lane, uint32_t ring_u32,
                                             uint32_t full0, uint32_t empty0, uint32_t qfull0, uint32_t qempty0,
                                             uint32_t qraw_u32, uint32_t* blk_s, Item* items, int* misc,
                                             volatile int* abort_word, const PlaneMaps* maps) {
-  constexpr int ST = C::kST, NSTAGE = C::kNStage, NARR = C::kNArr;
+  using C = I8Cfg;
+  constexpr int ST = C::kST, NSTAGE = C::kNStage, NARR = 2;   // (K, V)
   const int n_cta = gridDim.x, cta = blockIdx.x;
   const SeqLens sl(p, lane);
   const SkRange rng = sk_range<ST>(p, n_cta, cta, lane, sl, sk_place(p, cta));
@@ -405,18 +373,17 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   __syncthreads();  // (A) the range is published
   const int n_units = (int)(lo < hi ? hi - lo : 0);
   if (n_units == 0) {
-    if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl, nullptr);
+    if (pw == 0) per_sequence<false, C::kPartCols>(p, cta, n_cta, lane, sl, nullptr);
     return;
   }
 
-  constexpr int SPW = 8 / C::kProdWarps;       // 16-token sub-blocks per warp: 1, 2 or 4
+  constexpr int SPW = 8 / C::kProdWarps;       // 16-token sub-blocks per warp
   constexpr int RP = SPW * NARR;               // roles of this warp: (sub-block, array)
   const int role = pw * RP + (lane < RP ? lane : 0);
   const int sub = role / NARR, arr = role % NARR, sub_first = SPW * pw;
   const uint32_t my_bytes = 1024u;
-  const uint32_t my_dst = (uint32_t)(arr == 0 ? C::kOffKA : arr == 1 ? C::kOffVA : arr == 2 ? C::kOffKR : C::kOffVR) +
-                          (uint32_t)sub * my_bytes;
-  constexpr uint32_t kBytesSub = (FULL ? 4u : 2u) * 1024u;   // bytes of one sub-block
+  const uint32_t my_dst = (uint32_t)(arr == 0 ? C::kOffKA : C::kOffVA) + (uint32_t)sub * my_bytes;
+  constexpr uint32_t kBytesSub = 2u * 1024u;   // bytes of one sub-block
   uint32_t* my_blk = blk_s + pw * SPW * kI8PieceUnits;   // [SPW sub-blocks][kI8PieceUnits]
   int b = b_lo, len = sl.of(b), U = (len + ST - 1) / ST;
   int hkv = (int)sk_div(off_lo, U), u = (int)(off_lo - (long long)hkv * U);
@@ -438,9 +405,8 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         mbar_expect_tx(qfull0 + qi * 8, (uint32_t)(p.nq * p.G * LYNX_D * 2));
       }
       __syncwarp();
-      if (u == 0 && lane < kMaxQ && FULL) p.ws_dev[((size_t)b * p.Hkv + hkv) * kMaxQ + lane] = 0.0f;   // (see attn_combine_kernel)
       for (int j = lane; j < p.nq; j += 32)
-        bulk_g2s(qraw_u32 + (uint32_t)((qi * C::kColsPad + j * p.G) * LYNX_D * 2),
+        bulk_g2s(qraw_u32 + (uint32_t)((qi * C::kCols + j * p.G) * LYNX_D * 2),
                  p.q + (((size_t)b * p.nq_stride + j) * p.Hq + (size_t)hkv * p.G) * LYNX_D,
                  (uint32_t)(p.G * LYNX_D * 2), qfull0 + qi * 8);
     }
@@ -476,7 +442,7 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
         }
         __syncwarp();
         if (lane < RP && row != 0xFFFFFFFFu)
-          tma_box(ring_u32 + slot * C::kStageBytes + my_dst, &maps->m[arr], map_row(row, (arr & 1) == 0), bar);
+          tma_box(ring_u32 + slot * C::kStageBytes + my_dst, &maps->m[arr], map_row(row, arr == 0), bar);
       }
       __syncwarp();  // my_blk is rewritten by the next round
     }
@@ -498,15 +464,13 @@ __device__ __forceinline__ void i8_producer(const AttnParams& p, int pw, int lan
   }
   __syncwarp();
   bar_arrive(9, C::kThreads);
-  if (pw == 0) per_sequence<FULL, C::kPartCols>(p, cta, n_cta, lane, sl, items);
+  if (pw == 0) per_sequence<false, C::kPartCols>(p, cta, n_cta, lane, sl, items);
 }
 
-// Largest |q| of a piece's raw queries, by 128 threads (index i of 0..127), reduced over the
-// warp; the caller combines the warps.
-template <int CP>
+// Largest |q| of a piece's raw queries, by nthr threads (index i), reduced over the warp; the caller combines the warps.
 __device__ __forceinline__ float i8_q_absmax(const unsigned char* qraw, int i, int nthr) {
   float amax = 0.0f;
-  for (int k = i; k < CP * 16; k += nthr) {
+  for (int k = i; k < I8Cfg::kCols * 16; k += nthr) {
     const uint4 v = reinterpret_cast<const uint4*>(qraw)[k];
     const uint32_t ww[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -661,11 +625,9 @@ __device__ __noinline__ bool seq_wait(const volatile int* ctr, int need, volatil
   }
 }
 
-template <bool FULL, int CP>
-__global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(const AttnParams p,
-                                                                               const __grid_constant__ PlaneMaps maps) {
-  using C = I8Cfg<FULL, CP>;
-  constexpr int NSTAGE = C::kNStage, T = C::kTeams, G = C::kGroups, CG = C::kCG, TT = C::kTeamThreads;
+__global__ void __launch_bounds__(I8Cfg::kThreads, 1) attn_i8_kernel(const AttnParams p, const __grid_constant__ PlaneMaps maps) {
+  using C = I8Cfg;
+  constexpr int NSTAGE = C::kNStage, T = C::kTeams, G = C::kGroups, CP = C::kCols, CG = C::kCG, TT = C::kTeamThreads;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -717,7 +679,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (warp >= C::kProdWarp0) {
-    i8_producer<C, FULL>(p, warp - C::kProdWarp0, lane, ring_u32, full0, empty0, qfull0, qempty0,
+    i8_producer(p, warp - C::kProdWarp0, lane, ring_u32, full0, empty0, qfull0, qempty0,
                          sbase + C::kOffQRaw, blk_s, items, misc, abort_word, &maps);
     return;
   }
@@ -748,7 +710,6 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   const uint32_t lane_sel = (uint32_t)(w4 * 32) << 16;
   const uint32_t tm_s = tmem0 + tm * C::kTmTeam + C::kTmS + c0 + lane_sel;        // + plane * CP
   const uint32_t tm_o = tmem0 + tm * C::kTmTeam + C::kTmO + 4 * c0 + lane_sel;
-  const uint32_t tm_of = tmem0 + tm * C::kTmTeam + C::kTmOF + c0 + lane_sel;
   float* my_scal = reinterpret_cast<float*>(smem + C::kOffScal + tm * C::kTeamScal);
   float* qs_s = my_scal, *ref_s = my_scal + CP, *fac_s = my_scal + 2 * CP;
   int* lim_s = reinterpret_cast<int*>(my_scal + 3 * CP);
@@ -757,11 +718,10 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   float* my_red = my_scal + 8 * CP;               // [team warps][2 CG]
   float* my_lz = my_scal + 16 * CP;               // [2 CP]
   const int tw = grp * 4 + w4;                    // warp of the team
-  int* my_misc = misc + 64 * (1 + tm);
   Item* shared = reinterpret_cast<Item*>(misc + 64 + 16);   // [2] this CTA's first and last segment where others have part in it (zeroed)
   // named barriers of this team.  On bar_k and bar_p all but the issuing warp only arrive; each has an id of its own, so that
-  // between two arrivals of a warp there lies a barrier at which all warps synchronise (the restart question, or bar_p itself
-  // where they synchronise there): the phases stay apart even if the waits for products in between have given up.
+  // between two arrivals of a warp there lies a barrier at which all warps synchronise (the restart question): the phases stay apart
+  // even if the waits for products in between have given up.
   static_assert(T <= 4, "barrier ids: 1.. bar_tm, 5.. bar_p, 9 and 14 all teams, 10.. bar_k");
   const int bar_tm = 1 + tm, bar_p = 5 + tm, bar_k = 10 + tm;
   const uint32_t vtile = sbase + tm * C::kTeamBytes, ptile = vtile + C::kTile;
@@ -769,13 +729,12 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   const uint32_t tm_k = tmem0 + tm * C::kTmTeam + C::kTmK;
   const int dim_out = 32 * (r >> 5) + 8 * ((r >> 2) & 3) + 2 * (r & 3) + ((r >> 4) & 1);   // head dim of lane r of O
   // this thread's row of the P tile: 16-byte chunk j goes to position j ^ p_swz
-  const uint32_t p_swz = C::kPRow == 32 ? ((uint32_t)r >> 2) & 1u : C::kPRow == 64 ? ((uint32_t)r >> 1) & 3u : (uint32_t)r & 7u;
+  const uint32_t p_swz = (uint32_t)r & 7u;
   const uint32_t p_row = ptile + (uint32_t)r * C::kPRow;
   const float cb = p.sm_log2;
   // descriptor low words of the MMA operands (used by the team's issuing thread)
   const uint32_t qd_lo0 = i8_desc_lo(sbase + C::kOffQT, 16u), vd_lo = i8_desc_lo(vtile, 16384u), pd_lo = i8_desc_lo(ptile, 16384u);
-  constexpr uint32_t kQdHi = i8_desc_hi(1024u, 2u), kVdHi = i8_desc_hi(1024u, 2u),
-                     kPdHi = i8_desc_hi(8u * C::kPRow, (uint32_t)C::kPLayout);
+  constexpr uint32_t kQdHi = i8_desc_hi(1024u, 2u), kVdHi = i8_desc_hi(1024u, 2u), kPdHi = i8_desc_hi(8u * C::kPRow, 2u);
   uint32_t dep_cnt[T];                            // deposits made so far, per team (every team keeps the same count)
 #pragma unroll
   for (int i = 0; i < T; ++i) dep_cnt[i] = 0;
@@ -793,12 +752,12 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
     const int team_f = (gs_base + n_piece - 1) % T;       // team of the piece's last unit: it writes the piece's result
     if (u_first < n_piece) {
       const bool finisher = tm == team_f;
-      if (!FULL && finisher && tt == 0 && item.n_contrib > 1) shared[gs_base == 0 ? 0 : 1] = item;   // (see behind the loop)
+      if (finisher && tt == 0 && item.n_contrib > 1) shared[gs_base == 0 ? 0 : 1] = item;   // (see behind the loop)
       const int full_lim = p.causal ? len - p.tail + 1 : len;
       // ---- the piece's queries: fixed-point exponent, sum of q per column, causal limits ----------
       const unsigned char* qb = qraw + qi * CP * 256;
       {
-        const float am = i8_q_absmax<CP>(qb, tt, TT);
+        const float am = i8_q_absmax(qb, tt, TT);
         if (lane == 0) amax_s[tw] = am;
         for (int c = tw; c < CP; c += C::kTeamWarps) {
           const uint2 v = *reinterpret_cast<const uint2*>(qb + c * 256 + lane * 8);
@@ -815,17 +774,15 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
 #pragma unroll
       for (int i = 0; i < C::kTeamWarps; ++i) amax = fmaxf(amax, amax_s[i]);
       const int e = i8_q_exponent(amax);
-      const float ca = p.sm_log2 * __int_as_float((127 - e) << 23) * ((FULL || C::kRawK) ? 1.0f : 16.0f);
+      const float ca = p.sm_log2 * __int_as_float((127 - e) << 23) * 16.0f;
       const uint32_t qt = sbase + C::kOffQT + qi * C::kQTile;
       if (u_first == 0) {
         // this team owns the piece's first unit: it writes the three balanced s8 digit planes of
         // q_int = rint(q 2^e), rows plane * CP + column.  (The slot's previous planes belong to the piece
         // before last, which every team has left: the queries of this piece were loaded after that.)
-        // Eight entries per thread and step: the first product of a launch waits for this, and 32 by a quarter of the threads took
-        // longer than the first planes to arrive (one layer of 4096 tokens, from a graph: 4 columns 10.85 -> 9.91 us, 16 columns 17.2 ->
-        // 16.3 us, with the decision's ticket ahead of the output's stores).
+        // Eight entries per thread and step: the first product of a launch waits for this.
         const float up = __int_as_float((127 + e) << 23);
-        constexpr int NP = C::kQPlanes;
+        constexpr int NP = 3;
 #pragma unroll 1
         for (int it = tt; it < CP * 16; it += TT) {
           const int c = it >> 4, j = (it >> 2) & 3, w = it & 3;   // column, 32 dims of the row, 8 of them
@@ -843,13 +800,10 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
               const int qv = __float2int_rn(f * up);
               qv2[par] = max(-4194303, min(4194303, qv));
             }
-            // half 0 / 1 of the row: even / odd dims -- or, where K goes in as raw bytes, what multiplies the
-            // byte pair m (dims 2m, 2m+1; odd value) and its low nibble (16 x even value - odd value)
-            int val[2] = {qv2[0], qv2[1]};
-            if (C::kRawK) { val[0] = qv2[1]; val[1] = 16 * qv2[0] - qv2[1]; }
+            // half 0 / 1 of the row: even / odd dims
 #pragma unroll
             for (int par = 0; par < 2; ++par) {
-              int qv = val[par];
+              int qv = qv2[par];
 #pragma unroll
               for (int pln = 0; pln < NP; ++pln) {
                 const int dgt = (int)(signed char)(qv & 0xFF);
@@ -863,7 +817,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             const int n = pln * CP + c;
 #pragma unroll
             for (int par = 0; par < 2; ++par) {
-              const int chunk = C::kRawK ? 4 * par + j : 2 * j + par;   // 16 bytes of the row's 128
+              const int chunk = 2 * j + par;   // 16 bytes of the row's 128
               const uint32_t a = qt + (uint32_t)n * 128u + ((uint32_t)(chunk ^ (n & 7)) << 4) + 4u * w;
               asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(acc[pln][par]) : "memory");
             }
@@ -877,7 +831,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       }
 
       uint64_t l2[CG / 2], zs2[CG / 2];   // softmax sums, two columns per register pair
-      float of_r[C::kOfInTmem ? 1 : CG];   // FP32 copy of O where tensor memory has no room for it
+      float of_r[CG];                     // FP32 copy of O (tensor memory has no room for it)
 #pragma unroll
       for (int c = 0; c < CG / 2; ++c) { l2[c] = 0ull; zs2[c] = 0ull; }
       bool fresh = true, have_of = false;
@@ -887,47 +841,27 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       // Ends the current accumulation (the team's last P.V is complete): the int32 accumulators, four
       // byte planes per column, are added to the FP32 copy and the sum is scaled by fac_s[] (the change
       // of the reference exponents).
-      // (rolled where the copy is in tensor memory: this code lies in the unit loop, whose size the instruction caches feel)
-      constexpr int kDrainUnroll = C::kOfInTmem ? 1 : CG / 4;
       auto drain = [&](bool scale) {
         if (units_in_acc > 0) {
           tc_fence_after();
-#pragma unroll kDrainUnroll
+#pragma unroll
           for (int c4 = 0; c4 < CG / 4; ++c4) {
-            uint32_t a[16], of[4];
+            uint32_t a[16];
             TmemRegs<16>::ld(tm_o + c4 * 16, a);
-            if (C::kOfInTmem && have_of) TmemRegs<4>::ld(tm_of + c4 * 4, of);
             tc_wait_ld();
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
               const float v = fmaf(fmaf(fmaf((float)(int)a[4 * k + 3], 256.0f, (float)(int)a[4 * k + 2]), 256.0f,
                                         (float)(int)a[4 * k + 1]), 256.0f, (float)(int)a[4 * k]);
-              const float old = !have_of ? 0.0f : C::kOfInTmem ? __uint_as_float(of[k]) : of_r[C::kOfInTmem ? 0 : c4 * 4 + k];
-              const float nw = (old + v) * (scale ? fac_s[c0 + c4 * 4 + k] : 1.0f);
-              of[k] = __float_as_uint(nw);
-              if (!C::kOfInTmem) of_r[C::kOfInTmem ? 0 : c4 * 4 + k] = nw;
+              const float old = !have_of ? 0.0f : of_r[c4 * 4 + k];
+              of_r[c4 * 4 + k] = (old + v) * (scale ? fac_s[c0 + c4 * 4 + k] : 1.0f);
             }
-            if (C::kOfInTmem) TmemRegs<4>::st(tm_of + c4 * 4, of);
           }
-          if (C::kOfInTmem) tc_wait_st();
           have_of = true;
           units_in_acc = 0;
         } else if (have_of && scale) {
-#pragma unroll kDrainUnroll
-          for (int c4 = 0; c4 < CG / 4; ++c4) {
-            if (C::kOfInTmem) {
-              uint32_t of[4];
-              TmemRegs<4>::ld(tm_of + c4 * 4, of);
-              tc_wait_ld();
 #pragma unroll
-              for (int k = 0; k < 4; ++k) of[k] = __float_as_uint(__uint_as_float(of[k]) * fac_s[c0 + c4 * 4 + k]);
-              TmemRegs<4>::st(tm_of + c4 * 4, of);
-            } else {
-#pragma unroll
-              for (int k = 0; k < 4; ++k) of_r[C::kOfInTmem ? 0 : c4 * 4 + k] *= fac_s[c0 + c4 * 4 + k];
-            }
-          }
-          if (C::kOfInTmem) tc_wait_st();
+          for (int c = 0; c < CG; ++c) of_r[c] *= fac_s[c0 + c];
         }
       };
 
@@ -978,18 +912,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           ack_pending = false;
         }
         // ---- K levels (free: the team's previous Q.K^T has been waited for), then Q.K^T; V tile (free
-        // once the team's previous P.V is complete).  With two column groups one expands K, the other V.
-        if (G == 1 || grp == 0) {
-          i8_expand_k_tmem<FULL, C::kRawK>(st + C::kOffKA, st + C::kOffKR, r, tm_k + lane_sel);
+        // once the team's previous P.V is complete): one group expands K, the other V.
+        if (grp == 0) {
+          i8_expand_k_tmem<false, false>(st + C::kOffKA, 0u, r, tm_k + lane_sel);
           tc_wait_st();
         } else {
           if (n_own > 0) mbar_wait(pvdone0 + tm * 8, (n_own - 1) & 1, abort_word);
-          i8_expand<FULL>(st + C::kOffVA, st + C::kOffVR, vtile, w4, lane);
+          i8_expand<false>(st + C::kOffVA, 0u, vtile, w4, lane);
         }
         tc_fence_before();
         // (only the issuing warp waits for the others' K levels: they go on to the V tile.  An elected lane issues: the
-        // operands stay on the uniform datapath, see tc_elect.  Both together: one layer of 131072 tokens 42.4 -> 40.0 us
-        // at 4 columns, 16 ragged sequences at 16 columns 340 -> 335 us, 4096 tokens at 16 columns 29.0 -> 27.8 us.)
+        // operands stay on the uniform datapath, see tc_elect.)
         if (tw != 0) bar_arrive(bar_k, TT);
         else named_bar(bar_k, TT);
         if (tw == 0) {
@@ -1005,20 +938,17 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           }
         }
         __syncwarp();
-        if (G == 1 || grp == 0) {   // (the other group has waited already)
-          if (n_own > 0) mbar_wait(pvdone0 + tm * 8, (n_own - 1) & 1, abort_word);
-        }
-        if (G == 1) i8_expand<FULL>(st + C::kOffVA, st + C::kOffVR, vtile, w4, lane);
+        if (grp == 0 && n_own > 0) mbar_wait(pvdone0 + tm * 8, (n_own - 1) & 1, abort_word);   // (the other group has waited already)
         __syncwarp();
         if (lane == 0) mbar_arrive(empty0 + slot * 8);
         const bool valid = tok < len;
         if (!valid) { km = make_float2(0.f, 0.f); vm = make_float2(0.f, 0.f); }
-        const float sve = fmaxf(FULL ? vm.x : 16.0f * vm.x, 9.094947e-13f);   // floor 2^-40
+        const float sve = fmaxf(16.0f * vm.x, 9.094947e-13f);   // floor 2^-40
         const float al = km.x * ca;
-        const float be = (FULL ? km.y : fmaf(km.x, 8.0f, km.y)) * cb;
+        const float be = fmaf(km.x, 8.0f, km.y) * cb;
         const float lsv = lg2_approx(sve);
         const float ia = valid ? rcp_approx(sve) : 0.0f;
-        const float ib = (FULL ? vm.y : fmaf(vm.x, 8.0f, vm.y)) * ia;
+        const float ib = fmaf(vm.x, 8.0f, vm.y) * ia;
 
         // ---- scores of this thread's token -------------------------------------------------------
         mbar_wait(sfull0 + tm * 8, n_own & 1, abort_word);
@@ -1026,25 +956,19 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
         // y = log2 of the weight relative to the column's reference exponent, two columns per register pair
         uint64_t y2[CG / 2];
         {
-          uint32_t s0[CG], s1[CG], s2[CG], s3[C::kRawK ? CG : 1];
+          uint32_t s0[CG], s1[CG], s2[CG];
           TmemRegs<CG>::ld(tm_s, s0);
           TmemRegs<CG>::ld(tm_s + CP, s1);
           TmemRegs<CG>::ld(tm_s + 2 * CP, s2);
-          if (C::kRawK) TmemRegs<CG>::ld(tm_s + 3 * CP, s3);
           tc_wait_ld();
           const uint64_t al2 = f2_pack(al, al), be2 = f2_pack(be, be), lsv2 = f2_pack(lsv, lsv);
-          const uint64_t k256 = C::kRawK ? f2_pack(65536.0f, 65536.0f) : f2_pack(256.0f, 256.0f);
+          const uint64_t k256 = f2_pack(256.0f, 256.0f);
           const float* ref_r = fresh ? zero_s : ref_s;   // (a piece's first unit: relative to zero)
 #pragma unroll
           for (int c = 0; c < CG / 2; ++c) {
-            uint64_t hi, lo;   // the digit-plane sums put together: exact in int32 two planes at a time
-            if (C::kRawK) {
-              hi = f2_pack((float)((int)s3[2 * c] * 256 + (int)s2[2 * c]), (float)((int)s3[2 * c + 1] * 256 + (int)s2[2 * c + 1]));
-              lo = f2_pack((float)((int)s1[2 * c] * 256 + (int)s0[2 * c]), (float)((int)s1[2 * c + 1] * 256 + (int)s0[2 * c + 1]));
-            } else {
-              hi = f2_pack((float)((int)s2[2 * c] * 256 + (int)s1[2 * c]), (float)((int)s2[2 * c + 1] * 256 + (int)s1[2 * c + 1]));
-              lo = f2_pack((float)(int)s0[2 * c], (float)(int)s0[2 * c + 1]);
-            }
+            // the digit-plane sums put together: exact in int32 two planes at a time
+            const uint64_t hi = f2_pack((float)((int)s2[2 * c] * 256 + (int)s1[2 * c]), (float)((int)s2[2 * c + 1] * 256 + (int)s1[2 * c + 1]));
+            const uint64_t lo = f2_pack((float)(int)s0[2 * c], (float)(int)s0[2 * c + 1]);
             const uint64_t qs2 = *reinterpret_cast<const uint64_t*>(qs_s + c0 + 2 * c);
             const uint64_t rf2 = *reinterpret_cast<const uint64_t*>(ref_r + c0 + 2 * c);
             y2[c] = f2_fma(f2_fma(hi, k256, lo), al2, f2_fma(be2, qs2, f2_sub(lsv2, rf2)));
@@ -1068,17 +992,10 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           f2_unpack(y2[c], a, b);
           ymax = max3(ymax, a, b);
         }
-        // A restart of the accumulation (new reference exponents, the int32 sums drained into the FP32 copy)
-        // is a decision of the whole team: one P.V covers all columns.  Where it is known beforehand (first
-        // unit of a piece, sums about to overflow) it is taken first.  Otherwise every thread writes its
-        // weights at once and a thread whose weight would leave the u32 range raises a flag, which all
-        // look at after the barrier that completes the P tile anyway: the common case has no barrier of
-        // its own for the question.
+        // A restart of the accumulation (new reference exponents, the int32 sums drained into the FP32 copy) is a decision of the whole
+        // team: one P.V covers all columns.
         const bool forced = fresh || units_in_acc >= C::kDrainUnits;   // uniform over the team
         const bool over = ymax > 31.5f;
-        // (two flags in turn: a warp may be on its way into the next unit while another looks at this one's, if the waits in
-        // between have given up)
-        volatile int* raise_flag = my_misc + 2 + (n_own & 1);
         auto restart = [&]() {
 #pragma unroll
           for (int c = 0; c < CG; ++c) {   // (rare path: back to absolute exponents x = y + ref)
@@ -1088,7 +1005,6 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             if (lane == 0) my_red[tw * CG + c] = mx;
           }
           named_bar(bar_tm, TT);
-          if (tt == 0) *raise_flag = 0;
           if (tt < CP) {
             const float* mr = my_red + (tt / CG) * 4 * CG + (tt % CG);   // the four warps of the column's group
             const float mx = fmaxf(fmaxf(mr[0], mr[CG]), fmaxf(mr[2 * CG], mr[3 * CG]));
@@ -1113,8 +1029,9 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
           drain(true);   // (the team's previous P.V has been waited for)
           fresh = false;
         };
-        // weights of this thread's token into its row of the P tile; `commit`: add them to the softmax sums
-        auto weights = [&](bool commit) {
+        if (bar_or(bar_tm, TT, forced || over)) restart();
+        // ---- weights of this thread's token into its row of the P tile -------------------------------------
+        {
           uint32_t wi[CG];
           const uint64_t ia2 = f2_pack(ia, ia), ib2 = f2_pack(ib, ib);
 #pragma unroll
@@ -1124,11 +1041,9 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
             const float wa = ex2_ftz(a), wb = ex2_ftz(b);
             asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c]) : "f"(wa));
             asm("cvt.rni.u32.f32 %0, %1;" : "=r"(wi[2 * c + 1]) : "f"(wb));
-            if (commit) {   // (not for weights beyond the range: they may be infinite)
-              const uint64_t w2 = f2_pack(wa, wb);
-              l2[c] = f2_fma(w2, ia2, l2[c]);
-              zs2[c] = f2_fma(w2, ib2, zs2[c]);
-            }
+            const uint64_t w2 = f2_pack(wa, wb);
+            l2[c] = f2_fma(w2, ia2, l2[c]);
+            zs2[c] = f2_fma(w2, ib2, zs2[c]);
           }
 #pragma unroll
           for (int j = 0; j < CG / 4; ++j)
@@ -1137,27 +1052,9 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
                            "r"(wi[4 * j + 2]), "r"(wi[4 * j + 3]) : "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           tc_fence_before();
-          // the P tile and the V tile are complete, S has been read: the issuing warp waits for it, the others only where
-          // the restart flag is looked at afterwards
-          if (C::kVoteFirst && tw != 0) bar_arrive(bar_p, TT);
+          // the P tile and the V tile are complete, S has been read: the issuing warp waits for it
+          if (tw != 0) bar_arrive(bar_p, TT);
           else named_bar(bar_p, TT);
-        };
-        if (C::kVoteFirst) {   // (every instance but the 4-column anchor one measures faster with the question asked first)
-          if (bar_or(bar_tm, TT, forced || over)) restart();
-          weights(true);
-        } else {
-          if (!forced && over) *raise_flag = 1;
-          // (a thread beyond the range keeps its weights out of the sums: after the restart they are different ones.  A loop, so
-          // that the unit loop holds one copy of either step)
-          bool again = forced, commit = forced || !over;
-#pragma unroll 1
-          for (;;) {
-            if (again) restart();
-            weights(commit);
-            if (again || *raise_flag == 0) break;   // uniform: read after the barrier; cleared inside restart()
-            again = true;
-            commit = over;
-          }
         }
         if (tw == 0) {
           tc_fence_after();
@@ -1179,18 +1076,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
       drain(false);   // the FP32 copy now holds this team's part of O
       float of[CG];
 #pragma unroll
-      for (int c4 = 0; c4 < CG / 4; ++c4) {
-        if (C::kOfInTmem) {
-          uint32_t t[4];
-          TmemRegs<4>::ld(tm_of + c4 * 4, t);
-          tc_wait_ld();
-#pragma unroll
-          for (int k = 0; k < 4; ++k) of[c4 * 4 + k] = __uint_as_float(t[k]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) of[c4 * 4 + k] = of_r[C::kOfInTmem ? 0 : c4 * 4 + k];
-        }
-      }
+      for (int c = 0; c < CG; ++c) of[c] = of_r[c];
       tc_fence_before();
       // totals of l and zs over the 128 token lanes of every column group
       {
@@ -1295,7 +1181,7 @@ __global__ void __launch_bounds__(I8Cfg<FULL, CP>::kThreads, 1) attn_i8_kernel(c
   tc_fence_before();
   // (a thread sees what its own team has noted: whose slots are its own.  Here, not behind a piece, where it holds up the next: 12
   // ragged sequences of up to 9000 tokens, 8 columns, 36.5 -> 35.3 us)
-  const auto any_shared = [&]() { return !FULL && p.inline_merge && (shared[0].n_contrib > 1 || shared[1].n_contrib > 1); };
+  const auto any_shared = [&]() { return p.inline_merge && (shared[0].n_contrib > 1 || shared[1].n_contrib > 1); };
   if (any_shared()) __threadfence();
   named_bar(9, C::kThreads);   // (the producers have arrived there behind their last copy)
   if (any_shared()) i8_join_shared<C>(p, shared, tid, misc);
@@ -1357,10 +1243,9 @@ lynx_status launch_units(AttnParams p, cudaStream_t st) {
   return launch_status();
 }
 
-template <bool FULL, int CP>
-lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
-  using C = I8Cfg<FULL, CP>;
+inline lynx_status launch_i8(const AttnParams& p, cudaStream_t st) {
+  using C = I8Cfg;
   constexpr int kMin = 2;
-  const lynx_status rc = launch_units<FULL, PlaneMaps, C::kSmem, C::kThreads, C::kST, kMin, attn_i8_kernel<FULL, CP>>(p, st);
+  const lynx_status rc = launch_units<false, PlaneMaps, C::kSmem, C::kThreads, C::kST, kMin, attn_i8_kernel>(p, st);
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }

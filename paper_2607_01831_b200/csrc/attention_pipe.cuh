@@ -74,8 +74,8 @@ struct PipeCfg {
   static constexpr int kThreads = 32 * (kWarpQ + 2), kTeams = kSG, kTeamWarps = 4, kTeamThreads = 128;
   static constexpr int kDoneThreads = kSG * 128 + 128 + 64;   // softmax warpgroups, producers, products
   static constexpr int kDrainUnits = 256;   // a group's units after which the int32 sums could overflow (128 * 255 * 255 or 240 each)
-  // registers per thread after the split; launched with 80, 72 or 64 each: 256 * 128 + 512 * 56, 384 * 104 + 512 * 48, 512 * 80 + 512 * 48
-  static constexpr int kRegSoft = kSG == 2 ? 128 : kSG == 3 ? 104 : 80, kRegRest = kSG == 2 ? 56 : 48;
+  // registers per thread after the split; launched with 72 or 64 each: 384 * 104 + 512 * 48, 512 * 80 + 512 * 48
+  static constexpr int kRegSoft = kSG == 3 ? 104 : 80, kRegRest = 48;
 };
 
 template <int N>

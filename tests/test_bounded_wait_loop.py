@@ -59,7 +59,8 @@ def test_waiting_loop(tmp_path):
 def test_memory_is_given_back_behind_what_is_in_flight():
     """The warps that issue copies and products arrive at a barrier behind their last one; tensor memory is released, and with it
     the CTA can end, behind that barrier and the pause."""
-    for name, bar in (("attention_i8.cuh", r"named_bar\(9, C::kThreads\)"), ("attention_f16.cuh", r"named_bar\(5, C::kDoneThreads\)")):
+    for name, bar in (("attention_i8.cuh", r"named_bar\(9, C::kThreads\)"), ("attention_f16.cuh", r"named_bar\(5, C::kDoneThreads\)"),
+                      ("attention_pipe.cuh", r"named_bar\(9, C::kDoneThreads\)")):
         code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
         done, land, free = (re.search(x, code).start() for x in (bar, r"land_after_abort\(", r"tcgen05\.dealloc"))
         assert done < land < free
@@ -67,7 +68,7 @@ def test_memory_is_given_back_behind_what_is_in_flight():
 
 
 def test_every_wait_of_the_kernels_goes_through_it():
-    text = "".join(open(os.path.join(CSRC, n)).read() for n in ("attention.cu", "attention_i8.cuh", "attention_f16.cuh"))
+    text = "".join(open(os.path.join(CSRC, n)).read() for n in ("attention.cu", "attention_i8.cuh", "attention_f16.cuh", "attention_pipe.cuh"))
     loops = re.findall(r"mbar_try_wait\(bar, parity\)", text)
     assert len(loops) == 3                                          # mbar_wait's own, and one in each bounded wait
     assert len(re.findall(r"\bbounded_wait\(", text)) == 2

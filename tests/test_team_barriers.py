@@ -134,9 +134,9 @@ def _decisions(flag_of, warps=4, units=8, orders=400):
 
 
 def test_all_warps_take_the_restart_or_none_does():
-    text = _team_barriers()[1]
-    expr = re.search(r"raise_flag = my_misc \+ 2([^;]*);", text).group(1)
-    assert _decisions(lambda u: eval("0" + expr, {"n_own": u})) == 0
+    """The question is asked at a barrier that gives all threads one answer; a flag in memory would have to be one per unit."""
+    assert re.findall(r"([^\n]*)\brestart\(\);", _team_barriers()[1]) == ["        if (bar_or(bar_tm, TT, forced || over)) "]
+    assert _decisions(lambda u: u) == 0
 
 
 def test_one_flag_for_all_units_would_split_the_team():

@@ -73,7 +73,10 @@ struct PipeCfg {
   static_assert(kTmOF + kSG * CP <= 512, "tensor memory");
   static constexpr int kThreads = 32 * (kWarpQ + 2), kTeams = kSG, kTeamWarps = 4, kTeamThreads = 128;
   static constexpr int kDoneThreads = kSG * 128 + 128 + 64;   // softmax warpgroups, producers, products
-  static constexpr int kDrainUnits = 256;   // a group's units after which the int32 sums could overflow (128 * 255 * 255 or 240 each)
+  // A group's units between drains: a unit adds up to 128 * 128 * 255 to the sum of a byte plane of full codes, 128 * 240 * 255 of an
+  // Anchor's odd dims, so that 514 or 274 could pass int32.
+  static constexpr int kDrainUnits = 256;
+  static_assert(128ll * (FULL ? 128 : 240) * 255 * kDrainUnits < 1ll << 31, "no sum overflows");
   // registers per thread after the split; launched with 72 or 64 each: 384 * 104 + 512 * 48, 512 * 80 + 512 * 48
   static constexpr int kRegSoft = kSG == 3 ? 104 : 80, kRegRest = 48;
 };

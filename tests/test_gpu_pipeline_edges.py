@@ -137,7 +137,41 @@ def test_sums_are_drained_before_they_could_overflow():
                 sl = slice(h * G, h * G + G)
                 ref = torch.softmax(q[0, :, sl].double().reshape(-1, 128) @ kd.T / math.sqrt(128), 1) @ vd
                 got = o[0, :, sl].double().reshape(-1, 128)
-                # (a mean of 132096 values is 1 / 360 of one, and the integer kernels form it as the difference of two sums of the size of
-                # a zero point, here up to 5.5, with some four roundings: 4 * 2^-24 * 5.5 for every element)
-                bound = REL * ref.norm() + 4 * 2.0 ** -24 * 5.5 * ref.numel() ** 0.5
+                # (a mean of 132096 values is 1 / 360 of one.  Anchor levels count from the zero point: the mean is the difference of two
+                # sums of its size, here up to 5.5, with some four roundings.  Full codes count from the middle of their row, half a unit
+                # away from zero at most where rows are 128 normal values)
+                bound = REL * ref.norm() + 4 * 2.0 ** -24 * (0.5 if full else 5.5) * ref.numel() ** 0.5
                 assert (got - ref).norm() <= bound, (G, n_q, full, h, ((got - ref).norm() / bound).item())
+
+
+@pytest.mark.parametrize("full", [False, True])
+@pytest.mark.parametrize("G,n_q", [(1, 4), (1, 8), (1, 16), (2, 16)])
+def test_sums_that_would_overflow(G, n_q, full):
+    """A CTA for each head and 2120 units for each CTA: 530 for each of four softmax groups, 706 of three, 1060 of two.  Every unit has one
+    token whose weight is 2^-12 over the others', so that these are 255 in a byte plane, and values at the ends of their rows: without drains
+    a sum of full codes passes 2^31 at 514 units, of an Anchor's odd dims at 274 (kDrainUnits).  All units are the same two blocks, so that the
+    result is one unit's.  Bound: the sums of weights in 32 bits, at most half an ulp for each of a thread's additions and either sum; a sum
+    that wraps around is off by more than the result."""
+    heads, units, bt = 148, 2120, 64
+    v = torch.empty(2, heads, bt, 128)
+    v[..., :64], v[..., 64:] = 2.0, -1.0                  # codes 255 and 0, Anchor levels 15 and 0
+    k = torch.zeros(2, heads, bt, 128)
+    k[..., 1] = 1.0                                       # (a scale for every row)
+    k[0, :, 0, 0] = 1.0
+    q = torch.zeros(1, n_q, heads * G, 128)
+    q[..., 0] = 0.0015                                    # 0.0015 / sqrt(128) log2(e) = 1.9e-4
+    K, V = (lynx.split_quantize(x.to(torch.bfloat16).cuda()) for x in (k, v))
+    q = q.to(torch.bfloat16).cuda()
+    nb = units * 2
+    table = torch.arange(2, dtype=torch.int32, device="cuda").repeat(units).view(1, nb)
+    geo = lynx.Geometry(heads * G, heads, bt, 2, nb)
+    ws = lynx.make_workspace(geo, 1, n_q, "cuda")
+    call = lynx.merge_verify_attention if full else lynx.anchor_attention
+    o = call(geo, q, K, V, table, torch.tensor([units * 128], dtype=torch.int32, device="cuda"), ws, causal=False)
+    o = (o[0] if full else o)[0].double()
+    lynx.check(ws)
+    kd, vd = (_values(p, full).permute(1, 0, 2, 3).reshape(heads, 128, 128) for p in (K, V))
+    s = q[0].double().permute(1, 0, 2).reshape(heads, G * n_q, 128) @ kd.transpose(1, 2) / math.sqrt(128)
+    ref = (torch.softmax(s, 2) @ vd).reshape(heads * G, n_q, 128).permute(1, 0, 2)
+    adds = units // 2 * 4                                 # (two groups, four tokens of a unit to a thread)
+    assert (o - ref).abs().max() <= 2 * adds * 2.0 ** -24 * ref.abs().max(), (o - ref).abs().max().item()

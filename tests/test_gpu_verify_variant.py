@@ -36,7 +36,8 @@ def _kernels(call):
     return names
 
 
-@pytest.mark.parametrize("B,H,blocks,ints", [(200, 8, 32, False), (1200, 2, 191, False), (1200, 2, 192, True), (1, 4, 8192, True), (1, 4, 7103, False), (1, 4, 7104, True)])
+@pytest.mark.parametrize("B,H,blocks,ints", [(200, 8, 32, False), (1200, 2, 191, False), (1200, 2, 192, True), (1, 4, 7103, False), (1, 4, 7104, True),
+                                            (1, 4, 113600 // 16, False), (1, 4, 131072 // 16, True)])   # (tables of test_gpu_verify_wide_precision.py)
 def test_variant(B, H, blocks, ints):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     if sms != 148:

@@ -1,10 +1,12 @@
 """The hand-offs of attn_pipe_kernel, played through on the host: every stage's waits and arrivals in the order of the kernel, over
-random pieces and random orders of the warps' steps.  No warp may be left waiting, no buffer may be written before its readers have
-left it, and no barrier may be two phases ahead of somebody who waits for it (a wait knows the parity of a phase only).  Barrier ids
+random pieces, restarts and orders of the warps' steps.  No warp may be left waiting, no buffer may be written before its readers have
+left it -- the accumulators while a product adds to them or a group reads them, the P tiles that carry a group's sums at the end of a
+piece, among them --, and no barrier may be two phases ahead of somebody who waits for it (a wait knows the parity of a phase only).  Barrier ids
 and the order in which a CTA gives its memory back are read from the source."""
 import os
 import random
 import re
+import subprocess
 
 import pytest
 
@@ -44,6 +46,8 @@ def _play(pieces, SG, NB, NV, PB, NT, ring_k, ring_v, rng):
     kready, sfull, sfree = B(NB, 4), B(NB, 1), B(NB, 4)
     vready, pready, pvdone = B(NV, 4), B(SG * PB, 4), B(NP, 1)
     users = {}                      # buffer -> unit that is in it, and how many may still read it
+    restart = [rng.random() < 0.3 for _ in range(n)]      # a unit that raises its group's references
+    adding, reading, mail = [False] * SG, [0] * SG, [False] * SG   # a P.V, warps that read the sums, sums in the group's P tiles
 
     def put(buf, unit, readers, writers=1):
         old = users.get(buf)
@@ -113,7 +117,10 @@ def _play(pieces, SG, NB, NV, PB, NT, ring_k, ring_v, rng):
             gb = gs % SG * PB + gs // SG % PB
             yield from _wait(vready[gs % NV], gs // NV)
             yield from _wait(pready[gb], gs // (SG * PB))
+            assert reading[gs % SG] == 0, "a product into sums that are being read"
+            adding[gs % SG] = True
             yield
+            adding[gs % SG] = False
             get(("vtile", gs % NV), gs)
             get(("p", gb), gs)
             pvdone[gs % NP].arrive()
@@ -132,6 +139,13 @@ def _play(pieces, SG, NB, NV, PB, NT, ring_k, ring_v, rng):
         meet[key] = meet.get(key, 0) + 1
         while meet[key] < count:
             yield
+
+    def read_sums(g):
+        assert not adding[g], "sums read under a product"
+        reading[g] += 1
+        yield
+        assert not adding[g]
+        reading[g] -= 1
 
     def softmax(g, w):
         base = 0
@@ -153,13 +167,24 @@ def _play(pieces, SG, NB, NV, PB, NT, ring_k, ring_v, rng):
                 if gs >= SG * PB:
                     yield from _wait(pvdone[(gs - SG * PB) % NP], (gs - SG * PB) // NP)
                 yield from together(("vote", gs), 4)
+                if restart[gs] and gs - SG >= base:           # (not a piece's first unit: nothing to drain)
+                    if PB > 1:
+                        yield from _wait(pvdone[(gs - SG) % NP], (gs - SG) // NP)
+                    yield from read_sums(g)
+                assert not mail[g], "weights over sums that have not been read"
                 put(("p", gb), gs, 1)
                 yield
                 pready[gb].arrive()
             if last is not None:
                 yield from _wait(pvdone[last % NP], last // NP)
+                yield from read_sums(g)
+            tiles = [users.get(("p", g * PB + i)) for i in range(PB)]
+            assert all(t is None or t[1] == 0 for t in tiles), "sums over weights that have not been read"
+            mail[g] = True
             yield from together(("mail", ic), 4 * SG)
+            assert all(mail), "sums of every group"
             yield from together(("left", ic), 4 * SG)
+            mail[g] = False
             get(("item", ic % 2), ic)
             qempty[ic % 2].arrive()
             base += m
@@ -184,8 +209,9 @@ def _play(pieces, SG, NB, NV, PB, NT, ring_k, ring_v, rng):
         assert idle < 2000, "warps wait for one another"
 
 
-# softmax groups, scores, V tiles, P tiles of a group, metadata, rings: as PipeCfg has them at 16 columns (full codes, Anchor) and below
-CONFIGS = [(3, 3, 3, 2, 6, 3, 3), (3, 3, 3, 2, 8, 6, 6), (4, 4, 3, 1, 8, 3, 4), (4, 4, 3, 1, 8, 7, 8)]
+# softmax groups, scores, V tiles, P tiles of a group, metadata, rings: PipeCfg's at full codes with 16 columns, Anchor with 16, full and
+# Anchor below
+CONFIGS = [(3, 3, 3, 2, 6, 3, 3), (3, 3, 3, 2, 8, 5, 6), (4, 4, 3, 1, 8, 4, 4), (4, 4, 3, 1, 8, 8, 8)]
 
 
 @pytest.mark.parametrize("cfg", CONFIGS)
@@ -196,10 +222,21 @@ def test_no_warp_waits_for_ever_and_no_buffer_is_taken_early(cfg):
         _play(pieces, *cfg, rng)
 
 
-def test_the_games_configurations_are_the_kernels():
-    code = _code()
-    assert "kSG = CP == 16 ? 3 : 4" in code and "kNB = CP == 16 ? 3 : 4, kNV = 3, kPB = CP == 16 ? 2 : 1, kNP = 4 * kPB" in code
-    assert "kNT = FULL && CP == 16 ? 6 : 8" in code
+def test_the_games_configurations_are_the_kernels(tmp_path):
+    """PipeCfg as it stands in the source, compiled for the host: every pair of full codes or not and columns."""
+    text = open(os.path.join(CSRC, "attention_pipe.cuh")).read()
+    cfg = re.search(r"template <bool FULL, int CP>\nstruct PipeCfg \{.*?\n\};\n", text, re.S).group(0)
+    units = re.search(r"constexpr int kI8PieceUnits = \d+;", open(os.path.join(CSRC, "attention_i8.cuh")).read()).group(0)
+    show = "".join(f"show<PipeCfg<{f}, {cp}>>();" for f in ("true", "false") for cp in (4, 8, 16))
+    src, exe = tmp_path / "c.cpp", tmp_path / "c"
+    src.write_text("#include <cstdint>\n#include <cstdio>\n" + units + "\n" + cfg + """
+template <class C> void show() {
+  std::printf("%d %d %d %d %d %d %d %d\\n", C::kSG, C::kNB, C::kNV, C::kPB, C::kNT, C::kRingK, C::kRingV, C::kNP);
+}
+int main() {""" + show + "}")
+    subprocess.run(["g++", "-std=c++17", "-x", "c++", str(src), "-o", str(exe)], check=True)
+    lines = [tuple(map(int, x.split())) for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines()]
+    assert len(lines) == 6 and {x[:7] for x in lines} == set(CONFIGS) and all(x[7] == 4 * x[3] for x in lines)
 
 
 def test_memory_is_given_back_behind_what_is_in_flight():

@@ -143,8 +143,9 @@ lynx_status lynx_anchor_attention(const lynx_shape* shape, const void* q_bf16, i
  * 17..64 columns (up to 16 positions) are one launch of a kernel whose weights are two FP16 terms each
  * (22 bits), summed in FP32, or up to 32 columns on long contexts integers (steps of 2^-26 of the largest, rounded
  * without a bias), summed exactly; a longer window runs as slices of whole positions (a pass over the planes each).
- * Which of the two follows from the table's size (max_blocks_per_seq of 3072 tokens and more, and 3072 per SM in all), so
- * that results may differ in their rounding between tables of different widths.  With several launches first_reject is taken over the whole window from the deviations.
+ * Which of the two follows from the table's size (max_blocks_per_seq of more than 512 tokens, and 3072 per SM in all), so
+ * that results may differ in their rounding between tables of different widths.  With several launches first_reject is
+ * taken over the whole window from the deviations.
  * Value rows of any finite scale are handled with up to 32 columns.  With 33..64 columns per launch a value
  * row whose scale reaches 16 (a range of 4080 or more) is recorded in the status word and lynx_check
  * returns LYNX_ERR_RANGE: that is the range this width is specified and tested for. */

@@ -1139,14 +1139,14 @@ lynx_status launch_f16(AttnParams p, cudaStream_t st) {
   return rc != LYNX_OK ? rc : launch_combine(p, C::kPartCols, C::kST, kMin, st);
 }
 
-// P.V on integers where a table gives each CTA 24 units or more and has room for as many in a sequence: they take less per unit, 0.3 us
-// more at the end of a piece, and some 4000 cycles whenever a reference is raised, which outliers do mostly in a piece's first units.  us,
-// FP16 / integers, 32 columns, log-normal and outlier values: one sequence of 16384 (7 units per CTA) 24.0 / 23.1 and 25.2 / 26.1, 4 of 7056
-// (12) 31.2 / 28.6 and 32.3 / 32.7, 200 of 500 (42, in pieces of 4) 150.2 / 153.4 and 153.2 / 167.7, 24 of 4000 (41, in pieces of 32) 84.5 / 75.4 and
-// 85.7 / 80.8, one of 131072 (55) 80.0 / 72.3 and 82.5 / 77.5, 4 of 32768 (55) 87.2 / 77.9 and 90.0 / 83.0.  The host does not know the lengths: short
-// sequences in a wide table go there, too.  (Both variants in one kernel that decides by the lengths: the instruction caches, 72.1 -> 75.1 us for
-// one sequence of 131072, 16.0 -> 16.6 for one of 4096; each role's two codes side by side 73.5 and 18.1.)
+// P.V on integers where a table gives each CTA 24 units or more and has room for five in a sequence: they take less per unit, 0.3 us more
+// at the end of a piece, and some 4000 cycles whenever a reference is raised, which outliers do mostly in a piece's first units.  us, FP16 /
+// integers, 32 columns, log-normal and outlier values: one sequence of 16384 (7 units per CTA) 24.0 / 23.1 and 25.2 / 26.1, 4 of 7056 (12) 31.2 /
+// 28.6 and 32.3 / 32.7; 24 units and more: 200 of 500 (pieces of 4) 148.7 / 153.2 and 153.1 / 166.6, 160 of 600 (5) 156 / 145 and 158 / 155, 100 of
+// 1000 130.5 / 117.0 and 130.5 / 125.2, 24 of 4000 84.5 / 75.4 and 85.7 / 80.8, one of 131072 80.0 / 72.3 and 82.5 / 77.5.  The host does not know the
+// lengths: short sequences in a wide table go there, too.  (Both variants in one kernel that decides by the lengths: the instruction caches,
+// 72.1 -> 75.1 us for one sequence of 131072, 16.0 -> 16.6 for one of 4096; each role's two codes side by side 73.5 and 18.1.)
 inline bool f16_int_pv(const AttnParams& p) {
   const long long tokens = (long long)p.max_blocks * p.bt;
-  return tokens >= 24 * 128 && tokens * p.B * p.Hkv >= 24ll * 128 * sm_count();
+  return tokens > 4 * 128 && tokens * p.B * p.Hkv >= 24ll * 128 * sm_count();
 }

@@ -1,5 +1,5 @@
 """Verification with 17..32 columns goes through integer products for the values where a table gives CTAs 24 units of 128 tokens and
-has room for as many in a sequence: many short sequences in a table of their own width do not (they would lose by it), few long ones do.
+has room for five in a sequence: many short sequences in a table of their own width do not (they would lose by it), few long ones do.
 By the names of the kernels of a captured call."""
 import ctypes
 
@@ -36,7 +36,7 @@ def _kernels(call):
     return names
 
 
-@pytest.mark.parametrize("B,H,blocks,ints", [(200, 8, 32, False), (1200, 2, 191, False), (1200, 2, 192, True), (1, 4, 7103, False), (1, 4, 7104, True),
+@pytest.mark.parametrize("B,H,blocks,ints", [(200, 8, 32, False), (1200, 2, 32, False), (1200, 2, 33, True), (1, 4, 7103, False), (1, 4, 7104, True),
                                             (1, 4, 113600 // 16, False), (1, 4, 131072 // 16, True)])   # (tables of test_gpu_verify_wide_precision.py)
 def test_variant(B, H, blocks, ints):
     sms = torch.cuda.get_device_properties(0).multi_processor_count

@@ -303,9 +303,10 @@ __global__ void __launch_bounds__(PipeCfg<FULL, CP>::kThreads, 1) attn_pipe_kern
           if (gs >= SG * PB) mbar_wait_in(pvdone + ((gs - SG * PB) % NP) * 8, ((gs - SG * PB) / NP) & 1, abort_word);   // P free
           // ---- a piece's first unit, a weight that would leave the u32 range, sums about to overflow: new references ----
           if (bar_or(bar_g, 128, fresh || units_in_acc >= C::kDrainUnits || ymax > 3.5f)) {
-            // (At 8 and 16 columns by exchanging halves, as the sums: a maximum per column and instruction took 2 us of a piece at 16, now 0.9;
-            // 64 sequences of 16 tokens 27.2 -> 24.1 us, 16 ragged long ones 242 -> 241.  At 4 columns 1 % slower.)
-            if constexpr (CP > 4) {
+            // (By exchanging halves, as the sums: a maximum per column and instruction took 2 us of a piece at 16 columns, now 0.9; 64
+            // sequences of 16 tokens 27.2 -> 24.1 us, 16 ragged long ones 242 -> 241; verification at 8 columns 23.6 -> 22.7.  At 4 columns 1 %
+            // slower, Anchor at 8 0.5 % on long contexts.)
+            if constexpr (CP == 16 || (FULL && CP == 8)) {
               float x[CP];   // (back to absolute exponents x = y + ref)
 #pragma unroll
               for (int c = 0; c < CP / 2; ++c) {

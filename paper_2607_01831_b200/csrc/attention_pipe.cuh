@@ -13,7 +13,7 @@
 // a unit takes is the longest stage, 600 to 1000 cycles.  us, teams -> stages: 16 layers of two sequences of 131072 tokens, 8
 // columns, 912 -> 790 (before the power cap sets in; among other passes 1026 -> 963), one layer of 131072 tokens, 4 columns, 37.1 ->
 // 35.0, of 4096 10.5 -> 9.4; 16 ragged sequences, 16 columns, 276 -> 243 (303 -> 283), 4 columns with a BF16 tail 166 -> 153; two
-// sequences of 16000, 8 columns, 22.2 -> 19.4; verification of one layer of 4096 tokens, 16 columns, 16.8 -> 16.5.
+// sequences of 16000, 8 columns, 22.2 -> 19.4; verification of one layer of 4096 tokens, 16 columns, 16.8 -> 14.4.
 //
 // Exponents are relative to the column's largest weight and the weights scaled by 2^28 afterwards: an exponent of 28 would carry
 // four times the rounding of one below 8.
